@@ -445,95 +445,136 @@ mask_positions_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
     }
 }
 
-struct MaskPosGroup {                   // the keys of four nodes l, up to 128 each: lane x holds keys x, x+32, x+64, x+96
-    int32_t ps[4][4];
-    float v[4][4];
-    int32_t len[4], beg[4], pbeg[4];
+// Bound by the load/store unit: per 32 multiply-adds two accesses of the accumulators (about three bank conflicts each) and
+// the position and value loads.  So every row makes one pass over its nodes: a warp's accumulators are as long as the block's
+// key list, and the CTA runs as many of its warps as then fit its shared memory (a list beyond an eighth of it is
+// taken in segments).  Rows are handed to the warps by a counter.  N = 32768 cloud, 297 M multiply-adds: 853 -> 660 us
+// (fixed segments of 4096 keys made two passes of half the rows; four shuffles per node were 14 % of the unit's work).
+constexpr int MVP_WARPS = 16;
+constexpr int MVP_MIN_WARPS = 8;
+constexpr int MVP_ROOM = 212 * 256;      // accumulators (fp32) of a CTA at most: what an SM's shared memory holds
+
+struct MaskPosGroup {                   // the keys of two nodes l, up to 128 each: lane x holds keys x, x+32, x+64, x+96
+    int32_t ps[2][4];
+    float v[2][4];
 };
 
-__global__ void __launch_bounds__(MASK_WARPS * 32)
-mask_values_pos_kernel(int32_t N, const int32_t* __restrict__ phi_rowptr, const int32_t* __restrict__ phi_col,
-                       const float* __restrict__ phi_val, const int32_t* __restrict__ phi_pos,
-                       const int32_t* __restrict__ t_rowptr, const float* __restrict__ t_val,
-                       const unsigned short* __restrict__ pos16, const int32_t* __restrict__ mk_off,
-                       const int32_t* __restrict__ mk_cnt, __nv_bfloat16* __restrict__ mk_val)
+// nodes: (Phi_il, length and start of row l of Psi^T, start of node l's positions) of the 32 non-zeros a warp works on: read back
+// as one broadcast each, which costs the load/store unit a quarter of what four shuffles do
+template <bool SEGMENTED>
+__device__ __forceinline__ void mask_row_pass(int32_t pbeg, int32_t pend, int32_t seg0, int32_t seglen, int lane, float* acc,
+                                              int4* nodes, const int32_t* __restrict__ phi_col,
+                                              const float* __restrict__ phi_val, const int32_t* __restrict__ phi_pos,
+                                              const int32_t* __restrict__ t_rowptr, const float* __restrict__ t_val,
+                                              const unsigned short* __restrict__ pos16)
 {
-    extern __shared__ float smem_acc[];         // the warps' accumulators
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int GROUPS = BQ / MASK_ROWS;
-    const int32_t nblocks = (N + BQ - 1) / BQ;
-    const int32_t blk = mk_cnt[nblocks + blockIdx.x / GROUPS];     // blocks by decreasing key count
-    const int32_t rg = blockIdx.x % GROUPS;
-    float* acc = smem_acc + (size_t)warp * MASK_SEG;
-    const int32_t off = mk_off[blk], cnt = mk_cnt[blk];
-    for (int32_t x = lane; x < MASK_SEG; x += 32) acc[x] = 0.0f;
-    __syncwarp();
-    const int32_t r0 = blk * BQ;
-    for (int32_t seg0 = 0; seg0 < cnt; seg0 += MASK_SEG) {
-        const int32_t seglen = min(MASK_SEG, cnt - seg0);       // a multiple of the tile, hence of 8
-        for (int32_t rr = rg * MASK_ROWS + warp; rr < (rg + 1) * MASK_ROWS; rr += MASK_WARPS) {
-            const int32_t r = r0 + rr;
-            if (r < N) {
-                const int32_t pbeg = phi_rowptr[r], pend = phi_rowptr[r + 1];
-                for (int32_t p0 = pbeg; p0 < pend; p0 += 32) {
-                    // 32 non-zeros of the row at a time: lane x holds Phi_il, the start and length of row l_x of Psi^T
-                    // and the start of node l_x's positions
-                    const int32_t n = min(32, pend - p0);
-                    const int32_t my_l = lane < n ? __ldg(phi_col + p0 + lane) : 0;
-                    const float my_phi = lane < n ? __ldg(phi_val + p0 + lane) : 0.0f;
-                    const int32_t my_pbeg = lane < n ? __ldg(phi_pos + p0 + lane) : 0;
-                    const int32_t my_beg = lane < n ? __ldg(t_rowptr + my_l) : 0;
-                    const int32_t my_len = lane < n ? __ldg(t_rowptr + my_l + 1) - my_beg : 0;
-                    auto fetch = [&](int32_t e0, MaskPosGroup& gq) {
+    auto place = [&](int32_t ps) { return SEGMENTED ? ((uint32_t)(ps - seg0) < (uint32_t)seglen ? ps - seg0 : -1) : ps; };
+    for (int32_t p0 = pbeg; p0 < pend; p0 += 32) {
+        const int32_t n = min(32, pend - p0);
+        int4 mine = make_int4(0, 0, 0, 0);
+        if (lane < n) {
+            const int32_t l = __ldg(phi_col + p0 + lane);
+            mine.x = __float_as_int(__ldg(phi_val + p0 + lane));
+            mine.w = __ldg(phi_pos + p0 + lane);
+            mine.z = __ldg(t_rowptr + l);
+            mine.y = __ldg(t_rowptr + l + 1) - mine.z;
+        }
+        __syncwarp();
+        nodes[lane] = mine;
+        __syncwarp();
+        auto fetch = [&](int32_t e0, MaskPosGroup& gq) {
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            gq.beg[e] = __shfl_sync(0xffffffffu, my_beg, (e0 + e) & 31);
-                            gq.pbeg[e] = __shfl_sync(0xffffffffu, my_pbeg, (e0 + e) & 31);
-                            gq.len[e] = e0 + e < n ? __shfl_sync(0xffffffffu, my_len, (e0 + e) & 31) : 0;
+            for (int e = 0; e < 2; ++e) {
+                const int4 nd = nodes[e0 + e];
 #pragma unroll
-                            for (int sl = 0; sl < 4; ++sl) {
-                                const int32_t x = sl * 32 + lane;
-                                const bool valid = x < gq.len[e];
-                                gq.ps[e][sl] = valid ? (int32_t)__ldg(pos16 + (size_t)gq.pbeg[e] + x) : -1;
-                                gq.v[e][sl] = valid ? __ldg(t_val + gq.beg[e] + x) : 0.0f;
-                            }
-                        }
-                    };
-                    auto add = [&](int32_t e0, MaskPosGroup& gq) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float phi = __shfl_sync(0xffffffffu, my_phi, (e0 + e) & 31);
-                            float a[4];
-                            int32_t ps[4];
-                            // one node's keys are distinct: a lane's four additions go side by side
-#pragma unroll
-                            for (int sl = 0; sl < 4; ++sl) {
-                                const int32_t x = gq.ps[e][sl] - seg0;
-                                ps[sl] = (gq.ps[e][sl] >= 0 && x >= 0 && x < seglen) ? x : -1;
-                                a[sl] = ps[sl] >= 0 ? acc[ps[sl]] : 0.0f;
-                            }
-#pragma unroll
-                            for (int sl = 0; sl < 4; ++sl)
-                                if (ps[sl] >= 0) acc[ps[sl]] = fmaf(phi, gq.v[e][sl], a[sl]);
-                            for (int32_t x = 128 + lane; x < gq.len[e]; x += 32) {      // nodes with more than 128 keys
-                                const int32_t y = (int32_t)__ldg(pos16 + (size_t)gq.pbeg[e] + x) - seg0;
-                                if (y >= 0 && y < seglen) acc[y] = fmaf(phi, __ldg(t_val + gq.beg[e] + x), acc[y]);
-                            }
-                            __syncwarp();
-                        }
-                    };
-                    MaskPosGroup ga, gb;
-                    fetch(0, ga);
-                    for (int32_t e0 = 0; e0 < n; e0 += 8) {
-                        if (e0 + 4 < n) fetch(e0 + 4, gb);
-                        add(e0, ga);
-                        if (e0 + 4 < n) {
-                            if (e0 + 8 < n) fetch(e0 + 8, ga);
-                            add(e0 + 4, gb);
-                        }
-                    }
+                for (int sl = 0; sl < 4; ++sl) {
+                    const int32_t x = sl * 32 + lane;
+                    const bool valid = x < nd.y;
+                    gq.ps[e][sl] = valid ? (int32_t)__ldg(pos16 + (size_t)nd.w + x) : -1;
+                    gq.v[e][sl] = valid ? __ldg(t_val + nd.z + x) : 0.0f;
                 }
             }
+        };
+        auto add = [&](int32_t e0, MaskPosGroup& gq) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int4 nd = nodes[e0 + e];
+                const float phi = __int_as_float(nd.x);
+                float a[4];
+                int32_t ps[4];
+                // one node's keys are distinct: a lane's four additions go side by side
+#pragma unroll
+                for (int sl = 0; sl < 4; ++sl) {
+                    ps[sl] = place(gq.ps[e][sl]);
+                    a[sl] = ps[sl] >= 0 ? acc[ps[sl]] : 0.0f;
+                }
+#pragma unroll
+                for (int sl = 0; sl < 4; ++sl)
+                    if (ps[sl] >= 0) acc[ps[sl]] = fmaf(phi, gq.v[e][sl], a[sl]);
+                for (int32_t x = 128 + lane; x < nd.y; x += 32) {      // nodes with more than 128 keys
+                    const int32_t y = place((int32_t)__ldg(pos16 + (size_t)nd.w + x));
+                    if (y >= 0) acc[y] = fmaf(phi, __ldg(t_val + nd.z + x), acc[y]);
+                }
+                __syncwarp();
+            }
+        };
+        MaskPosGroup g[3];
+        fetch(0, g[0]);
+        fetch(2, g[1]);
+        for (int32_t e0 = 0; e0 < n; e0 += 6) {
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {
+                if (e0 + 2 * u < n) {
+                    if (e0 + 2 * u + 4 < n) fetch(e0 + 2 * u + 4, g[(u + 2) % 3]);
+                    add(e0 + 2 * u, g[u]);
+                }
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(MVP_WARPS * 32)
+mask_values_pos_kernel(int32_t N, int32_t rows_per_cta, int32_t room, const int32_t* __restrict__ phi_rowptr,
+                       const int32_t* __restrict__ phi_col, const float* __restrict__ phi_val,
+                       const int32_t* __restrict__ phi_pos, const int32_t* __restrict__ t_rowptr,
+                       const float* __restrict__ t_val, const unsigned short* __restrict__ pos16,
+                       const int32_t* __restrict__ mk_off, const int32_t* __restrict__ mk_cnt,
+                       __nv_bfloat16* __restrict__ mk_val)
+{
+    extern __shared__ __align__(16) float smem_acc[];         // the warps' accumulators, `room` floats in all
+    __shared__ int32_t next_row;
+    __shared__ int4 nodes[MVP_WARPS][32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t groups = BQ / rows_per_cta;
+    const int32_t nblocks = (N + BQ - 1) / BQ;
+    const int32_t blk = mk_cnt[nblocks + blockIdx.x / groups];     // blocks by decreasing key count
+    const int32_t rr0 = (blockIdx.x % groups) * rows_per_cta;
+    const int32_t off = mk_off[blk], cnt = mk_cnt[blk];
+    if (cnt == 0) return;
+    // warps that run and accumulators of each (a multiple of 8: they are read as float4 pairs)
+    const int32_t nw = min(MVP_WARPS, max(MVP_MIN_WARPS, room / cnt));
+    const int32_t seg = min(cnt, room / nw & ~7);
+    if (tid == 0) next_row = 0;
+    __syncthreads();
+    if (warp >= nw) return;
+    float* acc = smem_acc + (size_t)warp * seg;
+    for (int32_t x = lane; x < seg; x += 32) acc[x] = 0.0f;
+    __syncwarp();
+    const int32_t r0 = blk * BQ;
+    for (;;) {
+        int32_t rr = 0;
+        if (lane == 0) rr = atomicAdd(&next_row, 1);
+        rr = __shfl_sync(0xffffffffu, rr, 0);
+        if (rr >= rows_per_cta) break;
+        rr += rr0;
+        const int32_t r = r0 + rr;
+        const int32_t pbeg = r < N ? phi_rowptr[r] : 0, pend = r < N ? phi_rowptr[r + 1] : 0;
+        for (int32_t seg0 = 0; seg0 < cnt; seg0 += seg) {
+            const int32_t seglen = min(seg, cnt - seg0);           // a multiple of 8
+            if (seg == cnt)
+                mask_row_pass<false>(pbeg, pend, 0, cnt, lane, acc, nodes[warp], phi_col, phi_val, phi_pos, t_rowptr, t_val, pos16);
+            else
+                mask_row_pass<true>(pbeg, pend, seg0, seglen, lane, acc, nodes[warp], phi_col, phi_val, phi_pos, t_rowptr, t_val, pos16);
             // the row's values of this segment, eight keys (16 bytes) per lane at a time; the accumulators are
             // cleared for the next row as they are read
             for (int32_t c8 = lane; c8 < seglen / 8; c8 += 32) {
@@ -911,14 +952,18 @@ int launch_mask_values(grf_ctx* ctx, grf_features* feat, bool by_position)
     const int32_t N = feat->phi.rows, Nk = feat->psi.rows, nblocks = feat->plan_blocks;
     const size_t words = ((size_t)Nk + 31) / 32;
     if (by_position) {
-        const size_t smem_acc = (size_t)MASK_WARPS * MASK_SEG * sizeof(float);
+        // accumulators for sixteen rows of the longest list, up to an SM's shared memory; few blocks: fewer rows per CTA
+        const int64_t want = (int64_t)MVP_WARPS * (K.longest > 0 ? K.longest : KT);
+        const int32_t room = (int32_t)(want < MVP_ROOM ? want : MVP_ROOM);
+        const int32_t rows_per_cta = nblocks * 4 >= 2 * ctx->sm_count ? 32 : 16;
+        const size_t smem_acc = (size_t)room * sizeof(float);
         GRF_CUDA_TRY(cudaFuncSetAttribute(mask_values_pos_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_acc));
         grf_launch_scope scope(ctx, 8);
-        mask_values_pos_kernel<<<nblocks * (BQ / MASK_ROWS), MASK_WARPS * 32, smem_acc, ctx->stream>>>(
-            N, (const int32_t*)feat->phi.rowptr.ptr, (const int32_t*)feat->phi.col.ptr, (const float*)feat->phi.val.ptr,
-            (const int32_t*)K.phi_pos.ptr, (const int32_t*)feat->psit.rowptr.ptr, (const float*)feat->psit.val.ptr,
-            (const unsigned short*)K.pos16.ptr, (const int32_t*)K.off.ptr, (const int32_t*)K.cnt.ptr,
-            (__nv_bfloat16*)K.val.ptr);
+        mask_values_pos_kernel<<<nblocks * (BQ / rows_per_cta), MVP_WARPS * 32, smem_acc, ctx->stream>>>(
+            N, rows_per_cta, room, (const int32_t*)feat->phi.rowptr.ptr, (const int32_t*)feat->phi.col.ptr,
+            (const float*)feat->phi.val.ptr, (const int32_t*)K.phi_pos.ptr, (const int32_t*)feat->psit.rowptr.ptr,
+            (const float*)feat->psit.val.ptr, (const unsigned short*)K.pos16.ptr, (const int32_t*)K.off.ptr,
+            (const int32_t*)K.cnt.ptr, (__nv_bfloat16*)K.val.ptr);
     } else {
         const size_t smem_values = ((words + 1) & ~(size_t)1) * 8 + (size_t)MASK_WARPS * MASK_SEG * sizeof(float);
         GRF_CUDA_TRY(cudaFuncSetAttribute(mask_values_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_values));
@@ -1005,6 +1050,7 @@ extern "C" int grf_features_materialise(grf_ctx* ctx, grf_features* feat)
     // total means it did not) and both bitmaps fit shared memory; otherwise once per (row, node)
     const int64_t total_pos = ctx->pinned[6];
     const size_t smem_pos = (words + ((size_t)R + 31) / 32) * 8;
+    K.longest = ctx->pinned[7];
     const bool by_position = total_pos >= 0 && ctx->pinned[7] <= 65535 && smem_pos <= 96 * 1024;
     const size_t val_bytes = (size_t)entries * BQ * sizeof(__nv_bfloat16);
     if (val_bytes > ((size_t)8 << 30)) return GRF_ERR_TOO_LARGE;   // no locality: the S/z route serves this object

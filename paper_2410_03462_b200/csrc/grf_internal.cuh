@@ -103,6 +103,7 @@ struct grf_mask_dev {
     bool by_position = false;       // which of the two value kernels the structure serves
     int32_t blocks = 0;
     int64_t entries = 0;            // padded key entries over all blocks
+    int32_t longest = 0;            // longest key list of a block
     grf_buf off, cnt, key;          // cnt holds [blocks] padded counts, then [blocks] the blocks by decreasing count
     grf_buf bits;                   // per block one bit per key: the block's key set
     // build scratch: where each node's key positions start (within its block; the blocks' offsets), the positions,
