@@ -187,9 +187,12 @@ size_t grf_attn_workspace_bytes(int32_t G, int32_t R, int32_t m, int32_t d, int 
  * GRF_DTYPE_F32 or _BF16 (bf16: S is stored in bf16, sums are carried in fp32).  den_out: optional
  * DEVICE fp32 [G][N] receiving the denominators.  A row whose denominator is exactly 0 yields out = 0.
  * m, d in {8, 16, 32, 64, 128}.  workspace: DEVICE, 256-byte aligned.  Summation order is fixed, so
- * results are run-to-run identical.  Asynchronous, except that the first bf16 call with m and d multiples of 16
- * after the features were created, resampled or re-modulated prepares a per-block plan of Phi inside the feature
- * object, which waits for the stream once (so a feature object must not be used by two threads at the same time).
+ * results are run-to-run identical.  Where the same sum is cheaper in the other order (Mhat = Phi Psi^T first, as
+ * grf_masked_attn_mhat evaluates it), a bf16 batch takes that order; the choice depends on the features' sizes and on
+ * G, m, d only, never on earlier calls, and the workspace is then not touched.
+ * Asynchronous, except that the first bf16 call with m and d multiples of 16
+ * after the features were created, resampled or re-modulated prepares a per-block plan of Phi, and where it takes the
+ * other order the mask, inside the feature object, which waits for the stream (so a feature object must not be used by two threads at the same time).
  */
 int grf_masked_linear_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d,
                            int dtype, const void* phiQ, const void* phiK, const void* V,
@@ -278,7 +281,8 @@ int grf_ctx_check(grf_ctx* ctx);
 
 /* Chooses the attention kernels for bf16 problems: 1 (default) = tensor-core kernels where they apply (state
  * build: m a multiple of 16 and d <= 64; gather-contract: a block plan exists and m, d are multiples of 16);
- * 0 = plain-ALU kernels always.  Results agree within the stated tolerance. */
+ * 0 = plain-ALU kernels always; 2 = the tensor-core kernels, and grf_masked_linear_attn always goes through the
+ * per-node states.  Results agree within the stated tolerance. */
 int grf_ctx_use_tensor_cores(grf_ctx* ctx, int enable);
 
 /* The block plan of Phi that the tensor-core gather uses (built here if absent; waits for the stream then): HOST

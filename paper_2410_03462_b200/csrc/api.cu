@@ -115,6 +115,7 @@ extern "C" int grf_ctx_use_tensor_cores(grf_ctx* ctx, int enable)
 {
     if (!ctx) return GRF_ERR_INVALID;
     ctx->use_tensor_cores = enable != 0;
+    ctx->states_only = enable == 2;
     return GRF_OK;
 }
 
@@ -289,6 +290,10 @@ extern "C" int grf_features_from_csr(grf_ctx* ctx, int32_t N, int32_t R,
 
 static bool dim_ok(int32_t x) { return x == 8 || x == 16 || x == 32 || x == 64 || x == 128; }
 static size_t elem_size(int dtype) { return dtype == GRF_DTYPE_F32 ? 4 : 2; }
+static bool aligned16(const void* a, const void* b, const void* c, const void* d)
+{
+    return (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 15u) == 0;
+}
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // per-problem workspace: R records (state tile in the storage type, then z in fp32), 256-byte aligned
@@ -305,19 +310,14 @@ extern "C" size_t grf_attn_workspace_bytes(int32_t G, int32_t R, int32_t m, int3
     return ws_per_problem(R, m, d, dtype) * (size_t)G;
 }
 
-extern "C" int grf_masked_linear_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m,
-                                      int32_t d, int dtype, const void* phiQ, const void* phiK, const void* V,
-                                      void* out, float* den_out, void* workspace, size_t workspace_bytes)
+// The attention of G problems once the route is known: over the mask in one launch, or through the per-node states in
+// chunks of as many problems as the workspace holds.
+static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int32_t G, int32_t N, int32_t m, int32_t d,
+                       int dtype, const void* phiQ, const void* phiK, const void* V, void* out, float* den_out,
+                       void* workspace, size_t workspace_bytes)
 {
-    if (!ctx || !feat || !phiQ || !phiK || !V || !out || !workspace) return GRF_ERR_INVALID;
-    if (G <= 0 || N <= 0 || !dim_ok(m) || !dim_ok(d)) return GRF_ERR_INVALID;
-    if (dtype != GRF_DTYPE_F32 && dtype != GRF_DTYPE_BF16) return GRF_ERR_INVALID;
-    if (feat->phi.rows != N || feat->psit.cols != N || feat->phi.cols != feat->psit.rows) return GRF_ERR_INVALID;
-    if (((uintptr_t)workspace & 255) != 0) return GRF_ERR_INVALID;
-    const int32_t R = feat->phi.cols;
-    const size_t per = ws_per_problem(R, m, d, dtype);
-    if (workspace_bytes < per) return GRF_ERR_WORKSPACE;
-    GRF_CUDA_TRY(cudaSetDevice(ctx->device));
+    if (by_mask) return grf_mhat_launch(ctx, feat, G, N, m, phiQ, phiK, V, out, den_out);
+    const size_t per = ws_per_problem(feat->phi.cols, m, d, dtype);
     int64_t chunk = (int64_t)(workspace_bytes / per);
     if (chunk > G) chunk = G;
     if (chunk > 65535) chunk = 65535;
@@ -346,6 +346,24 @@ extern "C" int grf_masked_linear_attn(grf_ctx* ctx, const grf_features* feat, in
         GRF_TRY(rc);
     }
     return GRF_OK;
+}
+
+extern "C" int grf_masked_linear_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m,
+                                      int32_t d, int dtype, const void* phiQ, const void* phiK, const void* V,
+                                      void* out, float* den_out, void* workspace, size_t workspace_bytes)
+{
+    if (!ctx || !feat || !phiQ || !phiK || !V || !out || !workspace) return GRF_ERR_INVALID;
+    if (G <= 0 || N <= 0 || !dim_ok(m) || !dim_ok(d)) return GRF_ERR_INVALID;
+    if (dtype != GRF_DTYPE_F32 && dtype != GRF_DTYPE_BF16) return GRF_ERR_INVALID;
+    if (feat->phi.rows != N || feat->psit.cols != N || feat->phi.cols != feat->psit.rows) return GRF_ERR_INVALID;
+    if (((uintptr_t)workspace & 255) != 0) return GRF_ERR_INVALID;
+    const int32_t R = feat->phi.cols;
+    const size_t per = ws_per_problem(R, m, d, dtype);
+    if (workspace_bytes < per) return GRF_ERR_WORKSPACE;
+    GRF_CUDA_TRY(cudaSetDevice(ctx->device));
+    bool by_mask = false;
+    if (aligned16(phiQ, phiK, V, out)) GRF_TRY(grf_linear_by_mask(ctx, feat, G, N, m, d, dtype, &by_mask));
+    return linear_attn(ctx, feat, by_mask, G, N, m, d, dtype, phiQ, phiK, V, out, den_out, workspace, workspace_bytes);
 }
 
 static int check_graph_host(int32_t N, const int32_t* rowptr, const int32_t* col)
@@ -395,11 +413,7 @@ extern "C" int grf_step_host(grf_ctx* ctx, int32_t N, const int32_t* rowptr, con
         }
         GRF_CUDA_TRY(cudaEventCreateWithFlags(&ctx->down_done, cudaEventDisableTiming));
     }
-    // Two parts on the route through the per-node states, whose kernels lose more on small batches than the finer
-    // overlap returns (four parts were measured slower there); four on the route over the mask, whose attention is
-    // short, so that most of the outputs leave while later parts are computed.
-    const bool mask_shape = ctx->prefer_mask_route && dtype == GRF_DTYPE_BF16 && d == 64 && (m == 16 || m == 32 || m == 64);
-    const int want_parts = mask_shape ? grf_ctx::HOST_PARTS : 2;
+    const int want_parts = grf_ctx::HOST_PARTS;
     const int parts = G >= 2 * want_parts ? want_parts : (G >= 2 ? 2 : 1);
     const int32_t gp = (G + parts - 1) / parts;           // problems per part
     for (int p = 0; p < parts; ++p) {
@@ -414,32 +428,36 @@ extern "C" int grf_step_host(grf_ctx* ctx, int32_t N, const int32_t* rowptr, con
     }
     GRF_TRY(grf_sample(ctx, N, (const int32_t*)ctx->h_rowptr.ptr, (const int32_t*)ctx->h_col.ptr,
                        (const float*)ctx->h_w.ptr, seed, n_walks, p_halt, max_len, f_phi, f_psi, &ctx->h_feat));
-    // route: over the materialised mask when the caller prefers it and the shape and the graph allow it
+    // route: over the materialised mask when the caller prefers it and the shape and the graph allow it, or when the
+    // whole batch is cheaper that way (the parts below follow one decision, so the split does not change the bits)
     bool by_mask = false;
     if (ctx->prefer_mask_route && dtype == GRF_DTYPE_BF16 && d == 64 && (m == 16 || m == 32 || m == 64)) {
         const int rc = grf_features_materialise(ctx, ctx->h_feat);
         if (rc == GRF_OK) by_mask = true;
         else if (rc != GRF_ERR_TOO_LARGE) return rc;          // too large = no locality: the S/z route serves it
+    } else {
+        GRF_TRY(grf_linear_by_mask(ctx, ctx->h_feat, G, N, m, d, dtype, &by_mask));
     }
+    // Inputs always travel in the parts above.  The attention follows part by part over the mask (it is short, so most of
+    // the outputs leave while later parts are computed), and in two steps through the per-node states, whose kernels lose
+    // more on small batches than the finer overlap returns.
+    const int per_step = by_mask ? 1 : (parts + 1) / 2;        // upload parts per attention step
+    const int32_t gs = gp * per_step;
     // workspace: one part's records if that is modest, else chunks of about 1 GiB
     const size_t per = by_mask ? 256 : ws_per_problem(N, m, d, dtype);
-    size_t want = per * (size_t)gp;
+    size_t want = per * (size_t)(gs < G ? gs : G);
     const size_t cap = (size_t)1 << 31;
     if (want > cap) want = per * (cap / per > 0 ? cap / per : 1);
     GRF_TRY(grf_buf_reserve(&ctx->h_ws, want));
-    for (int p = 0; p < parts; ++p) {
-        const int32_t g0 = p * gp, gc = g0 + gp <= G ? gp : G - g0;
+    for (int p = 0; p * per_step < parts; ++p) {
+        const int32_t g0 = p * gs, gc = g0 + gs <= G ? gs : G - g0;
         if (gc <= 0) break;
         const size_t qo = (size_t)g0 * N * m * es, vo = (size_t)g0 * N * d * es;
-        GRF_CUDA_TRY(cudaStreamWaitEvent(s, ctx->up_done[p], 0));
-        if (by_mask)
-            GRF_TRY(grf_masked_attn_mhat(ctx, ctx->h_feat, gc, N, m, d, dtype, (const char*)ctx->h_q.ptr + qo,
-                                         (const char*)ctx->h_k.ptr + qo, (const char*)ctx->h_v.ptr + vo,
-                                         (char*)ctx->h_out.ptr + vo, nullptr));
-        else
-            GRF_TRY(grf_masked_linear_attn(ctx, ctx->h_feat, gc, N, m, d, dtype, (const char*)ctx->h_q.ptr + qo,
-                                           (const char*)ctx->h_k.ptr + qo, (const char*)ctx->h_v.ptr + vo,
-                                           (char*)ctx->h_out.ptr + vo, nullptr, ctx->h_ws.ptr, ctx->h_ws.bytes));
+        for (int u = p * per_step; u < (p + 1) * per_step && u < parts; ++u)
+            if (u * gp < G) GRF_CUDA_TRY(cudaStreamWaitEvent(s, ctx->up_done[u], 0));
+        GRF_TRY(linear_attn(ctx, ctx->h_feat, by_mask, gc, N, m, d, dtype, (const char*)ctx->h_q.ptr + qo,
+                            (const char*)ctx->h_k.ptr + qo, (const char*)ctx->h_v.ptr + vo, (char*)ctx->h_out.ptr + vo,
+                            nullptr, ctx->h_ws.ptr, ctx->h_ws.bytes));
         GRF_CUDA_TRY(cudaEventRecord(ctx->part_done[p], s));
         GRF_CUDA_TRY(cudaStreamWaitEvent(ctx->down_stream, ctx->part_done[p], 0));
         GRF_CUDA_TRY(cudaMemcpyAsync((char*)out + vo, (const char*)ctx->h_out.ptr + vo, (size_t)gc * N * d * es,

@@ -940,11 +940,20 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
 
 }  // namespace
 
-void grf_mask_invalidate(grf_features* feat) { feat->mask.ready = false; feat->mask.structure_ready = false; }
+void grf_mask_invalidate(grf_features* feat)
+{
+    grf_mask_dev& K = feat->mask;
+    K.ready = K.requested = K.refused = K.lists_ready = K.structure_ready = false;
+}
 // Phi's and Psi's values changed, their structure did not (re-modulation): key lists and positions stay
-void grf_mask_values_stale(grf_features* feat) { feat->mask.ready = false; }
+void grf_mask_values_stale(grf_features* feat) { feat->mask.ready = feat->mask.requested = false; }
 
 namespace {
+int reserve_with_headroom(grf_buf* b, size_t bytes)
+{
+    return b->bytes >= bytes ? GRF_OK : grf_buf_reserve(b, bytes + bytes / 8 + 256);
+}
+
 // The values of the mask from the present values of Phi and Psi^T, over key lists (and positions) that are in place.
 int launch_mask_values(grf_ctx* ctx, grf_features* feat, bool by_position)
 {
@@ -982,31 +991,16 @@ void grf_mask_release(grf_features* feat)
     grf_mask_dev& K = feat->mask;
     grf_buf_release(&K.off); grf_buf_release(&K.cnt); grf_buf_release(&K.key); grf_buf_release(&K.bits); grf_buf_release(&K.val); grf_buf_release(&K.node_off);
     grf_buf_release(&K.blk_pos); grf_buf_release(&K.pos16); grf_buf_release(&K.phi_pos);
-    K.ready = false;
-    K.structure_ready = false;
+    grf_mask_invalidate(feat);
 }
 
-extern "C" int grf_features_materialise(grf_ctx* ctx, grf_features* feat)
+// Key sets of the blocks, their counts and offsets, where every node's key positions will start: all sizes that the rest
+// of the build and the choice of the route need.  Waits for the stream.
+static int prepare_mask_lists(grf_ctx* ctx, grf_features* feat)
 {
-    if (!ctx || !feat) return GRF_ERR_INVALID;
-    GRF_CUDA_TRY(cudaSetDevice(ctx->device));
     grf_mask_dev& K = feat->mask;
-    K.ready = false;
-    if (K.structure_ready && feat->plan_ready && !feat->plan_stale) {
-        // same walks, new coefficients: the key lists and positions still hold
-        GRF_TRY(launch_mask_values(ctx, feat, K.by_position));
-        K.ready = true;
-        return GRF_OK;
-    }
-    K.structure_ready = false;
-    const int32_t N = feat->phi.rows, Nk = feat->psi.rows;
+    const int32_t Nk = feat->psi.rows, nblocks = feat->plan_blocks;
     const size_t words = ((size_t)Nk + 31) / 32;
-    // the values kernel keeps the key bitmap, its prefix counts and the accumulators in shared memory
-    const size_t smem_values = ((words + 1) & ~(size_t)1) * 8 + (size_t)MASK_WARPS * MASK_SEG * sizeof(float);
-    if (smem_values > 200 * 1024) return GRF_ERR_TOO_LARGE;
-    GRF_TRY(grf_ensure_block_plan(ctx, feat, false));         // the node lists only
-    if (!feat->plan_ready) return GRF_ERR_TOO_LARGE;          // rows of a block share too little
-    const int32_t nblocks = feat->plan_blocks;
     GRF_TRY(grf_buf_reserve(&K.cnt, sizeof(int32_t) * 2 * (size_t)nblocks));
     GRF_TRY(grf_buf_reserve(&K.off, sizeof(int32_t) * ((size_t)nblocks + 1)));
     GRF_TRY(grf_buf_reserve(&K.bits, sizeof(uint32_t) * 2 * (size_t)nblocks * words));
@@ -1023,12 +1017,8 @@ extern "C" int grf_features_materialise(grf_ctx* ctx, grf_features* feat)
     GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 5, (const int32_t*)K.off.ptr + nblocks, sizeof(int32_t),
                                  cudaMemcpyDeviceToHost, ctx->stream));
     // where every node's key positions will start (per block, then over the blocks), and the longest key list
-    const int32_t R = feat->psit.rows;
     // (buffers whose size follows the sample grow with head-room: resampling changes the sizes a little every time,
     // and a reallocation stalls the device)
-    auto reserve_with_headroom = [](grf_buf* b, size_t bytes) {
-        return b->bytes >= bytes ? GRF_OK : grf_buf_reserve(b, bytes + bytes / 8 + 256);
-    };
     GRF_TRY(reserve_with_headroom(&K.node_off, sizeof(int32_t) * (size_t)(feat->plan_entries > 0 ? feat->plan_entries : 1)));
     GRF_TRY(grf_buf_reserve(&K.blk_pos, sizeof(int32_t) * (2 * (size_t)nblocks + 2)));
     int32_t* blk_pos = (int32_t*)K.blk_pos.ptr;                 // offsets [nblocks + 1], totals [nblocks], longest list
@@ -1044,18 +1034,52 @@ extern "C" int grf_features_materialise(grf_ctx* ctx, grf_features* feat)
     GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 6, blk_pos + nblocks, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 7, blk_pos + 2 * nblocks + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     GRF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));          // the sizes of the key lists are known only now
-    const int64_t entries = ctx->pinned[5];
-    if (entries < 0) return GRF_ERR_TOO_LARGE;
-    // positions are looked up once per (block, node) when they fit 16 bits, their number fits an int32 (a negative
-    // total means it did not) and both bitmaps fit shared memory; otherwise once per (row, node)
-    const int64_t total_pos = ctx->pinned[6];
-    const size_t smem_pos = (words + ((size_t)R + 31) / 32) * 8;
+    K.blocks = nblocks;
+    K.entries = ctx->pinned[5];
+    K.positions = ctx->pinned[6];
     K.longest = ctx->pinned[7];
-    const bool by_position = total_pos >= 0 && ctx->pinned[7] <= 65535 && smem_pos <= 96 * 1024;
-    const size_t val_bytes = (size_t)entries * BQ * sizeof(__nv_bfloat16);
-    if (val_bytes > ((size_t)8 << 30)) return GRF_ERR_TOO_LARGE;   // no locality: the S/z route serves this object
-    if (K.key.bytes < (size_t)entries * 4) GRF_TRY(grf_buf_reserve(&K.key, ((size_t)entries + (size_t)entries / 8 + 64) * 4));
-    if (K.val.bytes < val_bytes) GRF_TRY(grf_buf_reserve(&K.val, val_bytes + val_bytes / 8 + 256));
+    K.lists_ready = true;
+    // (a negative sum means that it passed 2^31); no locality: the S/z route serves this object
+    K.refused = K.entries < 0 || (size_t)K.entries * BQ * sizeof(__nv_bfloat16) > ((size_t)8 << 30);
+    return GRF_OK;
+}
+
+// Shared memory of the row-by-row values kernel: the key bitmap, its prefix counts and the accumulators.
+static bool mask_fits_smem(const grf_features* feat)
+{
+    const size_t words = ((size_t)feat->psi.rows + 31) / 32;
+    return ((words + 1) & ~(size_t)1) * 8 + (size_t)MASK_WARPS * MASK_SEG * sizeof(float) <= 200 * 1024;
+}
+
+// Forms the mask of the present features (or only its values, where the key lists still hold).
+static int build_mask(grf_ctx* ctx, grf_features* feat)
+{
+    grf_mask_dev& K = feat->mask;
+    K.ready = false;
+    if (K.structure_ready && feat->plan_ready && !feat->plan_stale) {
+        // same walks, new coefficients: the key lists and positions still hold
+        GRF_TRY(launch_mask_values(ctx, feat, K.by_position));
+        K.ready = true;
+        return GRF_OK;
+    }
+    K.structure_ready = false;
+    const int32_t N = feat->phi.rows, Nk = feat->psi.rows, R = feat->psit.rows;
+    if (!mask_fits_smem(feat)) return GRF_ERR_TOO_LARGE;
+    GRF_TRY(grf_ensure_block_plan(ctx, feat, false));         // the node lists only
+    if (!feat->plan_ready) return GRF_ERR_TOO_LARGE;          // rows of a block share too little
+    if (!K.lists_ready) GRF_TRY(prepare_mask_lists(ctx, feat));
+    if (K.refused) return GRF_ERR_TOO_LARGE;
+    const int32_t nblocks = feat->plan_blocks;
+    const int64_t entries = K.entries;
+    const size_t words = ((size_t)Nk + 31) / 32;
+    int32_t* blk_pos = (int32_t*)K.blk_pos.ptr;
+    // positions are looked up once per (block, node) when they fit 16 bits, their number fits an int32 and both bitmaps
+    // fit shared memory; otherwise once per (row, node)
+    const int64_t total_pos = K.positions;
+    const size_t smem_pos = (words + ((size_t)R + 31) / 32) * 8;
+    const bool by_position = total_pos >= 0 && K.longest <= 65535 && smem_pos <= 96 * 1024;
+    GRF_TRY(reserve_with_headroom(&K.key, (size_t)entries * 4));
+    GRF_TRY(reserve_with_headroom(&K.val, (size_t)entries * BQ * sizeof(__nv_bfloat16)));
     {
         grf_launch_scope scope(ctx, 8);
         mask_list_kernel<<<nblocks, 256, 0, ctx->stream>>>(Nk, (const uint32_t*)K.bits.ptr, (const int32_t*)K.off.ptr,
@@ -1080,17 +1104,71 @@ extern "C" int grf_features_materialise(grf_ctx* ctx, grf_features* feat)
     }
     GRF_TRY(launch_mask_values(ctx, feat, by_position));
     GRF_CUDA_TRY(cudaGetLastError());
-    K.blocks = nblocks;
-    K.entries = entries;
     K.by_position = by_position;
     K.structure_ready = true;
     K.ready = true;
     return GRF_OK;
 }
 
+extern "C" int grf_features_materialise(grf_ctx* ctx, grf_features* feat)
+{
+    if (!ctx || !feat) return GRF_ERR_INVALID;
+    GRF_CUDA_TRY(cudaSetDevice(ctx->device));
+    feat->mask.requested = false;
+    GRF_TRY(build_mask(ctx, feat));
+    feat->mask.requested = true;
+    return GRF_OK;
+}
+
+static bool mhat_shape(int32_t m, int32_t d, int dtype)
+{
+    return dtype == GRF_DTYPE_BF16 && d == 64 && (m == 16 || m == 32 || m == 64);
+}
+
+// Which association of the product serves a batch of grf_masked_linear_attn: the per-node states of Eq. 12, or the
+// mask formed first.  The choice depends on the features' sizes and the batch only (never on earlier calls), so equal
+// calls give equal bits.  Times in nanoseconds, fitted on a B200 to clouds, grids and expanders of 2^6 .. 2^17 nodes:
+//   states   per problem: 0.52 per node-list entry (a state tile into shared memory) and 0.04 per non-zero (a key's rows
+//            into a state, z into a denominator), both at m = 32 and in proportion to m;
+//   mask     per problem: 2.5 per 64-key tile and 15 per block; once: 0.0022 per multiply-add of Phi Psi^T (non-zeros of Phi
+//            times the mean row of Psi^T, again for every further segment of the lists), 500 per block for the lists,
+//            80 000 for the launches and the wait.
+// The mask is charged as if this call had to form it, although frozen features keep it: a batch too small for that keeps
+// to the states.
+int grf_linear_by_mask(grf_ctx* ctx, const grf_features* cfeat, int32_t G, int32_t N, int32_t m, int32_t d, int dtype,
+                       bool* by_mask)
+{
+    *by_mask = false;
+    grf_features* feat = const_cast<grf_features*>(cfeat);     // the mask is a cache inside the object, like the block plan
+    grf_mask_dev& K = feat->mask;
+    if (!ctx->use_tensor_cores || ctx->states_only || !mhat_shape(m, d, dtype)) return GRF_OK;
+    if (feat->psi.rows != N || !mask_fits_smem(feat)) return GRF_OK;
+    GRF_TRY(grf_ensure_block_plan(ctx, feat, false));
+    if (!feat->plan_ready || K.refused) return GRF_OK;
+    const double scale = m / 32.0;
+    const double nnz = 0.5 * ((double)feat->phi.nnz + (double)feat->psi.nnz);
+    const double states = G * scale * (0.52 * (double)feat->plan_entries + 0.04 * nnz);
+    const double macs = (double)feat->phi.nnz * (double)feat->psi.nnz / feat->psit.rows;
+    const double build = 80000.0 + 500.0 * feat->plan_blocks + 0.0022 * macs;
+    if (build > states) return GRF_OK;                          // already without the attention itself
+    if (!K.lists_ready) GRF_TRY(prepare_mask_lists(ctx, feat));
+    if (K.refused || (int64_t)G * K.blocks > 0x7fffffffll || (int64_t)G * N > 0x7fffffffll) return GRF_OK;
+    const double attn = G * (2.5 * scale * (double)(K.entries / KT) + 15.0 * K.blocks);
+    const double lists = (double)K.entries / K.blocks / (MVP_ROOM / MVP_MIN_WARPS);     // mean list, in accumulator segments
+    const double more = lists > 1.0 ? 0.0022 * macs * (lists - 1.0) : 0.0;
+    if (build + more + attn > states) return GRF_OK;
+    if (!K.ready) {
+        const int rc = build_mask(ctx, feat);
+        if (rc == GRF_ERR_TOO_LARGE || rc == GRF_ERR_NOMEM) { K.refused = true; return GRF_OK; }
+        GRF_TRY(rc);
+    }
+    *by_mask = true;
+    return GRF_OK;
+}
+
 extern "C" int grf_mask_stats(const grf_features* feat, int32_t* blocks, int64_t* key_entries, int64_t* bytes)
 {
-    if (!feat || !feat->mask.ready) return GRF_ERR_INVALID;
+    if (!feat || !feat->mask.ready || !feat->mask.requested) return GRF_ERR_INVALID;
     if (blocks) *blocks = feat->mask.blocks;
     if (key_entries) *key_entries = feat->mask.entries;
     if (bytes) *bytes = feat->mask.entries * (int64_t)(BQ * sizeof(__nv_bfloat16) + sizeof(int32_t));
@@ -1100,7 +1178,7 @@ extern "C" int grf_mask_stats(const grf_features* feat, int32_t* blocks, int64_t
 extern "C" int grf_mask_rows(grf_ctx* ctx, const grf_features* feat, int32_t n, const int32_t* rows, float* out)
 {
     if (!ctx || !feat || n <= 0 || !rows || !out) return GRF_ERR_INVALID;
-    if (!feat->mask.ready) return GRF_ERR_INVALID;
+    if (!feat->mask.ready || !feat->mask.requested) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
     const grf_mask_dev& K = feat->mask;
     {
@@ -1130,16 +1208,22 @@ static int launch_mhat(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_
     return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
 }
 
+int grf_mhat_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, const void* phiQ,
+                    const void* phiK, const void* V, void* out, float* den_out)
+{
+    if (m == 16) return launch_mhat<16>(ctx, feat, G, N, phiQ, phiK, V, out, den_out);
+    if (m == 32) return launch_mhat<32>(ctx, feat, G, N, phiQ, phiK, V, out, den_out);
+    return launch_mhat<64>(ctx, feat, G, N, phiQ, phiK, V, out, den_out);
+}
+
 extern "C" int grf_masked_attn_mhat(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d,
                                     int dtype, const void* phiQ, const void* phiK, const void* V, void* out, float* den_out)
 {
     if (!ctx || !feat || !phiQ || !phiK || !V || !out || G <= 0 || N <= 0) return GRF_ERR_INVALID;
-    if (dtype != GRF_DTYPE_BF16 || d != 64 || (m != 16 && m != 32 && m != 64)) return GRF_ERR_INVALID;
-    if (!feat->mask.ready || feat->phi.rows != N || feat->psi.rows != N) return GRF_ERR_INVALID;
+    if (!mhat_shape(m, d, dtype)) return GRF_ERR_INVALID;
+    if (!feat->mask.ready || !feat->mask.requested || feat->phi.rows != N || feat->psi.rows != N) return GRF_ERR_INVALID;
     if ((int64_t)G * N > 0x7fffffffll || (int64_t)G * feat->mask.blocks > 0x7fffffffll) return GRF_ERR_TOO_LARGE;
     if (((uintptr_t)phiQ | (uintptr_t)phiK | (uintptr_t)V | (uintptr_t)out) & 15u) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
-    if (m == 16) return launch_mhat<16>(ctx, feat, G, N, phiQ, phiK, V, out, den_out);
-    if (m == 32) return launch_mhat<32>(ctx, feat, G, N, phiQ, phiK, V, out, den_out);
-    return launch_mhat<64>(ctx, feat, G, N, phiQ, phiK, V, out, den_out);
+    return grf_mhat_launch(ctx, feat, G, N, m, phiQ, phiK, V, out, den_out);
 }

@@ -54,6 +54,7 @@ struct grf_ctx {
     int32_t* pinned = nullptr;      // small pinned host block for read-backs
     int* error_word = nullptr;      // device word set by a kernel that gave up a bounded wait
     bool use_tensor_cores = true;
+    bool states_only = false;       // grf_masked_linear_attn never takes the mask (grf_ctx_use_tensor_cores(ctx, 2))
     bool prefer_mask_route = false; // grf_step_host evaluates the attention over the materialised mask where it can
     bool check_graphs = false;      // grf_sample validates the device-resident CSR first (debugging aid)
     // optional per-launch timing
@@ -98,12 +99,16 @@ struct grf_kept_walks {
 // and zero values) and the block's values in bf16, laid out [group of 8 keys][row of the block][8 keys].
 #define GRF_MASK_TILE 64
 struct grf_mask_dev {
-    bool ready = false;
+    bool ready = false;             // the blocks hold the mask of the present features
+    bool requested = false;         // the caller asked for it (grf_features_materialise); else it is grf_masked_linear_attn's own
+    bool refused = false;           // its blocks would be too large for the present structure: not tried again
+    bool lists_ready = false;       // key sets, counts and sizes match the features' structure (what deciding the route needs)
+    int64_t positions = 0;          // (node, key) pairs over all blocks, -1 when they passed 2^31
+    int32_t longest = 0;            // longest key list of a block
     bool structure_ready = false;   // key lists (and positions) match the features' structure; values may be stale
     bool by_position = false;       // which of the two value kernels the structure serves
     int32_t blocks = 0;
     int64_t entries = 0;            // padded key entries over all blocks
-    int32_t longest = 0;            // longest key list of a block
     grf_buf off, cnt, key;          // cnt holds [blocks] padded counts, then [blocks] the blocks by decreasing count
     grf_buf bits;                   // per block one bit per key: the block's key set
     // build scratch: where each node's key positions start (within its block; the blocks' offsets), the positions,
@@ -165,6 +170,11 @@ int grf_gather_contract_alu(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int
 // attn_mhat.cu
 void grf_mask_invalidate(grf_features* feat);
 void grf_mask_values_stale(grf_features* feat);
+// Whether grf_masked_linear_attn evaluates this batch over the materialised mask; forms the mask when it does.
+int grf_linear_by_mask(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, int dtype,
+                       bool* by_mask);
+int grf_mhat_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, const void* phiQ,
+                    const void* phiK, const void* V, void* out, float* den_out);
 void grf_mask_release(grf_features* feat);
 // attn_gather_tc.cu
 int grf_build_block_plan(grf_ctx* ctx, grf_features* feat, bool with_coef = true);
