@@ -296,10 +296,10 @@ static bool aligned16(const void* a, const void* b, const void* c, const void* d
 }
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// per-problem workspace: R records (state tile in the storage type, then z in fp32), 256-byte aligned
+// per-problem workspace, 256-byte aligned
 static size_t ws_per_problem(int32_t R, int32_t m, int32_t d, int dtype)
 {
-    // one record per node: the state tile, z (fp32) and, with bf16 storage, z once more in bf16
+    // per node: the state tile, z (fp32) and, with bf16 storage, room for z once more in bf16
     return align256((size_t)R * ((size_t)m * d * elem_size(dtype) + (size_t)m * sizeof(float) +
                                  (dtype == GRF_DTYPE_BF16 ? (size_t)m * 2 : 0)));
 }
@@ -323,12 +323,10 @@ static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int
     if (chunk > 65535) chunk = 65535;
     const size_t es = elem_size(dtype);
     // the plan's build waits for the stream once: do it before the attention kernels are queued, not between them
-    // (only for shapes the tensor-core gather covers: other shapes never read the plan)
-    if (dtype == GRF_DTYPE_BF16 && ctx->use_tensor_cores && m % 16 == 0 && d % 16 == 0)
-        GRF_TRY(grf_ensure_block_plan(ctx, feat));
+    bool tc_gather = false;
+    GRF_TRY(grf_gather_by_tensor_cores(ctx, feat, m, d, dtype, &tc_gather));
     for (int64_t g0 = 0; g0 < G; g0 += chunk) {
         const int32_t gc = (int32_t)((G - g0) < chunk ? (G - g0) : chunk);
-        // chunk layout: records [gc][R], contiguous
         const char* k_ptr = (const char*)phiK + (size_t)g0 * N * m * es;
         const char* v_ptr = (const char*)V + (size_t)g0 * N * d * es;
         const char* q_ptr = (const char*)phiQ + (size_t)g0 * N * m * es;
@@ -336,14 +334,11 @@ static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int
         float* den_ptr = den_out ? den_out + (size_t)g0 * N : nullptr;
         int rs = 1;
         if (dtype == GRF_DTYPE_BF16 && ctx->use_tensor_cores)
-            rs = grf_build_states_tc(ctx, feat->psit, gc, N, m, d, k_ptr, v_ptr, workspace);
-        if (rs > 0) rs = grf_build_states(ctx, feat->psit, gc, N, m, d, dtype, k_ptr, v_ptr, workspace);
+            rs = grf_build_states_tc(ctx, feat->psit, gc, N, m, d, k_ptr, v_ptr, workspace, !tc_gather);
+        if (rs > 0) rs = grf_build_states(ctx, feat->psit, gc, N, m, d, dtype, k_ptr, v_ptr, workspace, !tc_gather);
         GRF_TRY(rs);
-        int rc = 1;
-        if (dtype == GRF_DTYPE_BF16 && ctx->use_tensor_cores)
-            rc = grf_gather_contract_tc(ctx, feat, gc, N, m, d, q_ptr, workspace, o_ptr, den_ptr);
-        if (rc > 0) rc = grf_gather_contract_alu(ctx, feat->phi, gc, N, m, d, dtype, q_ptr, workspace, o_ptr, den_ptr);
-        GRF_TRY(rc);
+        if (tc_gather) GRF_TRY(grf_gather_contract_tc(ctx, feat, gc, N, m, d, q_ptr, workspace, o_ptr, den_ptr));
+        else GRF_TRY(grf_gather_contract_alu(ctx, feat->phi, gc, N, m, d, dtype, q_ptr, workspace, o_ptr, den_ptr));
     }
     return GRF_OK;
 }

@@ -1,139 +1,272 @@
-// Gather-and-contract with normalisation (Alg. 1 step 5, Eq. 12):
+// Gather-and-contract with normalisation (Alg. 1 step 5, Eq. 12) on the plain ALUs (any supported m, d; fp32 or bf16):
 //   num_i = sum_l Phi_il phi(q_i)^T S_l,  den_i = sum_l Phi_il phi(q_i)^T z_l,  out_i = num_i / den_i.
 //
-// Plain-ALU kernel (any supported m, d; fp32 or bf16 storage): one warp per (problem g, query i).  A tile
-// is read as consecutive 16-byte chunks (512 contiguous bytes per warp-wide load); sums are carried in
-// fp32 in a fixed order.
+// What bounds it is the delivery of state tiles: every non-zero of Phi brings m x d values to the SM, and on graphs
+// without locality nothing is shared.  From HBM that is 6 TB/s, from L2 up to 19 TB/s, so the columns of a problem's
+// tiles are taken in slices whose bytes over all nodes fit L2 (the grid runs through the rows of one slice before it
+// starts the next): HBM then sees each record once.  A group of lanes takes one node's slice, one 16-byte chunk (CH
+// consecutive feature rows a of one column b) per lane, and adds Phi_il times it to T_i = sum_l Phi_il S_l in registers;
+// phi(q_i) enters once, at the end.  What limits a slice is then the latency of L2 at one load per warp and 64 warps per
+// SM; fewer warps with more loads each were slower.  Expanders, 4 heads, m = 32, d = 64, bf16: N = 2^18 34.0 -> 23.5 ms
+// (10.4 TB/s into the SMs), N = 2^16 6.8 ms by the tensor-core gather -> 3.6 ms (17 TB/s).  Sums are carried in fp32 in a
+// fixed order.
+#include <type_traits>
+
 #include "grf_internal.cuh"
 
 namespace {
 
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// a 16-byte chunk as packed pairs of fp32, and one element of a row
 template <typename T> struct Chunk;
 template <> struct Chunk<float> {
-    __device__ static __forceinline__ void load(const float* p, float (&v)[4])
+    static constexpr int PAIRS = 2;
+    __device__ static __forceinline__ void widen(const uint4& x, uint64_t (&v)[2])
     {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(p));
-        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+        v[0] = (uint64_t)x.y << 32 | x.x;
+        v[1] = (uint64_t)x.w << 32 | x.z;
     }
-    __device__ static __forceinline__ void store1(float* p, float x) { *p = x; }
+    __device__ static __forceinline__ float get(const float* p) { return __ldg(p); }
+    __device__ static __forceinline__ void put(float* p, float x) { *p = x; }
 };
 template <> struct Chunk<__nv_bfloat16> {
-    __device__ static __forceinline__ void load(const __nv_bfloat16* p, float (&v)[8])
+    static constexpr int PAIRS = 4;
+    __device__ static __forceinline__ void widen(const uint4& x, uint64_t (&v)[4])
     {
-        const uint4 x = __ldg(reinterpret_cast<const uint4*>(p));
         const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            v[2 * q] = __uint_as_float(w[q] << 16);
-            v[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
-        }
+        for (int q = 0; q < 4; ++q) v[q] = pack2(__uint_as_float(w[q] << 16), __uint_as_float(w[q] & 0xffff0000u));
     }
-    __device__ static __forceinline__ void store1(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
+    __device__ static __forceinline__ float get(const __nv_bfloat16* p)
+    {
+        return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p)) << 16);
+    }
+    __device__ static __forceinline__ void put(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
 };
-
-template <typename T> __device__ __forceinline__ float to_f32(T x);
-template <> __device__ __forceinline__ float to_f32<float>(float x) { return x; }
-template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 x) { return __bfloat162float(x); }
 
 constexpr int GATHER_WARPS = 4;
 
+// Denominators: a warp per (problem, query), M / 4 lanes per node on z_l in fp32.
 template <typename T, int M, int D>
 __global__ void __launch_bounds__(GATHER_WARPS * 32)
-gather_contract_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                       const float* __restrict__ val, const T* __restrict__ phiQ,
-                       const unsigned char* __restrict__ records, T* __restrict__ out, float* __restrict__ den_out)
+gather_denominators_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                           const float* __restrict__ val, const T* __restrict__ phiQ,
+                           const unsigned char* __restrict__ states, float* __restrict__ den)
 {
-    constexpr int CH = grf_tile_chunk<T>();
-    constexpr int NCHUNK = (M / CH) * D;            // 16-byte chunks per tile, chunk x = (a / CH) * D + b
-    constexpr int NACC = D >= 32 ? D / 32 : 1;      // output columns per lane
-    __shared__ float qs[GATHER_WARPS][M];
-
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int32_t i = blockIdx.x * GATHER_WARPS + warp;
-    const int32_t g = blockIdx.y;
+    constexpr int LPN = M / 4, NPS = 32 / LPN;          // lanes per node, nodes side by side
+    const int lane = threadIdx.x & 31, sub = lane / LPN, pl = lane % LPN;
+    const int32_t i = blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5), g = blockIdx.y;
     if (i >= N) return;
-    const T* qrow = phiQ + ((size_t)g * N + i) * M;
-    for (int a = lane; a < M; a += 32) qs[warp][a] = to_f32(qrow[a]);
-    __syncwarp();
-
-    float acc[NACC];
-#pragma unroll
-    for (int j = 0; j < NACC; ++j) acc[j] = 0.0f;
-    float den = 0.0f;
-
-    constexpr size_t REC = grf_record_bytes<T>(M, D);
-    const unsigned char* recs = records + (size_t)g * R * REC;
-    for (int32_t p = rowptr[i]; p < rowptr[i + 1]; ++p) {
-        const int32_t l = __ldg(col + p);
-        const float phi = __ldg(val + p);
-        const T* tile = reinterpret_cast<const T*>(recs + (size_t)l * REC);
-        const float* zl = reinterpret_cast<const float*>(recs + (size_t)l * REC + (size_t)M * D * sizeof(T));
-#pragma unroll
-        for (int x0 = 0; x0 < NCHUNK; x0 += 32) {
-            const int x = x0 + lane;
-            if (NCHUNK % 32 == 0 || x < NCHUNK) {
-                const int kc = D >= 32 ? x0 / D : x / D;
-                float s[CH];
-                Chunk<T>::load(tile + (size_t)x * CH, s);
-                float dot = 0.0f;
-#pragma unroll
-                for (int c = 0; c < CH; ++c) dot = fmaf(qs[warp][kc * CH + c], s[c], dot);
-                acc[D >= 32 ? (x0 % D) / 32 : 0] = fmaf(phi, dot, acc[D >= 32 ? (x0 % D) / 32 : 0]);
+    const unsigned char* zbase = states + (size_t)g * grf_states_stride<T>(R, M, D) + grf_z_at<T>(true, 0, R, M, D) + (size_t)pl * 16;
+    uint64_t z[2] = {0ull, 0ull};
+    const int32_t beg = rowptr[i], end = rowptr[i + 1];
+    for (int32_t p0 = beg; p0 < end; p0 += 32) {
+        const int32_t n = min(32, end - p0);
+        const int32_t my_l = lane < n ? __ldcs(col + p0 + lane) : 0;
+        const float my_phi = lane < n ? __ldcs(val + p0 + lane) : 0.0f;
+#pragma unroll 4
+        for (int32_t j = 0; j < n; j += NPS) {
+            const int32_t l = __shfl_sync(0xffffffffu, my_l, (j + sub) & 31);
+            const float phi = __shfl_sync(0xffffffffu, my_phi, (j + sub) & 31);
+            if (j + sub < n) {
+                uint64_t v[2];
+                Chunk<float>::widen(__ldg(reinterpret_cast<const uint4*>(zbase + (size_t)l * (M * 4))), v);
+                const uint64_t phi2 = pack2(phi, phi);
+                z[0] = fma2(phi2, v[0], z[0]);
+                z[1] = fma2(phi2, v[1], z[1]);
             }
         }
-        for (int a = lane; a < M; a += 32) den = fmaf(phi * qs[warp][a], __ldg(zl + a), den);
     }
-    if (D < 32) {
-        // lanes with the same column b = lane % D hold partial sums over different row chunks
+    const T* qrow = phiQ + ((size_t)g * N + i) * M + pl * 4;
+    float a[4];
+    unpack2(z[0], a[0], a[1]);
+    unpack2(z[1], a[2], a[3]);
+    float d = 0.0f;
 #pragma unroll
-        for (int off = D; off < 32; off <<= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], off);
-    }
+    for (int e = 0; e < 4; ++e) d = fmaf(Chunk<T>::get(qrow + e), a[e], d);
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
+    for (int off = 1; off < 32; off <<= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
+    if (lane == 0) den[(size_t)g * N + i] = d;
+}
 
-    const float inv = den != 0.0f ? 1.0f / den : 0.0f;
-    T* orow = out + ((size_t)g * N + i) * D;
-    if (D >= 32) {
+// Lanes of one node's slice and columns of a slice, for LANES lanes wanted and CPL chunks per lane.
+template <typename T, int M, int D, int LANES, int CPL> struct SliceShape {
+    static constexpr int CH = grf_tile_chunk<T>();
+    static constexpr int KC = M / CH;                                        // chunks along the feature rows a
+    static constexpr int LPN = KC >= LANES ? KC : (KC * D < LANES ? KC * D : LANES);
+    static constexpr int SB = LPN / KC;                                      // columns side by side
+    static constexpr int NB = SB * CPL <= D ? CPL : D / SB;                  // columns per lane
+    static constexpr int COLS = SB * NB;                                     // columns of a slice
+    static constexpr int SLICES = D / COLS;
+};
+
+// a chunk of a tile, kept in L2 in preference to the streams
+__device__ __forceinline__ uint4 load_tile(const unsigned char* p, uint64_t policy)
+{
+    uint4 x;
+    asm volatile("ld.global.nc.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
+        : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "l"(p), "l"(policy));
+    return x;
+}
+
+template <typename T, int M, int D, int LANES, int CPL>
+__global__ void __launch_bounds__(GATHER_WARPS * 32, CPL == 1 ? 16 : 6)
+gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                     const float* __restrict__ val, const T* __restrict__ phiQ, const unsigned char* __restrict__ states,
+                     T* __restrict__ out, const float* __restrict__ den)
+{
+    using Sh = SliceShape<T, M, D, LANES, CPL>;
+    constexpr int CH = Sh::CH, LPN = Sh::LPN, NPS = 32 / LPN, NB = Sh::NB, KC = Sh::KC, P = Chunk<T>::PAIRS;
+    const int lane = threadIdx.x & 31, sub = lane / LPN, pl = lane % LPN;
+    const int kc = pl % KC, b = pl / KC;                 // this lane's chunk along a, and its first column of the slice
+    const int32_t i = blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5);
+    const int32_t slice = blockIdx.y, g = blockIdx.z;
+    if (i >= N) return;
+    const int b0 = slice * Sh::COLS + b;
+    // this lane's first chunk; chunk y lies y * SB columns further on: LPN consecutive chunks per group of lanes
+    const unsigned char* base = states + (size_t)g * grf_states_stride<T>(R, M, D) + grf_chunk_at<T>(true, 0, kc * CH, b0, M, D);
+    uint64_t policy;
+    asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(policy));
+    // entries are taken 32 at a time, and the next 32 are read before these are used (streamed: the matrix is read once per
+    // slice and must not push the slice out of L2)
+    const int32_t my_rp = __ldg(rowptr + i + min(lane, 1));
+    int32_t beg = __shfl_sync(0xffffffffu, my_rp, 0);
+    const int32_t end = __shfl_sync(0xffffffffu, my_rp, 1);
+    int32_t next_l = beg + lane < end ? __ldcs(col + beg + lane) : 0;
+    float next_phi = beg + lane < end ? __ldcs(val + beg + lane) : 0.0f;
+    uint64_t acc[NB][P];
 #pragma unroll
-        for (int j = 0; j < NACC; ++j) Chunk<T>::store1(orow + j * 32 + lane, acc[j] * inv);
-    } else if (lane < D) {
-        Chunk<T>::store1(orow + lane, acc[0] * inv);
+    for (int y = 0; y < NB; ++y)
+#pragma unroll
+        for (int q = 0; q < P; ++q) acc[y][q] = 0ull;
+    while (beg < end) {
+        const int32_t n = min(32, end - beg);
+        const int32_t my_l = next_l;
+        const float my_phi = next_phi;
+        beg += n;
+        next_l = beg + lane < end ? __ldcs(col + beg + lane) : 0;
+        next_phi = beg + lane < end ? __ldcs(val + beg + lane) : 0.0f;
+        constexpr int UNROLL = NB >= 4 ? 2 : 4;
+#pragma unroll UNROLL
+        for (int32_t j = 0; j < n; j += NPS) {
+            const int32_t l = __shfl_sync(0xffffffffu, my_l, (j + sub) & 31);
+            const float phi = __shfl_sync(0xffffffffu, my_phi, (j + sub) & 31);
+            if (j + sub < n) {
+                const unsigned char* tile = base + (size_t)l * (M * D * sizeof(T));
+                const uint64_t phi2 = pack2(phi, phi);
+#pragma unroll
+                for (int y = 0; y < NB; ++y) {
+                    uint64_t v[P];
+                    Chunk<T>::widen(load_tile(tile + y * LPN * 16, policy), v);
+#pragma unroll
+                    for (int q = 0; q < P; ++q) acc[y][q] = fma2(phi2, v[q], acc[y][q]);
+                }
+            }
+        }
     }
-    if (lane == 0 && den_out) den_out[(size_t)g * N + i] = den;
+    // contract with phi(q): over this lane's rows a, then over the lanes along a and the nodes side by side
+    const T* qrow = phiQ + ((size_t)g * N + i) * M;
+    const float dn = den[(size_t)g * N + i];
+    float s[NB];
+    uint64_t qv[P];
+    Chunk<T>::widen(__ldg(reinterpret_cast<const uint4*>(qrow + kc * CH)), qv);
+#pragma unroll
+    for (int y = 0; y < NB; ++y) {
+        uint64_t t = 0ull;
+#pragma unroll
+        for (int q = 0; q < P; ++q) t = fma2(qv[q], acc[y][q], t);
+        float s1;
+        unpack2(t, s[y], s1);
+        s[y] += s1;
+    }
+    const float inv = dn != 0.0f ? 1.0f / dn : 0.0f;
+    T* orow = out + ((size_t)g * N + i) * D;
+#pragma unroll
+    for (int y = 0; y < NB; ++y) {
+#pragma unroll
+        for (int off = 1; off < KC; off <<= 1) s[y] += __shfl_xor_sync(0xffffffffu, s[y], off);
+#pragma unroll
+        for (int off = LPN; off < 32; off <<= 1) s[y] += __shfl_xor_sync(0xffffffffu, s[y], off);
+        if (sub == 0 && kc == 0) Chunk<T>::put(orow + b0 + y * Sh::SB, s[y] * inv);
+    }
+}
+
+// Bytes of a slice over all nodes that still stay in L2 beside the streams.  (Measured at 2^17 and 2^18 nodes: half of it
+// doubles the passes over the matrix, 23 -> 36 ms; twice of it misses L2, 23 -> 31 ms.)
+constexpr size_t SLICE_L2_BYTES = (size_t)72 << 20;
+
+template <typename T, int M, int D>
+int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, const void* phiQ, const void* states, void* out,
+              float* den_out)
+{
+    float* den = den_out;
+    if (!den) {
+        GRF_TRY(grf_buf_reserve(&ctx->den_scratch, sizeof(float) * (size_t)G * N));
+        den = (float*)ctx->den_scratch.ptr;
+    }
+    const int32_t* rp = (const int32_t*)phi.rowptr.ptr;
+    const int32_t* cl = (const int32_t*)phi.col.ptr;
+    const float* vl = (const float*)phi.val.ptr;
+    const int blocks = grf_ceil_div(N, GATHER_WARPS);
+    {
+        grf_launch_scope scope(ctx, 6);
+        gather_denominators_kernel<T, M, D><<<dim3(blocks, G), GATHER_WARPS * 32, 0, ctx->stream>>>(
+            N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, den);
+    }
+    grf_launch_scope scope(ctx, 5);
+    // The widest slice that fits L2: fewer passes over the matrix.
+    auto launch = [&](auto lanes, auto cpl) {
+        using Sh = SliceShape<T, M, D, decltype(lanes)::value, decltype(cpl)::value>;
+        gather_sliced_kernel<T, M, D, decltype(lanes)::value, decltype(cpl)::value>
+            <<<dim3(blocks, Sh::SLICES, G), GATHER_WARPS * 32, 0, ctx->stream>>>(
+                N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, (T*)out, den);
+    };
+    using std::integral_constant;
+    const size_t R = (size_t)phi.cols;
+    if (R * 2048 <= SLICE_L2_BYTES) launch(integral_constant<int, 32>(), integral_constant<int, 4>());
+    else if (R * 512 <= SLICE_L2_BYTES) launch(integral_constant<int, 32>(), integral_constant<int, 1>());
+    else if (R * 256 <= SLICE_L2_BYTES) launch(integral_constant<int, 16>(), integral_constant<int, 1>());
+    else launch(integral_constant<int, 8>(), integral_constant<int, 1>());
+    return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
 }
 
 template <typename T, int M>
 int launch_m(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t d,
-             const void* phiQ, const void* records, void* out, float* den_out)
+             const void* phiQ, const void* states, void* out, float* den_out)
 {
-    const dim3 grid(grf_ceil_div(N, GATHER_WARPS), G);
-#define GRF_GATHER_CASE(DD)                                                                                  \
-    case DD:                                                                                                 \
-        gather_contract_kernel<T, M, DD><<<grid, GATHER_WARPS * 32, 0, ctx->stream>>>(                       \
-            N, phi.cols, (const int32_t*)phi.rowptr.ptr, (const int32_t*)phi.col.ptr,                        \
-            (const float*)phi.val.ptr, (const T*)phiQ, (const unsigned char*)records, (T*)out, den_out);                   \
-        break;
-    {
-        grf_launch_scope scope(ctx, 5);
-        switch (d) {
-            GRF_GATHER_CASE(8) GRF_GATHER_CASE(16) GRF_GATHER_CASE(32) GRF_GATHER_CASE(64) GRF_GATHER_CASE(128)
-            default: return GRF_ERR_INVALID;
-        }
+    switch (d) {
+        case 8: return launch_md<T, M, 8>(ctx, phi, G, N, phiQ, states, out, den_out);
+        case 16: return launch_md<T, M, 16>(ctx, phi, G, N, phiQ, states, out, den_out);
+        case 32: return launch_md<T, M, 32>(ctx, phi, G, N, phiQ, states, out, den_out);
+        case 64: return launch_md<T, M, 64>(ctx, phi, G, N, phiQ, states, out, den_out);
+        case 128: return launch_md<T, M, 128>(ctx, phi, G, N, phiQ, states, out, den_out);
+        default: return GRF_ERR_INVALID;
     }
-#undef GRF_GATHER_CASE
-    return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
 }
 
 template <typename T>
 int launch_t(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t m, int32_t d,
-             const void* phiQ, const void* records, void* out, float* den_out)
+             const void* phiQ, const void* states, void* out, float* den_out)
 {
     switch (m) {
-        case 8: return launch_m<T, 8>(ctx, phi, G, N, d, phiQ, records, out, den_out);
-        case 16: return launch_m<T, 16>(ctx, phi, G, N, d, phiQ, records, out, den_out);
-        case 32: return launch_m<T, 32>(ctx, phi, G, N, d, phiQ, records, out, den_out);
-        case 64: return launch_m<T, 64>(ctx, phi, G, N, d, phiQ, records, out, den_out);
-        case 128: return launch_m<T, 128>(ctx, phi, G, N, d, phiQ, records, out, den_out);
+        case 8: return launch_m<T, 8>(ctx, phi, G, N, d, phiQ, states, out, den_out);
+        case 16: return launch_m<T, 16>(ctx, phi, G, N, d, phiQ, states, out, den_out);
+        case 32: return launch_m<T, 32>(ctx, phi, G, N, d, phiQ, states, out, den_out);
+        case 64: return launch_m<T, 64>(ctx, phi, G, N, d, phiQ, states, out, den_out);
+        case 128: return launch_m<T, 128>(ctx, phi, G, N, d, phiQ, states, out, den_out);
         default: return GRF_ERR_INVALID;
     }
 }
@@ -141,10 +274,10 @@ int launch_t(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t
 }  // namespace
 
 int grf_gather_contract_alu(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t m, int32_t d,
-                            int dtype, const void* phiQ, const void* records, void* out, float* den_out)
+                            int dtype, const void* phiQ, const void* states, void* out, float* den_out)
 {
     if (G > 65535) return GRF_ERR_TOO_LARGE;
-    if (dtype == GRF_DTYPE_F32) return launch_t<float>(ctx, phi, G, N, m, d, phiQ, records, out, den_out);
-    if (dtype == GRF_DTYPE_BF16) return launch_t<__nv_bfloat16>(ctx, phi, G, N, m, d, phiQ, records, out, den_out);
+    if (dtype == GRF_DTYPE_F32) return launch_t<float>(ctx, phi, G, N, m, d, phiQ, states, out, den_out);
+    if (dtype == GRF_DTYPE_BF16) return launch_t<__nv_bfloat16>(ctx, phi, G, N, m, d, phiQ, states, out, den_out);
     return GRF_ERR_INVALID;
 }

@@ -93,9 +93,9 @@ __device__ __forceinline__ void state_mma_issuer(int32_t nnodes, const int32_t* 
 template <int M, int D, int ACC_COLS>
 __device__ __forceinline__ void state_epilogue(int warp, int lane, int32_t g, int32_t R, int32_t l0, int32_t l1,
                                                uint32_t acc_full0, uint32_t acc_free0, uint32_t tmem_base,
-                                               volatile int* abort_flag, unsigned char* __restrict__ records)
+                                               volatile int* abort_flag, unsigned char* __restrict__ states, bool by_column)
 {
-    constexpr size_t REC = grf_record_bytes<__nv_bfloat16>(M, D);
+    unsigned char* base = states + (size_t)g * grf_states_stride<__nv_bfloat16>(R, M, D);
     const int row = warp * 32 + lane;                   // accumulator row = TMEM lane
     const bool warp_has_rows = warp * 32 <= D;          // S rows 0..D-1 and the z row D
     int32_t nn = 0;
@@ -107,9 +107,7 @@ __device__ __forceinline__ void state_epilogue(int warp, int lane, int32_t g, in
         if (!ok) break;
         fence_after_sync();
         if (warp_has_rows) {
-            unsigned char* rec = records + ((size_t)g * R + l) * REC;
-            __nv_bfloat16* tile = reinterpret_cast<__nv_bfloat16*>(rec);
-            float* zl = reinterpret_cast<float*>(rec + (size_t)M * D * 2);
+            float* zl = reinterpret_cast<float*>(base + grf_z_at<__nv_bfloat16>(by_column, l, R, M, D));
             const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * ACC_COLS);
 #pragma unroll
             for (int c0 = 0; c0 < M; c0 += 16) {
@@ -126,7 +124,7 @@ __device__ __forceinline__ void state_epilogue(int warp, int lane, int32_t g, in
                                                                       __uint_as_float(r[8 * half + 2 * e + 1]));
                             w[e] = *reinterpret_cast<uint32_t*>(&t2);
                         }
-                        *reinterpret_cast<uint4*>(tile + grf_tile_index<__nv_bfloat16>(c0 + 8 * half, row, D)) =
+                        *reinterpret_cast<uint4*>(base + grf_chunk_at<__nv_bfloat16>(by_column, l, c0 + 8 * half, row, M, D)) =
                             make_uint4(w[0], w[1], w[2], w[3]);
                     }
                 } else if (row == D) {
@@ -134,6 +132,7 @@ __device__ __forceinline__ void state_epilogue(int warp, int lane, int32_t g, in
                     for (int e = 0; e < 16; e += 4)
                         *reinterpret_cast<float4*>(zl + c0 + e) = make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]),
                                                                               __uint_as_float(r[e + 2]), __uint_as_float(r[e + 3]));
+                    if (by_column) continue;
                     // and once more in bf16, for the denominators kernel
                     uint32_t zw[8];
 #pragma unroll
@@ -141,7 +140,7 @@ __device__ __forceinline__ void state_epilogue(int warp, int lane, int32_t g, in
                         __nv_bfloat162 t2 = __floats2bfloat162_rn(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1]));
                         zw[e] = *reinterpret_cast<uint32_t*>(&t2);
                     }
-                    uint4* zb = reinterpret_cast<uint4*>(rec + (size_t)M * D * 2 + (size_t)M * 4 + (size_t)c0 * 2);
+                    uint4* zb = reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(zl) + (size_t)M * 4 + (size_t)c0 * 2);
                     zb[0] = make_uint4(zw[0], zw[1], zw[2], zw[3]);
                     zb[1] = make_uint4(zw[4], zw[5], zw[6], zw[7]);
                 }
@@ -157,8 +156,8 @@ template <int M, int D>
 __global__ void __launch_bounds__(ST_THREADS)
 build_states_tc_kernel(int32_t R, int32_t N, const int32_t* __restrict__ t_rowptr, const int32_t* __restrict__ t_col,
                        const float* __restrict__ t_val, const __nv_bfloat16* __restrict__ phiK,
-                       const __nv_bfloat16* __restrict__ V, unsigned char* __restrict__ records,
-                       int* __restrict__ error_word)
+                       const __nv_bfloat16* __restrict__ V, unsigned char* __restrict__ states,
+                       bool by_column, int* __restrict__ error_word)
 {
     using Sh = StShape<M, D>;
     constexpr int NS = Sh::NS;
@@ -325,7 +324,7 @@ build_states_tc_kernel(int32_t R, int32_t N, const int32_t* __restrict__ t_rowpt
         });
     } else {
         // ------------------------------------------------------------ epilogue: accumulator -> record
-        state_epilogue<M, D, Sh::ACC_COLS>(warp, lane, g, R, l0, l1, acc_full(0), acc_free(0), tmem_base, &abort_flag, records);
+        state_epilogue<M, D, Sh::ACC_COLS>(warp, lane, g, R, l0, l1, acc_full(0), acc_free(0), tmem_base, &abort_flag, states, by_column);
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -338,7 +337,7 @@ build_states_tc_kernel(int32_t R, int32_t N, const int32_t* __restrict__ t_rowpt
 
 template <int M, int D>
 int launch_state_tc(grf_ctx* ctx, const grf_csr_dev& psit, int32_t G, int32_t N, const void* phiK, const void* V,
-                    void* records)
+                    void* states, bool by_column)
 {
     using Sh = StShape<M, D>;
     GRF_CUDA_TRY(cudaFuncSetAttribute(build_states_tc_kernel<M, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::SMEM));
@@ -347,7 +346,7 @@ int launch_state_tc(grf_ctx* ctx, const grf_csr_dev& psit, int32_t G, int32_t N,
         grf_launch_scope scope(ctx, 4);
         build_states_tc_kernel<M, D><<<grid, ST_THREADS, Sh::SMEM, ctx->stream>>>(
             psit.rows, N, (const int32_t*)psit.rowptr.ptr, (const int32_t*)psit.col.ptr, (const float*)psit.val.ptr,
-            (const __nv_bfloat16*)phiK, (const __nv_bfloat16*)V, (unsigned char*)records, ctx->error_word);
+            (const __nv_bfloat16*)phiK, (const __nv_bfloat16*)V, (unsigned char*)states, by_column, ctx->error_word);
     }
     return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
 }
@@ -383,8 +382,8 @@ template <int M>
 __global__ void __launch_bounds__(ST_THREADS)
 build_states_tma_kernel(int32_t R, int32_t N, const int32_t* __restrict__ t_rowptr, const int32_t* __restrict__ t_col,
                         const float* __restrict__ t_val, const __nv_bfloat16* __restrict__ phiK,
-                        const __grid_constant__ CUtensorMap map_v, unsigned char* __restrict__ records,
-                        int* __restrict__ error_word)
+                        const __grid_constant__ CUtensorMap map_v, unsigned char* __restrict__ states,
+                        bool by_column, int* __restrict__ error_word)
 {
     using Sh = TmaShape<M>;
     constexpr int NS = Sh::NS, D = Sh::D;
@@ -550,7 +549,7 @@ build_states_tma_kernel(int32_t R, int32_t N, const int32_t* __restrict__ t_rowp
         });
     } else {
         // ------------------------------------------------------------ epilogue: accumulator -> record
-        state_epilogue<M, D, Sh::ACC_COLS>(warp, lane, g, R, l0, l1, acc_full(0), acc_free(0), tmem_base, &abort_flag, records);
+        state_epilogue<M, D, Sh::ACC_COLS>(warp, lane, g, R, l0, l1, acc_full(0), acc_free(0), tmem_base, &abort_flag, states, by_column);
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -564,7 +563,7 @@ build_states_tma_kernel(int32_t R, int32_t N, const int32_t* __restrict__ t_rowp
 // 1 when the tensor maps cannot be made (the caller then takes the kernel above)
 template <int M>
 int launch_state_tma(grf_ctx* ctx, const grf_csr_dev& psit, int32_t G, int32_t N, const void* phiK, const void* V,
-                     void* records)
+                     void* states, bool by_column)
 {
     using Sh = TmaShape<M>;
     if ((int64_t)G * N > 0x7fffffffll) return 1;
@@ -576,7 +575,7 @@ int launch_state_tma(grf_ctx* ctx, const grf_csr_dev& psit, int32_t G, int32_t N
         grf_launch_scope scope(ctx, 4);
         build_states_tma_kernel<M><<<grid, ST_THREADS, Sh::SMEM, ctx->stream>>>(
             psit.rows, N, (const int32_t*)psit.rowptr.ptr, (const int32_t*)psit.col.ptr, (const float*)psit.val.ptr,
-            (const __nv_bfloat16*)phiK, map_v, (unsigned char*)records, ctx->error_word);
+            (const __nv_bfloat16*)phiK, map_v, (unsigned char*)states, by_column, ctx->error_word);
     }
     return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
 }
@@ -585,17 +584,17 @@ int launch_state_tma(grf_ctx* ctx, const grf_csr_dev& psit, int32_t G, int32_t N
 
 // Returns GRF_OK after launching, or 1 when this shape has no tensor-core path (the caller falls back).
 int grf_build_states_tc(grf_ctx* ctx, const grf_csr_dev& psit, int32_t G, int32_t N, int32_t m, int32_t d,
-                        const void* phiK, const void* V, void* records)
+                        const void* phiK, const void* V, void* states, bool by_column)
 {
     if (G > 65535) return 1;
     if (d == 64 && (m == 16 || m == 32 || m == 64)) {
-        const int rc = m == 16 ? launch_state_tma<16>(ctx, psit, G, N, phiK, V, records)
-                     : m == 32 ? launch_state_tma<32>(ctx, psit, G, N, phiK, V, records)
-                               : launch_state_tma<64>(ctx, psit, G, N, phiK, V, records);
+        const int rc = m == 16 ? launch_state_tma<16>(ctx, psit, G, N, phiK, V, states, by_column)
+                     : m == 32 ? launch_state_tma<32>(ctx, psit, G, N, phiK, V, states, by_column)
+                               : launch_state_tma<64>(ctx, psit, G, N, phiK, V, states, by_column);
         if (rc != 1) return rc;
     }
 #define GRF_ST_CASE(MM, DD) \
-    if (m == MM && d == DD) return launch_state_tc<MM, DD>(ctx, psit, G, N, phiK, V, records);
+    if (m == MM && d == DD) return launch_state_tc<MM, DD>(ctx, psit, G, N, phiK, V, states, by_column);
     GRF_ST_CASE(16, 16) GRF_ST_CASE(16, 32) GRF_ST_CASE(16, 64)
     GRF_ST_CASE(32, 16) GRF_ST_CASE(32, 32) GRF_ST_CASE(32, 64)
     GRF_ST_CASE(64, 16) GRF_ST_CASE(64, 32) GRF_ST_CASE(64, 64)

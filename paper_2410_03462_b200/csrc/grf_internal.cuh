@@ -161,12 +161,13 @@ int grf_transpose_launch(grf_ctx* ctx, int32_t rows, int32_t cols, int64_t nnz,
                          int32_t* t_rowptr, int32_t* t_col, float* t_val);
 
 // attn_state.cu / attn_gather.cu
+// by_column: the states in the ALU gather's layout (below) instead of the tensor-core gather's records
 int grf_build_states(grf_ctx* ctx, const grf_csr_dev& psit, int32_t G, int32_t N, int32_t m, int32_t d, int dtype,
-                     const void* phiK, const void* V, void* records);
+                     const void* phiK, const void* V, void* states, bool by_column);
 int grf_build_states_tc(grf_ctx* ctx, const grf_csr_dev& psit, int32_t G, int32_t N, int32_t m, int32_t d,
-                        const void* phiK, const void* V, void* records);
+                        const void* phiK, const void* V, void* states, bool by_column);
 int grf_gather_contract_alu(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t m, int32_t d,
-                            int dtype, const void* phiQ, const void* records, void* out, float* den_out);
+                            int dtype, const void* phiQ, const void* states, void* out, float* den_out);
 // attn_mhat.cu
 void grf_mask_invalidate(grf_features* feat);
 void grf_mask_values_stale(grf_features* feat);
@@ -179,25 +180,44 @@ void grf_mask_release(grf_features* feat);
 // attn_gather_tc.cu
 int grf_build_block_plan(grf_ctx* ctx, grf_features* feat, bool with_coef = true);
 int grf_ensure_block_plan(grf_ctx* ctx, const grf_features* feat, bool with_coef = true);   // builds it if Phi changed since the last build
+// Which gather serves this object and shape (prepares the block plan it needs).
+int grf_gather_by_tensor_cores(grf_ctx* ctx, const grf_features* feat, int32_t m, int32_t d, int dtype, bool* yes);
 int grf_gather_contract_tc(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d,
                            const void* phiQ, const void* records, void* out, float* den_out);
 
-// Layout of one state tile S_l (m x d) inside the workspace: 16-byte chunks that hold CH consecutive feature
-// rows a of one column b, ordered [a / CH][b][a % CH].  With bf16 (CH = 8) this is the K-major, unswizzled
-// shared-memory operand layout of the tensor-core gather kernel (8-row core matrices of 128 contiguous
-// bytes), so a tile is brought in with one contiguous bulk copy; the ALU kernels read the same chunks.
+// Where the states of one problem lie inside the workspace; R nodes, E = bytes of an element of T.
+//
+// For the tensor-core gather: one record per node, the state tile S_l (m x d), then z_l (m fp32 values), then z_l once more
+// in bf16 (the denominators kernel reads that copy: half the bytes per (query, node) pair).  The tile is made of 16-byte
+// chunks that hold 8 consecutive feature rows a of one column b, ordered [a / 8][b][a % 8]: the K-major, unswizzled
+// shared-memory operand layout (8-row core matrices of 128 contiguous bytes), so a tile is brought in with one contiguous
+// bulk copy.
+//
+// For the ALU gather (by column): all tiles first, each [b][a] so that any range of columns is contiguous, then all z_l in
+// fp32; tiles and z_l start on whole cache lines.
+//
+// Both fit the R * (m d E + 4 m (+ 2 m with bf16)) bytes that a problem's workspace has.
 template <typename T> __host__ __device__ constexpr int grf_tile_chunk() { return 16 / (int)sizeof(T); }
-template <typename T> __host__ __device__ constexpr size_t grf_tile_index(int a, int b, int D)
-{
-    return ((size_t)(a / grf_tile_chunk<T>()) * D + b) * grf_tile_chunk<T>() + (a % grf_tile_chunk<T>());
-}
-
-// The workspace holds one record per (problem, node): the state tile S_l, then z_l (m fp32 values) and, with
-// bf16 storage, z_l once more rounded to bf16 (the denominators kernel of the tensor-core path reads that copy:
-// half the bytes per (query, node) pair).
 template <typename T> __host__ __device__ constexpr size_t grf_record_bytes(int M, int D)
 {
     return (size_t)M * D * sizeof(T) + (size_t)M * sizeof(float) + (sizeof(T) == 2 ? (size_t)M * 2 : 0);
+}
+// bytes from one problem's states to the next one's
+template <typename T> __host__ __device__ constexpr size_t grf_states_stride(size_t R, int M, int D)
+{
+    return (R * grf_record_bytes<T>(M, D) + 255) & ~(size_t)255;
+}
+// tile chunk holding feature rows a .. a + 7 (fp32: a + 3) of column b, and z_l, of node l
+template <typename T> __host__ __device__ constexpr size_t grf_chunk_at(bool by_column, size_t l, int a, int b, int M, int D)
+{
+    constexpr int CH = grf_tile_chunk<T>();
+    return by_column ? l * ((size_t)M * D * sizeof(T)) + ((size_t)b * M + a) * sizeof(T)
+                     : l * grf_record_bytes<T>(M, D) + ((size_t)(a / CH) * D + b) * 16;
+}
+template <typename T> __host__ __device__ constexpr size_t grf_z_at(bool by_column, size_t l, size_t R, int M, int D)
+{
+    return by_column ? R * ((size_t)M * D * sizeof(T)) + l * ((size_t)M * sizeof(float))
+                     : l * grf_record_bytes<T>(M, D) + (size_t)M * D * sizeof(T);
 }
 
 static inline int grf_ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }

@@ -39,3 +39,41 @@ def test_both_routes_match_oracle(N, G, m):
         api.masked_attn_mhat(ctx, feat, qd, kd, vd)
     feat.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("R,m,d", [(300, 32, 64), (36863, 32, 64), (36865, 128, 8), (147457, 16, 32), (294913, 8, 16)])
+def test_sliced_gather_widths(R, m, d, dtype):
+    """The plain-ALU gather takes tiles whole or in slices of 512, 256 or 128 bytes by the number of nodes: rows of Phi
+    with 0, 1, 31, 32, 33 and 70 non-zeros over few and many nodes."""
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    rng = np.random.default_rng(R + m)
+    N, G = 67, 2
+
+    def csr(lengths):
+        cols = [np.sort(rng.choice(R, size=n, replace=False)) for n in lengths]
+        rp = np.concatenate([[0], np.cumsum([len(c) for c in cols])]).astype(np.int32)
+        c = np.concatenate(cols).astype(np.int32)
+        return oracle.CSR(rp, c, rng.uniform(0.1, 1.0, c.size).astype(np.float32), None, (N, R))
+
+    Phi = csr([(0, 1, 31, 32, 33, 70)[i % 6] for i in range(N)])
+    # every node that a row of Phi touches has keys
+    keys = np.tile(np.unique(Phi.col), 2)
+    Psi = csr([3] * N)
+    Psi.col[:] = np.sort(rng.choice(np.unique(keys), size=(N, 3)), axis=1).ravel()
+    dup = [i for i in range(N) if len(set(Psi.col[3 * i:3 * i + 3])) < 3]
+    for i in dup:
+        Psi.col[3 * i:3 * i + 3] = np.sort(np.unique(keys)[[0, 5, 9]])
+    PsiT = oracle.transpose(Psi)
+    feat = api.features_from_csr(ctx, N, R, (Phi.rowptr, Phi.col, Phi.val), (Psi.rowptr, Psi.col, Psi.val))
+    q, k, v = tensors.qkv(G, N, m, d, dtype, 5)
+    q = (q.float() + 0.1).to(q.dtype)
+    k = (k.float() + 0.1).to(k.dtype)
+    ref = oracle.attn_sparse(tensors.widen(q), tensors.widen(k), tensors.widen(v), Phi, PsiT)
+    B.grf_ctx_use_tensor_cores(ctx.handle, 0)
+    out, den = api.masked_linear_attn(ctx, feat, q.cuda(), k.cuda(), v.cuda(), want_den=True)
+    B.grf_ctx_check(ctx.handle)
+    helpers.assert_attn_close(out.float().cpu().numpy(), ref, helpers.TOL[dtype], den.cpu().numpy(), f"R={R}", min_ok=0.3)
+    feat.free()
+    ctx.close()
