@@ -61,7 +61,7 @@ extern "C" int grf_ctx_destroy(grf_ctx* ctx)
     if (!ctx) return GRF_ERR_INVALID;
     cudaSetDevice(ctx->device);
     cudaStreamSynchronize(ctx->stream);
-    grf_buf* bufs[] = {&ctx->stage_col, &ctx->stage_val, &ctx->counts, &ctx->rowptr2, &ctx->scan_blocks,
+    grf_buf* bufs[] = {&ctx->edge_records, &ctx->stage_col, &ctx->stage_val, &ctx->counts, &ctx->rowptr2, &ctx->scan_blocks,
                        &ctx->stage_dep_start, &ctx->stage_dep_t, &ctx->stage_dep_load, &ctx->dep_counts, &ctx->dep_rowptr2,
                        &ctx->t_cursor, &ctx->t_tmp_col, &ctx->t_tmp_val, &ctx->den_scratch, &ctx->h_rowptr, &ctx->h_col, &ctx->h_w,
                        &ctx->h_q, &ctx->h_k, &ctx->h_v, &ctx->h_out, &ctx->h_ws};

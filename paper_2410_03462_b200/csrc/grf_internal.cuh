@@ -34,6 +34,7 @@ struct grf_ctx {
     int64_t launches = 0;
     // sampler scratch
     grf_buf stage_col, stage_val;   // merged rows at a fixed stride, before compaction
+    grf_buf edge_records;           // the graph's edges as the walks read them
     grf_buf counts;                 // per-row nonzero counts (both matrices)
     grf_buf rowptr2;                // scanned counts, [2][N+1]
     grf_buf scan_blocks;            // block totals of the two-level scan
@@ -143,6 +144,7 @@ struct grf_walk_params {
     float inv_keep, inv_n;
     int32_t cap;        // n_walks * (max_len + 1)
     int32_t seq_bits;   // ceil(log2(cap)), at least 1
+    int32_t last_step[2];   // last step with a non-zero coefficient, per ensemble: no walk goes further
     float f[2][GRF_MAX_WALK_LEN + 1];
 };
 int grf_walk_params_init(grf_walk_params* p, int32_t N, uint64_t seed, int32_t n_walks, float p_halt,

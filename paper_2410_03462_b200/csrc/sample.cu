@@ -33,71 +33,157 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t
     out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
 }
 
-// State of one walker; `advance` takes the hop after step t (halting coin first).
-struct Walker {
-    int32_t v;
-    float load;
-    uint32_t words[4];
-    bool alive;
+// factor of the load for a hop along an edge of weight w out of a node of degree deg (Eq. 9)
+__device__ __forceinline__ float hop_weight(float w, int32_t deg, float inv_keep)
+{
+    return __fmul_rn(__fmul_rn(w, (float)deg), inv_keep);
+}
 
-    __device__ __forceinline__ void advance(const grf_walk_params& P, const int32_t* __restrict__ rowptr,
-                                            const int32_t* __restrict__ col, const float* __restrict__ w,
-                                            int32_t e, int32_t i, int32_t k, int32_t t)
+// State of one walker.
+struct Walker {
+    int32_t v, beg, deg;     // where it stands, and that node's edges
+    float load;
+
+    // by the records of edge_records_kernel: one gather
+    __device__ __forceinline__ void hop(uint32_t r_next, const int4* __restrict__ edges)
     {
-        if ((t & 1) == 0)
-            philox4x32_10((uint32_t)i, (uint32_t)k, (uint32_t)(t >> 1), (uint32_t)e, P.key0, P.key1, words);
-        const uint32_t r_halt = (t & 1) ? words[2] : words[0];
-        const uint32_t r_next = (t & 1) ? words[3] : words[1];
-        if (r_halt < P.halt_threshold) { alive = false; return; }
-        const int32_t beg = __ldg(rowptr + v);
-        const int32_t deg = __ldg(rowptr + v + 1) - beg;
-        if (deg == 0) { alive = false; return; }
+        const int4 r = __ldg(edges + (beg + (int32_t)__umulhi(r_next, (uint32_t)deg)));
+        v = r.x; load = __fmul_rn(load, __int_as_float(r.y)); beg = r.z; deg = r.w;
+    }
+    // by the CSR arrays: four
+    __device__ __forceinline__ void hop(uint32_t r_next, const grf_walk_params& P, const int32_t* __restrict__ rowptr,
+                                        const int32_t* __restrict__ col, const float* __restrict__ w)
+    {
         const int32_t eidx = beg + (int32_t)__umulhi(r_next, (uint32_t)deg);
-        float step = __fmul_rn(__ldg(w + eidx), (float)deg);
-        step = __fmul_rn(step, P.inv_keep);
-        load = __fmul_rn(load, step);
+        load = __fmul_rn(load, hop_weight(__ldg(w + eidx), deg, P.inv_keep));
         v = __ldg(col + eidx);
+        beg = __ldg(rowptr + v);
+        deg = __ldg(rowptr + v + 1) - beg;
     }
 };
 
-// Bitonic sort of 32 * E keys held E per lane (key x = lane * E + r sits in register r of its lane): partners
-// closer than E are registers of the same lane, the others are reached with one shuffle.  Same network as
-// the shared-memory loop it replaces, so the result is the same sorted row.
+// One 16-byte record per edge u -> v: v, the factor of the hop's load, and where v's own edges are.  A hop of a warp's 32
+// walkers then costs one gather instead of four, and fewer instructions.  Eight lanes per row.
+__global__ void __launch_bounds__(256)
+edge_records_kernel(int32_t N, int64_t room, float inv_keep, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                    const float* __restrict__ w, int4* __restrict__ edges)
+{
+    if (rowptr[N] > room) return;
+    const int32_t u = blockIdx.x * 32 + (threadIdx.x >> 3);
+    if (u >= N) return;
+    const int32_t beg = rowptr[u], end = rowptr[u + 1];
+    for (int32_t p = beg + (threadIdx.x & 7); p < end; p += 8) {
+        const int32_t v = col[p], vb = rowptr[v];
+        edges[p] = make_int4(v, __float_as_int(hop_weight(w[p], end - beg, inv_keep)), vb, rowptr[v + 1] - vb);
+    }
+}
+
+// the smaller of v and x, or the larger where `larger` is set: one comparison, one selection
+__device__ __forceinline__ uint32_t min_or_max(uint32_t v, uint32_t x, bool larger)
+{
+    uint32_t r;
+    asm("{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %3, 0;\n\t"
+        "setp.lt.xor.u32 p, %1, %2, q;\n\t"
+        "selp.u32 %0, %1, %2, p;\n\t}"
+        : "=r"(r) : "r"(v), "r"(x), "r"((uint32_t)larger));
+    return r;
+}
+
+// Bitonic sort of 32 * E keys held E per lane (key x = lane * E + r sits in register r of its lane): partners closer than E
+// are registers of the same lane, the others are reached with one shuffle.  Every merge starts by comparing x with its
+// mirror image in the block, so all comparators point the same way: two instructions per pair in a lane, three per key
+// across lanes.
+//
+// Then, from the same registers, the places among the first cnt keys where a new column (key >> seq_bits) begins: written
+// in order to heads, their number returned.
 template <int E>
-__device__ __forceinline__ void sort_in_registers(uint32_t* keys, int lane)
+__device__ __forceinline__ int32_t sort_in_registers(uint32_t* keys, int lane, int32_t cnt, int32_t seq_bits,
+                                                     unsigned short* heads)
 {
     uint32_t v[E];
 #pragma unroll
-    for (int r = 0; r < E; ++r) v[r] = keys[lane * E + r];
+    for (int r = 0; r < E; ++r) v[r] = keys[r * 32 + lane];          // any order will do
 #pragma unroll
     for (int k = 2; k <= 32 * E; k <<= 1) {
+        if (k <= E) {
 #pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            if (j >= E) {
-                const int lj = j / E;
-                const bool keep_min = ((lane & lj) == 0) == (((lane * E) & k) == 0);
-#pragma unroll
-                for (int r = 0; r < E; ++r) {
-                    const uint32_t p = __shfl_xor_sync(0xffffffffu, v[r], lj);
-                    v[r] = keep_min ? min(v[r], p) : max(v[r], p);
+            for (int r = 0; r < E; ++r)
+                if ((r & (k >> 1)) == 0) {
+                    const int x = r ^ (k - 1);
+                    const uint32_t mn = min(v[r], v[x]), mx = max(v[r], v[x]);
+                    v[r] = mn; v[x] = mx;
                 }
+        } else {
+            const int lm = k / E - 1;                                 // mirrored lane, mirrored register
+            const bool larger = (lane & (k / E / 2)) != 0;
+            uint32_t p[E];
+#pragma unroll
+            for (int r = 0; r < E; ++r) p[r] = __shfl_xor_sync(0xffffffffu, v[E - 1 - r], lm);
+#pragma unroll
+            for (int r = 0; r < E; ++r) v[r] = min_or_max(v[r], p[r], larger);
+        }
+#pragma unroll
+        for (int j = k >> 2; j > 0; j >>= 1) {
+            if (j >= E) {
+                const bool larger = (lane & (j / E)) != 0;
+#pragma unroll
+                for (int r = 0; r < E; ++r) v[r] = min_or_max(v[r], __shfl_xor_sync(0xffffffffu, v[r], j / E), larger);
             } else {
 #pragma unroll
-                for (int r = 0; r < E; ++r) {
+                for (int r = 0; r < E; ++r)
                     if ((r & j) == 0) {
-                        const bool up = k < E ? (r & k) == 0 : ((lane * E) & k) == 0;
                         const uint32_t mn = min(v[r], v[r | j]), mx = max(v[r], v[r | j]);
-                        v[r] = up ? mn : mx;
-                        v[r | j] = up ? mx : mn;
+                        v[r] = mn; v[r | j] = mx;
                     }
-                }
             }
         }
     }
+    __syncwarp();
 #pragma unroll
     for (int r = 0; r < E; ++r) keys[lane * E + r] = v[r];
+    uint32_t before = __shfl_up_sync(0xffffffffu, v[E - 1], 1) >> seq_bits;
+    if (lane == 0) before = 0xffffffffu;                    // no column is that large: the first key is a head
+    uint32_t head = 0;
+    int32_t mine = 0;
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        const uint32_t c = v[r] >> seq_bits;
+        if (c != before && lane * E + r < cnt) { head |= 1u << r; ++mine; }
+        before = c;
+    }
+    int32_t inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    int32_t at = inc - mine;
+#pragma unroll
+    for (int r = 0; r < E; ++r)
+        if (head >> r & 1u) heads[at++] = (unsigned short)(lane * E + r);
+    return __shfl_sync(0xffffffffu, inc, 31);
 }
 
+// shared memory of one warp: keys, the deposits' values by sequence number, the starts of the distinct columns
+__host__ __device__ __forceinline__ size_t walk_smem_bytes(int32_t key_slots, int32_t cap)
+{
+    return ((size_t)key_slots * 4 + (size_t)cap * 4 + (size_t)key_slots * 2 + 15) & ~(size_t)15;
+}
+
+// One warp per row; what bounds it is instruction issue, the ALU pipe first (2 290 warp instructions per row of 240
+// deposits: hops 650, Philox 360, sort 680, sums 600).
+//   walks   lanes are walkers, all at the same step; one block of random words serves two hops, a hop is one gather (the
+//           records above), and steps behind the last non-zero coefficient are not taken.
+//   sort    the deposits' keys (column, walk, step).  The first deposit of every walk lies at the source, so without
+//           KEEP only walk 0's is sorted (it holds the source's place in the row): 32 walks of a cloud leave 208 keys
+//           instead of 240, which fit the 256-key network.
+//   sums    the distinct columns are found first, then every lane adds one column's deposits in sorted order (the
+//           source's first deposits are added where their walk begins), so a column with many deposits delays 31 others
+//           once, not once per 32 deposits.
+// N = 20011 cloud (40 022 rows, 32 walks of up to 12 hops): 200 us before these three, 130 with them.  (Sums over values laid
+// out in sorted order first, which spares the key look-ups, cost as much as they saved.)
+//
 // KEEP: the row's deposits themselves are kept as well (for grf_remodulate): every prefix deposits whatever its
 // coefficient, the sorted list of (step, load) pairs of the row goes to a staging area of stride P.cap, and every
 // merged entry records where its deposits begin in that list.  The values are computed by the same operations in
@@ -105,8 +191,7 @@ __device__ __forceinline__ void sort_in_registers(uint32_t* keys, int lane)
 template <bool KEEP>
 __global__ void __launch_bounds__(256)
 walk_merge_kernel(const __grid_constant__ grf_walk_params P,
-                  const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, const float* __restrict__ w,
-                  int32_t stage_stride, int32_t* __restrict__ stage_col, float* __restrict__ stage_val,
+                  const int32_t* __restrict__ rowptr, const int4* __restrict__ edges, int64_t edge_room, int32_t stage_stride, int32_t* __restrict__ stage_col, float* __restrict__ stage_val,
                   int32_t* __restrict__ counts,
                   int32_t* __restrict__ stage_dep_start, unsigned char* __restrict__ stage_dep_t,
                   float* __restrict__ stage_dep_load, int32_t* __restrict__ dep_counts)
@@ -116,36 +201,63 @@ walk_merge_kernel(const __grid_constant__ grf_walk_params P,
     const int warp = threadIdx.x >> 5;
     const int warps = blockDim.x >> 5;
     const int32_t row = blockIdx.x * warps + warp;
-    if (row >= 2 * P.N) return;
+    if (row >= 2 * P.N || __ldg(rowptr + P.N) > edge_room) return;      // no records: the host makes room and comes again
     const int32_t e = row >= P.N ? 1 : 0;
     const int32_t i = row - e * P.N;
 
     const int32_t key_slots = max(32, 1 << P.seq_bits);   // the sort pads a row to at least one key per lane
-    uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw) + (size_t)warp * (key_slots + P.cap);
+    unsigned char* mine = smem_raw + (size_t)warp * walk_smem_bytes(key_slots, P.cap);
+    uint32_t* keys = reinterpret_cast<uint32_t*>(mine);
     float* vals = reinterpret_cast<float*>(keys + key_slots);
+    unsigned short* heads = reinterpret_cast<unsigned short*>(vals + P.cap);
     const uint32_t lt_mask = (1u << lane) - 1u;
     const int32_t Lp1 = P.max_len + 1;
+    const int32_t steps = KEEP ? P.max_len : P.last_step[e];
+    // value of a deposit before the first hop: (f_0 * 1) / n
+    const float first = __fmul_rn(__fmul_rn(P.f[e][0], 1.0f), P.inv_n);
+    const bool at_source = !KEEP && P.f[e][0] != 0.0f;
+
+    const int32_t src_beg = __ldg(rowptr + i), src_deg = __ldg(rowptr + i + 1) - src_beg;
 
     // ---- walks: lanes are walkers, all at the same step t
     int32_t cnt = 0;
+    if (at_source) {
+        if (lane == 0) keys[0] = (uint32_t)i << P.seq_bits;
+        cnt = 1;
+    }
     for (int32_t k0 = 0; k0 < P.n_walks; k0 += 32) {
         const int32_t k = k0 + lane;
         Walker wk;
-        wk.v = i; wk.load = 1.0f; wk.alive = k < P.n_walks;
-        wk.words[0] = wk.words[1] = wk.words[2] = wk.words[3] = 0;
-        for (int32_t t = 0;; ++t) {
+        wk.v = i; wk.beg = src_beg; wk.deg = src_deg; wk.load = 1.0f;
+        bool alive = k < P.n_walks;
+        float* my_vals = vals + k * Lp1;
+        uint32_t word_key = (uint32_t)(k * Lp1);                 // the deposit's sequence number
+        auto deposit = [&](int32_t t, uint32_t mask) {
             const float ft = P.f[e][t];
-            const bool dep = wk.alive && (KEEP || ft != 0.0f);
-            const uint32_t dm = __ballot_sync(0xffffffffu, dep);
-            if (dep) {
-                const int32_t seq = k * Lp1 + t;
-                keys[cnt + __popc(dm & lt_mask)] = ((uint32_t)wk.v << P.seq_bits) | (uint32_t)seq;
-                vals[seq] = KEEP ? wk.load : __fmul_rn(__fmul_rn(ft, wk.load), P.inv_n);
+            if (KEEP || ft != 0.0f) {
+                if (alive) {
+                    keys[cnt + __popc(mask & lt_mask)] = ((uint32_t)wk.v << P.seq_bits) | (word_key + (uint32_t)t);
+                    my_vals[t] = KEEP ? wk.load : __fmul_rn(__fmul_rn(ft, wk.load), P.inv_n);
+                }
+                cnt += __popc(mask);
             }
-            cnt += __popc(dm);
-            if (t == P.max_len) break;
-            if (wk.alive) wk.advance(P, rowptr, col, w, e, i, k, t);
-            if (__ballot_sync(0xffffffffu, wk.alive) == 0u) break;
+        };
+        if (KEEP) deposit(0, __ballot_sync(0xffffffffu, alive));
+        // a block of random words serves two hops: words 0 and 2 are the halting coins, 1 and 3 pick the neighbours
+        for (int32_t t = 0; t < steps; t += 2) {
+            uint32_t words[4];
+            philox4x32_10((uint32_t)i, (uint32_t)k, (uint32_t)(t >> 1), (uint32_t)e, P.key0, P.key1, words);
+            alive = alive && words[0] >= P.halt_threshold && wk.deg != 0;
+            uint32_t mask = __ballot_sync(0xffffffffu, alive);
+            if (mask == 0u) break;
+            if (alive) wk.hop(words[1], edges);
+            deposit(t + 1, mask);
+            if (t + 1 >= steps) break;
+            alive = alive && words[2] >= P.halt_threshold && wk.deg != 0;
+            mask = __ballot_sync(0xffffffffu, alive);
+            if (mask == 0u) break;
+            if (alive) wk.hop(words[3], edges);
+            deposit(t + 2, mask);
         }
     }
     __syncwarp();
@@ -155,63 +267,72 @@ walk_merge_kernel(const __grid_constant__ grf_walk_params P,
     while (Psort < cnt) Psort <<= 1;
     for (int32_t x = cnt + lane; x < Psort; x += 32) keys[x] = 0xffffffffu;
     __syncwarp();
+    int32_t r = 0;                                        // distinct columns
     if (Psort <= 512) {
         switch (Psort) {
-            case 32: sort_in_registers<1>(keys, lane); break;
-            case 64: sort_in_registers<2>(keys, lane); break;
-            case 128: sort_in_registers<4>(keys, lane); break;
-            case 256: sort_in_registers<8>(keys, lane); break;
-            default: sort_in_registers<16>(keys, lane); break;
+            case 32: r = sort_in_registers<1>(keys, lane, cnt, P.seq_bits, heads); break;
+            case 64: r = sort_in_registers<2>(keys, lane, cnt, P.seq_bits, heads); break;
+            case 128: r = sort_in_registers<4>(keys, lane, cnt, P.seq_bits, heads); break;
+            case 256: r = sort_in_registers<8>(keys, lane, cnt, P.seq_bits, heads); break;
+            default: r = sort_in_registers<16>(keys, lane, cnt, P.seq_bits, heads); break;
         }
-        __syncwarp();
-    } else
-    for (int32_t k = 2; k <= Psort; k <<= 1)
-        for (int32_t j = k >> 1; j > 0; j >>= 1) {
-            for (int32_t idx = lane; idx < (Psort >> 1); idx += 32) {
-                const int32_t a = ((idx & ~(j - 1)) << 1) | (idx & (j - 1));
-                const int32_t b = a | j;
-                const uint32_t ka = keys[a], kb = keys[b];
-                const bool up = (a & k) == 0;
-                if ((ka > kb) == up) { keys[a] = kb; keys[b] = ka; }
+    } else {
+        for (int32_t k = 2; k <= Psort; k <<= 1)
+            for (int32_t j = k >> 1; j > 0; j >>= 1) {
+                for (int32_t idx = lane; idx < (Psort >> 1); idx += 32) {
+                    const int32_t a = ((idx & ~(j - 1)) << 1) | (idx & (j - 1));
+                    const int32_t b = a | j;
+                    const uint32_t ka = keys[a], kb = keys[b];
+                    const bool up = (a & k) == 0;
+                    if ((ka > kb) == up) { keys[a] = kb; keys[b] = ka; }
+                }
+                __syncwarp();
             }
-            __syncwarp();
+        for (int32_t base = 0; base < cnt; base += 32) {
+            const int32_t p = base + lane;
+            const bool head = p < cnt && (p == 0 || (keys[p - 1] >> P.seq_bits) != (keys[p] >> P.seq_bits));
+            const uint32_t hm = __ballot_sync(0xffffffffu, head);
+            if (head) heads[r + __popc(hm & lt_mask)] = (unsigned short)p;
+            r += __popc(hm);
         }
-
-    // ---- add equal columns in sorted order; one lane per distinct column
+    }
+    __syncwarp();
     const uint32_t seq_mask = (1u << P.seq_bits) - 1u;
-    int32_t r = 0;
     const size_t out_base = (size_t)row * stage_stride;
     const size_t dep_base = (size_t)row * P.cap;
+    if (KEEP)
+        for (int32_t p = lane; p < cnt; p += 32) {
+            stage_dep_t[dep_base + p] = (unsigned char)((int32_t)(keys[p] & seq_mask) % Lp1);
+            stage_dep_load[dep_base + p] = vals[keys[p] & seq_mask];
+        }
+
+    // ---- add every column's deposits in sorted order; one lane per distinct column
     // value of the deposit with sequence number seq = walk * (max_len + 1) + t
     auto term = [&](uint32_t seq) {
         if (!KEEP) return vals[seq];
         const int32_t t = (int32_t)seq % Lp1;
         return __fmul_rn(__fmul_rn(P.f[e][t], vals[seq]), P.inv_n);
     };
-    for (int32_t base = 0; base < cnt; base += 32) {
-        const int32_t p = base + lane;
-        const bool valid = p < cnt;
-        const uint32_t key = valid ? keys[p] : 0u;
-        const uint32_t c = key >> P.seq_bits;
-        const bool head = valid && (p == 0 || (keys[p - 1] >> P.seq_bits) != c);
-        const uint32_t hm = __ballot_sync(0xffffffffu, head);
-        if (KEEP && valid) {
-            stage_dep_t[dep_base + p] = (unsigned char)((int32_t)(key & seq_mask) % Lp1);
-            stage_dep_load[dep_base + p] = vals[key & seq_mask];
-        }
-        if (head) {
-            float s = term(key & seq_mask);
-            for (int32_t q = p + 1; q < cnt; ++q) {
-                const uint32_t kq = keys[q];
-                if ((kq >> P.seq_bits) != c) break;
-                s = __fadd_rn(s, term(kq & seq_mask));
+    for (int32_t d = lane; d < r; d += 32) {
+        const int32_t p = heads[d], end = d + 1 < r ? heads[d + 1] : cnt;
+        const uint32_t c = keys[p] >> P.seq_bits;
+        float s;
+        if (at_source && c == (uint32_t)i) {
+            s = first;                                   // walk 0 begins
+            int32_t begun = Lp1;                         // sequence number at which the next walk begins
+            for (int32_t q = p + 1; q < end; ++q) {
+                const int32_t seq = (int32_t)(keys[q] & seq_mask);
+                for (; begun <= seq; begun += Lp1) s = __fadd_rn(s, first);
+                s = __fadd_rn(s, vals[seq]);
             }
-            const int32_t rank = r + __popc(hm & lt_mask);
-            stage_col[out_base + rank] = (int32_t)c;
-            stage_val[out_base + rank] = s;
-            if (KEEP) stage_dep_start[out_base + rank] = p;
+            for (; begun < P.cap; begun += Lp1) s = __fadd_rn(s, first);
+        } else {
+            s = term(keys[p] & seq_mask);
+            for (int32_t q = p + 1; q < end; ++q) s = __fadd_rn(s, term(keys[q] & seq_mask));
         }
-        r += __popc(hm);
+        stage_col[out_base + d] = (int32_t)c;
+        stage_val[out_base + d] = s;
+        if (KEEP) stage_dep_start[out_base + d] = p;
     }
     if (lane == 0) {
         counts[row] = r;
@@ -328,14 +449,15 @@ debug_walks_kernel(const __grid_constant__ grf_walk_params P,
     int32_t* tr = traj + id * Lp1;
     float* ld = load + id * Lp1;
     Walker wk;
-    wk.v = i; wk.load = 1.0f; wk.alive = true;
-    wk.words[0] = wk.words[1] = wk.words[2] = wk.words[3] = 0;
+    wk.v = i; wk.beg = rowptr[i]; wk.deg = rowptr[i + 1] - wk.beg; wk.load = 1.0f;
+    uint32_t words[4] = {0, 0, 0, 0};
     int32_t t = 0;
     for (;; ++t) {
         tr[t] = wk.v; ld[t] = wk.load;
         if (t == P.max_len) break;
-        wk.advance(P, rowptr, col, w, e, i, k, t);
-        if (!wk.alive) break;
+        if ((t & 1) == 0) philox4x32_10((uint32_t)i, (uint32_t)k, (uint32_t)(t >> 1), (uint32_t)e, P.key0, P.key1, words);
+        if (((t & 1) ? words[2] : words[0]) < P.halt_threshold || wk.deg == 0) break;
+        wk.hop((t & 1) ? words[3] : words[1], P, rowptr, col, w);
     }
     for (++t; t < Lp1; ++t) { tr[t] = -1; ld[t] = 0.0f; }
 }
@@ -356,12 +478,6 @@ check_graph_kernel(int32_t N, const int32_t* __restrict__ rowptr, const int32_t*
             if (c < 0 || c >= N) *bad = 1;
         }
     }
-}
-
-size_t walk_smem_per_warp(const grf_walk_params& P)
-{
-    const size_t key_slots = (1 << P.seq_bits) < 32 ? 32 : (size_t)(1 << P.seq_bits);
-    return (key_slots + (size_t)P.cap) * 4;
 }
 
 }  // namespace
@@ -390,7 +506,16 @@ int grf_walk_params_init(grf_walk_params* p, int32_t N, uint64_t seed, int32_t n
         p->f[0][t] = t <= max_len ? f_phi[t] : 0.0f;
         p->f[1][t] = t <= max_len ? f_psi[t] : 0.0f;
     }
+    for (int e = 0; e < 2; ++e) {
+        p->last_step[e] = max_len;
+        while (p->last_step[e] > 0 && p->f[e][p->last_step[e]] == 0.0f) --p->last_step[e];
+    }
     return GRF_OK;
+}
+
+static int reserve_edges(grf_ctx* ctx, int32_t E)
+{
+    return E < 0 ? GRF_ERR_INVALID : grf_buf_reserve(&ctx->edge_records, sizeof(int4) * ((size_t)E + (size_t)E / 8 + 64));
 }
 
 static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& P,
@@ -406,6 +531,14 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     GRF_TRY(grf_csr_reserve(&feat->phi, N, N, 0));
     GRF_TRY(grf_csr_reserve(&feat->psi, N, N, 0));
 
+    if (ctx->edge_records.bytes == 0) {
+        GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 10, rowptr + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+        GRF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        GRF_TRY(reserve_edges(ctx, ctx->pinned[10]));
+    }
+    int4* edges = (int4*)ctx->edge_records.ptr;
+    const int64_t edge_room = (int64_t)(ctx->edge_records.bytes / sizeof(int4));
+
     const bool keep = ctx->keep_walks;
     feat->kept.valid = false;
     feat->kept.perm_valid = false;
@@ -417,7 +550,7 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
         GRF_TRY(grf_buf_reserve(&ctx->dep_rowptr2, 2 * ((size_t)N + 1) * sizeof(int32_t)));
     }
 
-    const size_t per_warp = walk_smem_per_warp(P);
+    const size_t per_warp = walk_smem_bytes(1 << P.seq_bits < 32 ? 32 : 1 << P.seq_bits, P.cap);
     int warps = (int)((200u * 1024u) / per_warp);
     if (warps > 8) warps = 8;
     if (warps < 1) warps = 1;
@@ -426,15 +559,16 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     GRF_CUDA_TRY(cudaFuncSetAttribute(walk_merge_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     GRF_CUDA_TRY(cudaFuncSetAttribute(walk_merge_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     {
-        grf_launch_scope scope(ctx, 0);
+        grf_launch_scope scope(ctx, 0, 2);
+        edge_records_kernel<<<grf_ceil_div(N, 32), 256, 0, ctx->stream>>>(N, edge_room, P.inv_keep, rowptr, col, w, edges);
         if (keep)
             walk_merge_kernel<true><<<grf_ceil_div(rows2, warps), warps * 32, smem, ctx->stream>>>(
-                P, rowptr, col, w, stride, (int32_t*)ctx->stage_col.ptr, (float*)ctx->stage_val.ptr,
+                P, rowptr, edges, edge_room, stride, (int32_t*)ctx->stage_col.ptr, (float*)ctx->stage_val.ptr,
                 (int32_t*)ctx->counts.ptr, (int32_t*)ctx->stage_dep_start.ptr, (unsigned char*)ctx->stage_dep_t.ptr,
                 (float*)ctx->stage_dep_load.ptr, (int32_t*)ctx->dep_counts.ptr);
         else
             walk_merge_kernel<false><<<grf_ceil_div(rows2, warps), warps * 32, smem, ctx->stream>>>(
-                P, rowptr, col, w, stride, (int32_t*)ctx->stage_col.ptr, (float*)ctx->stage_val.ptr,
+                P, rowptr, edges, edge_room, stride, (int32_t*)ctx->stage_col.ptr, (float*)ctx->stage_val.ptr,
                 (int32_t*)ctx->counts.ptr, nullptr, nullptr, nullptr, nullptr);
     }
     GRF_CUDA_TRY(cudaGetLastError());
@@ -456,8 +590,14 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 0, scan_out + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 1, scan_out + 2 * N + 1, sizeof(int32_t), cudaMemcpyDeviceToHost,
                                  ctx->stream));
+    GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 10, rowptr + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     GRF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
     const int64_t nnz_phi = ctx->pinned[0], nnz_psi = ctx->pinned[1];
+    if (ctx->pinned[10] > edge_room) {
+        // the graph has more edges than the records have room for (their number is known on the device only): once more
+        GRF_TRY(reserve_edges(ctx, ctx->pinned[10]));
+        return sample_into(ctx, feat, P, rowptr, col, w);
+    }
 
     // column/value arrays, grown with head-room so that resampling rarely reallocates
     const int64_t cap_phi = nnz_phi + nnz_phi / 8 + 64, cap_psi = nnz_psi + nnz_psi / 8 + 64;
