@@ -74,7 +74,8 @@ int grf_deconvolve(const double* alpha, int32_t len, double* f_out);
  * Deposits of a row that hit the same column are added in ascending (walk, t) order.
  *
  * Limits: n_walks*(max_len+1) <= 16384 and N * 2^ceil(log2(n_walks*(max_len+1))) <= 2^32, else
- * GRF_ERR_TOO_LARGE.  The call waits once for the device (it reads back the two nonzero counts).
+ * GRF_ERR_TOO_LARGE.  Samples of more than 4 M possible entries per matrix make the call wait once for the device (it reads
+ * back the two nonzero counts); smaller ones do not wait, and the first call that needs the counts does.
  */
 int grf_sample(grf_ctx* ctx, int32_t N, const int32_t* rowptr, const int32_t* col, const float* w,
                uint64_t seed, int32_t n_walks, float p_halt, int32_t max_len,

@@ -46,6 +46,7 @@ extern "C" int grf_ctx_create(grf_ctx** out, int device, void* cuda_stream)
     c->stream = (cudaStream_t)cuda_stream;
     if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
         cudaMallocHost((void**)&c->pinned, 64) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->sizes_ready, cudaEventDisableTiming) != cudaSuccess ||
         cudaMalloc((void**)&c->error_word, 2 * sizeof(int)) != cudaSuccess ||
         cudaMemset(c->error_word, 0, 2 * sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
@@ -61,9 +62,11 @@ extern "C" int grf_ctx_destroy(grf_ctx* ctx)
     if (!ctx) return GRF_ERR_INVALID;
     cudaSetDevice(ctx->device);
     cudaStreamSynchronize(ctx->stream);
-    grf_buf* bufs[] = {&ctx->edge_records, &ctx->stage_col, &ctx->stage_val, &ctx->counts, &ctx->rowptr2, &ctx->scan_blocks,
+    grf_settle_sizes(ctx);
+    if (ctx->sizes_ready) cudaEventDestroy(ctx->sizes_ready);
+    grf_buf* bufs[] = {&ctx->edge_records, &ctx->stage_col, &ctx->stage_val, &ctx->counts, &ctx->scan_blocks,
                        &ctx->stage_dep_start, &ctx->stage_dep_t, &ctx->stage_dep_load, &ctx->dep_counts, &ctx->dep_rowptr2,
-                       &ctx->t_cursor, &ctx->t_tmp_col, &ctx->t_tmp_val, &ctx->den_scratch, &ctx->h_rowptr, &ctx->h_col, &ctx->h_w,
+                       &ctx->t_cursor, &ctx->t_tmp, &ctx->den_scratch, &ctx->h_rowptr, &ctx->h_col, &ctx->h_w,
                        &ctx->h_q, &ctx->h_k, &ctx->h_v, &ctx->h_out, &ctx->h_ws};
     for (grf_buf* b : bufs) grf_buf_release(b);
     if (ctx->h_feat) grf_features_free(ctx->h_feat);
@@ -189,6 +192,7 @@ extern "C" int grf_attn_flops(const grf_features* feat, int32_t m, int32_t d, in
                               int64_t* unmasked_linear, int64_t* softmax)
 {
     if (!feat || m <= 0 || d <= 0) return GRF_ERR_INVALID;
+    GRF_TRY(grf_features_sizes(feat));
     const int64_t N = feat->phi.rows;
     const int64_t per_nonzero = (int64_t)m + 2 * (int64_t)m * (d + 1);     // scale phi(.), then multiply-add into [S_l | z_l]
     if (masked) *masked = (feat->phi.nnz + feat->psit.nnz) * per_nonzero + N * d;
@@ -206,6 +210,7 @@ extern "C" int grf_features_free(grf_features* feat)
 {
     if (!feat) return GRF_ERR_INVALID;
     cudaSetDevice(feat->device);
+    if (feat->sizes_from) { feat->sizes_from->sizes_of = nullptr; feat->sizes_from = nullptr; }
     csr_release(&feat->phi); csr_release(&feat->psi); csr_release(&feat->psit);
     grf_buf_release(&feat->plan_off); grf_buf_release(&feat->plan_cnt);
     grf_buf_release(&feat->plan_col); grf_buf_release(&feat->plan_total); grf_buf_release(&feat->plan_coef);
@@ -222,6 +227,7 @@ extern "C" int grf_features_view(const grf_features* feat, int which, int32_t* r
                                  const int32_t** rowptr, const int32_t** col, const float** val)
 {
     if (!feat || which < 0 || which > 2) return GRF_ERR_INVALID;
+    GRF_TRY(grf_features_sizes(feat));
     const grf_csr_dev& m = which == 0 ? feat->phi : (which == 1 ? feat->psi : feat->psit);
     if (rows) *rows = m.rows;
     if (cols) *cols = m.cols;
@@ -236,6 +242,7 @@ extern "C" int grf_features_copy(grf_ctx* ctx, const grf_features* feat, int whi
                                  float* val)
 {
     if (!ctx || !feat || which < 0 || which > 2 || !rowptr) return GRF_ERR_INVALID;
+    GRF_TRY(grf_features_sizes(feat));
     const grf_csr_dev& m = which == 0 ? feat->phi : (which == 1 ? feat->psi : feat->psit);
     if (m.nnz > 0 && (!col || !val)) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
@@ -255,6 +262,7 @@ extern "C" int grf_features_from_csr(grf_ctx* ctx, int32_t N, int32_t R,
 {
     if (!ctx || !out || N <= 0 || R <= 0 || !phi_rowptr || !psi_rowptr) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
+    GRF_TRY(grf_settle_sizes(ctx));                 // the pinned block is used again below
     GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 0, phi_rowptr + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 1, psi_rowptr + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     GRF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));

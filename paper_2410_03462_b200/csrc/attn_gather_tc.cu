@@ -548,6 +548,7 @@ static int build_plan_coefficients(grf_ctx* ctx, grf_features* feat)
 
 int grf_build_block_plan(grf_ctx* ctx, grf_features* feat, bool with_coef)
 {
+    GRF_TRY(grf_features_sizes(feat));
     grf_csr_dev& phi = feat->phi;
     feat->plan_ready = false;
     feat->plan_coef_ready = false;

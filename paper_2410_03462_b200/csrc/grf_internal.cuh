@@ -35,14 +35,14 @@ struct grf_ctx {
     // sampler scratch
     grf_buf stage_col, stage_val;   // merged rows at a fixed stride, before compaction
     grf_buf edge_records;           // the graph's edges as the walks read them
-    grf_buf counts;                 // per-row nonzero counts (both matrices)
-    grf_buf rowptr2;                // scanned counts, [2][N+1]
+    grf_buf counts;                 // nonzeros per row of both matrices, then per column of Psi: three arrays of 16-byte aligned length
     grf_buf scan_blocks;            // block totals of the two-level scan
     // sampler scratch when the walks' deposits are kept (grf_ctx_keep_walks)
     bool keep_walks = false;
     grf_buf stage_dep_start, stage_dep_t, stage_dep_load, dep_counts, dep_rowptr2;
     // transpose scratch
-    grf_buf t_cursor, t_tmp_col, t_tmp_val;
+    grf_buf t_cursor;               // per column: count, then scatter cursor; number of long buckets; their list
+    grf_buf t_tmp;                  // unordered buckets of (row, value)
     grf_buf den_scratch;            // denominators of the tensor-core gather path when the caller wants none
     // host-buffer path
     grf_buf h_rowptr, h_col, h_w, h_q, h_k, h_v, h_out, h_ws;
@@ -53,6 +53,9 @@ struct grf_ctx {
     cudaStream_t copy_stream = nullptr, down_stream = nullptr;
     cudaEvent_t up_done[HOST_PARTS] = {}, part_done[HOST_PARTS] = {}, down_done = nullptr;
     int32_t* pinned = nullptr;      // small pinned host block for read-backs
+    // the sample whose sizes the kernels have left, or will leave, in the pinned block, and the event behind them
+    grf_features* sizes_of = nullptr;
+    cudaEvent_t sizes_ready = nullptr;
     int* error_word = nullptr;      // device word set by a kernel that gave up a bounded wait
     bool use_tensor_cores = true;
     bool states_only = false;       // grf_masked_linear_attn never takes the mask (grf_ctx_use_tensor_cores(ctx, 2))
@@ -121,6 +124,7 @@ struct grf_mask_dev {
 struct grf_features {
     int device = 0;
     grf_csr_dev phi, psi, psit;
+    grf_ctx* sizes_from = nullptr;  // context that still owes this object its sizes (nnz): grf_features_sizes fetches them
     grf_kept_walks kept;
     grf_mask_dev mask;
     // block plan of Phi: per block of GRF_PLAN_BLOCK rows, the sorted distinct columns
@@ -136,6 +140,9 @@ struct grf_features {
 int grf_buf_reserve(grf_buf* b, size_t bytes);          // grows (contents not preserved)
 void grf_buf_release(grf_buf* b);
 int grf_csr_reserve(grf_csr_dev* m, int32_t rows, int32_t cols, int64_t nnz_cap);
+int grf_settle_sizes(grf_ctx* ctx);
+// before nnz of a matrix is read
+static inline int grf_features_sizes(const grf_features* feat) { return feat->sizes_from ? grf_settle_sizes(feat->sizes_from) : GRF_OK; }
 
 // sample.cu
 struct grf_walk_params {
@@ -157,7 +164,19 @@ int grf_exclusive_scan(grf_ctx* ctx, const int32_t* in, int32_t* out, int32_t n,
 int grf_exclusive_scan_scratch(cudaStream_t stream, const int32_t* in, int32_t* out, int32_t n, int32_t segments,
                                int32_t* totals);
 
+// The same for up to three arrays of one length n <= GRF_SCAN_DIRECT_MAX in one launch (in: 16-byte aligned): out[n] is the
+// total, which also goes to host_total (pinned host memory); copy, if any, receives out[0 .. n-1] once more.
+#define GRF_SCAN_DIRECT_MAX (1 << 18)
+struct grf_scan_job { const int32_t* in; int32_t* out; int32_t* copy; int32_t* host_total; };
+struct grf_scan_jobs { grf_scan_job job[3]; };
+int grf_scan_jobs_launch(grf_ctx* ctx, cudaStream_t stream, const grf_scan_jobs& jobs, int count, int32_t n);
+
 // transpose.cu
+// Last step of a regrouping by column: every bucket of (row, value) pairs is ordered by row into t_col, t_val.  long_count
+// (zero before) and long_list: scratch for the buckets too long to rank; rows bounds a bucket's length.
+int grf_order_buckets(cudaStream_t stream, int32_t rows, int32_t cols, const int32_t* t_rowptr, int2* tmp, int32_t* long_count,
+                      int32_t* long_list, int32_t* t_col, float* t_val);
+int grf_reserve_buckets(grf_ctx* ctx, int64_t nnz);
 int grf_transpose_launch(grf_ctx* ctx, int32_t rows, int32_t cols, int64_t nnz,
                          const int32_t* rowptr, const int32_t* col, const float* val,
                          int32_t* t_rowptr, int32_t* t_col, float* t_val);

@@ -44,33 +44,40 @@ struct Walker {
     int32_t v, beg, deg;     // where it stands, and that node's edges
     float load;
 
-    // by the records of edge_records_kernel: one gather
-    __device__ __forceinline__ void hop(uint32_t r_next, const int4* __restrict__ edges)
-    {
-        const int4 r = __ldg(edges + (beg + (int32_t)__umulhi(r_next, (uint32_t)deg)));
-        v = r.x; load = __fmul_rn(load, __int_as_float(r.y)); beg = r.z; deg = r.w;
-    }
-    // by the CSR arrays: four
+    // edges: the records of edge_records_kernel, or null: then the CSR arrays are read
     __device__ __forceinline__ void hop(uint32_t r_next, const grf_walk_params& P, const int32_t* __restrict__ rowptr,
-                                        const int32_t* __restrict__ col, const float* __restrict__ w)
+                                        const int32_t* __restrict__ col, const float* __restrict__ w,
+                                        const int4* __restrict__ edges)
     {
         const int32_t eidx = beg + (int32_t)__umulhi(r_next, (uint32_t)deg);
-        load = __fmul_rn(load, hop_weight(__ldg(w + eidx), deg, P.inv_keep));
-        v = __ldg(col + eidx);
-        beg = __ldg(rowptr + v);
-        deg = __ldg(rowptr + v + 1) - beg;
+        if (edges) {
+            const int4 r = __ldg(edges + eidx);
+            v = r.x; load = __fmul_rn(load, __int_as_float(r.y)); beg = r.z; deg = r.w;
+        } else {
+            load = __fmul_rn(load, hop_weight(__ldg(w + eidx), deg, P.inv_keep));
+            v = __ldg(col + eidx);
+            beg = __ldg(rowptr + v);
+            deg = __ldg(rowptr + v + 1) - beg;
+        }
     }
 };
 
 // One 16-byte record per edge u -> v: v, the factor of the hop's load, and where v's own edges are.  A hop of a warp's 32
-// walkers then costs one gather instead of four, and fewer instructions.  Eight lanes per row.
+// walkers then costs one gather instead of four, and fewer instructions.  Eight lanes per row.  (How many edges a graph has
+// is known on the device only: the records have the room that earlier graphs needed, and a larger graph is walked through
+// its CSR arrays once.)
+// It also clears what the walk kernel counts into and tells the host how many edges there are.
 __global__ void __launch_bounds__(256)
 edge_records_kernel(int32_t N, int64_t room, float inv_keep, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                    const float* __restrict__ w, int4* __restrict__ edges)
+                    const float* __restrict__ w, int4* __restrict__ edges, int32_t* __restrict__ col_counts,
+                    int32_t* __restrict__ long_count, int32_t* __restrict__ host_edges)
 {
-    if (rowptr[N] > room) return;
+    const int32_t E = rowptr[N];
+    if (blockIdx.x == 0 && threadIdx.x == 0) { *host_edges = E; *long_count = 0; }
     const int32_t u = blockIdx.x * 32 + (threadIdx.x >> 3);
     if (u >= N) return;
+    if ((threadIdx.x & 7) == 0) col_counts[u] = 0;
+    if (E > room) return;
     const int32_t beg = rowptr[u], end = rowptr[u + 1];
     for (int32_t p = beg + (threadIdx.x & 7); p < end; p += 8) {
         const int32_t v = col[p], vb = rowptr[v];
@@ -191,17 +198,17 @@ __host__ __device__ __forceinline__ size_t walk_smem_bytes(int32_t key_slots, in
 template <bool KEEP>
 __global__ void __launch_bounds__(256)
 walk_merge_kernel(const __grid_constant__ grf_walk_params P,
-                  const int32_t* __restrict__ rowptr, const int4* __restrict__ edges, int64_t edge_room, int32_t stage_stride, int32_t* __restrict__ stage_col, float* __restrict__ stage_val,
-                  int32_t* __restrict__ counts,
-                  int32_t* __restrict__ stage_dep_start, unsigned char* __restrict__ stage_dep_t,
-                  float* __restrict__ stage_dep_load, int32_t* __restrict__ dep_counts)
+                  const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, const float* __restrict__ w,
+                  const int4* __restrict__ edge_records, int64_t edge_room, int32_t stage_stride, int32_t* __restrict__ stage_col, float* __restrict__ stage_val,
+                  int32_t* __restrict__ counts, int32_t counts_stride, int32_t* __restrict__ stage_dep_start,
+                  unsigned char* __restrict__ stage_dep_t, float* __restrict__ stage_dep_load, int32_t* __restrict__ dep_counts)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int warps = blockDim.x >> 5;
     const int32_t row = blockIdx.x * warps + warp;
-    if (row >= 2 * P.N || __ldg(rowptr + P.N) > edge_room) return;      // no records: the host makes room and comes again
+    if (row >= 2 * P.N) return;
     const int32_t e = row >= P.N ? 1 : 0;
     const int32_t i = row - e * P.N;
 
@@ -217,6 +224,7 @@ walk_merge_kernel(const __grid_constant__ grf_walk_params P,
     const float first = __fmul_rn(__fmul_rn(P.f[e][0], 1.0f), P.inv_n);
     const bool at_source = !KEEP && P.f[e][0] != 0.0f;
 
+    const int4* edges = __ldg(rowptr + P.N) <= edge_room ? edge_records : nullptr;
     const int32_t src_beg = __ldg(rowptr + i), src_deg = __ldg(rowptr + i + 1) - src_beg;
 
     // ---- walks: lanes are walkers, all at the same step t
@@ -250,13 +258,13 @@ walk_merge_kernel(const __grid_constant__ grf_walk_params P,
             alive = alive && words[0] >= P.halt_threshold && wk.deg != 0;
             uint32_t mask = __ballot_sync(0xffffffffu, alive);
             if (mask == 0u) break;
-            if (alive) wk.hop(words[1], edges);
+            if (alive) wk.hop(words[1], P, rowptr, col, w, edges);
             deposit(t + 1, mask);
             if (t + 1 >= steps) break;
             alive = alive && words[2] >= P.halt_threshold && wk.deg != 0;
             mask = __ballot_sync(0xffffffffu, alive);
             if (mask == 0u) break;
-            if (alive) wk.hop(words[3], edges);
+            if (alive) wk.hop(words[3], P, rowptr, col, w, edges);
             deposit(t + 2, mask);
         }
     }
@@ -333,10 +341,11 @@ walk_merge_kernel(const __grid_constant__ grf_walk_params P,
         stage_col[out_base + d] = (int32_t)c;
         stage_val[out_base + d] = s;
         if (KEEP) stage_dep_start[out_base + d] = p;
+        if (e == 1) atomicAdd(counts + 2 * (size_t)counts_stride + c, 1);      // entries per column of Psi
     }
     if (lane == 0) {
-        counts[row] = r;
-        if (KEEP) dep_counts[row] = cnt;
+        counts[(size_t)e * counts_stride + i] = r;
+        if (KEEP) dep_counts[(size_t)e * counts_stride + i] = cnt;
     }
 }
 
@@ -409,27 +418,31 @@ remodulate_kernel(const __grid_constant__ grf_remod_params P, int32_t e, int64_t
     val[p] = s;
 }
 
-// Copies each merged row from the fixed-stride staging area to its place in the CSR arrays.
+// Copies each merged row from the fixed-stride staging area to its place in the CSR arrays, and Psi's entries at once into
+// their column's bucket of Psi^T (in arrival order; the buckets are ordered afterwards).
 __global__ void __launch_bounds__(256)
-compact_rows_kernel(int32_t N, int32_t stage_stride, const int32_t* __restrict__ stage_col,
-                    const float* __restrict__ stage_val,
-                    const int32_t* __restrict__ rowptr_phi, const int32_t* __restrict__ rowptr_psi,
-                    int32_t* __restrict__ col_phi, float* __restrict__ val_phi,
-                    int32_t* __restrict__ col_psi, float* __restrict__ val_psi)
+place_rows_kernel(int32_t N, int32_t stage_stride, const int32_t* __restrict__ stage_col,
+                  const float* __restrict__ stage_val,
+                  const int32_t* __restrict__ rowptr_phi, const int32_t* __restrict__ rowptr_psi,
+                  int32_t* __restrict__ col_phi, float* __restrict__ val_phi,
+                  int32_t* __restrict__ col_psi, float* __restrict__ val_psi, int32_t* __restrict__ cursor,
+                  int2* __restrict__ buckets)
 {
     const int lane = threadIdx.x & 31;
     const int32_t row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= 2 * N) return;
-    const int32_t e = row >= N ? 1 : 0;
-    const int32_t i = row - e * N;
+    // the rows of Psi first: their scatter takes longer
+    const int32_t e = row >= N ? 0 : 1;
+    const int32_t i = row - (1 - e) * N;
     const int32_t* rp = e ? rowptr_psi : rowptr_phi;
-    int32_t* oc = e ? col_psi : col_phi;
-    float* ov = e ? val_psi : val_phi;
     const int32_t beg = rp[i], len = rp[i + 1] - beg;
-    const size_t src = (size_t)row * stage_stride;
+    const size_t src = (size_t)(e * N + i) * stage_stride;
     for (int32_t x = lane; x < len; x += 32) {
-        oc[beg + x] = stage_col[src + x];
-        ov[beg + x] = stage_val[src + x];
+        const int32_t c = stage_col[src + x];
+        const float v = stage_val[src + x];
+        (e ? col_psi : col_phi)[beg + x] = c;
+        (e ? val_psi : val_phi)[beg + x] = v;
+        if (e) buckets[atomicAdd(cursor + c, 1)] = make_int2(i, __float_as_int(v));
     }
 }
 
@@ -457,7 +470,7 @@ debug_walks_kernel(const __grid_constant__ grf_walk_params P,
         if (t == P.max_len) break;
         if ((t & 1) == 0) philox4x32_10((uint32_t)i, (uint32_t)k, (uint32_t)(t >> 1), (uint32_t)e, P.key0, P.key1, words);
         if (((t & 1) ? words[2] : words[0]) < P.halt_threshold || wk.deg == 0) break;
-        wk.hop((t & 1) ? words[3] : words[1], P, rowptr, col, w);
+        wk.hop((t & 1) ? words[3] : words[1], P, rowptr, col, w, nullptr);
     }
     for (++t; t < Lp1; ++t) { tr[t] = -1; ld[t] = 0.0f; }
 }
@@ -513,10 +526,27 @@ int grf_walk_params_init(grf_walk_params* p, int32_t N, uint64_t seed, int32_t n
     return GRF_OK;
 }
 
-static int reserve_edges(grf_ctx* ctx, int32_t E)
+// Row pointers of Phi, Psi and Psi^T (and the scatter cursors of the latter) from the counts; totals to pinned[0], pinned[1].
+static int sample_row_pointers(grf_ctx* ctx, grf_features* feat, int32_t N, int32_t stride_counts, int32_t* cursor)
 {
-    return E < 0 ? GRF_ERR_INVALID : grf_buf_reserve(&ctx->edge_records, sizeof(int4) * ((size_t)E + (size_t)E / 8 + 64));
+    const int32_t* counts = (const int32_t*)ctx->counts.ptr;
+    int32_t* out[3] = {(int32_t*)feat->phi.rowptr.ptr, (int32_t*)feat->psi.rowptr.ptr, (int32_t*)feat->psit.rowptr.ptr};
+    if (N <= GRF_SCAN_DIRECT_MAX) {
+        grf_scan_jobs jobs = {};
+        for (int x = 0; x < 3; ++x)
+            jobs.job[x] = {counts + (size_t)x * stride_counts, out[x], x == 2 ? cursor : nullptr, x == 2 ? nullptr : ctx->pinned + x};
+        return grf_scan_jobs_launch(ctx, ctx->stream, jobs, 3, N);
+    }
+    for (int x = 0; x < 3; ++x) GRF_TRY(grf_exclusive_scan(ctx, counts + (size_t)x * stride_counts, out[x], N, 1));
+    GRF_CUDA_TRY(cudaMemcpyAsync(cursor, out[2], (size_t)N * sizeof(int32_t), cudaMemcpyDeviceToDevice, ctx->stream));
+    for (int x = 0; x < 2; ++x)
+        GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + x, out[x] + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+    return GRF_OK;
 }
+
+// Up to this many entries per matrix the arrays are made for the largest sample there can be, so that nothing has to be
+// known about it before the kernels are queued, and grf_sample does not wait.
+constexpr int64_t SAMPLE_WHOLE_ENTRIES = 4 << 20;
 
 static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& P,
                        const int32_t* rowptr, const int32_t* col, const float* w)
@@ -524,30 +554,35 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     const int32_t N = P.N;
     const int32_t stride = P.cap < N ? P.cap : N;   // a row cannot hold more distinct columns than N
     const size_t rows2 = 2 * (size_t)N;
+    GRF_TRY(grf_settle_sizes(ctx));                 // an earlier sample's sizes are still in the pinned block
+    const int64_t most = (int64_t)N * stride;
+    const bool whole = most <= SAMPLE_WHOLE_ENTRIES && !ctx->keep_walks;
+    const int32_t stride_counts = (N + 3) & ~3;
     GRF_TRY(grf_buf_reserve(&ctx->stage_col, rows2 * stride * sizeof(int32_t)));
     GRF_TRY(grf_buf_reserve(&ctx->stage_val, rows2 * stride * sizeof(float)));
-    GRF_TRY(grf_buf_reserve(&ctx->counts, rows2 * sizeof(int32_t)));
-    GRF_TRY(grf_buf_reserve(&ctx->rowptr2, 2 * ((size_t)N + 1) * sizeof(int32_t)));
-    GRF_TRY(grf_csr_reserve(&feat->phi, N, N, 0));
-    GRF_TRY(grf_csr_reserve(&feat->psi, N, N, 0));
+    GRF_TRY(grf_buf_reserve(&ctx->counts, 3 * (size_t)stride_counts * sizeof(int32_t)));
+    GRF_TRY(grf_buf_reserve(&ctx->t_cursor, sizeof(int32_t) * (3 * (size_t)N + 1)));
+    GRF_TRY(grf_csr_reserve(&feat->phi, N, N, whole ? most : 0));
+    GRF_TRY(grf_csr_reserve(&feat->psi, N, N, whole ? most : 0));
+    GRF_TRY(grf_csr_reserve(&feat->psit, N, N, whole ? most : 0));
+    if (whole) GRF_TRY(grf_reserve_buckets(ctx, most));
+    int32_t* counts = (int32_t*)ctx->counts.ptr;
+    int32_t *long_count = (int32_t*)ctx->t_cursor.ptr, *cursor = long_count + 1, *long_list = cursor + N;
 
-    if (ctx->edge_records.bytes == 0) {
-        GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 10, rowptr + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
-        GRF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-        GRF_TRY(reserve_edges(ctx, ctx->pinned[10]));
-    }
     int4* edges = (int4*)ctx->edge_records.ptr;
     const int64_t edge_room = (int64_t)(ctx->edge_records.bytes / sizeof(int4));
 
     const bool keep = ctx->keep_walks;
     feat->kept.valid = false;
     feat->kept.perm_valid = false;
+    int32_t* dep_scan[2] = {nullptr, nullptr};
     if (keep) {
         GRF_TRY(grf_buf_reserve(&ctx->stage_dep_start, rows2 * stride * sizeof(int32_t)));
         GRF_TRY(grf_buf_reserve(&ctx->stage_dep_t, rows2 * (size_t)P.cap));
         GRF_TRY(grf_buf_reserve(&ctx->stage_dep_load, rows2 * (size_t)P.cap * sizeof(float)));
-        GRF_TRY(grf_buf_reserve(&ctx->dep_counts, rows2 * sizeof(int32_t)));
+        GRF_TRY(grf_buf_reserve(&ctx->dep_counts, 2 * (size_t)stride_counts * sizeof(int32_t)));
         GRF_TRY(grf_buf_reserve(&ctx->dep_rowptr2, 2 * ((size_t)N + 1) * sizeof(int32_t)));
+        for (int e = 0; e < 2; ++e) dep_scan[e] = (int32_t*)ctx->dep_rowptr2.ptr + (size_t)e * (N + 1);
     }
 
     const size_t per_warp = walk_smem_bytes(1 << P.seq_bits < 32 ? 32 : 1 << P.seq_bits, P.cap);
@@ -556,70 +591,63 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     if (warps < 1) warps = 1;
     const size_t smem = per_warp * warps;
     static_assert(sizeof(grf_walk_params) <= 4096, "kernel parameter block too large");
-    GRF_CUDA_TRY(cudaFuncSetAttribute(walk_merge_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    GRF_CUDA_TRY(cudaFuncSetAttribute(walk_merge_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    GRF_CUDA_TRY(cudaFuncSetAttribute(keep ? walk_merge_kernel<true> : walk_merge_kernel<false>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     {
         grf_launch_scope scope(ctx, 0, 2);
-        edge_records_kernel<<<grf_ceil_div(N, 32), 256, 0, ctx->stream>>>(N, edge_room, P.inv_keep, rowptr, col, w, edges);
+        edge_records_kernel<<<grf_ceil_div(N, 32), 256, 0, ctx->stream>>>(
+            N, edge_room, P.inv_keep, rowptr, col, w, edges, counts + 2 * (size_t)stride_counts, long_count, ctx->pinned + 10);
         if (keep)
             walk_merge_kernel<true><<<grf_ceil_div(rows2, warps), warps * 32, smem, ctx->stream>>>(
-                P, rowptr, edges, edge_room, stride, (int32_t*)ctx->stage_col.ptr, (float*)ctx->stage_val.ptr,
-                (int32_t*)ctx->counts.ptr, (int32_t*)ctx->stage_dep_start.ptr, (unsigned char*)ctx->stage_dep_t.ptr,
+                P, rowptr, col, w, edges, edge_room, stride, (int32_t*)ctx->stage_col.ptr, (float*)ctx->stage_val.ptr,
+                counts, stride_counts, (int32_t*)ctx->stage_dep_start.ptr, (unsigned char*)ctx->stage_dep_t.ptr,
                 (float*)ctx->stage_dep_load.ptr, (int32_t*)ctx->dep_counts.ptr);
         else
             walk_merge_kernel<false><<<grf_ceil_div(rows2, warps), warps * 32, smem, ctx->stream>>>(
-                P, rowptr, edges, edge_room, stride, (int32_t*)ctx->stage_col.ptr, (float*)ctx->stage_val.ptr,
-                (int32_t*)ctx->counts.ptr, nullptr, nullptr, nullptr, nullptr);
+                P, rowptr, col, w, edges, edge_room, stride, (int32_t*)ctx->stage_col.ptr, (float*)ctx->stage_val.ptr,
+                counts, stride_counts, nullptr, nullptr, nullptr, nullptr);
     }
     GRF_CUDA_TRY(cudaGetLastError());
-
-    // counts -> row pointers of Phi (segment 0) and Psi (segment 1)
-    int32_t* scan_out = (int32_t*)ctx->rowptr2.ptr;
-    GRF_TRY(grf_exclusive_scan(ctx, (const int32_t*)ctx->counts.ptr, scan_out, N, 2));
-    int32_t* dep_scan = (int32_t*)ctx->dep_rowptr2.ptr;
-    if (keep) {
-        GRF_TRY(grf_exclusive_scan(ctx, (const int32_t*)ctx->dep_counts.ptr, dep_scan, N, 2));
-        GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 2, dep_scan + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
-        GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 3, dep_scan + 2 * N + 1, sizeof(int32_t), cudaMemcpyDeviceToHost,
-                                     ctx->stream));
+    GRF_TRY(sample_row_pointers(ctx, feat, N, stride_counts, cursor));
+    if (keep)
+        for (int e = 0; e < 2; ++e) {
+            GRF_TRY(grf_exclusive_scan(ctx, (const int32_t*)ctx->dep_counts.ptr + (size_t)e * stride_counts, dep_scan[e], N, 1));
+            GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 2 + e, dep_scan[e] + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+        }
+    GRF_CUDA_TRY(cudaEventRecord(ctx->sizes_ready, ctx->stream));
+    ctx->sizes_of = feat;
+    feat->sizes_from = ctx;
+    feat->plan_stale = true;       // the block plan of Phi is built by the first attention call that needs it
+    feat->plan_ready = false;
+    grf_mask_invalidate(feat);
+    if (!whole) {
+        // column/value arrays, grown with head-room so that resampling rarely reallocates
+        GRF_TRY(grf_settle_sizes(ctx));
+        const int64_t nnz_phi = feat->phi.nnz, nnz_psi = feat->psi.nnz;
+        const int64_t cap_phi = nnz_phi + nnz_phi / 8 + 64, cap_psi = nnz_psi + nnz_psi / 8 + 64;
+        if (feat->phi.col.bytes < (size_t)nnz_phi * 4) GRF_TRY(grf_csr_reserve(&feat->phi, N, N, cap_phi));
+        if (feat->psi.col.bytes < (size_t)nnz_psi * 4) GRF_TRY(grf_csr_reserve(&feat->psi, N, N, cap_psi));
+        if (feat->psit.col.bytes < (size_t)nnz_psi * 4) GRF_TRY(grf_csr_reserve(&feat->psit, N, N, cap_psi));
+        GRF_TRY(grf_reserve_buckets(ctx, nnz_psi));
     }
-    GRF_CUDA_TRY(cudaMemcpyAsync(feat->phi.rowptr.ptr, scan_out, ((size_t)N + 1) * sizeof(int32_t),
-                                 cudaMemcpyDeviceToDevice, ctx->stream));
-    GRF_CUDA_TRY(cudaMemcpyAsync(feat->psi.rowptr.ptr, scan_out + N + 1, ((size_t)N + 1) * sizeof(int32_t),
-                                 cudaMemcpyDeviceToDevice, ctx->stream));
-    GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 0, scan_out + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
-    GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 1, scan_out + 2 * N + 1, sizeof(int32_t), cudaMemcpyDeviceToHost,
-                                 ctx->stream));
-    GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 10, rowptr + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
-    GRF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-    const int64_t nnz_phi = ctx->pinned[0], nnz_psi = ctx->pinned[1];
-    if (ctx->pinned[10] > edge_room) {
-        // the graph has more edges than the records have room for (their number is known on the device only): once more
-        GRF_TRY(reserve_edges(ctx, ctx->pinned[10]));
-        return sample_into(ctx, feat, P, rowptr, col, w);
-    }
-
-    // column/value arrays, grown with head-room so that resampling rarely reallocates
-    const int64_t cap_phi = nnz_phi + nnz_phi / 8 + 64, cap_psi = nnz_psi + nnz_psi / 8 + 64;
-    if (feat->phi.col.bytes < (size_t)nnz_phi * 4) GRF_TRY(grf_csr_reserve(&feat->phi, N, N, cap_phi));
-    if (feat->psi.col.bytes < (size_t)nnz_psi * 4) GRF_TRY(grf_csr_reserve(&feat->psi, N, N, cap_psi));
-    if (feat->psit.col.bytes < (size_t)nnz_psi * 4 || feat->psit.rowptr.bytes < ((size_t)N + 1) * 4)
-        GRF_TRY(grf_csr_reserve(&feat->psit, N, N, cap_psi));
-    feat->phi.nnz = nnz_phi; feat->psi.nnz = nnz_psi; feat->psit.nnz = nnz_psi;
-    feat->psit.rows = N; feat->psit.cols = N;
-
+    int2* buckets = (int2*)ctx->t_tmp.ptr;
     {
         grf_launch_scope scope(ctx, 2);
-        compact_rows_kernel<<<grf_ceil_div(rows2, 8), 256, 0, ctx->stream>>>(
+        place_rows_kernel<<<grf_ceil_div(rows2, 8), 256, 0, ctx->stream>>>(
             N, stride, (const int32_t*)ctx->stage_col.ptr, (const float*)ctx->stage_val.ptr,
             (const int32_t*)feat->phi.rowptr.ptr, (const int32_t*)feat->psi.rowptr.ptr,
             (int32_t*)feat->phi.col.ptr, (float*)feat->phi.val.ptr,
-            (int32_t*)feat->psi.col.ptr, (float*)feat->psi.val.ptr);
+            (int32_t*)feat->psi.col.ptr, (float*)feat->psi.val.ptr, cursor, buckets);
+    }
+    {
+        grf_launch_scope scope(ctx, 3, 2);
+        GRF_TRY(grf_order_buckets(ctx->stream, N, N, (const int32_t*)feat->psit.rowptr.ptr, buckets, long_count, long_list,
+                                  (int32_t*)feat->psit.col.ptr, (float*)feat->psit.val.ptr));
     }
     GRF_CUDA_TRY(cudaGetLastError());
     if (keep) {
         grf_kept_walks& K = feat->kept;
-        const int64_t nnz_e[2] = {nnz_phi, nnz_psi};
+        const int64_t nnz_e[2] = {feat->phi.nnz, feat->psi.nnz};
         for (int e = 0; e < 2; ++e) {
             K.deposits[e] = ctx->pinned[2 + e];
             const size_t dcap = (size_t)K.deposits[e] + (size_t)K.deposits[e] / 8 + 64;
@@ -633,7 +661,7 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
             compact_deposits_kernel<<<grf_ceil_div(rows2, 8), 256, 0, ctx->stream>>>(
                 N, stride, P.cap, (const int32_t*)ctx->stage_dep_start.ptr, (const unsigned char*)ctx->stage_dep_t.ptr,
                 (const float*)ctx->stage_dep_load.ptr, (const int32_t*)feat->phi.rowptr.ptr,
-                (const int32_t*)feat->psi.rowptr.ptr, dep_scan,
+                (const int32_t*)feat->psi.rowptr.ptr, (const int32_t*)ctx->dep_rowptr2.ptr,
                 (int32_t*)K.dep_ptr[0].ptr, (unsigned char*)K.dep_t[0].ptr, (float*)K.dep_load[0].ptr,
                 (int32_t*)K.dep_ptr[1].ptr, (unsigned char*)K.dep_t[1].ptr, (float*)K.dep_load[1].ptr);
         }
@@ -641,14 +669,22 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
         K.n_walks = P.n_walks; K.max_len = P.max_len; K.valid = true;
         K.perm_valid = false;
     }
+    return GRF_OK;
+}
 
-    GRF_TRY(grf_transpose_launch(ctx, N, N, nnz_psi, (const int32_t*)feat->psi.rowptr.ptr,
-                                 (const int32_t*)feat->psi.col.ptr, (const float*)feat->psi.val.ptr,
-                                 (int32_t*)feat->psit.rowptr.ptr, (int32_t*)feat->psit.col.ptr,
-                                 (float*)feat->psit.val.ptr));
-    feat->plan_stale = true;       // the block plan of Phi is built by the first attention call that needs it
-    feat->plan_ready = false;
-    grf_mask_invalidate(feat);
+// The sizes of the last sample of this context: waits for them if they have not been read yet.
+int grf_settle_sizes(grf_ctx* ctx)
+{
+    grf_features* feat = ctx->sizes_of;
+    if (!feat) return GRF_OK;
+    ctx->sizes_of = nullptr;
+    feat->sizes_from = nullptr;
+    GRF_CUDA_TRY(cudaEventSynchronize(ctx->sizes_ready));
+    feat->phi.nnz = ctx->pinned[0];
+    feat->psi.nnz = feat->psit.nnz = ctx->pinned[1];
+    const int64_t E = ctx->pinned[10];
+    if (E > (int64_t)(ctx->edge_records.bytes / sizeof(int4)))
+        GRF_TRY(grf_buf_reserve(&ctx->edge_records, sizeof(int4) * ((size_t)E + (size_t)E / 8 + 64)));
     return GRF_OK;
 }
 
@@ -713,6 +749,7 @@ extern "C" int grf_ctx_keep_walks(grf_ctx* ctx, int enable)
 extern "C" int grf_remodulate(grf_ctx* ctx, grf_features* feat, int32_t max_len, const float* f_phi, const float* f_psi)
 {
     if (!ctx || !feat || !f_phi) return GRF_ERR_INVALID;
+    GRF_TRY(grf_features_sizes(feat));
     grf_kept_walks& K = feat->kept;
     if (!K.valid || max_len != K.max_len) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
