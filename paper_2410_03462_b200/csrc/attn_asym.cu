@@ -5,143 +5,195 @@
 // over the nodes l that the walkers out of node i visited: m + d multiply-adds per non-zero of Phi, no
 // per-node states at all.
 //
-// One warp per query and two problems (they share the row's indices and mask values).  Non-zeros are taken
-// 32 at a time: lane t computes the whole dot product of the batch's t-th key row with the query (the query
-// sits in shared memory and is read as a broadcast), then
-// the lanes spread over the d output columns and the batch's value rows are added one after the other, each
-// read as one coalesced row.  The exponentials are taken relative to a running maximum of the scores, which
-// cancels in the quotient; sums are carried in fp32 in a fixed order, so results are run-to-run identical.
+// One warp per query and two problems (they share the row's indices and mask values), non-zeros 32 at a time.  What bounds the
+// kernel is the number of cache lines that its loads touch (one per key row and one per value row at the least):
+//   scores   M / CH lanes take one key row, 16 bytes each, so an instruction reads 32 CH / M whole rows (a lane per key
+//            touched M / CH lines more often than needed: 4 per key at m = 32, bf16); the partial dot products of the
+//            instructions are summed and spread over the lanes by one exchange per halving, which leaves every lane one key;
+//   values   D / CH lanes take one value row, 16 bytes each, so an instruction adds 32 CH / D rows; the groups are summed once
+//            per query.
+// The exponentials are taken relative to a running maximum of the scores, which cancels in the quotient; sums are carried
+// in fp32 in a fixed order, so results are run-to-run identical.
+// N = 32768 cloud, 8 problems, m = 32, d = 64, bf16, softmax: 684 us with a lane per key and a warp per value row.
 #include "grf_internal.cuh"
 
 namespace {
 
+__device__ __forceinline__ uint64_t pair_of(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void split_pair(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma_pair(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul_pair(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// sixteen bytes of a row as packed pairs of fp32, and back
 template <typename T> struct Row;
 template <> struct Row<float> {
     static constexpr int CH = 4;
-    __device__ static __forceinline__ void load(const float* p, float (&v)[4])
+    __device__ static __forceinline__ void widen(const uint4& x, uint64_t (&v)[2])
     {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(p));
-        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+        v[0] = pair_of(__uint_as_float(x.x), __uint_as_float(x.y));
+        v[1] = pair_of(__uint_as_float(x.z), __uint_as_float(x.w));
     }
-    __device__ static __forceinline__ float get(const float* p) { return __ldg(p); }
-    __device__ static __forceinline__ void put(float* p, float x) { *p = x; }
+    __device__ static __forceinline__ void store(float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
 };
 template <> struct Row<__nv_bfloat16> {
     static constexpr int CH = 8;
-    __device__ static __forceinline__ void load(const __nv_bfloat16* p, float (&v)[8])
+    __device__ static __forceinline__ void widen(const uint4& x, uint64_t (&v)[4])
     {
-        const uint4 x = __ldg(reinterpret_cast<const uint4*>(p));
         const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            v[2 * q] = __uint_as_float(w[q] << 16);
-            v[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
-        }
+        for (int q = 0; q < 4; ++q) v[q] = pair_of(__uint_as_float(w[q] << 16), __uint_as_float(w[q] & 0xffff0000u));
     }
-    __device__ static __forceinline__ float get(const __nv_bfloat16* p)
+    __device__ static __forceinline__ void store(__nv_bfloat16* p, const float (&v)[8])
     {
-        return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p)) << 16);
+        uint32_t w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+            w[q] = *reinterpret_cast<uint32_t*>(&h);
+        }
+        *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
     }
-    __device__ static __forceinline__ void put(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
 };
+
+// sixteen bytes, or zeros where there is no row to read
+template <typename T> __device__ __forceinline__ uint4 row_piece(const T* p, bool valid)
+{
+    return valid ? __ldg(reinterpret_cast<const uint4*>(p)) : make_uint4(0u, 0u, 0u, 0u);
+}
 
 constexpr int ASYM_WARPS = 8;
 constexpr int ASYM_GH = 2;      // problems per warp: they share the row's indices and mask values
 
 template <typename T, int M, int D, bool SOFTMAX>
-__global__ void __launch_bounds__(ASYM_WARPS * 32)
+__global__ void __launch_bounds__(ASYM_WARPS * 32, 4)
 asym_attention_kernel(int32_t G, int32_t N, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                       const float* __restrict__ val, const T* __restrict__ Q, const T* __restrict__ K,
                       const T* __restrict__ V, T* __restrict__ out, float* __restrict__ den_out)
 {
-    constexpr int CH = Row<T>::CH;
-    constexpr int EPL = D >= 32 ? D / 32 : 1;        // output columns per lane
-    constexpr int GH = ASYM_GH;
-    __shared__ float qs[ASYM_WARPS][GH][M];
-
+    constexpr int CH = Row<T>::CH, P = CH / 2, GH = ASYM_GH;
+    constexpr int KL = M / CH, KPI = 32 / KL;        // lanes per key row, key rows per instruction
+    constexpr int VL = D / CH, VPI = 32 / VL;        // lanes per value row, value rows per instruction
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t i = blockIdx.x * ASYM_WARPS + warp;
     const int32_t g0 = blockIdx.y * GH;
     if (i >= N) return;
+    const int ks = lane % KL, vs = lane % VL, vg = lane / VL;
+    // within a batch of 32 non-zeros this lane owns number (lane % KL) * KPI + lane / KL: the one whose score the exchange
+    // below leaves here
+    const int own = ks * KPI + lane / KL;
+
+    uint64_t q[GH][P], acc[GH][P];
+    float den[GH], run_max[GH];                      // this lane's share of the denominators; softmax: running maxima
+    const T* Kh[GH];
+    const T* Vh[GH];
 #pragma unroll
     for (int h = 0; h < GH; ++h) {
         const int32_t g = min(g0 + h, G - 1);        // a problem beyond the batch repeats the last one and is not written
-        const T* qrow = Q + ((size_t)g * N + i) * M;
-        for (int a = lane; a < M; a += 32) qs[warp][h][a] = Row<T>::get(qrow + a);
-    }
-    __syncwarp();
-    const bool col_lane = lane * EPL < D;            // lanes that own output columns
-
-    float acc[GH][EPL];
-    float den[GH], run_max[GH];                      // this lane's share of the denominators; softmax: running maxima
-#pragma unroll
-    for (int h = 0; h < GH; ++h) {
+        Row<T>::widen(row_piece(Q + ((size_t)g * N + i) * M + ks * CH, true), q[h]);
+        Kh[h] = K + (size_t)g * N * M + ks * CH;
+        Vh[h] = V + (size_t)g * N * D + vs * CH;
         den[h] = 0.0f; run_max[h] = -INFINITY;
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) acc[h][e] = 0.0f;
+        for (int e = 0; e < P; ++e) acc[h][e] = 0ull;
     }
 
     const int32_t beg = rowptr[i], end = rowptr[i + 1];
     for (int32_t p0 = beg; p0 < end; p0 += 32) {
         const int32_t n = min(32, end - p0);
-        const bool valid = lane < n;
-        const int32_t l = valid ? __ldg(col + p0 + lane) : 0;
-        const float phi = valid ? __ldg(val + p0 + lane) : 0.0f;
+        const bool valid = own < n;
+        const int32_t l = valid ? __ldg(col + p0 + own) : 0;
+        const float phi = valid ? __ldg(val + p0 + own) : 0.0f;
         float w[GH];
 #pragma unroll
         for (int h = 0; h < GH; ++h) {
-            const int32_t g = min(g0 + h, G - 1);
-            // score of this lane's key: the whole dot product in one lane
-            float s = 0.0f;
-            if (valid) {
-                const T* krow = K + ((size_t)g * N + l) * M;
+            // number it * KPI + lane / KL of the batch belongs to lane (lane / KL) * KL + it
+            float part[KL];
+            constexpr int KB = KL < 4 ? KL : 4;                      // loads on their way together
 #pragma unroll
-                for (int c = 0; c < M / CH; ++c) {
-                    float v[CH];
-                    Row<T>::load(krow + c * CH, v);
+            for (int i0 = 0; i0 < KL; i0 += KB) {
+                uint4 x[KB];
 #pragma unroll
-                    for (int e = 0; e < CH; ++e) s = fmaf(v[e], qs[warp][h][c * CH + e], s);
+                for (int u = 0; u < KB; ++u) {
+                    const int32_t lk = __shfl_sync(0xffffffffu, l, (lane / KL) * KL + i0 + u);
+                    x[u] = row_piece(Kh[h] + (size_t)lk * M, (i0 + u) * KPI + lane / KL < n);
+                }
+#pragma unroll
+                for (int u = 0; u < KB; ++u) {
+                    uint64_t k[P], s2 = 0ull;
+                    Row<T>::widen(x[u], k);
+#pragma unroll
+                    for (int e = 0; e < P; ++e) s2 = fma_pair(k[e], q[h][e], s2);
+                    float lo, hi;
+                    split_pair(s2, lo, hi);
+                    part[i0 + u] = lo + hi;
                 }
             }
+            // sum over the KL lanes of a key row; lane ks keeps the sum of instruction ks
+#pragma unroll
+            for (int off = KL / 2; off > 0; off >>= 1) {
+                const bool upper = (ks & off) != 0;
+#pragma unroll
+                for (int x = 0; x < off; ++x) {
+                    const float keep = upper ? part[x + off] : part[x], give = upper ? part[x] : part[x + off];
+                    part[x] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+                }
+            }
+            const float s = part[0];
             if (SOFTMAX) {
                 float bmax = valid ? s : -INFINITY;
 #pragma unroll
                 for (int off = 1; off < 32; off <<= 1) bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, off));
                 const float new_max = fmaxf(run_max[h], bmax);
-                const float rescale = __expf(run_max[h] - new_max);     // 0 on the first batch (run_max = -inf)
+                if (new_max > run_max[h]) {
+                    const float rescale = __expf(run_max[h] - new_max);     // 0 on the first batch (run_max = -inf)
+                    const uint64_t r2 = pair_of(rescale, rescale);
 #pragma unroll
-                for (int e = 0; e < EPL; ++e) acc[h][e] *= rescale;
-                den[h] *= rescale;
-                run_max[h] = new_max;
+                    for (int e = 0; e < P; ++e) acc[h][e] = mul_pair(acc[h][e], r2);
+                    den[h] *= rescale;
+                    run_max[h] = new_max;
+                }
                 w[h] = valid ? phi * __expf(s - new_max) : 0.0f;
             } else {
                 w[h] = phi * s;
             }
             den[h] += w[h];
         }
-        // the batch's value rows, one after the other, lanes across the output columns
-        for (int32_t t = 0; t < n; ++t) {
-            const int32_t lt = __shfl_sync(0xffffffffu, l, t);
+        // the batch's value rows, VPI at a time
+        constexpr int VB = 32 / VPI < 4 ? 32 / VPI : 4;              // loads of a problem on their way together
+        for (int t0 = 0; t0 < n; t0 += VPI * VB) {
 #pragma unroll
             for (int h = 0; h < GH; ++h) {
-                const float wt = __shfl_sync(0xffffffffu, w[h], t);
-                const int32_t g = min(g0 + h, G - 1);
-                if (col_lane) {
-                    const T* vrow = V + ((size_t)g * N + lt) * D + lane * EPL;
-                    if constexpr (sizeof(T) == 2 && EPL == 2) {
-                        const uint32_t x = __ldg(reinterpret_cast<const uint32_t*>(vrow));
-                        acc[h][0] = fmaf(wt, __uint_as_float(x << 16), acc[h][0]);
-                        acc[h][1] = fmaf(wt, __uint_as_float(x & 0xffff0000u), acc[h][1]);
-                    } else if constexpr (sizeof(T) == 2 && EPL == 4) {
-                        const uint2 x = __ldg(reinterpret_cast<const uint2*>(vrow));
-                        acc[h][0] = fmaf(wt, __uint_as_float(x.x << 16), acc[h][0]);
-                        acc[h][1] = fmaf(wt, __uint_as_float(x.x & 0xffff0000u), acc[h][1]);
-                        acc[h][2] = fmaf(wt, __uint_as_float(x.y << 16), acc[h][2]);
-                        acc[h][3] = fmaf(wt, __uint_as_float(x.y & 0xffff0000u), acc[h][3]);
-                    } else {
+                uint4 x[VB];
+                float wt[VB];
 #pragma unroll
-                        for (int e = 0; e < EPL; ++e) acc[h][e] = fmaf(wt, Row<T>::get(vrow + e), acc[h][e]);
-                    }
+                for (int u = 0; u < VB; ++u) {
+                    const int b = t0 + u * VPI + vg, src = (b % KPI) * KL + b / KPI;     // the lane that owns number b
+                    const int32_t lv = __shfl_sync(0xffffffffu, l, src & 31);
+                    wt[u] = __shfl_sync(0xffffffffu, w[h], src & 31);
+                    x[u] = row_piece(Vh[h] + (size_t)lv * D, b < n);
+                }
+#pragma unroll
+                for (int u = 0; u < VB; ++u) {
+                    uint64_t v[P];
+                    Row<T>::widen(x[u], v);
+                    const uint64_t w2 = pair_of(wt[u], wt[u]);
+#pragma unroll
+                    for (int e = 0; e < P; ++e) acc[h][e] = fma_pair(w2, v[e], acc[h][e]);
                 }
             }
         }
@@ -153,11 +205,16 @@ asym_attention_kernel(int32_t G, int32_t N, const int32_t* __restrict__ rowptr, 
         for (int off = 1; off < 32; off <<= 1) dn += __shfl_xor_sync(0xffffffffu, dn, off);
         if (g0 + h >= G) break;
         const float inv = dn != 0.0f ? 1.0f / dn : 0.0f;
-        if (col_lane) {
-            T* orow = out + ((size_t)(g0 + h) * N + i) * D + lane * EPL;
+        float o[CH];
 #pragma unroll
-            for (int e = 0; e < EPL; ++e) Row<T>::put(orow + e, acc[h][e] * inv);
+        for (int e = 0; e < P; ++e) split_pair(acc[h][e], o[2 * e], o[2 * e + 1]);
+#pragma unroll
+        for (int e = 0; e < CH; ++e) {
+#pragma unroll
+            for (int off = VL; off < 32; off <<= 1) o[e] += __shfl_xor_sync(0xffffffffu, o[e], off);
+            o[e] *= inv;
         }
+        if (vg == 0) Row<T>::store(out + ((size_t)(g0 + h) * N + i) * D + vs * CH, o);
         // with the softmax kernel the reported denominator is relative to exp(max score of the row)
         if (lane == 0 && den_out) den_out[(size_t)(g0 + h) * N + i] = dn;
     }
