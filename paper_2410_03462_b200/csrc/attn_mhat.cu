@@ -27,101 +27,31 @@ constexpr int BQ = GRF_PLAN_BLOCK;      // queries per block
 constexpr int KT = GRF_MASK_TILE;       // keys per tile
 
 // ---------------------------------------------------------------------------------------------------
-// Key sets: one CTA per block of rows marks, in a bitmap, the keys of Psi^T's rows over the block's node list.
-// A warp takes 32 nodes at a time (lane x holds node x's extent in Psi^T) and fetches the keys of four nodes
-// together, so that several loads are in flight.  The bitmap and the count (padded to whole tiles) are kept.
+// Structure of the mask: one CTA per block of rows, everything that does not depend on values.
+//   keys       the union of Psi^T's rows over the block's node list, marked in a bitmap (a bit is looked at before it is
+//              set: a block reaches each of its keys about thirty times), counted, and written as the block's key list,
+//              padded to whole tiles with the last key (whose mask values there are zeros);
+//   positions  for every node of the list the accumulator (by position in the key list) of each of its keys, 16 bits each;
+//              for every non-zero Phi_il of the block's rows where node l's positions begin.
+// A warp takes 32 nodes at a time (lane x holds node x's extent in Psi^T) and fetches the keys of two nodes together.
+// Blocks take their places in the lists by atomic additions, so the order of the blocks inside the arrays varies; nothing
+// depends on it.  A block whose part does not fit the room that the host has made writes none of it: the totals tell
+// the host how much is needed.  The last CTA to finish orders the blocks by decreasing key count.
+// One kernel for all of this, at the N = 32768 cloud: 237 us in five kernels and two prefix sums before, 178 us now (issue
+// slots 69 % busy while an SM has blocks, the blocks with the longest lists end last).
 
-constexpr int MASK_BITMAP_THREADS = 1024;     // one CTA per block: many warps, each with a few batches of 32 nodes
+constexpr int MS_THREADS = 768;
 
-__global__ void __launch_bounds__(MASK_BITMAP_THREADS)
-mask_bitmap_kernel(int32_t Nk, const int32_t* __restrict__ plan_off, const int32_t* __restrict__ plan_cnt,
-                   const int32_t* __restrict__ plan_col, const int32_t* __restrict__ t_rowptr,
-                   const int32_t* __restrict__ t_col, uint32_t* __restrict__ bits, int32_t* __restrict__ mk_cnt)
+struct grf_mask_totals {                // zeroed before the launch; host[0..2] = entries, positions, longest list
+    unsigned long long entries, positions;
+    int32_t longest, finished;
+};
+
+// exclusive prefix sum of one value per thread over MS_THREADS threads; *total (shared) = the sum
+__device__ __forceinline__ int32_t ms_scan(int32_t x, int32_t* warp_sums, int32_t* total)
 {
-    extern __shared__ uint32_t bitmap[];        // one bit per key
-    __shared__ int32_t warp_sums[8];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t blk = blockIdx.x;
-    const int32_t words = (Nk + 31) >> 5;
-    for (int32_t x = tid; x < words; x += MASK_BITMAP_THREADS) bitmap[x] = 0u;
-    __syncthreads();
-    const int32_t* ulist = plan_col + plan_off[blk];
-    const int32_t ucnt = plan_cnt[blk];
-    for (int32_t u0 = warp * 32; u0 < ucnt; u0 += MASK_BITMAP_THREADS) {
-        const int32_t n = min(32, ucnt - u0);
-        const int32_t my_l = lane < n ? __ldg(ulist + u0 + lane) : 0;
-        const int32_t my_beg = lane < n ? __ldg(t_rowptr + my_l) : 0;
-        const int32_t my_end = lane < n ? __ldg(t_rowptr + my_l + 1) : 0;
-        for (int32_t e0 = 0; e0 < n; e0 += 4) {
-            int32_t jj[4][4];
-            int32_t ebeg[4], eend[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                ebeg[e] = e0 + e < n ? __shfl_sync(0xffffffffu, my_beg, (e0 + e) & 31) : 0;
-                eend[e] = e0 + e < n ? __shfl_sync(0xffffffffu, my_end, (e0 + e) & 31) : 0;
-#pragma unroll
-                for (int sl = 0; sl < 4; ++sl) {
-                    const int32_t q = ebeg[e] + sl * 32 + lane;
-                    jj[e][sl] = q < eend[e] ? __ldg(t_col + q) : -1;
-                }
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-#pragma unroll
-                for (int sl = 0; sl < 4; ++sl)
-                    if (jj[e][sl] >= 0) atomicOr(&bitmap[jj[e][sl] >> 5], 1u << (jj[e][sl] & 31));
-                for (int32_t q = ebeg[e] + 128 + lane; q < eend[e]; q += 32) {
-                    const int32_t j = __ldg(t_col + q);
-                    atomicOr(&bitmap[j >> 5], 1u << (j & 31));
-                }
-            }
-        }
-    }
-    __syncthreads();
-    // the bitmap, and behind it the number of set bits before each of its words (the first 256 threads)
-    const int32_t per = (words + 255) / 256;
-    const int32_t w0 = min(words, min(tid, 256) * per), w1 = tid < 256 ? min(words, w0 + per) : w0;
-    int32_t mine = 0;
-    for (int32_t x = w0; x < w1; ++x) mine += __popc(bitmap[x]);
-    int32_t inc = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-    }
-    if (lane == 31 && warp < 8) warp_sums[warp] = inc;
-    __syncthreads();
-    if (tid >= 256) return;
-    int32_t run = inc - mine;
-    for (int w = 0; w < warp; ++w) run += warp_sums[w];
-    uint32_t* dst = bits + (size_t)blk * 2 * words;
-    for (int32_t x = w0; x < w1; ++x) {
-        const uint32_t b = bitmap[x];
-        dst[x] = b;
-        dst[words + x] = (uint32_t)run;
-        run += __popc(b);
-    }
-    if (tid == 255) mk_cnt[blk] = (run + KT - 1) / KT * KT;
-}
-
-// Key lists: the set bits of a block's bitmap in ascending order, padded to whole tiles with the last key
-// (whose mask values in the padding are zeros).
-__global__ void __launch_bounds__(256)
-mask_list_kernel(int32_t Nk, const uint32_t* __restrict__ bits, const int32_t* __restrict__ mk_off,
-                 const int32_t* __restrict__ mk_cnt, int32_t* __restrict__ mk_key)
-{
-    __shared__ int32_t warp_sums[8];
-    __shared__ int32_t block_total;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t blk = blockIdx.x;
-    const int32_t words = (Nk + 31) >> 5;
-    const uint32_t* bitmap = bits + (size_t)blk * 2 * words;
-    // each thread owns a contiguous range of words so that the list comes out sorted
-    const int32_t per = (words + 255) / 256;
-    const int32_t w0 = min(words, tid * per), w1 = min(words, w0 + per);
-    int32_t mine = 0;
-    for (int32_t x = w0; x < w1; ++x) mine += __popc(bitmap[x]);
-    int32_t inc = mine;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t inc = x;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
@@ -129,37 +59,181 @@ mask_list_kernel(int32_t Nk, const uint32_t* __restrict__ bits, const int32_t* _
     }
     if (lane == 31) warp_sums[warp] = inc;
     __syncthreads();
-    int32_t before = inc - mine;
-    for (int w = 0; w < warp; ++w) before += warp_sums[w];
-    if (tid == 255) block_total = before + mine;
-    const int32_t base_off = mk_off[blk];
-    int32_t o = base_off + before;
-    for (int32_t x = w0; x < w1; ++x) {
-        uint32_t b = bitmap[x];
-        while (b) {
-            const int k = __ffs(b) - 1;
-            b &= b - 1;
-            mk_key[o++] = (x << 5) + k;
+    if (warp == 0) {
+        int32_t w = lane < MS_THREADS / 32 ? warp_sums[lane] : 0;
+        const int32_t own = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
         }
+        warp_sums[lane] = w - own;
+        if (lane == 31) *total = w;
     }
     __syncthreads();
-    const int32_t padded = mk_cnt[blk];
-    if (block_total > 0)
-        for (int32_t e = block_total + tid; e < padded; e += 256) mk_key[base_off + e] = mk_key[base_off + block_total - 1];
+    const int32_t r = inc - x + warp_sums[warp];
+    __syncthreads();
+    return r;
 }
 
-// order[r] = the block with the r-th largest key list (ties: lower index first), stored behind the counts
-__global__ void __launch_bounds__(256) mask_order_kernel(int32_t nblocks, int32_t* __restrict__ mk_cnt)
+// bits set before each word of a bitmap; returns their number
+__device__ __forceinline__ int32_t ms_ranks(const uint32_t* bits, int32_t* before, int32_t words, int32_t* warp_sums, int32_t* total)
 {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nblocks) return;
-    const int32_t c = mk_cnt[i];
-    int32_t rank = 0;
-    for (int32_t j = 0; j < nblocks; ++j) {
-        const int32_t cj = mk_cnt[j];
-        rank += (cj > c || (cj == c && j < i)) ? 1 : 0;
+    const int32_t per = (words + MS_THREADS - 1) / MS_THREADS;
+    const int32_t w0 = min(words, (int32_t)threadIdx.x * per), w1 = min(words, w0 + per);
+    int32_t mine = 0;
+    for (int32_t x = w0; x < w1; ++x) mine += __popc(bits[x]);
+    int32_t run = ms_scan(mine, warp_sums, total);
+    for (int32_t x = w0; x < w1; ++x) { before[x] = run; run += __popc(bits[x]); }
+    __syncthreads();
+    return *total;
+}
+
+// Where the accumulator of position p lies: the 16-byte quarters of a group of sixteen change places from pair to pair of
+// groups, so that lanes which read whole neighbouring groups meet in no bank.
+__host__ __device__ __forceinline__ uint32_t mask_slot(uint32_t p) { return p ^ ((p >> 5 & 3u) << 2); }
+
+__global__ void __launch_bounds__(MS_THREADS, 2)
+mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restrict__ phi_rowptr, const int32_t* __restrict__ phi_col,
+                      const int32_t* __restrict__ plan_off, const int32_t* __restrict__ plan_cnt,
+                      const int32_t* __restrict__ plan_col, const int32_t* __restrict__ t_rowptr,
+                      const int32_t* __restrict__ t_col, int64_t key_room, int64_t pos_room, uint32_t* __restrict__ bits_out,
+                      int32_t* node_off, int32_t* __restrict__ mk_off, int32_t* __restrict__ mk_cnt,
+                      int32_t* __restrict__ mk_key, unsigned short* __restrict__ pos16, int32_t* __restrict__ phi_pos,
+                      grf_mask_totals* totals, int32_t* host)
+{
+    extern __shared__ uint32_t smem_ms[];       // key bitmap, its ranks, node bitmap, its ranks
+    __shared__ int32_t warp_sums[32];
+    __shared__ int32_t total, last_cta;
+    __shared__ unsigned long long base_keys, base_pos;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t blk = blockIdx.x, nblocks = gridDim.x;
+    const int32_t wk = (Nk + 31) >> 5, wr = (R + 31) >> 5;
+    uint32_t* kbits = smem_ms;
+    int32_t* kbefore = reinterpret_cast<int32_t*>(smem_ms + wk);
+    uint32_t* nbits = smem_ms + 2 * wk;
+    int32_t* nbefore = reinterpret_cast<int32_t*>(smem_ms + 2 * wk + wr);
+    for (int32_t x = tid; x < wk; x += MS_THREADS) kbits[x] = 0u;
+    for (int32_t x = tid; x < wr; x += MS_THREADS) nbits[x] = 0u;
+    __syncthreads();
+    const int32_t uoff = plan_off[blk], ucnt = plan_cnt[blk];
+    const int32_t* ulist = plan_col + uoff;
+
+    // ---- nodes: bitmap, where their positions begin (the padding at the list's end repeats the last node; it gets a
+    // place of its own that nobody uses)
+    int32_t npos = 0;
+    for (int32_t u0 = 0; u0 < ucnt; u0 += MS_THREADS) {
+        const int32_t u = u0 + tid;
+        int32_t len = 0;
+        if (u < ucnt) {
+            const int32_t l = __ldg(ulist + u);
+            len = __ldg(t_rowptr + l + 1) - __ldg(t_rowptr + l);
+            if (!(nbits[l >> 5] >> (l & 31) & 1u)) atomicOr(&nbits[l >> 5], 1u << (l & 31));
+        }
+        const int32_t at = ms_scan(len, warp_sums, &total);
+        if (u < ucnt) node_off[uoff + u] = npos + at;
+        npos += total;
+        __syncthreads();
     }
-    mk_cnt[nblocks + rank] = i;
+
+    // ---- keys
+    auto each_key = [&](auto&& use) {
+        for (int32_t u0 = warp * 32; u0 < ucnt; u0 += MS_THREADS) {
+            const int32_t n = min(32, ucnt - u0);
+            const int32_t my_l = lane < n ? __ldg(ulist + u0 + lane) : 0;
+            const int32_t my_beg = lane < n ? __ldg(t_rowptr + my_l) : 0;
+            const int32_t my_len = lane < n ? __ldg(t_rowptr + my_l + 1) - my_beg : 0;
+            for (int32_t e0 = 0; e0 < n; e0 += 2) {
+                int32_t j[2][4], beg[2], len[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    beg[e] = __shfl_sync(0xffffffffu, my_beg, (e0 + e) & 31);
+                    len[e] = e0 + e < n ? __shfl_sync(0xffffffffu, my_len, (e0 + e) & 31) : 0;
+#pragma unroll
+                    for (int sl = 0; sl < 4; ++sl) j[e][sl] = sl * 32 + lane < len[e] ? __ldg(t_col + beg[e] + sl * 32 + lane) : -1;
+                }
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                    for (int sl = 0; sl < 4; ++sl)
+                        if (j[e][sl] >= 0) use(u0 + e0 + e, sl * 32 + lane, j[e][sl]);
+                    for (int32_t x = 128 + lane; x < len[e]; x += 32) use(u0 + e0 + e, x, __ldg(t_col + beg[e] + x));
+                }
+            }
+        }
+    };
+    each_key([&](int32_t, int32_t, int32_t k) {
+        if (!(kbits[k >> 5] >> (k & 31) & 1u)) atomicOr(&kbits[k >> 5], 1u << (k & 31));
+    });
+    __syncthreads();
+    const int32_t keys = ms_ranks(kbits, kbefore, wk, warp_sums, &total);
+    ms_ranks(nbits, nbefore, wr, warp_sums, &total);
+    const int32_t padded = (keys + KT - 1) / KT * KT;
+    if (tid == 0) {
+        base_keys = atomicAdd(&totals->entries, (unsigned long long)padded);
+        base_pos = atomicAdd(&totals->positions, (unsigned long long)npos);
+        atomicMax(&totals->longest, padded);
+        mk_cnt[blk] = padded;
+        mk_off[blk] = (int32_t)base_keys;
+    }
+    __syncthreads();
+    if ((int64_t)base_keys + padded <= key_room) {
+        int32_t* list = mk_key + base_keys;
+        const int32_t per = (wk + MS_THREADS - 1) / MS_THREADS;
+        const int32_t w0 = min(wk, tid * per), w1 = min(wk, w0 + per);
+        for (int32_t x = w0; x < w1; ++x) {
+            uint32_t b = kbits[x];
+            int32_t o = kbefore[x];
+            while (b) {
+                const int k = (x << 5) + __ffs(b) - 1;
+                b &= b - 1;
+                if (o == keys - 1)
+                    for (int32_t e = keys; e < padded; ++e) list[e] = k;
+                list[o++] = k;
+            }
+        }
+    }
+    if (bits_out) {                             // for the kernel that looks positions up row by row
+        uint32_t* dst = bits_out + (size_t)blk * 2 * wk;
+        for (int32_t x = tid; x < wk; x += MS_THREADS) { dst[x] = kbits[x]; dst[wk + x] = (uint32_t)kbefore[x]; }
+    }
+    if ((int64_t)base_pos + npos <= pos_room && padded <= 65536) {
+        unsigned short* pos = pos16 + base_pos;
+        each_key([&](int32_t u, int32_t x, int32_t k) {
+            pos[node_off[uoff + u] + x] = (unsigned short)mask_slot((uint32_t)(kbefore[k >> 5] + __popc(kbits[k >> 5] & ((1u << (k & 31)) - 1u))));
+        });
+        const int32_t r0 = blk * BQ, r1 = min(N, r0 + BQ);
+        for (int32_t p = phi_rowptr[r0] + tid, end = phi_rowptr[r1]; p < end; p += MS_THREADS) {
+            const int32_t l = __ldg(phi_col + p);
+            const int32_t u = nbefore[l >> 5] + __popc(nbits[l >> 5] & ((1u << (l & 31)) - 1u));
+            phi_pos[p] = (int32_t)base_pos + node_off[uoff + u];
+        }
+    }
+
+    // ---- the last CTA: sizes to the host, blocks by decreasing key count (ties: lower index first) behind the counts
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last_cta = atomicAdd(&totals->finished, 1) == nblocks - 1;
+    __syncthreads();
+    if (!last_cta) return;
+    __threadfence();
+    const volatile int32_t* counts = mk_cnt;
+    for (int32_t i = tid; i < nblocks; i += MS_THREADS) {
+        const int32_t c = counts[i];
+        int32_t rank = 0;
+        for (int32_t j = 0; j < nblocks; ++j) {
+            const int32_t cj = counts[j];
+            rank += (cj > c || (cj == c && j < i)) ? 1 : 0;
+        }
+        mk_cnt[nblocks + rank] = i;
+    }
+    if (tid == 0) {
+        const volatile grf_mask_totals* t = totals;
+        const unsigned long long e = t->entries, p = t->positions;
+        host[0] = e > 0x7fffffffull ? -1 : (int32_t)e;
+        host[1] = p > 0x7fffffffull ? -1 : (int32_t)p;
+        host[2] = t->longest;
+    }
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -171,6 +245,32 @@ __global__ void __launch_bounds__(256) mask_order_kernel(int32_t nblocks, int32_
 // so no two lanes meet at one position, and the warp is synchronised between two l: the order of every sum is
 // fixed.  The keys of four nodes are fetched together and the next four are on their way while these are added.
 // Lists longer than a segment take further passes.
+
+// A segment of a row's accumulators -> the mask blocks, sixteen keys per lane at a time: 32 bytes, a whole sector, at
+// [group of 16 keys][row of the block] (in groups of 8 the half sectors cost 90 us of 660).  Cleared for the next row
+// as they are read.
+// SLOTS: the accumulators lie where mask_slot says.
+template <bool SLOTS>
+__device__ __forceinline__ void store_mask_row(float* acc, int32_t len, int lane, __nv_bfloat16* __restrict__ mk_val,
+                                               int32_t first_key, int32_t first_acc, int32_t rr)
+{
+    for (int32_t c = lane; c < len / 16; c += 32) {
+        float4* a4 = reinterpret_cast<float4*>(acc + c * 16);
+        const int turn = SLOTS ? ((first_acc / 16 + c) >> 1) & 3 : 0;
+        uint32_t w[8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 x = a4[q ^ turn];
+            a4[q ^ turn] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(x.x, x.y), hi = __floats2bfloat162_rn(x.z, x.w);
+            w[2 * q] = *reinterpret_cast<const uint32_t*>(&lo);
+            w[2 * q + 1] = *reinterpret_cast<const uint32_t*>(&hi);
+        }
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                     ::"l"(mk_val + ((size_t)(first_key / 16 + c) * BQ + rr) * 16), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
+                       "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+    }
+}
 
 constexpr int MASK_SEG = 4096;          // accumulators per warp
 constexpr int MASK_WARPS = 4;
@@ -212,7 +312,7 @@ mask_values_kernel(int32_t N, int32_t Nk, const int32_t* __restrict__ phi_rowptr
     __syncthreads();
     const int32_t r0 = blk * BQ;
     for (int32_t seg0 = 0; seg0 < cnt; seg0 += MASK_SEG) {
-        const int32_t seglen = min(MASK_SEG, cnt - seg0);       // a multiple of the tile, hence of 8
+        const int32_t seglen = min(MASK_SEG, cnt - seg0);       // a multiple of the tile, hence of 16
         auto position = [&](int32_t j) {
             const int32_t ps = before_word[j >> 5] + __popc(bitmap[j >> 5] & ((1u << (j & 31)) - 1u)) - seg0;
             return (ps >= 0 && ps < seglen) ? ps : -1;
@@ -276,19 +376,7 @@ mask_values_kernel(int32_t N, int32_t Nk, const int32_t* __restrict__ phi_rowptr
                     }
                 }
             }
-            // the row's values of this segment, eight keys (16 bytes) per lane at a time; the accumulators are
-            // cleared for the next row as they are read
-            for (int32_t c8 = lane; c8 < seglen / 8; c8 += 32) {
-                float4* a4 = reinterpret_cast<float4*>(acc + c8 * 8);
-                const float4 x0 = a4[0], x1 = a4[1];
-                a4[0] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                a4[1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                const __nv_bfloat162 h0 = __floats2bfloat162_rn(x0.x, x0.y), h1 = __floats2bfloat162_rn(x0.z, x0.w);
-                const __nv_bfloat162 h2 = __floats2bfloat162_rn(x1.x, x1.y), h3 = __floats2bfloat162_rn(x1.z, x1.w);
-                uint4* dst = reinterpret_cast<uint4*>(mk_val + ((size_t)((off + seg0) / 8 + c8) * BQ + rr) * 8);
-                *dst = make_uint4(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1),
-                                  *reinterpret_cast<const uint32_t*>(&h2), *reinterpret_cast<const uint32_t*>(&h3));
-            }
+            store_mask_row<false>(acc, seglen, lane, mk_val, off + seg0, seg0, rr);
             __syncwarp();
         }
     }
@@ -298,168 +386,24 @@ mask_values_kernel(int32_t N, int32_t Nk, const int32_t* __restrict__ phi_rowptr
 // The same sums with the positions looked up once per (block, node) instead of once per (row, node): a node of a
 // block's list is used by nine of the block's rows on average, and the look-up (two shared-memory reads and a
 // population count per key) was most of the work of every addition.
-//   mask_node_offsets_kernel  per block: where each node's positions start (running sum of the lengths of the
-//                             nodes' rows of Psi^T over the block's list) and the block's total;
-//   mask_positions_kernel     per block: the position in the block's key list of every key of every node of the
-//                             list (16 bits each), and for every non-zero Phi_il of the block's rows where the
-//                             positions of node l start;
-//   mask_values_pos_kernel    the row-by-row accumulation, reading positions instead of keys.
-
-__global__ void __launch_bounds__(256)
-mask_node_offsets_kernel(const int32_t* __restrict__ plan_off, const int32_t* __restrict__ plan_cnt,
-                         const int32_t* __restrict__ plan_col, const int32_t* __restrict__ t_rowptr,
-                         int32_t* __restrict__ node_off, int32_t* __restrict__ blk_total,
-                         const int32_t* __restrict__ mk_cnt, int32_t* __restrict__ longest_list)
-{
-    __shared__ int32_t warp_sums[8];
-    __shared__ int32_t carry_s;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t blk = blockIdx.x;
-    const int32_t uoff = plan_off[blk], ucnt = plan_cnt[blk];
-    if (tid == 0) carry_s = 0;
-    __syncthreads();
-    for (int32_t base = 0; base < ucnt; base += 256) {
-        const int32_t u = base + tid;
-        int32_t len = 0;
-        if (u < ucnt) {
-            const int32_t l = plan_col[uoff + u];
-            len = t_rowptr[l + 1] - t_rowptr[l];
-        }
-        int32_t inc = len;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        if (lane == 31) warp_sums[warp] = inc;
-        __syncthreads();
-        int32_t before = carry_s + inc - len;
-        for (int w = 0; w < warp; ++w) before += warp_sums[w];
-        if (u < ucnt) node_off[uoff + u] = before;
-        __syncthreads();
-        if (tid == 255) carry_s = before + len;
-        __syncthreads();
-    }
-    if (tid == 0) {
-        blk_total[blk] = carry_s;
-        atomicMax(longest_list, mk_cnt[blk]);        // positions are kept in 16 bits: the host checks this
-    }
-}
-
-constexpr int MASK_POS_PARTS = 4;
-
-__global__ void __launch_bounds__(256)
-mask_positions_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restrict__ phi_rowptr,
-                      const int32_t* __restrict__ phi_col, const int32_t* __restrict__ plan_off,
-                      const int32_t* __restrict__ plan_cnt, const int32_t* __restrict__ plan_col,
-                      const int32_t* __restrict__ t_rowptr, const int32_t* __restrict__ t_col,
-                      const uint32_t* __restrict__ bits, const int32_t* __restrict__ node_off,
-                      const int32_t* __restrict__ blk_pos, unsigned short* __restrict__ pos16, int32_t* __restrict__ phi_pos)
-{
-    extern __shared__ uint32_t smem_pos[];      // key bitmap, its prefix counts, node bitmap, its prefix counts
-    __shared__ int32_t warp_sums[8];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // MASK_POS_PARTS CTAs share a block: each takes every MASK_POS_PARTS-th batch of nodes and slice of non-zeros
-    const int32_t blk = blockIdx.x / MASK_POS_PARTS, part = blockIdx.x % MASK_POS_PARTS;
-    const int32_t wk = (Nk + 31) >> 5, wr = (R + 31) >> 5;
-    uint32_t* kbits = smem_pos;
-    int32_t* kbefore = reinterpret_cast<int32_t*>(smem_pos + wk);
-    uint32_t* nbits = smem_pos + 2 * wk;
-    int32_t* nbefore = reinterpret_cast<int32_t*>(smem_pos + 2 * wk + wr);
-    const uint32_t* src = bits + (size_t)blk * 2 * wk;
-    for (int32_t x = tid; x < wk; x += 256) { kbits[x] = src[x]; kbefore[x] = (int32_t)src[wk + x]; }
-    for (int32_t x = tid; x < wr; x += 256) nbits[x] = 0u;
-    __syncthreads();
-    const int32_t uoff = plan_off[blk], ucnt = plan_cnt[blk];
-    const int32_t* ulist = plan_col + uoff;
-    for (int32_t u = tid; u < ucnt; u += 256) {
-        const int32_t l = ulist[u];
-        atomicOr(&nbits[l >> 5], 1u << (l & 31));
-    }
-    __syncthreads();
-    {
-        const int32_t per = (wr + 255) / 256;
-        const int32_t w0 = min(wr, tid * per), w1 = min(wr, w0 + per);
-        int32_t mine = 0;
-        for (int32_t x = w0; x < w1; ++x) mine += __popc(nbits[x]);
-        int32_t inc = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        if (lane == 31) warp_sums[warp] = inc;
-        __syncthreads();
-        int32_t run = inc - mine;
-        for (int w = 0; w < warp; ++w) run += warp_sums[w];
-        for (int32_t x = w0; x < w1; ++x) { nbefore[x] = run; run += __popc(nbits[x]); }
-    }
-    __syncthreads();
-    const int32_t base = blk_pos[blk];
-    // positions of the keys of every node of the list; a warp takes 32 nodes at a time (lane x holds node x's extent
-    // in Psi^T and the start of its positions) and fetches the keys of four nodes together
-    for (int32_t u0 = (part * 8 + warp) * 32; u0 < ucnt; u0 += MASK_POS_PARTS * 8 * 32) {
-        const int32_t n = min(32, ucnt - u0);
-        const int32_t my_l = lane < n ? __ldg(ulist + u0 + lane) : 0;
-        const int32_t my_beg = lane < n ? __ldg(t_rowptr + my_l) : 0;
-        const int32_t my_end = lane < n ? __ldg(t_rowptr + my_l + 1) : 0;
-        const int32_t my_dst = lane < n ? base + node_off[uoff + u0 + lane] : 0;
-        for (int32_t e0 = 0; e0 < n; e0 += 4) {
-            int32_t jj[4][4];
-            int32_t ebeg[4], eend[4], edst[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                ebeg[e] = e0 + e < n ? __shfl_sync(0xffffffffu, my_beg, (e0 + e) & 31) : 0;
-                eend[e] = e0 + e < n ? __shfl_sync(0xffffffffu, my_end, (e0 + e) & 31) : 0;
-                edst[e] = __shfl_sync(0xffffffffu, my_dst, (e0 + e) & 31);
-#pragma unroll
-                for (int sl = 0; sl < 4; ++sl) {
-                    const int32_t q = ebeg[e] + sl * 32 + lane;
-                    jj[e][sl] = q < eend[e] ? __ldg(t_col + q) : -1;
-                }
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-#pragma unroll
-                for (int sl = 0; sl < 4; ++sl) {
-                    const int32_t j = jj[e][sl];
-                    if (j >= 0)
-                        pos16[(size_t)edst[e] + sl * 32 + lane] =
-                            (unsigned short)(kbefore[j >> 5] + __popc(kbits[j >> 5] & ((1u << (j & 31)) - 1u)));
-                }
-                for (int32_t q = ebeg[e] + 128 + lane; q < eend[e]; q += 32) {        // nodes with more than 128 keys
-                    const int32_t j = __ldg(t_col + q);
-                    pos16[(size_t)edst[e] + (q - ebeg[e])] =
-                        (unsigned short)(kbefore[j >> 5] + __popc(kbits[j >> 5] & ((1u << (j & 31)) - 1u)));
-                }
-            }
-        }
-    }
-    // where the positions of its node start, for every non-zero of the block's rows of Phi (the list holds a node
-    // once, apart from the padding at its end, which repeats the last node: the first occurrence counts)
-    const int32_t r0 = blk * BQ, r1 = min(N, r0 + BQ);
-    for (int32_t p = phi_rowptr[r0] + part * 256 + tid; p < phi_rowptr[r1]; p += MASK_POS_PARTS * 256) {
-        const int32_t l = __ldg(phi_col + p);
-        const int32_t u = nbefore[l >> 5] + __popc(nbits[l >> 5] & ((1u << (l & 31)) - 1u));
-        phi_pos[p] = base + node_off[uoff + u];
-    }
-}
-
+//
 // Bound by the load/store unit: per 32 multiply-adds two accesses of the accumulators (about three bank conflicts each) and
 // the position and value loads.  So every row makes one pass over its nodes: a warp's accumulators are as long as the block's
 // key list, and the CTA runs as many of its warps as then fit its shared memory (a list beyond an eighth of it is
-// taken in segments).  Rows are handed to the warps by a counter.  N = 32768 cloud, 297 M multiply-adds: 853 -> 660 us
-// (fixed segments of 4096 keys made two passes of half the rows; four shuffles per node were 14 % of the unit's work).
+// taken in segments).  Rows are handed to the warps by a counter.  N = 32768 cloud, 297 M multiply-adds: 853 -> 557 us
+// (fixed segments of 4096 keys made two passes of half the rows; four shuffles per node were 14 % of the unit's work; half
+// sectors in the output 10 %; 422 -> 222 M warp instructions).  The unit is busy 78 % of the time; what is left is its
+// bank conflicts (a node's 95 keys meet three times in a bank on average) and the loads.
 constexpr int MVP_WARPS = 16;
 constexpr int MVP_MIN_WARPS = 8;
 constexpr int MVP_ROOM = 212 * 256;      // accumulators (fp32) of a CTA at most: what an SM's shared memory holds
 
 struct MaskPosGroup {                   // the keys of two nodes l, up to 128 each: lane x holds keys x, x+32, x+64, x+96
     int32_t ps[2][4];
-    float v[2][4];
+    float v[2][4], phi[2];
 };
 
-// nodes: (Phi_il, length and start of row l of Psi^T, start of node l's positions) of the 32 non-zeros a warp works on: read back
+// nodes: (Phi_il, length of row l of Psi^T, start of its values, start of node l's positions) of the 32 non-zeros a warp works on: read back
 // as one broadcast each, which costs the load/store unit a quarter of what four shuffles do
 template <bool SEGMENTED>
 __device__ __forceinline__ void mask_row_pass(int32_t pbeg, int32_t pend, int32_t seg0, int32_t seglen, int lane, float* acc,
@@ -482,38 +426,43 @@ __device__ __forceinline__ void mask_row_pass(int32_t pbeg, int32_t pend, int32_
         __syncwarp();
         nodes[lane] = mine;
         __syncwarp();
+        const bool any_long = __any_sync(0xffffffffu, mine.y > 128);
         auto fetch = [&](int32_t e0, MaskPosGroup& gq) {
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const int4 nd = nodes[e0 + e];
+                gq.phi[e] = __int_as_float(nd.x);
+                const unsigned short* pp = pos16 + (uint32_t)nd.w + lane;
+                const float* vp = t_val + (uint32_t)nd.z + lane;
 #pragma unroll
                 for (int sl = 0; sl < 4; ++sl) {
-                    const int32_t x = sl * 32 + lane;
-                    const bool valid = x < nd.y;
-                    gq.ps[e][sl] = valid ? (int32_t)__ldg(pos16 + (size_t)nd.w + x) : -1;
-                    gq.v[e][sl] = valid ? __ldg(t_val + nd.z + x) : 0.0f;
+                    const bool valid = sl * 32 + lane < nd.y;
+                    gq.ps[e][sl] = valid ? (int32_t)__ldg(pp + sl * 32) : -1;
+                    gq.v[e][sl] = valid ? __ldg(vp + sl * 32) : 0.0f;
                 }
             }
         };
         auto add = [&](int32_t e0, MaskPosGroup& gq) {
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const int4 nd = nodes[e0 + e];
-                const float phi = __int_as_float(nd.x);
+                const float phi = gq.phi[e];
                 float a[4];
                 int32_t ps[4];
                 // one node's keys are distinct: a lane's four additions go side by side
 #pragma unroll
                 for (int sl = 0; sl < 4; ++sl) {
                     ps[sl] = place(gq.ps[e][sl]);
-                    a[sl] = ps[sl] >= 0 ? acc[ps[sl]] : 0.0f;
+                    if (ps[sl] >= 0) a[sl] = acc[ps[sl]];
                 }
 #pragma unroll
                 for (int sl = 0; sl < 4; ++sl)
                     if (ps[sl] >= 0) acc[ps[sl]] = fmaf(phi, gq.v[e][sl], a[sl]);
-                for (int32_t x = 128 + lane; x < nd.y; x += 32) {      // nodes with more than 128 keys
-                    const int32_t y = place((int32_t)__ldg(pos16 + (size_t)nd.w + x));
-                    if (y >= 0) acc[y] = fmaf(phi, __ldg(t_val + nd.z + x), acc[y]);
+                if (any_long) {                                             // nodes with more than 128 keys
+                    const int4 nd = nodes[e0 + e];
+                    for (int32_t x = 128 + lane; x < nd.y; x += 32) {
+                        const int32_t y = place((int32_t)__ldg(pos16 + (uint32_t)nd.w + x));
+                        if (y >= 0) acc[y] = fmaf(phi, __ldg(t_val + (uint32_t)nd.z + x), acc[y]);
+                    }
                 }
                 __syncwarp();
             }
@@ -551,9 +500,9 @@ mask_values_pos_kernel(int32_t N, int32_t rows_per_cta, int32_t room, const int3
     const int32_t rr0 = (blockIdx.x % groups) * rows_per_cta;
     const int32_t off = mk_off[blk], cnt = mk_cnt[blk];
     if (cnt == 0) return;
-    // warps that run and accumulators of each (a multiple of 8: they are read as float4 pairs)
+    // warps that run and accumulators of each (a multiple of 16: they leave sixteen at a time)
     const int32_t nw = min(MVP_WARPS, max(MVP_MIN_WARPS, room / cnt));
-    const int32_t seg = min(cnt, room / nw & ~7);
+    const int32_t seg = min(cnt, room / nw & ~15);
     if (tid == 0) next_row = 0;
     __syncthreads();
     if (warp >= nw) return;
@@ -570,24 +519,12 @@ mask_values_pos_kernel(int32_t N, int32_t rows_per_cta, int32_t room, const int3
         const int32_t r = r0 + rr;
         const int32_t pbeg = r < N ? phi_rowptr[r] : 0, pend = r < N ? phi_rowptr[r + 1] : 0;
         for (int32_t seg0 = 0; seg0 < cnt; seg0 += seg) {
-            const int32_t seglen = min(seg, cnt - seg0);           // a multiple of 8
+            const int32_t seglen = min(seg, cnt - seg0);           // a multiple of 16
             if (seg == cnt)
                 mask_row_pass<false>(pbeg, pend, 0, cnt, lane, acc, nodes[warp], phi_col, phi_val, phi_pos, t_rowptr, t_val, pos16);
             else
                 mask_row_pass<true>(pbeg, pend, seg0, seglen, lane, acc, nodes[warp], phi_col, phi_val, phi_pos, t_rowptr, t_val, pos16);
-            // the row's values of this segment, eight keys (16 bytes) per lane at a time; the accumulators are
-            // cleared for the next row as they are read
-            for (int32_t c8 = lane; c8 < seglen / 8; c8 += 32) {
-                float4* a4 = reinterpret_cast<float4*>(acc + c8 * 8);
-                const float4 x0 = a4[0], x1 = a4[1];
-                a4[0] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                a4[1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                const __nv_bfloat162 h0 = __floats2bfloat162_rn(x0.x, x0.y), h1 = __floats2bfloat162_rn(x0.z, x0.w);
-                const __nv_bfloat162 h2 = __floats2bfloat162_rn(x1.x, x1.y), h3 = __floats2bfloat162_rn(x1.z, x1.w);
-                uint4* dst = reinterpret_cast<uint4*>(mk_val + ((size_t)((off + seg0) / 8 + c8) * BQ + rr) * 8);
-                *dst = make_uint4(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1),
-                                  *reinterpret_cast<const uint32_t*>(&h2), *reinterpret_cast<const uint32_t*>(&h3));
-            }
+            store_mask_row<true>(acc, seglen, lane, mk_val, off + seg0, seg0, rr);
             __syncwarp();
         }
     }
@@ -609,7 +546,7 @@ mask_rows_kernel(int32_t Nk, const int32_t* __restrict__ rows, const int32_t* __
     for (int32_t e = threadIdx.x; e < cnt; e += 256) {
         const int32_t j = mk_key[off + e];
         if (e > 0 && mk_key[off + e - 1] == j) continue;
-        o[j] = __bfloat162float(mk_val[((size_t)((off + e) / 8) * BQ + rr) * 8 + ((off + e) & 7)]);
+        o[j] = __bfloat162float(mk_val[((size_t)((off + e) / 16) * BQ + rr) * 16 + ((off + e) & 15)]);
     }
 }
 
@@ -667,6 +604,11 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b)
     uint64_t r;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
+}
+__device__ __forceinline__ void ld_nc_32bytes(const uint4* p, uint4& a, uint4& b)
+{
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
 }
 constexpr int MH_ISSUER_S = 8, MH_ISSUER_O = 9, MH_PRODUCER0 = 10;
 
@@ -738,13 +680,14 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
         const int rr = (warp & 3) * 32 + lane;                   // row of the block = tensor-memory lane
         const int32_t row = blk * BQ + rr;
         const uint32_t lane_field = (uint32_t)((warp & 3) * 32) << 16;
-        const uint4* mrow = mk_val + (size_t)(off / 8) * BQ + rr;       // chunk x of this row: mrow[x * BQ]
+        const uint4* mrow = mk_val + ((size_t)(off / 16) * BQ + rr) * 2;   // keys 16x .. 16x+15 of this row: mrow[2 * x * BQ], and the next
         uint64_t den2[2] = {0ull, 0ull};                         // row sums, four partial sums in two packed pairs
         uint4 mk[KT / 8];
-        if (grp < T) {
+        auto load_mask = [&](int32_t t) {
 #pragma unroll
-            for (int c = 0; c < KT / 8; ++c) mk[c] = __ldg(mrow + (size_t)(grp * (KT / 8) + c) * BQ);
-        }
+            for (int c = 0; c < KT / 16; ++c) ld_nc_32bytes(mrow + (size_t)(t * (KT / 16) + c) * (2 * BQ), mk[2 * c], mk[2 * c + 1]);
+        };
+        if (grp < T) load_mask(grp);
         bool ok = true;
         int buf = grp;                                           // t % NB and the parity of t / NB, kept in step
         uint32_t par = 0u;
@@ -778,10 +721,7 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
                 tmem_st8(s_addr + (uint32_t)(c16 * 8), pw);
             }
             // this group's next tile: its mask values travel while the products run
-            if (t + 2 < T) {
-#pragma unroll
-                for (int c = 0; c < KT / 8; ++c) mk[c] = __ldg(mrow + (size_t)((t + 2) * (KT / 8) + c) * BQ);
-            }
+            if (t + 2 < T) load_mask(t + 2);
             tmem_st_wait();
             fence_before_sync();
             __syncwarp();
@@ -990,65 +930,67 @@ void grf_mask_release(grf_features* feat)
 {
     grf_mask_dev& K = feat->mask;
     grf_buf_release(&K.off); grf_buf_release(&K.cnt); grf_buf_release(&K.key); grf_buf_release(&K.bits); grf_buf_release(&K.val); grf_buf_release(&K.node_off);
-    grf_buf_release(&K.blk_pos); grf_buf_release(&K.pos16); grf_buf_release(&K.phi_pos);
+    grf_buf_release(&K.totals); grf_buf_release(&K.pos16); grf_buf_release(&K.phi_pos);
     grf_mask_invalidate(feat);
 }
 
-// Key sets of the blocks, their counts and offsets, where every node's key positions will start: all sizes that the rest
-// of the build and the choice of the route need.  Waits for the stream.
+// The structure kernel, and a wait for its sizes.  Its arrays have room from earlier builds; where that was not enough
+// (once for a feature object, as a rule) it runs again with what it has found to be needed.
 static int prepare_mask_lists(grf_ctx* ctx, grf_features* feat)
 {
     grf_mask_dev& K = feat->mask;
-    const int32_t Nk = feat->psi.rows, nblocks = feat->plan_blocks;
-    const size_t words = ((size_t)Nk + 31) / 32;
+    const int32_t N = feat->phi.rows, Nk = feat->psi.rows, R = feat->psit.rows, nblocks = feat->plan_blocks;
+    const size_t words = ((size_t)Nk + 31) / 32, smem = (words + ((size_t)R + 31) / 32) * 8;
     GRF_TRY(grf_buf_reserve(&K.cnt, sizeof(int32_t) * 2 * (size_t)nblocks));
-    GRF_TRY(grf_buf_reserve(&K.off, sizeof(int32_t) * ((size_t)nblocks + 1)));
-    GRF_TRY(grf_buf_reserve(&K.bits, sizeof(uint32_t) * 2 * (size_t)nblocks * words));
-    GRF_CUDA_TRY(cudaFuncSetAttribute(mask_bitmap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(words * 4)));
-    {
-        grf_launch_scope scope(ctx, 8);
-        mask_bitmap_kernel<<<nblocks, MASK_BITMAP_THREADS, words * 4, ctx->stream>>>(
-            Nk, (const int32_t*)feat->plan_off.ptr, (const int32_t*)feat->plan_cnt.ptr, (const int32_t*)feat->plan_col.ptr,
-            (const int32_t*)feat->psit.rowptr.ptr, (const int32_t*)feat->psit.col.ptr, (uint32_t*)K.bits.ptr,
-            (int32_t*)K.cnt.ptr);
-    }
-    GRF_CUDA_TRY(cudaGetLastError());
-    GRF_TRY(grf_exclusive_scan(ctx, (const int32_t*)K.cnt.ptr, (int32_t*)K.off.ptr, nblocks, 1));
-    GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 5, (const int32_t*)K.off.ptr + nblocks, sizeof(int32_t),
-                                 cudaMemcpyDeviceToHost, ctx->stream));
-    // where every node's key positions will start (per block, then over the blocks), and the longest key list
-    // (buffers whose size follows the sample grow with head-room: resampling changes the sizes a little every time,
-    // and a reallocation stalls the device)
+    GRF_TRY(grf_buf_reserve(&K.off, sizeof(int32_t) * (size_t)nblocks));
+    GRF_TRY(grf_buf_reserve(&K.totals, sizeof(grf_mask_totals)));
     GRF_TRY(reserve_with_headroom(&K.node_off, sizeof(int32_t) * (size_t)(feat->plan_entries > 0 ? feat->plan_entries : 1)));
-    GRF_TRY(grf_buf_reserve(&K.blk_pos, sizeof(int32_t) * (2 * (size_t)nblocks + 2)));
-    int32_t* blk_pos = (int32_t*)K.blk_pos.ptr;                 // offsets [nblocks + 1], totals [nblocks], longest list
-    GRF_CUDA_TRY(cudaMemsetAsync(blk_pos + 2 * nblocks + 1, 0, sizeof(int32_t), ctx->stream));
-    {
-        grf_launch_scope scope(ctx, 8);
-        mask_node_offsets_kernel<<<nblocks, 256, 0, ctx->stream>>>(
-            (const int32_t*)feat->plan_off.ptr, (const int32_t*)feat->plan_cnt.ptr, (const int32_t*)feat->plan_col.ptr,
-            (const int32_t*)feat->psit.rowptr.ptr, (int32_t*)K.node_off.ptr, blk_pos + nblocks + 1,
-            (const int32_t*)K.cnt.ptr, blk_pos + 2 * nblocks + 1);
+    GRF_TRY(reserve_with_headroom(&K.phi_pos, sizeof(int32_t) * (size_t)(feat->phi.nnz + 1)));
+    GRF_CUDA_TRY(cudaFuncSetAttribute(mask_structure_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    K.by_position = true;
+    for (int attempt = 0; attempt < 3; ++attempt) {
+        const int64_t key_room = (int64_t)(K.key.bytes / sizeof(int32_t));
+        const int64_t pos_room = K.by_position ? (int64_t)(K.pos16.bytes / sizeof(unsigned short)) : -1;
+        GRF_CUDA_TRY(cudaMemsetAsync(K.totals.ptr, 0, sizeof(grf_mask_totals), ctx->stream));
+        {
+            grf_launch_scope scope(ctx, 8);
+            mask_structure_kernel<<<nblocks, MS_THREADS, smem, ctx->stream>>>(
+                N, Nk, R, (const int32_t*)feat->phi.rowptr.ptr, (const int32_t*)feat->phi.col.ptr,
+                (const int32_t*)feat->plan_off.ptr, (const int32_t*)feat->plan_cnt.ptr, (const int32_t*)feat->plan_col.ptr,
+                (const int32_t*)feat->psit.rowptr.ptr, (const int32_t*)feat->psit.col.ptr, key_room, pos_room,
+                K.by_position ? nullptr : (uint32_t*)K.bits.ptr, (int32_t*)K.node_off.ptr, (int32_t*)K.off.ptr,
+                (int32_t*)K.cnt.ptr, (int32_t*)K.key.ptr, (unsigned short*)K.pos16.ptr, (int32_t*)K.phi_pos.ptr,
+                (grf_mask_totals*)K.totals.ptr, ctx->pinned + 5);
+        }
+        GRF_CUDA_TRY(cudaGetLastError());
+        GRF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));      // the sizes of the key lists are known only now
+        K.blocks = nblocks;
+        K.entries = ctx->pinned[5];
+        K.positions = ctx->pinned[6];
+        K.longest = ctx->pinned[7];
+        // (a negative sum means that it passed 2^31); no locality: the S/z route serves this object
+        K.refused = K.entries < 0 || (size_t)K.entries * BQ * sizeof(__nv_bfloat16) > ((size_t)8 << 30);
+        if (K.refused) break;
+        // positions are looked up once per (block, node) when they fit 16 bits and their number an int32; otherwise once
+        // per (row, node), in the blocks' key bitmaps
+        const bool by_position = K.positions >= 0 && K.longest <= 65536;
+        if (by_position == K.by_position && K.entries <= key_room && (!by_position || K.positions <= pos_room)) break;
+        K.by_position = by_position;
+        GRF_TRY(reserve_with_headroom(&K.key, (size_t)K.entries * 4));
+        if (by_position) GRF_TRY(reserve_with_headroom(&K.pos16, sizeof(unsigned short) * (size_t)K.positions));
+        else GRF_TRY(grf_buf_reserve(&K.bits, sizeof(uint32_t) * 2 * (size_t)nblocks * words));
     }
-    GRF_TRY(grf_exclusive_scan(ctx, blk_pos + nblocks + 1, blk_pos, nblocks, 1));
-    GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 6, blk_pos + nblocks, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
-    GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 7, blk_pos + 2 * nblocks + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
-    GRF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));          // the sizes of the key lists are known only now
-    K.blocks = nblocks;
-    K.entries = ctx->pinned[5];
-    K.positions = ctx->pinned[6];
-    K.longest = ctx->pinned[7];
     K.lists_ready = true;
-    // (a negative sum means that it passed 2^31); no locality: the S/z route serves this object
-    K.refused = K.entries < 0 || (size_t)K.entries * BQ * sizeof(__nv_bfloat16) > ((size_t)8 << 30);
     return GRF_OK;
 }
 
-// Shared memory of the row-by-row values kernel: the key bitmap, its prefix counts and the accumulators.
+// Shared memory of the structure kernel (two bitmaps and their ranks) and of the row-by-row values kernel (the key bitmap,
+// its ranks and the accumulators).
 static bool mask_fits_smem(const grf_features* feat)
 {
-    const size_t words = ((size_t)feat->psi.rows + 31) / 32;
-    return ((words + 1) & ~(size_t)1) * 8 + (size_t)MASK_WARPS * MASK_SEG * sizeof(float) <= 200 * 1024;
+    const size_t words = ((size_t)feat->psi.rows + 31) / 32, node_words = ((size_t)feat->psit.rows + 31) / 32;
+    return ((words + 1) & ~(size_t)1) * 8 + (size_t)MASK_WARPS * MASK_SEG * sizeof(float) <= 200 * 1024 &&
+           (words + node_words) * 8 <= 200 * 1024;
 }
 
 // Forms the mask of the present features (or only its values, where the key lists still hold).
@@ -1063,48 +1005,13 @@ static int build_mask(grf_ctx* ctx, grf_features* feat)
         return GRF_OK;
     }
     K.structure_ready = false;
-    const int32_t N = feat->phi.rows, Nk = feat->psi.rows, R = feat->psit.rows;
     if (!mask_fits_smem(feat)) return GRF_ERR_TOO_LARGE;
     GRF_TRY(grf_ensure_block_plan(ctx, feat, false));         // the node lists only
     if (!feat->plan_ready) return GRF_ERR_TOO_LARGE;          // rows of a block share too little
     if (!K.lists_ready) GRF_TRY(prepare_mask_lists(ctx, feat));
     if (K.refused) return GRF_ERR_TOO_LARGE;
-    const int32_t nblocks = feat->plan_blocks;
-    const int64_t entries = K.entries;
-    const size_t words = ((size_t)Nk + 31) / 32;
-    int32_t* blk_pos = (int32_t*)K.blk_pos.ptr;
-    // positions are looked up once per (block, node) when they fit 16 bits, their number fits an int32 and both bitmaps
-    // fit shared memory; otherwise once per (row, node)
-    const int64_t total_pos = K.positions;
-    const size_t smem_pos = (words + ((size_t)R + 31) / 32) * 8;
-    const bool by_position = total_pos >= 0 && K.longest <= 65535 && smem_pos <= 96 * 1024;
-    GRF_TRY(reserve_with_headroom(&K.key, (size_t)entries * 4));
-    GRF_TRY(reserve_with_headroom(&K.val, (size_t)entries * BQ * sizeof(__nv_bfloat16)));
-    {
-        grf_launch_scope scope(ctx, 8);
-        mask_list_kernel<<<nblocks, 256, 0, ctx->stream>>>(Nk, (const uint32_t*)K.bits.ptr, (const int32_t*)K.off.ptr,
-                                                           (const int32_t*)K.cnt.ptr, (int32_t*)K.key.ptr);
-    }
-    {
-        grf_launch_scope scope(ctx, 8);
-        mask_order_kernel<<<grf_ceil_div(nblocks, 256), 256, 0, ctx->stream>>>(nblocks, (int32_t*)K.cnt.ptr);
-    }
-    if (by_position) {
-        GRF_TRY(reserve_with_headroom(&K.pos16, sizeof(unsigned short) * (size_t)(total_pos + 1)));
-        GRF_TRY(reserve_with_headroom(&K.phi_pos, sizeof(int32_t) * (size_t)(feat->phi.nnz + 1)));
-        GRF_CUDA_TRY(cudaFuncSetAttribute(mask_positions_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_pos));
-        {
-            grf_launch_scope scope(ctx, 8);
-            mask_positions_kernel<<<nblocks * MASK_POS_PARTS, 256, smem_pos, ctx->stream>>>(
-                N, Nk, R, (const int32_t*)feat->phi.rowptr.ptr, (const int32_t*)feat->phi.col.ptr,
-                (const int32_t*)feat->plan_off.ptr, (const int32_t*)feat->plan_cnt.ptr, (const int32_t*)feat->plan_col.ptr,
-                (const int32_t*)feat->psit.rowptr.ptr, (const int32_t*)feat->psit.col.ptr, (const uint32_t*)K.bits.ptr,
-                (const int32_t*)K.node_off.ptr, blk_pos, (unsigned short*)K.pos16.ptr, (int32_t*)K.phi_pos.ptr);
-        }
-    }
-    GRF_TRY(launch_mask_values(ctx, feat, by_position));
-    GRF_CUDA_TRY(cudaGetLastError());
-    K.by_position = by_position;
+    GRF_TRY(reserve_with_headroom(&K.val, (size_t)K.entries * BQ * sizeof(__nv_bfloat16)));
+    GRF_TRY(launch_mask_values(ctx, feat, K.by_position));
     K.structure_ready = true;
     K.ready = true;
     return GRF_OK;
@@ -1128,11 +1035,12 @@ static bool mhat_shape(int32_t m, int32_t d, int dtype)
 // Which association of the product serves a batch of grf_masked_linear_attn: the per-node states of Eq. 12, or the
 // mask formed first.  The choice depends on the features' sizes and the batch only (never on earlier calls), so equal
 // calls give equal bits.  Times in nanoseconds, fitted on a B200 to clouds, grids and expanders of 2^6 .. 2^17 nodes:
-//   states   per problem: 0.52 per node-list entry (a state tile into shared memory) and 0.04 per non-zero (a key's rows
-//            into a state, z into a denominator), both at m = 32 and in proportion to m;
-//   mask     per problem: 2.5 per 64-key tile and 15 per block; once: 0.0022 per multiply-add of Phi Psi^T (non-zeros of Phi
-//            times the mean row of Psi^T, again for every further segment of the lists), 500 per block for the lists,
-//            80 000 for the launches and the wait.
+//   states   per problem: 0.52 per node-list entry (a state tile into shared memory) or 0.25 per non-zero (the same out of
+//            L2, for one query) and 0.04 per non-zero (a key's rows into a state, z into a denominator), all at m = 32 and
+//            in proportion to m;
+//   mask     per problem: 2.5 per 64-key tile and 15 per block; once: 0.0019 per multiply-add of Phi Psi^T (non-zeros of Phi
+//            times the mean row of Psi^T, again for every further segment of the lists), 0.002 per mask entry, 600 per
+//            block for the lists, 40 000 for the launches and the wait.
 // The mask is charged as if this call had to form it, although frozen features keep it: a batch too small for that keeps
 // to the states.
 int grf_linear_by_mask(grf_ctx* ctx, const grf_features* cfeat, int32_t G, int32_t N, int32_t m, int32_t d, int dtype,
@@ -1147,15 +1055,16 @@ int grf_linear_by_mask(grf_ctx* ctx, const grf_features* cfeat, int32_t G, int32
     if (!feat->plan_ready || K.refused) return GRF_OK;
     const double scale = m / 32.0;
     const double nnz = 0.5 * ((double)feat->phi.nnz + (double)feat->psi.nnz);
-    const double states = G * scale * (0.52 * (double)feat->plan_entries + 0.04 * nnz);
+    const double tiles = 0.52 * (double)feat->plan_entries, single = 0.25 * (double)feat->phi.nnz;
+    const double states = G * scale * ((tiles < single ? tiles : single) + 0.04 * nnz);
     const double macs = (double)feat->phi.nnz * (double)feat->psi.nnz / feat->psit.rows;
-    const double build = 80000.0 + 500.0 * feat->plan_blocks + 0.0022 * macs;
+    const double build = 40000.0 + 600.0 * feat->plan_blocks + 0.0019 * macs;
     if (build > states) return GRF_OK;                          // already without the attention itself
     if (!K.lists_ready) GRF_TRY(prepare_mask_lists(ctx, feat));
     if (K.refused || (int64_t)G * K.blocks > 0x7fffffffll || (int64_t)G * N > 0x7fffffffll) return GRF_OK;
     const double attn = G * (2.5 * scale * (double)(K.entries / KT) + 15.0 * K.blocks);
     const double lists = (double)K.entries / K.blocks / (MVP_ROOM / MVP_MIN_WARPS);     // mean list, in accumulator segments
-    const double more = lists > 1.0 ? 0.0022 * macs * (lists - 1.0) : 0.0;
+    const double more = (lists > 1.0 ? 0.0019 * macs * (lists - 1.0) : 0.0) + 0.002 * (double)K.entries * BQ;
     if (build + more + attn > states) return GRF_OK;
     if (!K.ready) {
         const int rc = build_mask(ctx, feat);

@@ -100,7 +100,7 @@ struct grf_kept_walks {
 
 // The mask estimate Mhat = Phi Psi^T held as dense blocks: for every block of GRF_PLAN_BLOCK consecutive rows the
 // sorted list of the keys j that any of its rows reaches (padded to a multiple of GRF_MASK_TILE with the last key
-// and zero values) and the block's values in bf16, laid out [group of 8 keys][row of the block][8 keys].
+// and zero values) and the block's values in bf16, laid out [group of 16 keys][row of the block][16 keys].
 #define GRF_MASK_TILE 64
 struct grf_mask_dev {
     bool ready = false;             // the blocks hold the mask of the present features
@@ -114,10 +114,11 @@ struct grf_mask_dev {
     int32_t blocks = 0;
     int64_t entries = 0;            // padded key entries over all blocks
     grf_buf off, cnt, key;          // cnt holds [blocks] padded counts, then [blocks] the blocks by decreasing count
-    grf_buf bits;                   // per block one bit per key: the block's key set
-    // build scratch: where each node's key positions start (within its block; the blocks' offsets), the positions,
-    // and per non-zero of Phi the start of its node's positions
-    grf_buf node_off, blk_pos, pos16, phi_pos;
+    grf_buf bits;                   // per block one bit per key and the ranks, where positions are looked up row by row
+    // build scratch: where each node's key positions start within its block, the positions, and per non-zero of Phi the
+    // start of its node's positions
+    grf_buf node_off, pos16, phi_pos;
+    grf_buf totals;                 // sizes as the structure kernel adds them up
     grf_buf val;
 };
 
