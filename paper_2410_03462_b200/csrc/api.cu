@@ -1,27 +1,95 @@
 // C-ABI entry points that are not kernels themselves: contexts, buffers, feature objects, the
 // attention driver (Alg. 1 step 5 in chunks of problems) and the host-buffer path.
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <new>
 
 #include <nvtx3/nvToolsExt.h>
 
 #include "grf_internal.cuh"
 
+// Device blocks that were given back, for the next object of about that size: making a feature object costs a dozen
+// cudaMalloc calls otherwise (3 .. 300 ms on a busy host, against 1.5 ms for sampling and attention at N = 32768), and
+// replacing one as many cudaFree calls.  At most POOL_BYTES per device; emptied when the last context goes and when
+// an allocation fails.  A block is given back only after the device has finished with it, as with cudaFree.
+namespace {
+
+struct block_pool {
+    static constexpr size_t POOL_BYTES = (size_t)1 << 30;
+    static constexpr int DEVICES = 64;
+    std::mutex lock;
+    std::multimap<size_t, void*> blocks[DEVICES];
+    size_t held[DEVICES] = {};
+    int contexts = 0;
+
+    void* take(int dev, size_t bytes, size_t* got)
+    {
+        std::lock_guard<std::mutex> g(lock);
+        auto it = blocks[dev].lower_bound(bytes);
+        if (it == blocks[dev].end() || it->first > bytes + bytes / 2 + 4096) return nullptr;
+        void* p = it->second;
+        *got = it->first;
+        held[dev] -= it->first;
+        blocks[dev].erase(it);
+        return p;
+    }
+    bool put(int dev, void* p, size_t bytes)
+    {
+        std::lock_guard<std::mutex> g(lock);
+        if (contexts == 0 || held[dev] + bytes > POOL_BYTES) return false;
+        blocks[dev].emplace(bytes, p);
+        held[dev] += bytes;
+        return true;
+    }
+    void empty(int dev)
+    {
+        std::lock_guard<std::mutex> g(lock);
+        for (auto& b : blocks[dev]) cudaFree(b.second);
+        blocks[dev].clear();
+        held[dev] = 0;
+    }
+};
+
+block_pool& pool() { static block_pool* p = new block_pool; return *p; }   // never destroyed: objects may outlive main()
+
+int current_device()
+{
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < block_pool::DEVICES ? dev : -1;
+}
+
+}  // namespace
+
 int grf_buf_reserve(grf_buf* b, size_t bytes)
 {
     if (bytes == 0) bytes = 1;
     if (b->bytes >= bytes) return GRF_OK;
-    if (b->ptr) { cudaFree(b->ptr); b->ptr = nullptr; b->bytes = 0; }
-    void* p = nullptr;
-    const cudaError_t e = cudaMalloc(&p, bytes);
-    if (e != cudaSuccess) { cudaGetLastError(); return GRF_ERR_NOMEM; }
+    if (b->ptr) {
+        cudaDeviceSynchronize();
+        grf_buf_release(b);
+    }
+    // rounded up to an eighth of its power of two, so that blocks of nearly equal objects serve one another
+    size_t step = 512;
+    while (step * 16 < bytes) step *= 2;
+    bytes = (bytes + step - 1) / step * step;
+    const int dev = current_device();
+    void* p = dev >= 0 ? pool().take(dev, bytes, &bytes) : nullptr;
+    if (!p && cudaMalloc(&p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        p = nullptr;
+        if (dev >= 0) pool().empty(dev);
+        if (cudaMalloc(&p, bytes) != cudaSuccess) { cudaGetLastError(); return GRF_ERR_NOMEM; }
+    }
     b->ptr = p; b->bytes = bytes;
     return GRF_OK;
 }
 
+// The device must have finished with the block: callers that cannot know it wait first.
 void grf_buf_release(grf_buf* b)
 {
-    if (b->ptr) cudaFree(b->ptr);
+    const int dev = current_device();
+    if (b->ptr && (dev < 0 || !pool().put(dev, b->ptr, b->bytes))) cudaFree(b->ptr);
     b->ptr = nullptr; b->bytes = 0;
 }
 
@@ -53,6 +121,10 @@ extern "C" int grf_ctx_create(grf_ctx** out, int device, void* cuda_stream)
         delete c;
         return GRF_ERR_CUDA;
     }
+    {
+        std::lock_guard<std::mutex> g(pool().lock);
+        ++pool().contexts;
+    }
     *out = c;
     return GRF_OK;
 }
@@ -61,7 +133,7 @@ extern "C" int grf_ctx_destroy(grf_ctx* ctx)
 {
     if (!ctx) return GRF_ERR_INVALID;
     cudaSetDevice(ctx->device);
-    cudaStreamSynchronize(ctx->stream);
+    cudaDeviceSynchronize();
     grf_settle_sizes(ctx);
     if (ctx->sizes_ready) cudaEventDestroy(ctx->sizes_ready);
     grf_buf* bufs[] = {&ctx->edge_records, &ctx->stage_col, &ctx->stage_val, &ctx->counts, &ctx->scan_blocks,
@@ -81,6 +153,18 @@ extern "C" int grf_ctx_destroy(grf_ctx* ctx)
     for (auto& t : ctx->timed) { cudaEventDestroy(t.beg); cudaEventDestroy(t.end); }
     for (cudaEvent_t e : ctx->free_events) cudaEventDestroy(e);
     delete ctx;
+    bool last = false;
+    {
+        std::lock_guard<std::mutex> g(pool().lock);
+        last = --pool().contexts == 0;
+    }
+    if (last) {
+        int before = 0;
+        cudaGetDevice(&before);
+        for (int dev = 0; dev < block_pool::DEVICES; ++dev)
+            if (pool().held[dev] > 0 && cudaSetDevice(dev) == cudaSuccess) pool().empty(dev);
+        cudaSetDevice(before);
+    }
     return GRF_OK;
 }
 
@@ -210,6 +294,7 @@ extern "C" int grf_features_free(grf_features* feat)
 {
     if (!feat) return GRF_ERR_INVALID;
     cudaSetDevice(feat->device);
+    cudaDeviceSynchronize();                        // its buffers may serve another object next
     if (feat->sizes_from) { feat->sizes_from->sizes_of = nullptr; feat->sizes_from = nullptr; }
     csr_release(&feat->phi); csr_release(&feat->psi); csr_release(&feat->psit);
     grf_buf_release(&feat->plan_off); grf_buf_release(&feat->plan_cnt);
