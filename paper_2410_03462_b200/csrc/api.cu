@@ -409,7 +409,7 @@ static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int
                        int dtype, const void* phiQ, const void* phiK, const void* V, void* out, float* den_out,
                        void* workspace, size_t workspace_bytes)
 {
-    if (by_mask) return grf_mhat_launch(ctx, feat, G, N, m, phiQ, phiK, V, out, den_out);
+    if (by_mask) return grf_mhat_launch(ctx, feat, G, N, m, d, phiQ, phiK, V, out, den_out);
     const size_t per = ws_per_problem(feat->phi.cols, m, d, dtype);
     int64_t chunk = (int64_t)(workspace_bytes / per);
     if (chunk > G) chunk = G;

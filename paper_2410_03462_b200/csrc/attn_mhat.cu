@@ -562,13 +562,14 @@ mask_rows_kernel(int32_t Nk, const int32_t* __restrict__ rows, const int32_t* __
 // (A round trip to tensor memory is about 230 cycles and the hand-overs add several hundred per tile: what bounds
 // the kernel is the length of that chain, not a pipe.)
 
-template <int M> struct MhShape {
-    static constexpr int D = 64;
+// M features of the keys, D values: 64, or 32 with half as long value rows.
+template <int M, int D> struct MhShape {
     // key/value stages in flight: two CTAs' rings then leave the SM the larger part of its L1, which serves the mask
     // values and the rows that neighbouring keys share (eight stages were 8 % slower at the point cloud, 25 % at the grid)
     static constexpr int NS = M <= 32 ? 5 : 3;
     static constexpr int NB = 3;                          // score buffers
-    static constexpr int V_BYTES = KT * 128;              // 64 value rows of 128 bytes, 128-byte swizzle
+    static constexpr int V_BYTES = KT * D * 2;            // 64 value rows of 128 or 64 bytes, swizzled over that length
+    static constexpr uint32_t V_SWIZZLE = D == 64 ? 2u : 4u;
     static constexpr int K_BYTES = KT * M * 2;            // [M/8][KT keys][8] bf16: K-major, unswizzled
     static constexpr int STAGE = V_BYTES + K_BYTES;
     static constexpr int Q_BYTES = BQ * M * 2;            // [M/8][128 rows][8] bf16
@@ -612,7 +613,7 @@ __device__ __forceinline__ void ld_nc_32bytes(const uint4* p, uint4& a, uint4& b
 }
 constexpr int MH_ISSUER_S = 8, MH_ISSUER_O = 9, MH_PRODUCER0 = 10;
 
-template <int M>
+template <int M, int D>
 __global__ void __launch_bounds__(MH_THREADS, 2)
 mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __restrict__ mk_off,
                       const int32_t* __restrict__ mk_cnt, const int32_t* __restrict__ mk_key,
@@ -620,8 +621,8 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
                       const __nv_bfloat16* __restrict__ phiK, const __nv_bfloat16* __restrict__ Vg,
                       __nv_bfloat16* __restrict__ out, float* __restrict__ den_out, int* __restrict__ error_word)
 {
-    using Sh = MhShape<M>;
-    constexpr int NS = Sh::NS, NB = Sh::NB, D = Sh::D;
+    using Sh = MhShape<M, D>;
+    constexpr int NS = Sh::NS, NB = Sh::NB;
     extern __shared__ unsigned char smem_dyn[];
     // kv_full, kv_empty per stage; s_full, p_full per score buffer; acc_done; den_ready; one drain barrier per issuer
     __shared__ __align__(8) unsigned long long bars[2 * NS + 2 * NB + 4];
@@ -772,9 +773,9 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
         }
     } else if (warp >= MH_PRODUCER0) {
         // ------------------------------------------------------------ producers: warp w takes keys 16w .. 16w+15 of every tile
-        // Lanes x and x + 16 hold key x of the warp's sixteen.  Rows travel as 16-byte pieces.  Value rows (128
-        // bytes): eight consecutive lanes copy one row, piece c of tile row r going to r * 128 + ((c ^ (r & 7)) * 16),
-        // the 128-byte swizzle the second product's operand descriptor names.  Key-feature rows: piece c of key y
+        // Lanes x and x + 16 hold key x of the warp's sixteen.  Rows travel as 16-byte pieces.  Value rows: D / 8
+        // consecutive lanes copy one row, into the swizzle that the second product's operand descriptor names (128-byte
+        // rows: piece c of row r at c ^ (r & 7); 64-byte rows: at c ^ (r / 2 & 3)).  Key-feature rows: piece c of key y
         // goes to (c * 64 + y) * 16; lanes 0-15 copy the even pieces, lanes 16-31 the odd ones.  A warp's copies of
         // one tile arrive on the stage's barrier by themselves as they land (the barrier counts all 128 producer
         // threads), so a producer never waits for its own copies; the issuing threads run the proxy fence between
@@ -783,7 +784,8 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
         const __nv_bfloat16* Kg = phiK + (size_t)g * N * M;
         const __nv_bfloat16* Vh = Vg + (size_t)g * N * D;
         const int ky = pw * 16 + (lane & 15);                   // this lane's key within the tile
-        const int vc = lane & 7;                                // its piece of a value row
+        constexpr int VP = D / 8;                               // pieces of a value row
+        const int vc = lane % VP;                               // its piece of a value row
         bool ok = true;
         const int32_t* kp = mk_key + off + ky;
         int32_t k1 = T > 0 ? __ldg(kp) : 0, k2 = T > 1 ? __ldg(kp + KT) : 0, k3 = T > 2 ? __ldg(kp + 2 * KT) : 0;
@@ -797,12 +799,13 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
             if (!ok) break;
             const uint32_t v_st = stage_base + (uint32_t)s * Sh::STAGE, k_st = v_st + Sh::V_BYTES;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int y = (lane >> 3) + 4 * i;              // key of the warp's sixteen
+            for (int i = 0; i < VP / 2; ++i) {
+                const int y = lane / VP + (32 / VP) * i;        // key of the warp's sixteen
                 const int32_t kv = __shfl_sync(0xffffffffu, k, y);
                 const int r = pw * 16 + y;
+                const int piece = D == 64 ? vc ^ (r & 7) : vc ^ (r >> 1 & 3);
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
-                             ::"r"(v_st + (uint32_t)(r * 128 + ((vc ^ (r & 7)) << 4))), "l"(Vh + (size_t)kv * D + vc * 8) : "memory");
+                             ::"r"(v_st + (uint32_t)(r * (D * 2) + piece * 16)), "l"(Vh + (size_t)kv * D + vc * 8) : "memory");
             }
 #pragma unroll
             for (int c2 = 0; c2 < M / 16; ++c2) {
@@ -844,6 +847,7 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
     } else {
         // ------------------------------------------------------------ O += P_t V_t (the whole warp runs the loop in step)
         constexpr uint32_t idesc_o = instr_desc(D, false, true);       // V is MN-major (rows of d values)
+        constexpr uint32_t ATOM = 8u * D * 2u;                         // eight value rows
         bool ok = true;
         int buf = 0;
         uint32_t par = 0u;
@@ -858,7 +862,7 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
             const uint32_t v_st = stage_base + (uint32_t)s * Sh::STAGE;
 #pragma unroll
             for (int ks = 0; ks < KT / 16; ++ks) {
-                const uint64_t bd = swizzled_desc(v_st + (uint32_t)ks * 2048u, 1024u, 1024u, 2);
+                const uint64_t bd = swizzled_desc(v_st + (uint32_t)ks * 2u * ATOM, ATOM, ATOM, Sh::V_SWIZZLE);
                 mma_bf16_ts(tmem_base + (uint32_t)Sh::O_COL, p_op + (uint32_t)ks * 8u, bd, idesc_o, (t > 0 || ks > 0) ? 1u : 0u);
             }
             mma_commit(kv_empty(s));                                   // frees the stage and the score buffer
@@ -1029,18 +1033,26 @@ extern "C" int grf_features_materialise(grf_ctx* ctx, grf_features* feat)
 
 static bool mhat_shape(int32_t m, int32_t d, int dtype)
 {
-    return dtype == GRF_DTYPE_BF16 && d == 64 && (m == 16 || m == 32 || m == 64);
+    return dtype == GRF_DTYPE_BF16 && (d == 64 || d == 32) && (m == 16 || m == 32 || m == 64);
 }
 
 // Which association of the product serves a batch of grf_masked_linear_attn: the per-node states of Eq. 12, or the
 // mask formed first.  The choice depends on the features' sizes and the batch only (never on earlier calls), so equal
 // calls give equal bits.  Times in nanoseconds, fitted on a B200 to clouds, grids and expanders of 2^6 .. 2^17 nodes:
-//   states   per problem: 0.52 per node-list entry (a state tile into shared memory) or 0.25 per non-zero (the same out of
-//            L2, for one query) and 0.04 per non-zero (a key's rows into a state, z into a denominator), all at m = 32 and
-//            in proportion to m;
-//   mask     per problem: 2.5 per 64-key tile and 15 per block; once: 0.0019 per multiply-add of Phi Psi^T (non-zeros of Phi
-//            times the mean row of Psi^T, again for every further segment of the lists), 0.002 per mask entry, 600 per
-//            block for the lists, 40 000 for the launches and the wait.
+//   states   per problem: 0.52 per node-list entry (a state tile into shared memory) or 0.17 per non-zero (the same out of
+//            L2, for one query) and 0.04 per non-zero (a key's rows into a state, z into a denominator); once, with the
+//            tiles: 150 per entry of a block's list (its chain of tiles: what few blocks wait for); 0.67 of all that at
+//            m = 16, 1.67 at m = 64 (measured at 32768 points, 8 problems: 2.0, 2.4, 4.4 ms at d = 64 and 1.8, 2.6, 4.6 ms
+//            at d = 32, which is therefore charged alike; by the mask 1.03, 1.05, 1.22 and 1.02, 1.04, 1.20); 20 000 for
+//            launches;
+//   mask     per problem: 2.5 per 64-key tile at m = 32 (0.8 of that at m = 16, 1.4 at m = 64) and 15 per block; once:
+//            0.0011 per multiply-add of Phi Psi^T (non-zeros of Phi times the mean row of Psi^T, again for every further
+//            segment of the lists), 0.004 per mask entry, 60 000 for launches and the wait (0.07 ms measured at 2048
+//            points, 0.14 at 4096, 0.20 at 8192, 0.41 at 16384, 0.74 at 32768).
+// The number of keys is not known before the lists are made, which is a quarter of the mask's cost, so it is estimated for
+// the decision: 2.5 per node-list entry where the rows of a block share their nodes (1.8 to 2.8 on clouds of 2048 to 32768
+// points), otherwise as many distinct keys as the blocks' nodes would draw at random.  With the lists there, the known
+// number may still turn the call back to the states if what is left to do costs more.
 // The mask is charged as if this call had to form it, although frozen features keep it: a batch too small for that keeps
 // to the states.
 int grf_linear_by_mask(grf_ctx* ctx, const grf_features* cfeat, int32_t G, int32_t N, int32_t m, int32_t d, int dtype,
@@ -1053,19 +1065,26 @@ int grf_linear_by_mask(grf_ctx* ctx, const grf_features* cfeat, int32_t G, int32
     if (feat->psi.rows != N || !mask_fits_smem(feat)) return GRF_OK;
     GRF_TRY(grf_ensure_block_plan(ctx, feat, false));
     if (!feat->plan_ready || K.refused) return GRF_OK;
-    const double scale = m / 32.0;
+    const double state_scale = (m + 16) / 48.0, mask_scale = (m + 48) / 80.0;
     const double nnz = 0.5 * ((double)feat->phi.nnz + (double)feat->psi.nnz);
-    const double tiles = 0.52 * (double)feat->plan_entries, single = 0.25 * (double)feat->phi.nnz;
-    const double states = G * scale * ((tiles < single ? tiles : single) + 0.04 * nnz);
+    const double tiles = G * 0.52 * (double)feat->plan_entries + 150.0 * (double)feat->plan_entries / feat->plan_blocks;
+    const double single = G * 0.17 * (double)feat->phi.nnz;
+    const double states = 20000.0 + state_scale * ((tiles < single ? tiles : single) + G * 0.04 * nnz);
     const double macs = (double)feat->phi.nnz * (double)feat->psi.nnz / feat->psit.rows;
-    const double build = 40000.0 + 600.0 * feat->plan_blocks + 0.0019 * macs;
-    if (build > states) return GRF_OK;                          // already without the attention itself
+    const double build = 60000.0 + 0.0011 * macs;
+    auto rest = [&](double entries) {                           // values and attention for lists of so many keys in all
+        const double lists = entries / feat->plan_blocks / (MVP_ROOM / MVP_MIN_WARPS);      // mean list, in accumulator segments
+        return (lists > 1.0 ? 0.0011 * macs * (lists - 1.0) : 0.0) + 0.004 * entries * BQ +
+               G * (2.5 * mask_scale * entries / KT + 15.0 * feat->plan_blocks);
+    };
+    const double list = (double)feat->plan_entries / feat->plan_blocks;
+    const double drawn = N * (1.0 - exp(-list * (double)feat->psi.nnz / feat->psit.rows / N));
+    const double shared = 2.5 * list < N ? 2.5 * list : N;
+    const double keys = 1.8 * (double)feat->plan_entries > (double)feat->phi.nnz ? drawn : shared;
+    if (build + rest(keys * feat->plan_blocks) > states) return GRF_OK;
     if (!K.lists_ready) GRF_TRY(prepare_mask_lists(ctx, feat));
     if (K.refused || (int64_t)G * K.blocks > 0x7fffffffll || (int64_t)G * N > 0x7fffffffll) return GRF_OK;
-    const double attn = G * (2.5 * scale * (double)(K.entries / KT) + 15.0 * K.blocks);
-    const double lists = (double)K.entries / K.blocks / (MVP_ROOM / MVP_MIN_WARPS);     // mean list, in accumulator segments
-    const double more = (lists > 1.0 ? 0.0019 * macs * (lists - 1.0) : 0.0) + 0.002 * (double)K.entries * BQ;
-    if (build + more + attn > states) return GRF_OK;
+    if (0.75 * build + rest((double)K.entries) > states) return GRF_OK;
     if (!K.ready) {
         const int rc = build_mask(ctx, feat);
         if (rc == GRF_ERR_TOO_LARGE || rc == GRF_ERR_NOMEM) { K.refused = true; return GRF_OK; }
@@ -1098,18 +1117,18 @@ extern "C" int grf_mask_rows(grf_ctx* ctx, const grf_features* feat, int32_t n, 
     return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
 }
 
-template <int M>
+template <int M, int D>
 static int launch_mhat(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, const void* phiQ, const void* phiK,
                        const void* V, void* out, float* den_out)
 {
-    using Sh = MhShape<M>;
+    using Sh = MhShape<M, D>;
     const grf_mask_dev& K = feat->mask;
     // at most two CTAs per SM: each holds half of the SM's tensor memory
     const size_t smem = Sh::SMEM > 78 * 1024 ? Sh::SMEM : 78 * 1024;
-    GRF_CUDA_TRY(cudaFuncSetAttribute(mhat_attention_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    GRF_CUDA_TRY(cudaFuncSetAttribute(mhat_attention_kernel<M, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     {
         grf_launch_scope scope(ctx, 9);
-        mhat_attention_kernel<M><<<(unsigned)K.blocks * (unsigned)G, MH_THREADS, smem, ctx->stream>>>(
+        mhat_attention_kernel<M, D><<<(unsigned)K.blocks * (unsigned)G, MH_THREADS, smem, ctx->stream>>>(
             G, K.blocks, N, (const int32_t*)K.off.ptr, (const int32_t*)K.cnt.ptr, (const int32_t*)K.key.ptr,
             (const uint4*)K.val.ptr, (const __nv_bfloat16*)phiQ, (const __nv_bfloat16*)phiK, (const __nv_bfloat16*)V,
             (__nv_bfloat16*)out, den_out, ctx->error_word);
@@ -1117,22 +1136,30 @@ static int launch_mhat(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_
     return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
 }
 
-int grf_mhat_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, const void* phiQ,
+template <int M>
+static int launch_mhat_values(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t d, const void* phiQ,
+                              const void* phiK, const void* V, void* out, float* den_out)
+{
+    return d == 32 ? launch_mhat<M, 32>(ctx, feat, G, N, phiQ, phiK, V, out, den_out)
+                   : launch_mhat<M, 64>(ctx, feat, G, N, phiQ, phiK, V, out, den_out);
+}
+
+int grf_mhat_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, const void* phiQ,
                     const void* phiK, const void* V, void* out, float* den_out)
 {
-    if (m == 16) return launch_mhat<16>(ctx, feat, G, N, phiQ, phiK, V, out, den_out);
-    if (m == 32) return launch_mhat<32>(ctx, feat, G, N, phiQ, phiK, V, out, den_out);
-    return launch_mhat<64>(ctx, feat, G, N, phiQ, phiK, V, out, den_out);
+    if (m == 16) return launch_mhat_values<16>(ctx, feat, G, N, d, phiQ, phiK, V, out, den_out);
+    if (m == 32) return launch_mhat_values<32>(ctx, feat, G, N, d, phiQ, phiK, V, out, den_out);
+    return launch_mhat_values<64>(ctx, feat, G, N, d, phiQ, phiK, V, out, den_out);
 }
 
 extern "C" int grf_masked_attn_mhat(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d,
                                     int dtype, const void* phiQ, const void* phiK, const void* V, void* out, float* den_out)
 {
     if (!ctx || !feat || !phiQ || !phiK || !V || !out || G <= 0 || N <= 0) return GRF_ERR_INVALID;
-    if (!mhat_shape(m, d, dtype)) return GRF_ERR_INVALID;
+    if (!mhat_shape(m, d, dtype) || d != 64) return GRF_ERR_INVALID;
     if (!feat->mask.ready || !feat->mask.requested || feat->phi.rows != N || feat->psi.rows != N) return GRF_ERR_INVALID;
     if ((int64_t)G * N > 0x7fffffffll || (int64_t)G * feat->mask.blocks > 0x7fffffffll) return GRF_ERR_TOO_LARGE;
     if (((uintptr_t)phiQ | (uintptr_t)phiK | (uintptr_t)V | (uintptr_t)out) & 15u) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
-    return grf_mhat_launch(ctx, feat, G, N, m, phiQ, phiK, V, out, den_out);
+    return grf_mhat_launch(ctx, feat, G, N, m, d, phiQ, phiK, V, out, den_out);
 }

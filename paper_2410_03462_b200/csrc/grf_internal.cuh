@@ -196,7 +196,7 @@ void grf_mask_values_stale(grf_features* feat);
 // Whether grf_masked_linear_attn evaluates this batch over the materialised mask; forms the mask when it does.
 int grf_linear_by_mask(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, int dtype,
                        bool* by_mask);
-int grf_mhat_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, const void* phiQ,
+int grf_mhat_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, const void* phiQ,
                     const void* phiK, const void* V, void* out, float* den_out);
 void grf_mask_release(grf_features* feat);
 // attn_gather_tc.cu

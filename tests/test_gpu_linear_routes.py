@@ -12,8 +12,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("m", [16, 32, 64])
-@pytest.mark.parametrize("N,G", [(127, 8), (129, 40), (1000, 96)])
-def test_both_routes_match_oracle(N, G, m):
+@pytest.mark.parametrize("N,G,d", [(127, 8, 64), (129, 40, 64), (1000, 96, 64), (128, 96, 32), (1000, 97, 32)])
+def test_both_routes_match_oracle(N, G, d, m):
     from paper_2410_03462_b200 import api, binding as B
     ctx = api.Context(0)
     w = configs.point_cloud_4096(N)
@@ -21,7 +21,7 @@ def test_both_routes_match_oracle(N, G, m):
     f = oracle.deconvolve(w.alpha).astype(np.float32)
     feat = api.sample(ctx, api.DeviceGraph(g), 3, w.n_walks, w.p_halt, w.max_len, f)
     Phi, _, PsiT, _, _ = helpers.oracle_features(w, g, 3, f)
-    q, k, v = tensors.qkv(G, N, m, 64, "bf16", 4)
+    q, k, v = tensors.qkv(G, N, m, d, "bf16", 4)
     qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
     one = slice(G - 1, G)
     ref = oracle.attn_sparse(tensors.widen(q[one]), tensors.widen(k[one]), tensors.widen(v[one]), Phi, PsiT)
@@ -33,7 +33,7 @@ def test_both_routes_match_oracle(N, G, m):
         helpers.assert_attn_close(out[mode][one].float().cpu().numpy(), ref, helpers.TOL["bf16"], den[one].cpu().numpy(),
                                   f"mode {mode}", same_sign=True)
     B.grf_ctx_use_tensor_cores(ctx.handle, 1)
-    small = B.grf_attn_workspace_bytes(1, N, m, 64, B.GRF_DTYPE_BF16)
+    small = B.grf_attn_workspace_bytes(1, N, m, d, B.GRF_DTYPE_BF16)
     assert torch.equal(out[1], api.masked_linear_attn(ctx, feat, qd, kd, vd, workspace_bytes=small))
     with pytest.raises(B.GrfError):         # the caller never asked for the mask
         api.masked_attn_mhat(ctx, feat, qd, kd, vd)
