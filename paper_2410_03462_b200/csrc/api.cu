@@ -202,7 +202,8 @@ extern "C" int grf_ctx_use_tensor_cores(grf_ctx* ctx, int enable)
 {
     if (!ctx) return GRF_ERR_INVALID;
     ctx->use_tensor_cores = enable != 0;
-    ctx->states_only = enable == 2;
+    ctx->states_only = enable == 2 || enable == 3;
+    ctx->tiles_only = enable == 3;
     return GRF_OK;
 }
 
@@ -404,8 +405,9 @@ extern "C" size_t grf_attn_workspace_bytes(int32_t G, int32_t R, int32_t m, int3
 }
 
 // The attention of G problems once the route is known: over the mask in one launch, or through the per-node states in
-// chunks of as many problems as the workspace holds.
-static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int32_t G, int32_t N, int32_t m, int32_t d,
+// chunks of as many problems as the workspace holds.  G_all is the size of the whole batch that they belong to: it picks
+// the gather, so that parts of a batch give the bits of the whole.
+static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int32_t G_all, int32_t G, int32_t N, int32_t m, int32_t d,
                        int dtype, const void* phiQ, const void* phiK, const void* V, void* out, float* den_out,
                        void* workspace, size_t workspace_bytes)
 {
@@ -417,7 +419,7 @@ static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int
     const size_t es = elem_size(dtype);
     // the plan's build waits for the stream once: do it before the attention kernels are queued, not between them
     bool tc_gather = false;
-    GRF_TRY(grf_gather_by_tensor_cores(ctx, feat, m, d, dtype, &tc_gather));
+    GRF_TRY(grf_gather_by_tensor_cores(ctx, feat, G_all, m, d, dtype, &tc_gather));
     for (int64_t g0 = 0; g0 < G; g0 += chunk) {
         const int32_t gc = (int32_t)((G - g0) < chunk ? (G - g0) : chunk);
         const char* k_ptr = (const char*)phiK + (size_t)g0 * N * m * es;
@@ -451,7 +453,7 @@ extern "C" int grf_masked_linear_attn(grf_ctx* ctx, const grf_features* feat, in
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
     bool by_mask = false;
     if (aligned16(phiQ, phiK, V, out)) GRF_TRY(grf_linear_by_mask(ctx, feat, G, N, m, d, dtype, &by_mask));
-    return linear_attn(ctx, feat, by_mask, G, N, m, d, dtype, phiQ, phiK, V, out, den_out, workspace, workspace_bytes);
+    return linear_attn(ctx, feat, by_mask, G, G, N, m, d, dtype, phiQ, phiK, V, out, den_out, workspace, workspace_bytes);
 }
 
 static int check_graph_host(int32_t N, const int32_t* rowptr, const int32_t* col)
@@ -543,7 +545,7 @@ extern "C" int grf_step_host(grf_ctx* ctx, int32_t N, const int32_t* rowptr, con
         const size_t qo = (size_t)g0 * N * m * es, vo = (size_t)g0 * N * d * es;
         for (int u = p * per_step; u < (p + 1) * per_step && u < parts; ++u)
             if (u * gp < G) GRF_CUDA_TRY(cudaStreamWaitEvent(s, ctx->up_done[u], 0));
-        GRF_TRY(linear_attn(ctx, ctx->h_feat, by_mask, gc, N, m, d, dtype, (const char*)ctx->h_q.ptr + qo,
+        GRF_TRY(linear_attn(ctx, ctx->h_feat, by_mask, G, gc, N, m, d, dtype, (const char*)ctx->h_q.ptr + qo,
                             (const char*)ctx->h_k.ptr + qo, (const char*)ctx->h_v.ptr + vo, (char*)ctx->h_out.ptr + vo,
                             nullptr, ctx->h_ws.ptr, ctx->h_ws.bytes));
         GRF_CUDA_TRY(cudaEventRecord(ctx->part_done[p], s));

@@ -652,15 +652,32 @@ int grf_ensure_block_plan(grf_ctx* ctx, const grf_features* feat, bool with_coef
     return GRF_OK;
 }
 
-// The tensor-core gather brings a tile into shared memory once per block of 128 queries that touches its node (0.52 ns per
-// list entry at m = 32, d = 64), the ALU gather once per query out of L2 (0.29 ns per non-zero): where fewer than 1.8
-// queries of a block share a node on average, as on expanders, the second is faster and needs no coefficient table.
-int grf_gather_by_tensor_cores(grf_ctx* ctx, const grf_features* feat, int32_t m, int32_t d, int dtype, bool* yes)
+// The tensor-core gather brings a tile into shared memory once per block of 128 queries that touches its node, the ALU gather
+// once per query out of L2.  In nanoseconds, fitted on a B200 to clouds, grids, lattices and expanders of 36 .. 65536 nodes:
+//   tiles    20 000 for the coefficient table; per problem 0.5 per list entry at m = 32 (0.67 of that at m = 16, 1.67 at
+//            m = 64); once 25 + 4.2 m per entry of a block's list, the chain that few blocks wait for;
+//   rows     8 000, and per problem 0.2 per non-zero at m = 32, d = 64, in proportion to m d and a part of its own.
+// us measured, tiles / rows: expander of 1024 nodes, 2 problems, m = 16: 109 / 27, of 4096 349 / 66; lattice of 400 27 / 11;
+// cloud of 2048, 4 problems, m = 16: 81 / 59, of 8192 169 / 262, of 32768 (8 problems, m = 32) 1386 / 4528.
+double grf_gather_tiles_ns(const grf_features* feat, int32_t G, int32_t m)
+{
+    const double entries = feat->plan_entries;
+    return 20000.0 + G * 0.5 * (m + 16) / 48.0 * entries + (25.0 + 4.2 * m) * entries / feat->plan_blocks;
+}
+double grf_gather_rows_ns(const grf_features* feat, int32_t G, int32_t m, int32_t d)
+{
+    return 8000.0 + G * 0.2 * ((double)m * d + 256.0) / 2304.0 * (double)feat->phi.nnz;
+}
+
+int grf_gather_by_tensor_cores(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t m, int32_t d, int dtype, bool* yes)
 {
     *yes = false;
     if (dtype != GRF_DTYPE_BF16 || !ctx->use_tensor_cores || m % 16 != 0 || d % 16 != 0) return GRF_OK;
+    const double rows = grf_gather_rows_ns(feat, G, m, d);
+    if (rows < GRF_PLAN_WORTH_NS && !ctx->tiles_only) return GRF_OK;
     GRF_TRY(grf_ensure_block_plan(ctx, feat, false));
-    if (!feat->plan_ready || 1.8 * (double)feat->plan_entries > (double)feat->phi.nnz) return GRF_OK;
+    if (!feat->plan_ready) return GRF_OK;
+    if (rows <= grf_gather_tiles_ns(feat, G, m) && !ctx->tiles_only) return GRF_OK;
     *yes = true;
     return grf_ensure_block_plan(ctx, feat);                  // with the coefficient table
 }

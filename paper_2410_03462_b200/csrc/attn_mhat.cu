@@ -1039,12 +1039,10 @@ static bool mhat_shape(int32_t m, int32_t d, int dtype)
 // Which association of the product serves a batch of grf_masked_linear_attn: the per-node states of Eq. 12, or the
 // mask formed first.  The choice depends on the features' sizes and the batch only (never on earlier calls), so equal
 // calls give equal bits.  Times in nanoseconds, fitted on a B200 to clouds, grids and expanders of 2^6 .. 2^17 nodes:
-//   states   per problem: 0.52 per node-list entry (a state tile into shared memory) or 0.17 per non-zero (the same out of
-//            L2, for one query) and 0.04 per non-zero (a key's rows into a state, z into a denominator); once, with the
-//            tiles: 150 per entry of a block's list (its chain of tiles: what few blocks wait for); 0.67 of all that at
-//            m = 16, 1.67 at m = 64 (measured at 32768 points, 8 problems: 2.0, 2.4, 4.4 ms at d = 64 and 1.8, 2.6, 4.6 ms
-//            at d = 32, which is therefore charged alike; by the mask 1.03, 1.05, 1.22 and 1.02, 1.04, 1.20); 20 000 for
-//            launches;
+//   states   the cheaper gather, 15 000 for launches, and per problem 0.04 per non-zero at m = 32 (a key's rows into a
+//            state, z into a denominator; 0.67 of that at m = 16, 1.67 at m = 64; measured at 32768 points, 8 problems,
+//            all kernels: 2.0, 2.4, 4.4 ms at d = 64 and 1.8, 2.6, 4.6 ms at d = 32, which is therefore charged alike;
+//            by the mask 1.03, 1.05, 1.22 and 1.02, 1.04, 1.20);
 //   mask     per problem: 2.5 per 64-key tile at m = 32 (0.8 of that at m = 16, 1.4 at m = 64) and 15 per block; once:
 //            0.0011 per multiply-add of Phi Psi^T (non-zeros of Phi times the mean row of Psi^T, again for every further
 //            segment of the lists), 0.004 per mask entry, 60 000 for launches and the wait (0.07 ms measured at 2048
@@ -1063,13 +1061,14 @@ int grf_linear_by_mask(grf_ctx* ctx, const grf_features* cfeat, int32_t G, int32
     grf_mask_dev& K = feat->mask;
     if (!ctx->use_tensor_cores || ctx->states_only || !mhat_shape(m, d, dtype)) return GRF_OK;
     if (feat->psi.rows != N || !mask_fits_smem(feat)) return GRF_OK;
+    const double rows = grf_gather_rows_ns(feat, G, m, d);
+    if (rows < GRF_PLAN_WORTH_NS) return GRF_OK;
     GRF_TRY(grf_ensure_block_plan(ctx, feat, false));
     if (!feat->plan_ready || K.refused) return GRF_OK;
     const double state_scale = (m + 16) / 48.0, mask_scale = (m + 48) / 80.0;
     const double nnz = 0.5 * ((double)feat->phi.nnz + (double)feat->psi.nnz);
-    const double tiles = G * 0.52 * (double)feat->plan_entries + 150.0 * (double)feat->plan_entries / feat->plan_blocks;
-    const double single = G * 0.17 * (double)feat->phi.nnz;
-    const double states = 20000.0 + state_scale * ((tiles < single ? tiles : single) + G * 0.04 * nnz);
+    const double tiles = grf_gather_tiles_ns(feat, G, m);
+    const double states = 15000.0 + (tiles < rows ? tiles : rows) + state_scale * G * 0.04 * nnz;
     const double macs = (double)feat->phi.nnz * (double)feat->psi.nnz / feat->psit.rows;
     const double build = 60000.0 + 0.0011 * macs;
     auto rest = [&](double entries) {                           // values and attention for lists of so many keys in all

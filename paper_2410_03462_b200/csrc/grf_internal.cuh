@@ -59,6 +59,7 @@ struct grf_ctx {
     int* error_word = nullptr;      // device word set by a kernel that gave up a bounded wait
     bool use_tensor_cores = true;
     bool states_only = false;       // grf_masked_linear_attn never takes the mask (grf_ctx_use_tensor_cores(ctx, 2))
+    bool tiles_only = false;        // the gather runs on the tensor cores wherever the shape allows it (3)
     bool prefer_mask_route = false; // grf_step_host evaluates the attention over the materialised mask where it can
     bool check_graphs = false;      // grf_sample validates the device-resident CSR first (debugging aid)
     // optional per-launch timing
@@ -202,8 +203,13 @@ void grf_mask_release(grf_features* feat);
 // attn_gather_tc.cu
 int grf_build_block_plan(grf_ctx* ctx, grf_features* feat, bool with_coef = true);
 int grf_ensure_block_plan(grf_ctx* ctx, const grf_features* feat, bool with_coef = true);   // builds it if Phi changed since the last build
+// Estimated times in nanoseconds of the two gathers for a batch of G problems; the first needs the block plan's sizes.
+double grf_gather_tiles_ns(const grf_features* feat, int32_t G, int32_t m);
+double grf_gather_rows_ns(const grf_features* feat, int32_t G, int32_t m, int32_t d);
+// Batches whose plain-ALU gather takes less than this gain nothing from a block plan, which alone takes half of it.
+constexpr double GRF_PLAN_WORTH_NS = 30000.0;
 // Which gather serves this object and shape (prepares the block plan it needs).
-int grf_gather_by_tensor_cores(grf_ctx* ctx, const grf_features* feat, int32_t m, int32_t d, int dtype, bool* yes);
+int grf_gather_by_tensor_cores(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t m, int32_t d, int dtype, bool* yes);
 int grf_gather_contract_tc(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d,
                            const void* phiQ, const void* records, void* out, float* den_out);
 

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("m", [16, 32, 64])
-@pytest.mark.parametrize("N,G,d", [(127, 8, 64), (129, 40, 64), (1000, 96, 64), (128, 96, 32), (1000, 97, 32)])
+@pytest.mark.parametrize("N,G,d", [(127, 8, 64), (129, 40, 64), (1000, 96, 64), (64, 2, 64), (1000, 2, 64), (128, 96, 32), (1000, 97, 32)])
 def test_both_routes_match_oracle(N, G, d, m):
     from paper_2410_03462_b200 import api, binding as B
     ctx = api.Context(0)
@@ -26,7 +26,7 @@ def test_both_routes_match_oracle(N, G, d, m):
     one = slice(G - 1, G)
     ref = oracle.attn_sparse(tensors.widen(q[one]), tensors.widen(k[one]), tensors.widen(v[one]), Phi, PsiT)
     out = {}
-    for mode in (1, 2):                     # 1: the cheaper route, 2: always the states
+    for mode in (1, 2, 3):                  # 1: the cheaper route, 2: always the states, 3: their gather on the tensor cores
         B.grf_ctx_use_tensor_cores(ctx.handle, mode)
         out[mode], den = api.masked_linear_attn(ctx, feat, qd, kd, vd, want_den=True)
         B.grf_ctx_check(ctx.handle)
@@ -35,6 +35,9 @@ def test_both_routes_match_oracle(N, G, d, m):
     B.grf_ctx_use_tensor_cores(ctx.handle, 1)
     small = B.grf_attn_workspace_bytes(1, N, m, d, B.GRF_DTYPE_BF16)
     assert torch.equal(out[1], api.masked_linear_attn(ctx, feat, qd, kd, vd, workspace_bytes=small))
+    B.grf_ctx_use_tensor_cores(ctx.handle, 2)
+    assert torch.equal(out[2], api.masked_linear_attn(ctx, feat, qd, kd, vd, workspace_bytes=small))
+    B.grf_ctx_use_tensor_cores(ctx.handle, 1)
     with pytest.raises(B.GrfError):         # the caller never asked for the mask
         api.masked_attn_mhat(ctx, feat, qd, kd, vd)
     feat.free()
