@@ -283,7 +283,7 @@ int grf_ctx_check(grf_ctx* ctx);
 /* Chooses the attention kernels for bf16 problems: 1 (default) = tensor-core kernels where they apply (state
  * build: m a multiple of 16 and d <= 64; gather-contract: a block plan exists and m, d are multiples of 16);
  * 0 = plain-ALU kernels always; 2 = the tensor-core kernels, and grf_masked_linear_attn always goes through the
- * per-node states; 3 = as 2, and the gather runs on the tensor cores wherever it can, not only where it is the faster.
+ * per-node states; 3 = as 2, on the tensor cores wherever they can be used, not only where they are the faster.
  * Results agree within the stated tolerance. */
 int grf_ctx_use_tensor_cores(grf_ctx* ctx, int enable);
 

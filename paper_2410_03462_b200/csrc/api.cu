@@ -406,7 +406,7 @@ extern "C" size_t grf_attn_workspace_bytes(int32_t G, int32_t R, int32_t m, int3
 
 // The attention of G problems once the route is known: over the mask in one launch, or through the per-node states in
 // chunks of as many problems as the workspace holds.  G_all is the size of the whole batch that they belong to: it picks
-// the gather, so that parts of a batch give the bits of the whole.
+// the kernels, so that parts of a batch give the bits of the whole.
 static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int32_t G_all, int32_t G, int32_t N, int32_t m, int32_t d,
                        int dtype, const void* phiQ, const void* phiK, const void* V, void* out, float* den_out,
                        void* workspace, size_t workspace_bytes)
@@ -419,6 +419,13 @@ static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int
     const size_t es = elem_size(dtype);
     // the plan's build waits for the stream once: do it before the attention kernels are queued, not between them
     bool tc_gather = false;
+    const bool tensor_cores = dtype == GRF_DTYPE_BF16 && ctx->use_tensor_cores;
+    if (tensor_cores) GRF_TRY(grf_features_sizes(feat));        // the choices below read them
+    // The tensor-core build takes 35 us at least (a bucket's chain of segments); the plain one 8 us and 0.27 ns per non-zero
+    // and problem at m = 32, d = 64.  us measured, plain / tensor cores: lattice of 400 nodes, 4 problems 10 / 36, grid of
+    // 196, 8 problems 29 / 44, expander of 1024, 2 problems, m = 16 29 / 44, 4 problems, m = 32 69 / 47.
+    const double plain_ns = 0.27 * ((double)m * d + 512.0) / 2560.0 * (double)G_all * (double)feat->psit.nnz;
+    const bool tc_states = tensor_cores && (plain_ns > 25000.0 || ctx->tiles_only);
     GRF_TRY(grf_gather_by_tensor_cores(ctx, feat, G_all, m, d, dtype, &tc_gather));
     for (int64_t g0 = 0; g0 < G; g0 += chunk) {
         const int32_t gc = (int32_t)((G - g0) < chunk ? (G - g0) : chunk);
@@ -428,7 +435,7 @@ static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int
         char* o_ptr = (char*)out + (size_t)g0 * N * d * es;
         float* den_ptr = den_out ? den_out + (size_t)g0 * N : nullptr;
         int rs = 1;
-        if (dtype == GRF_DTYPE_BF16 && ctx->use_tensor_cores)
+        if (tc_states)
             rs = grf_build_states_tc(ctx, feat->psit, gc, N, m, d, k_ptr, v_ptr, workspace, !tc_gather);
         if (rs > 0) rs = grf_build_states(ctx, feat->psit, gc, N, m, d, dtype, k_ptr, v_ptr, workspace, !tc_gather);
         GRF_TRY(rs);

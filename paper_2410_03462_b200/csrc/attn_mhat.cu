@@ -1061,6 +1061,7 @@ int grf_linear_by_mask(grf_ctx* ctx, const grf_features* cfeat, int32_t G, int32
     grf_mask_dev& K = feat->mask;
     if (!ctx->use_tensor_cores || ctx->states_only || !mhat_shape(m, d, dtype)) return GRF_OK;
     if (feat->psi.rows != N || !mask_fits_smem(feat)) return GRF_OK;
+    GRF_TRY(grf_features_sizes(feat));
     const double rows = grf_gather_rows_ns(feat, G, m, d);
     if (rows < GRF_PLAN_WORTH_NS) return GRF_OK;
     GRF_TRY(grf_ensure_block_plan(ctx, feat, false));

@@ -59,7 +59,7 @@ struct grf_ctx {
     int* error_word = nullptr;      // device word set by a kernel that gave up a bounded wait
     bool use_tensor_cores = true;
     bool states_only = false;       // grf_masked_linear_attn never takes the mask (grf_ctx_use_tensor_cores(ctx, 2))
-    bool tiles_only = false;        // the gather runs on the tensor cores wherever the shape allows it (3)
+    bool tiles_only = false;        // state build and gather run on the tensor cores wherever the shape allows it (3)
     bool prefer_mask_route = false; // grf_step_host evaluates the attention over the materialised mask where it can
     bool check_graphs = false;      // grf_sample validates the device-resident CSR first (debugging aid)
     // optional per-launch timing

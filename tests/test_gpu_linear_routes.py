@@ -26,7 +26,7 @@ def test_both_routes_match_oracle(N, G, d, m):
     one = slice(G - 1, G)
     ref = oracle.attn_sparse(tensors.widen(q[one]), tensors.widen(k[one]), tensors.widen(v[one]), Phi, PsiT)
     out = {}
-    for mode in (1, 2, 3):                  # 1: the cheaper route, 2: always the states, 3: their gather on the tensor cores
+    for mode in (1, 2, 3):                  # 1: the cheaper route, 2: always the states, 3: all on the tensor cores
         B.grf_ctx_use_tensor_cores(ctx.handle, mode)
         out[mode], den = api.masked_linear_attn(ctx, feat, qd, kd, vd, want_den=True)
         B.grf_ctx_check(ctx.handle)
