@@ -8,7 +8,8 @@ Prints ONE JSON line.
     python bench.py --suite        every workload, the unsorted point cloud, the scaling sweep and the operation
                                    counts of Sec. 4: a summary (.md) and one JSON line per run (.jsonl) in --suite-dir
 
-Routes: sz = Alg. 1 through the per-node states S_l, z_l (Eq. 12; the headline); mhat = Eqs. 1-2 over the
+Routes: sz = grf_masked_linear_attn (the headline): Alg. 1 through the per-node states S_l, z_l of Eq. 12 or over the mask,
+whichever the library's cost rule finds cheaper for the batch (`evaluated_by` in the output says which); mhat = Eqs. 1-2 over the
 materialised mask Phi Psi^T; asym = Alg. 2 (asymmetric features, Psi = I).
 
 With N > 1 (launched by torch.distributed.run) every rank runs the same-sized, independently seeded batch
@@ -386,12 +387,15 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
     B.grf_ctx_enable_timing(ctx.handle, False)
     nnz_phi, nnz_psi = feat.shape(0)[2], feat.shape(1)[2]
     plan_entries = mask_entries = None
-    if route == "sz" and w.dtype == "bf16":
+    by_mask = mhat or ktimes.get("mhat_attention", (0.0, 0))[1] > 0      # what grf_masked_linear_attn chose
+    if route == "sz" and w.dtype == "bf16" and not by_mask:
         try:
             plan_entries = B.grf_plan_stats(ctx.handle, feat.handle)[1]
         except B.GrfError:
             plan_entries = None                     # no plan: the plain-ALU gather ran
-    if mhat:
+    if by_mask:
+        if not mhat:
+            B.grf_features_materialise(ctx.handle, feat.handle)          # outside the timed region: the sizes are told to who asked
         mask_entries = B.grf_mask_stats(feat.handle)[1]
 
     # ---- end to end through the host-buffer entry point (pinned host memory; copies inside the timing)
@@ -441,7 +445,7 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
         counters = load_counters()
         alg = algorithmic_bytes(w, N, nnz_phi, nnz_psi, E)
         es = 2 if w.dtype == "bf16" else 4
-        if mhat:   # Q, K, V read once, out written once; the mask blocks written once, read once
+        if by_mask:   # Q, K, V read once, out written once; the mask blocks written once, read once
             mbytes = B.grf_mask_stats(feat.handle)[2]
             alg["mhat_attention"] = w.G * N * (2 * w.m + 2 * w.d) * es + mbytes
             alg["mask_build"] = mbytes + 2 * (nnz_phi + nnz_psi) * 8
@@ -471,6 +475,7 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
                 traffic = c["dram_bytes"] * w.G / c["heads"]
         binds = binding.get(dom, {}).get("binds")
         bound = {"tensor_issue": "tensor", "hbm": "hbm", "integer_issue": "alu"}.get(binds, "hbm" if binds is None else "smem")
+        note = "mhat" if by_mask else route
         step_text = {"sz": "grf_sample (both ensembles) + grf_masked_linear_attn",
                      "mhat": "grf_sample (both ensembles) + grf_features_materialise + grf_masked_attn_mhat",
                      "asym": "grf_sample (f_psi = delta_0) + grf_masked_attn_asym (Alg. 2, %s similarity)"
@@ -479,9 +484,10 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": steps,
             "warmup": warmup, "ms_per_step": total_ms / steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None,
-            "dtype": ("bf16" if w.dtype == "bf16" else "f32"), "dtype_note": DTYPE_NOTE[route] if w.dtype == "bf16" else "fp32 throughout",
+            "dtype": ("bf16" if w.dtype == "bf16" else "f32"), "dtype_note": DTYPE_NOTE[note] if w.dtype == "bf16" else "fp32 throughout",
             "data": "synthetic",
-            "config": {"workload": w.name, "route": route, "N": N, "edges": E, "batch": w.batch, "heads": w.heads, "m": w.m,
+            "config": {"workload": w.name, "route": route, "evaluated_by": "rows" if asym else "mask" if by_mask else "states",
+                       "N": N, "edges": E, "batch": w.batch, "heads": w.heads, "m": w.m,
                        "d": w.d, "n_walks": w.n_walks, "p_halt": w.p_halt, "max_len": w.max_len,
                        "nnz_phi": nnz_phi, "nnz_psi": nnz_psi,
                        "node_order": "as given" if "unsorted" in w.name else
@@ -511,7 +517,7 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
                        "walks_per_s": None if (frozen or remodulate) else 2 * N * w.n_walks / (statistics.mean(sample_ms) * 1e-3),
                        "attn_tokens_per_s": w.batch * N / (statistics.mean(attn_ms) * 1e-3),
                        "attn_hbm_frac": (2 * w.G * N * w.m * w.d * es + w.G * N * (2 * w.m + 2 * w.d) * es) / 1e9 /
-                                        (statistics.mean(attn_ms) * 1e-3) / pk["hbm_gbs"] if route == "sz" else None,
+                                        (statistics.mean(attn_ms) * 1e-3) / pk["hbm_gbs"] if route == "sz" and not by_mask else None,
                        "wall_s_timed_region": wall},
             "kernels": per_kernel,
         }
@@ -727,7 +733,7 @@ def main():
     ap.add_argument("--workload", default="pc32768")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--route", choices=["sz", "asym", "mhat"], default="sz",
-                    help="sz: Alg. 1 through per-node states (the default and the headline); mhat: Eqs. 1-2 over the "
+                    help="sz: grf_masked_linear_attn, states or mask by cost (the default and the headline); mhat: Eqs. 1-2 over the "
                          "materialised mask Phi Psi^T; asym: Alg. 2 (asymmetric features, Psi = I); the last two are "
                          "variants outside the headline metric")
     ap.add_argument("--frozen", action="store_true", help="features sampled (and prepared) once, outside the timed steps")
@@ -758,7 +764,7 @@ def main():
         else:
             res = measure(args, args.workload, args.route, not args.no_cpu_baseline, True, frozen=args.frozen,
                           remodulate=args.remodulate)
-            # beside the headline (the route through the per-node states, features resampled every step): the same
+            # beside the headline (grf_masked_linear_attn, features resampled every step): the same
             # workload on the route over the materialised mask, and both routes with frozen features, in short runs
             if res is not None and world == 1 and args.route == "sz" and not args.frozen and not args.remodulate and not args.no_other_routes:
                 w = make_workload(args.workload)
