@@ -572,7 +572,9 @@ mask_rows_kernel(int32_t Nk, const int32_t* __restrict__ rows, const int32_t* __
 template <int M, int D> struct MhShape {
     // key/value stages in flight: two CTAs' rings then leave the SM the larger part of its L1, which serves the mask
     // values and the rows that neighbouring keys share (eight stages were 8 % slower at the point cloud, 25 % at the grid)
-    static constexpr int NS = M <= 32 ? 5 : 3;
+    // (m = 64, d = 64, 8 problems at 32768 points: three stages 481 us, four 440, five 449; d = 32: 465, 418, 400;
+    // m = 32: four 324, five 313, six 313)
+    static constexpr int NS = M <= 32 || D == 32 ? 5 : 4;
     static constexpr int NB = 3;                          // score buffers
     static constexpr int V_BYTES = KT * D * 2;            // 64 value rows of 128 or 64 bytes, swizzled over that length
     static constexpr uint32_t V_SWIZZLE = D == 64 ? 2u : 4u;
