@@ -960,6 +960,16 @@ static int prepare_mask_lists(grf_ctx* ctx, grf_features* feat)
     GRF_TRY(reserve_with_headroom(&K.phi_pos, sizeof(int32_t) * (size_t)(feat->phi.nnz + 1)));
     GRF_CUDA_TRY(cudaFuncSetAttribute(mask_structure_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     K.by_position = true;
+    if (!K.key.ptr) {
+        // a first guess, so that the kernel need not run twice: 3 keys per node-list entry (see grf_linear_by_mask), and a
+        // mean row of Psi^T of positions for each; not where that is a lot of memory for a guess
+        const int64_t most = (int64_t)nblocks * ((Nk + KT - 1) / KT * KT), guess = 3 * feat->plan_entries;
+        const double positions = 1.125 * (double)feat->plan_entries * (double)feat->psi.nnz / R;
+        if (positions < (double)(128 << 20)) {
+            GRF_TRY(grf_buf_reserve(&K.key, sizeof(int32_t) * (size_t)((guess < most ? guess : most) + KT)));
+            GRF_TRY(grf_buf_reserve(&K.pos16, sizeof(unsigned short) * ((size_t)positions + 256)));
+        }
+    }
     for (int attempt = 0; attempt < 3; ++attempt) {
         const int64_t key_room = (int64_t)(K.key.bytes / sizeof(int32_t));
         const int64_t pos_room = K.by_position ? (int64_t)(K.pos16.bytes / sizeof(unsigned short)) : -1;
