@@ -233,6 +233,16 @@ def binding_report(w, N, nnz_phi, nnz_psi, ktimes, steps, pk, counters, plan_ent
         if issue is not None:
             fr["integer_issue"] = issue
         finish("walk_merge", r, fr)
+    ms, n = ktimes.get("mask_build", (0.0, 0))
+    if n and mask_entries:
+        # every multiply-add of Phi Psi^T reads a position and a value and reads and writes an accumulator: four accesses of
+        # the load/store unit, which takes one warp-wide access a cycle (148 SMs at 1.965 GHz)
+        t = ms / steps * 1e-3
+        macs = nnz_phi * nnz_psi / N / t / 1e9
+        peak = 148 * 32 * 1.965 / 4
+        hbm = (mask_entries * 260 + 2 * (nnz_phi + nnz_psi) * 8) / t / 1e9
+        finish("mask_build", {"multiply_adds_g_per_s": macs, "multiply_adds_peak_g_per_s": peak, "hbm_algorithmic_gbs": hbm},
+               {"load_store_unit": macs / peak, "hbm": hbm / pk["hbm_gbs"]})
     t = per_launch_s("mhat_attention")
     if t and mask_entries:
         issued = mask_entries * G * 2.0 * 128 * (m + d) / t / 1e12
@@ -455,13 +465,13 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
         for name, (ms, n) in ktimes.items():
             if n == 0:
                 continue
-            per = ms / n
+            per = ms / steps                        # the algorithmic bytes are those of a step, whatever the launches
             a = alg.get(name, 0)
             per_kernel[name] = {"ms_per_step": ms / steps, "launch_groups": n, "algorithmic_gb": a / 1e9,
                                 "achieved_gbs": a / 1e9 / (per * 1e-3), "hbm_frac": a / 1e9 / (per * 1e-3) / pk["hbm_gbs"]}
         dom = max(ktimes, key=lambda kname: ktimes[kname][0])
         dom_ms = ktimes[dom][0] / max(ktimes[dom][1], 1)
-        achieved = alg.get(dom, 0) / 1e9 / (dom_ms * 1e-3)
+        achieved = alg.get(dom, 0) / 1e9 / (ktimes[dom][0] / steps * 1e-3)
         binding = binding_report(w, N, nnz_phi, nnz_psi, ktimes, steps, pk, counters, plan_entries, mask_entries)
         # DRAM traffic of the dominant kernel from the tracked profile of the same sources, scaled to this run's heads
         traffic = None

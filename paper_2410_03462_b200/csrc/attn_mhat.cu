@@ -140,18 +140,21 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
     // ---- keys
     // nodes per warp and turn: as few as give every warp some (a short list would leave most of them idle), at most 32
     const int32_t turn = min(32, ((ucnt + MS_THREADS / 32 - 1) / (MS_THREADS / 32) + 1) & ~1);
-    auto each_key = [&](auto&& use) {
+    // (a node's number `of` comes with its extent, one load for 32 nodes, not with every key)
+    auto each_key = [&](const int32_t* of, auto&& use) {
         for (int32_t u0 = warp * turn; u0 < ucnt; u0 += turn * (MS_THREADS / 32)) {
             const int32_t n = min(turn, ucnt - u0);
             const int32_t my_l = lane < n ? __ldg(ulist + u0 + lane) : 0;
             const int32_t my_beg = lane < n ? __ldg(t_rowptr + my_l) : 0;
             const int32_t my_len = lane < n ? __ldg(t_rowptr + my_l + 1) - my_beg : 0;
+            const int32_t my_of = of && lane < n ? of[u0 + lane] : 0;
             for (int32_t e0 = 0; e0 < n; e0 += 2) {
-                int32_t j[2][4], beg[2], len[2];
+                int32_t j[2][4], beg[2], len[2], num[2];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                     beg[e] = __shfl_sync(0xffffffffu, my_beg, (e0 + e) & 31);
                     len[e] = e0 + e < n ? __shfl_sync(0xffffffffu, my_len, (e0 + e) & 31) : 0;
+                    num[e] = __shfl_sync(0xffffffffu, my_of, (e0 + e) & 31);
 #pragma unroll
                     for (int sl = 0; sl < 4; ++sl) j[e][sl] = sl * 32 + lane < len[e] ? __ldg(t_col + beg[e] + sl * 32 + lane) : -1;
                 }
@@ -159,13 +162,13 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
                 for (int e = 0; e < 2; ++e) {
 #pragma unroll
                     for (int sl = 0; sl < 4; ++sl)
-                        if (j[e][sl] >= 0) use(u0 + e0 + e, sl * 32 + lane, j[e][sl]);
-                    for (int32_t x = 128 + lane; x < len[e]; x += 32) use(u0 + e0 + e, x, __ldg(t_col + beg[e] + x));
+                        if (j[e][sl] >= 0) use(num[e] + sl * 32 + lane, j[e][sl]);
+                    for (int32_t x = 128 + lane; x < len[e]; x += 32) use(num[e] + x, __ldg(t_col + beg[e] + x));
                 }
             }
         }
     };
-    each_key([&](int32_t, int32_t, int32_t k) {
+    each_key(nullptr, [&](int32_t, int32_t k) {
         if (!(kbits[k >> 5] >> (k & 31) & 1u)) atomicOr(&kbits[k >> 5], 1u << (k & 31));
     });
     __syncthreads();
@@ -202,14 +205,22 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
     }
     if ((int64_t)base_pos + npos <= pos_room && padded <= 65536) {
         unsigned short* pos = pos16 + base_pos;
-        each_key([&](int32_t u, int32_t x, int32_t k) {
-            pos[node_off[uoff + u] + x] = (unsigned short)mask_slot((uint32_t)(kbefore[k >> 5] + __popc(kbits[k >> 5] & ((1u << (k & 31)) - 1u))));
+        each_key(node_off + uoff, [&](int32_t at, int32_t k) {
+            pos[at] = (unsigned short)mask_slot((uint32_t)(kbefore[k >> 5] + __popc(kbits[k >> 5] & ((1u << (k & 31)) - 1u))));
         });
         const int32_t r0 = blk * BQ, r1 = min(N, r0 + BQ);
-        for (int32_t p = phi_rowptr[r0] + tid, end = phi_rowptr[r1]; p < end; p += MS_THREADS) {
-            const int32_t l = __ldg(phi_col + p);
-            const int32_t u = nbefore[l >> 5] + __popc(nbits[l >> 5] & ((1u << (l & 31)) - 1u));
-            phi_pos[p] = (int32_t)base_pos + node_off[uoff + u];
+        const int32_t end = phi_rowptr[r1];
+        for (int32_t p0 = phi_rowptr[r0] + tid; p0 < end; p0 += 4 * MS_THREADS) {
+            int32_t at[4];                      // four in flight: two dependent loads each
+#pragma unroll
+            for (int q = 0; q < 4; ++q) at[q] = p0 + q * MS_THREADS < end ? __ldg(phi_col + p0 + q * MS_THREADS) : -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (at[q] >= 0)
+                    at[q] = node_off[uoff + nbefore[at[q] >> 5] + __popc(nbits[at[q] >> 5] & ((1u << (at[q] & 31)) - 1u))];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (p0 + q * MS_THREADS < end) phi_pos[p0 + q * MS_THREADS] = (int32_t)base_pos + at[q];
         }
     }
 
