@@ -138,8 +138,10 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
     }
 
     // ---- keys
-    // nodes per warp and turn: as few as give every warp some (a short list would leave most of them idle), at most 32
-    const int32_t turn = min(32, ((ucnt + MS_THREADS / 32 - 1) / (MS_THREADS / 32) + 1) & ~1);
+    // nodes per warp and turn, at most 32: equal shares for all warps in as few turns as it takes (with 32 each, a list of
+    // 166 nodes kept 6 warps busy and one of 908 took 5 of them a second turn)
+    const int32_t turns = (ucnt + MS_THREADS - 1) / MS_THREADS;
+    const int32_t turn = min(32, ((ucnt + turns * (MS_THREADS / 32) - 1) / max(1, turns * (MS_THREADS / 32)) + 1) & ~1);
     // (a node's number `of` comes with its extent, one load for 32 nodes, not with every key)
     auto each_key = [&](const int32_t* of, auto&& use) {
         for (int32_t u0 = warp * turn; u0 < ucnt; u0 += turn * (MS_THREADS / 32)) {
