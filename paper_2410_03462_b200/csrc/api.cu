@@ -59,12 +59,21 @@ int current_device()
     return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < block_pool::DEVICES ? dev : -1;
 }
 
+// Makes a block's device current for as long as something is done with the block.
+struct device_scope {
+    int before;
+    explicit device_scope(int dev) : before(current_device()) { if (dev >= 0 && dev != before) cudaSetDevice(dev); else before = -1; }
+    ~device_scope() { if (before >= 0) cudaSetDevice(before); }
+};
+
 }  // namespace
 
+// A buffer that already has a block grows on that block's device, whichever is current; an empty one takes the current.
 int grf_buf_reserve(grf_buf* b, size_t bytes)
 {
     if (bytes == 0) bytes = 1;
     if (b->bytes >= bytes) return GRF_OK;
+    const device_scope scope(b->ptr ? b->device : -1);
     if (b->ptr) {
         cudaDeviceSynchronize();
         grf_buf_release(b);
@@ -81,15 +90,14 @@ int grf_buf_reserve(grf_buf* b, size_t bytes)
         if (dev >= 0) pool().empty(dev);
         if (cudaMalloc(&p, bytes) != cudaSuccess) { cudaGetLastError(); return GRF_ERR_NOMEM; }
     }
-    b->ptr = p; b->bytes = bytes;
+    b->ptr = p; b->bytes = bytes; b->device = dev;
     return GRF_OK;
 }
 
 // The device must have finished with the block: callers that cannot know it wait first.
 void grf_buf_release(grf_buf* b)
 {
-    const int dev = current_device();
-    if (b->ptr && (dev < 0 || !pool().put(dev, b->ptr, b->bytes))) cudaFree(b->ptr);
+    if (b->ptr && (b->device < 0 || !pool().put(b->device, b->ptr, b->bytes))) cudaFree(b->ptr);
     b->ptr = nullptr; b->bytes = 0;
 }
 

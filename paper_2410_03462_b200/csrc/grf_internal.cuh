@@ -25,6 +25,7 @@
 struct grf_buf {
     void* ptr = nullptr;
     size_t bytes = 0;
+    int device = -1;                // of the block at ptr
 };
 
 struct grf_ctx {

@@ -677,6 +677,7 @@ int grf_settle_sizes(grf_ctx* ctx)
 {
     grf_features* feat = ctx->sizes_of;
     if (!feat) return GRF_OK;
+    GRF_CUDA_TRY(cudaSetDevice(ctx->device));       // called for objects of other devices than the current one
     ctx->sizes_of = nullptr;
     feat->sizes_from = nullptr;
     GRF_CUDA_TRY(cudaEventSynchronize(ctx->sizes_ready));
