@@ -11,7 +11,8 @@
  *     are ordinary host memory; the library never takes ownership of a caller's buffer;
  *   - all device work is enqueued on the context's stream; unless a call says otherwise it
  *     returns without waiting for that work;
- *   - a context is not thread-safe: one host thread at a time per context;
+ *   - a context is not thread-safe: one host thread at a time per context; a feature object likewise, but it is
+ *     independent of the context that sampled it: any context of its device may use it (the caller orders the streams);
  *   - matrices are CSR with int32 row pointers/column indices (ascending inside a row) and fp32 values.
  */
 #ifndef GRF_H

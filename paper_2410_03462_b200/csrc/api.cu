@@ -21,6 +21,10 @@ struct block_pool {
     std::mutex lock;
     std::multimap<size_t, void*> blocks[DEVICES];
     size_t held[DEVICES] = {};
+    // the same for the size slots of feature objects (pinning host memory waits for the device as well)
+    static constexpr int SLOTS = 64;
+    grf_size_slot slots[DEVICES][SLOTS];
+    int slots_held[DEVICES] = {};
     int contexts = 0;
 
     void* take(int dev, size_t bytes, size_t* got)
@@ -49,7 +53,28 @@ struct block_pool {
         blocks[dev].clear();
         held[dev] = 0;
     }
+    bool take_slot(int dev, grf_size_slot* s)
+    {
+        std::lock_guard<std::mutex> g(lock);
+        if (slots_held[dev] == 0) return false;
+        *s = slots[dev][--slots_held[dev]];
+        return true;
+    }
+    bool put_slot(int dev, const grf_size_slot& s)
+    {
+        std::lock_guard<std::mutex> g(lock);
+        if (contexts == 0 || slots_held[dev] == SLOTS) return false;
+        slots[dev][slots_held[dev]++] = s;
+        return true;
+    }
 };
+
+void slot_destroy(grf_size_slot* s)
+{
+    if (s->ready) cudaEventDestroy(s->ready);
+    if (s->host) cudaFreeHost(s->host);
+    *s = grf_size_slot();
+}
 
 block_pool& pool() { static block_pool* p = new block_pool; return *p; }   // never destroyed: objects may outlive main()
 
@@ -101,6 +126,35 @@ void grf_buf_release(grf_buf* b)
     b->ptr = nullptr; b->bytes = 0;
 }
 
+int grf_features_new(grf_features** out, int device)
+{
+    grf_features* f = new (std::nothrow) grf_features();
+    if (!f) return GRF_ERR_NOMEM;
+    f->device = device;
+    if (device >= block_pool::DEVICES || !pool().take_slot(device, &f->sizes)) {
+        int rc = GRF_OK;
+        if (cudaMallocHost((void**)&f->sizes.host, 64) != cudaSuccess) rc = GRF_ERR_NOMEM;
+        else if (cudaEventCreateWithFlags(&f->sizes.ready, cudaEventDisableTiming) != cudaSuccess) rc = GRF_ERR_CUDA;
+        if (rc != GRF_OK) {
+            cudaGetLastError();
+            slot_destroy(&f->sizes);
+            delete f;
+            return rc;
+        }
+    }
+    *out = f;
+    return GRF_OK;
+}
+
+int grf_settle_sizes(grf_features* feat)
+{
+    GRF_CUDA_TRY(cudaEventSynchronize(feat->sizes.ready));
+    feat->phi.nnz = feat->sizes.host[0];
+    feat->psi.nnz = feat->psit.nnz = feat->sizes.host[1];
+    feat->sizes_pending = false;
+    return GRF_OK;
+}
+
 int grf_csr_reserve(grf_csr_dev* m, int32_t rows, int32_t cols, int64_t nnz_cap)
 {
     m->rows = rows; m->cols = cols;
@@ -122,13 +176,13 @@ extern "C" int grf_ctx_create(grf_ctx** out, int device, void* cuda_stream)
     c->stream = (cudaStream_t)cuda_stream;
     if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
         cudaMallocHost((void**)&c->pinned, 64) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->sizes_ready, cudaEventDisableTiming) != cudaSuccess ||
         cudaMalloc((void**)&c->error_word, 2 * sizeof(int)) != cudaSuccess ||
         cudaMemset(c->error_word, 0, 2 * sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         delete c;
         return GRF_ERR_CUDA;
     }
+    memset(c->pinned, 0, 64);
     {
         std::lock_guard<std::mutex> g(pool().lock);
         ++pool().contexts;
@@ -142,8 +196,6 @@ extern "C" int grf_ctx_destroy(grf_ctx* ctx)
     if (!ctx) return GRF_ERR_INVALID;
     cudaSetDevice(ctx->device);
     cudaDeviceSynchronize();
-    grf_settle_sizes(ctx);
-    if (ctx->sizes_ready) cudaEventDestroy(ctx->sizes_ready);
     grf_buf* bufs[] = {&ctx->edge_records, &ctx->stage_col, &ctx->stage_val, &ctx->counts, &ctx->scan_blocks,
                        &ctx->stage_dep_start, &ctx->stage_dep_t, &ctx->stage_dep_load, &ctx->dep_counts, &ctx->dep_rowptr2,
                        &ctx->t_cursor, &ctx->t_tmp, &ctx->den_scratch, &ctx->h_rowptr, &ctx->h_col, &ctx->h_w,
@@ -170,7 +222,10 @@ extern "C" int grf_ctx_destroy(grf_ctx* ctx)
         int before = 0;
         cudaGetDevice(&before);
         for (int dev = 0; dev < block_pool::DEVICES; ++dev)
-            if (pool().held[dev] > 0 && cudaSetDevice(dev) == cudaSuccess) pool().empty(dev);
+            if ((pool().held[dev] > 0 || pool().slots_held[dev] > 0) && cudaSetDevice(dev) == cudaSuccess) {
+                pool().empty(dev);
+                for (grf_size_slot s; pool().take_slot(dev, &s);) slot_destroy(&s);
+            }
         cudaSetDevice(before);
     }
     return GRF_OK;
@@ -304,7 +359,6 @@ extern "C" int grf_features_free(grf_features* feat)
     if (!feat) return GRF_ERR_INVALID;
     cudaSetDevice(feat->device);
     cudaDeviceSynchronize();                        // its buffers may serve another object next
-    if (feat->sizes_from) { feat->sizes_from->sizes_of = nullptr; feat->sizes_from = nullptr; }
     csr_release(&feat->phi); csr_release(&feat->psi); csr_release(&feat->psit);
     grf_buf_release(&feat->plan_off); grf_buf_release(&feat->plan_cnt);
     grf_buf_release(&feat->plan_col); grf_buf_release(&feat->plan_total); grf_buf_release(&feat->plan_coef);
@@ -313,6 +367,7 @@ extern "C" int grf_features_free(grf_features* feat)
         grf_buf_release(&feat->kept.dep_ptr[e]); grf_buf_release(&feat->kept.dep_t[e]); grf_buf_release(&feat->kept.dep_load[e]);
     }
     grf_buf_release(&feat->kept.psit_perm);
+    if (feat->device >= block_pool::DEVICES || !pool().put_slot(feat->device, feat->sizes)) slot_destroy(&feat->sizes);
     delete feat;
     return GRF_OK;
 }
@@ -356,16 +411,14 @@ extern "C" int grf_features_from_csr(grf_ctx* ctx, int32_t N, int32_t R,
 {
     if (!ctx || !out || N <= 0 || R <= 0 || !phi_rowptr || !psi_rowptr) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
-    GRF_TRY(grf_settle_sizes(ctx));                 // the pinned block is used again below
     GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 0, phi_rowptr + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 1, psi_rowptr + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     GRF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
     const int64_t nnz_phi = ctx->pinned[0], nnz_psi = ctx->pinned[1];
     if (nnz_phi < 0 || nnz_psi < 0) return GRF_ERR_INVALID;
     if ((nnz_phi > 0 && (!phi_col || !phi_val)) || (nnz_psi > 0 && (!psi_col || !psi_val))) return GRF_ERR_INVALID;
-    grf_features* f = new (std::nothrow) grf_features();
-    if (!f) return GRF_ERR_NOMEM;
-    f->device = ctx->device;
+    grf_features* f = nullptr;
+    GRF_TRY(grf_features_new(&f, ctx->device));
     int rc = grf_csr_reserve(&f->phi, N, R, nnz_phi);
     if (rc == GRF_OK) rc = grf_csr_reserve(&f->psi, N, R, nnz_psi);
     if (rc == GRF_OK) rc = grf_csr_reserve(&f->psit, R, N, nnz_psi);

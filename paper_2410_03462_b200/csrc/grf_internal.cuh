@@ -53,10 +53,9 @@ struct grf_ctx {
     static constexpr int HOST_PARTS = 4;     // most parts grf_step_host splits a batch into
     cudaStream_t copy_stream = nullptr, down_stream = nullptr;
     cudaEvent_t up_done[HOST_PARTS] = {}, part_done[HOST_PARTS] = {}, down_done = nullptr;
-    int32_t* pinned = nullptr;      // small pinned host block for read-backs
-    // the sample whose sizes the kernels have left, or will leave, in the pinned block, and the event behind them
-    grf_features* sizes_of = nullptr;
-    cudaEvent_t sizes_ready = nullptr;
+    // small pinned host block for read-backs; [PINNED_EDGES]: edges of the graph of some earlier sample, written by its kernel
+    static constexpr int PINNED_EDGES = 10;
+    int32_t* pinned = nullptr;
     int* error_word = nullptr;      // device word set by a kernel that gave up a bounded wait
     bool use_tensor_cores = true;
     bool states_only = false;       // grf_masked_linear_attn never takes the mask (grf_ctx_use_tensor_cores(ctx, 2))
@@ -124,10 +123,18 @@ struct grf_mask_dev {
     grf_buf val;
 };
 
+// Where the kernels of a sample leave its sizes: non-zeros of Phi and Psi, deposits of both.  It belongs to the feature
+// object, not to the context that samples, so whichever context and thread has the object can read them.
+struct grf_size_slot {
+    int32_t* host = nullptr;        // pinned
+    cudaEvent_t ready = nullptr;    // behind the kernels that write them
+};
+
 struct grf_features {
     int device = 0;
     grf_csr_dev phi, psi, psit;
-    grf_ctx* sizes_from = nullptr;  // context that still owes this object its sizes (nnz): grf_features_sizes fetches them
+    grf_size_slot sizes;
+    bool sizes_pending = false;     // nnz of the matrices is still to be read from `sizes` (grf_features_sizes)
     grf_kept_walks kept;
     grf_mask_dev mask;
     // block plan of Phi: per block of GRF_PLAN_BLOCK rows, the sorted distinct columns
@@ -143,9 +150,13 @@ struct grf_features {
 int grf_buf_reserve(grf_buf* b, size_t bytes);          // grows (contents not preserved)
 void grf_buf_release(grf_buf* b);
 int grf_csr_reserve(grf_csr_dev* m, int32_t rows, int32_t cols, int64_t nnz_cap);
-int grf_settle_sizes(grf_ctx* ctx);
-// before nnz of a matrix is read
-static inline int grf_features_sizes(const grf_features* feat) { return feat->sizes_from ? grf_settle_sizes(feat->sizes_from) : GRF_OK; }
+int grf_features_new(grf_features** out, int device);   // empty; `device` is current
+int grf_settle_sizes(grf_features* feat);
+// before nnz of a matrix is read: waits for the sample's sizes if they have not been read yet
+static inline int grf_features_sizes(const grf_features* feat)
+{
+    return feat->sizes_pending ? grf_settle_sizes(const_cast<grf_features*>(feat)) : GRF_OK;
+}
 
 // sample.cu
 struct grf_walk_params {

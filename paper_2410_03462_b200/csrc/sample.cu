@@ -6,8 +6,6 @@
 // stay in shared memory: the warp sorts their keys by (column, walk, step) with a bitonic network (in
 // registers and shuffles for rows of up to 512 deposits), adds equal columns in that order and writes the
 // merged row once.
-#include <new>
-
 #include "grf_internal.cuh"
 
 namespace {
@@ -526,7 +524,7 @@ int grf_walk_params_init(grf_walk_params* p, int32_t N, uint64_t seed, int32_t n
     return GRF_OK;
 }
 
-// Row pointers of Phi, Psi and Psi^T (and the scatter cursors of the latter) from the counts; totals to pinned[0], pinned[1].
+// Row pointers of Phi, Psi and Psi^T (and the scatter cursors of the latter) from the counts; totals to the object's size slot.
 static int sample_row_pointers(grf_ctx* ctx, grf_features* feat, int32_t N, int32_t stride_counts, int32_t* cursor)
 {
     const int32_t* counts = (const int32_t*)ctx->counts.ptr;
@@ -534,13 +532,13 @@ static int sample_row_pointers(grf_ctx* ctx, grf_features* feat, int32_t N, int3
     if (N <= GRF_SCAN_DIRECT_MAX) {
         grf_scan_jobs jobs = {};
         for (int x = 0; x < 3; ++x)
-            jobs.job[x] = {counts + (size_t)x * stride_counts, out[x], x == 2 ? cursor : nullptr, x == 2 ? nullptr : ctx->pinned + x};
+            jobs.job[x] = {counts + (size_t)x * stride_counts, out[x], x == 2 ? cursor : nullptr, x == 2 ? nullptr : feat->sizes.host + x};
         return grf_scan_jobs_launch(ctx, ctx->stream, jobs, 3, N);
     }
     for (int x = 0; x < 3; ++x) GRF_TRY(grf_exclusive_scan(ctx, counts + (size_t)x * stride_counts, out[x], N, 1));
     GRF_CUDA_TRY(cudaMemcpyAsync(cursor, out[2], (size_t)N * sizeof(int32_t), cudaMemcpyDeviceToDevice, ctx->stream));
     for (int x = 0; x < 2; ++x)
-        GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + x, out[x] + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+        GRF_CUDA_TRY(cudaMemcpyAsync(feat->sizes.host + x, out[x] + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     return GRF_OK;
 }
 
@@ -554,7 +552,6 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     const int32_t N = P.N;
     const int32_t stride = P.cap < N ? P.cap : N;   // a row cannot hold more distinct columns than N
     const size_t rows2 = 2 * (size_t)N;
-    GRF_TRY(grf_settle_sizes(ctx));                 // an earlier sample's sizes are still in the pinned block
     const int64_t most = (int64_t)N * stride;
     const bool whole = most <= SAMPLE_WHOLE_ENTRIES && !ctx->keep_walks;
     const int32_t stride_counts = (N + 3) & ~3;
@@ -569,6 +566,11 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     int32_t* counts = (int32_t*)ctx->counts.ptr;
     int32_t *long_count = (int32_t*)ctx->t_cursor.ptr, *cursor = long_count + 1, *long_list = cursor + N;
 
+    // Room for the edge records by the last graph that is known: the kernels compare it with their own graph's edges and
+    // read the CSR arrays where it is too small.  (An earlier sample may be writing the number just now; either value will do.)
+    const int64_t edges_seen = *(volatile const int32_t*)(ctx->pinned + grf_ctx::PINNED_EDGES);
+    if (edges_seen > (int64_t)(ctx->edge_records.bytes / sizeof(int4)))
+        (void)grf_buf_reserve(&ctx->edge_records, sizeof(int4) * ((size_t)edges_seen + (size_t)edges_seen / 8 + 64));
     int4* edges = (int4*)ctx->edge_records.ptr;
     const int64_t edge_room = (int64_t)(ctx->edge_records.bytes / sizeof(int4));
 
@@ -596,7 +598,8 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     {
         grf_launch_scope scope(ctx, 0, 2);
         edge_records_kernel<<<grf_ceil_div(N, 32), 256, 0, ctx->stream>>>(
-            N, edge_room, P.inv_keep, rowptr, col, w, edges, counts + 2 * (size_t)stride_counts, long_count, ctx->pinned + 10);
+            N, edge_room, P.inv_keep, rowptr, col, w, edges, counts + 2 * (size_t)stride_counts, long_count,
+            ctx->pinned + grf_ctx::PINNED_EDGES);
         if (keep)
             walk_merge_kernel<true><<<grf_ceil_div(rows2, warps), warps * 32, smem, ctx->stream>>>(
                 P, rowptr, col, w, edges, edge_room, stride, (int32_t*)ctx->stage_col.ptr, (float*)ctx->stage_val.ptr,
@@ -612,17 +615,16 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     if (keep)
         for (int e = 0; e < 2; ++e) {
             GRF_TRY(grf_exclusive_scan(ctx, (const int32_t*)ctx->dep_counts.ptr + (size_t)e * stride_counts, dep_scan[e], N, 1));
-            GRF_CUDA_TRY(cudaMemcpyAsync(ctx->pinned + 2 + e, dep_scan[e] + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+            GRF_CUDA_TRY(cudaMemcpyAsync(feat->sizes.host + 2 + e, dep_scan[e] + N, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
         }
-    GRF_CUDA_TRY(cudaEventRecord(ctx->sizes_ready, ctx->stream));
-    ctx->sizes_of = feat;
-    feat->sizes_from = ctx;
+    GRF_CUDA_TRY(cudaEventRecord(feat->sizes.ready, ctx->stream));
+    feat->sizes_pending = true;
     feat->plan_stale = true;       // the block plan of Phi is built by the first attention call that needs it
     feat->plan_ready = false;
     grf_mask_invalidate(feat);
     if (!whole) {
         // column/value arrays, grown with head-room so that resampling rarely reallocates
-        GRF_TRY(grf_settle_sizes(ctx));
+        GRF_TRY(grf_settle_sizes(feat));
         const int64_t nnz_phi = feat->phi.nnz, nnz_psi = feat->psi.nnz;
         const int64_t cap_phi = nnz_phi + nnz_phi / 8 + 64, cap_psi = nnz_psi + nnz_psi / 8 + 64;
         if (feat->phi.col.bytes < (size_t)nnz_phi * 4) GRF_TRY(grf_csr_reserve(&feat->phi, N, N, cap_phi));
@@ -649,7 +651,7 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
         grf_kept_walks& K = feat->kept;
         const int64_t nnz_e[2] = {feat->phi.nnz, feat->psi.nnz};
         for (int e = 0; e < 2; ++e) {
-            K.deposits[e] = ctx->pinned[2 + e];
+            K.deposits[e] = feat->sizes.host[2 + e];
             const size_t dcap = (size_t)K.deposits[e] + (size_t)K.deposits[e] / 8 + 64;
             if (K.dep_ptr[e].bytes < ((size_t)nnz_e[e] + 1) * 4)
                 GRF_TRY(grf_buf_reserve(&K.dep_ptr[e], ((size_t)nnz_e[e] + (size_t)nnz_e[e] / 8 + 65) * 4));
@@ -672,23 +674,6 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     return GRF_OK;
 }
 
-// The sizes of the last sample of this context: waits for them if they have not been read yet.
-int grf_settle_sizes(grf_ctx* ctx)
-{
-    grf_features* feat = ctx->sizes_of;
-    if (!feat) return GRF_OK;
-    GRF_CUDA_TRY(cudaSetDevice(ctx->device));       // called for objects of other devices than the current one
-    ctx->sizes_of = nullptr;
-    feat->sizes_from = nullptr;
-    GRF_CUDA_TRY(cudaEventSynchronize(ctx->sizes_ready));
-    feat->phi.nnz = ctx->pinned[0];
-    feat->psi.nnz = feat->psit.nnz = ctx->pinned[1];
-    const int64_t E = ctx->pinned[10];
-    if (E > (int64_t)(ctx->edge_records.bytes / sizeof(int4)))
-        GRF_TRY(grf_buf_reserve(&ctx->edge_records, sizeof(int4) * ((size_t)E + (size_t)E / 8 + 64)));
-    return GRF_OK;
-}
-
 extern "C" int grf_sample(grf_ctx* ctx, int32_t N, const int32_t* rowptr, const int32_t* col, const float* w,
                           uint64_t seed, int32_t n_walks, float p_halt, int32_t max_len,
                           const float* f_phi, const float* f_psi, grf_features** inout)
@@ -707,11 +692,7 @@ extern "C" int grf_sample(grf_ctx* ctx, int32_t N, const int32_t* rowptr, const 
         if (ctx->pinned[9] != 0) return GRF_ERR_BADGRAPH;
     }
     grf_features* feat = *inout;
-    if (!feat) {
-        feat = new (std::nothrow) grf_features();
-        if (!feat) return GRF_ERR_NOMEM;
-        feat->device = ctx->device;
-    }
+    if (!feat) GRF_TRY(grf_features_new(&feat, ctx->device));
     const int rc = sample_into(ctx, feat, P, rowptr, col, w);
     if (rc != GRF_OK) {
         if (!*inout) grf_features_free(feat);

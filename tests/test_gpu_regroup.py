@@ -46,3 +46,37 @@ def test_sizes_of_interleaved_samples_and_growing_graphs():
     feat = api.sample(ctx, api.DeviceGraph(gs[0]), 5, w.n_walks, w.p_halt, w.max_len, f)
     feat.free()                       # freed before its sizes were read
     ctx.close()
+
+
+def test_objects_handed_from_one_context_to_another():
+    """A producer samples without reading sizes and goes on with larger graphs; a consumer thread with its own context
+    takes each object over."""
+    import threading
+
+    from paper_2410_03462_b200 import api
+    w = configs.tiny()
+    f = oracle.deconvolve(w.alpha).astype(np.float32)
+    gs = [graphs.grid_graph(n, n + 1, 0.25, n % 2 == 0) for n in (5, 8, 13, 21)]
+    producer, consumer = api.Context(0), api.Context(0)
+    feats, got, ready = [], [], [threading.Event() for _ in gs]
+
+    def consume():
+        for x in range(len(gs)):
+            ready[x].wait(60)
+            feats[x].ctx = consumer
+            got.append([feats[x].to_host(which) for which in range(3)])
+
+    t = threading.Thread(target=consume)
+    t.start()
+    for x, g in enumerate(gs):
+        feats.append(api.sample(producer, api.DeviceGraph(g), 11, w.n_walks, w.p_halt, w.max_len, f))
+        producer.stream.synchronize()              # the hand-over is the caller's to order
+        ready[x].set()
+    t.join()
+    for g, feat, matrices in zip(gs, feats, got):
+        want = oracle.sample(g.rowptr, g.col, g.w, 11, w.n_walks, w.p_halt, w.max_len, f)[:3]
+        for which in range(3):
+            helpers.assert_csr_equal(matrices[which], want[which], f"N={g.N} matrix {which}", val_rtol=0)
+        feat.free()
+    producer.close()
+    consumer.close()

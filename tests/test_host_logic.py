@@ -40,3 +40,41 @@ def test_sizes_read_while_another_device_is_current(fake):
     for c in (ctx0, ctx1):
         assert fake.lib.grf_ctx_destroy(c) == 0
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0 and fake.lib.fake_live(1) == 0
+
+
+def test_reading_sizes_leaves_the_sampling_context_alone(fake):
+    """One thread samples with its context while another, with its own context, takes the object on: whatever the second
+    does to learn the sizes neither allocates nor waits for the device, and needs nothing of the first context."""
+    ctx = fake.context(0)
+    fake.report(PHI=5000, PSI=6000, EDGES=900)
+    assert fake.lib.grf_ctx_destroy(fake.context(0)) == 0
+    rc, a = fake.sample(ctx, 100)
+    assert rc == 0
+    fake.report(PHI=4000, PSI=3000, EDGES=1800)
+    rc, b = fake.sample(ctx, 100)                 # the sizes of the first have not been read
+    assert rc == 0
+    mallocs, frees = fake.lib.fake_mallocs(), fake.lib.fake_frees()
+    fake.lib.fake_log_clear()
+    assert fake.nnz(a) == (0, 5000) and fake.nnz(a, 2) == (0, 6000)
+    assert fake.log() in ([], ["sync event"])
+    assert (mallocs, frees) == (fake.lib.fake_mallocs(), fake.lib.fake_frees())
+    assert fake.lib.grf_ctx_destroy(ctx) == 0     # before the second object's sizes were read
+    assert fake.nnz(b) == (0, 4000) and fake.nnz(b, 1) == (0, 3000)
+    assert fake.lib.grf_features_free(a) == 0 and fake.lib.grf_features_free(b) == 0
+    assert fake.errors() == 0
+
+
+def test_a_sample_does_not_wait_for_the_one_before(fake):
+    """... and the room for its edge records follows the graphs seen so far without a wait."""
+    ctx = fake.context(0)
+    fake.report(PHI=500, PSI=600, EDGES=900)
+    rc, feat = fake.sample(ctx, 100)
+    assert rc == 0 and fake.nnz(feat) == (0, 500)
+    assert fake.sample(ctx, 100, feat)[0] == 0    # arrays are as large as they get
+    fake.lib.fake_log_clear()
+    fake.report(PHI=510, PSI=610)
+    assert fake.sample(ctx, 100, feat)[0] == 0
+    assert not [x for x in fake.log() if x.startswith("sync")]
+    assert fake.nnz(feat) == (0, 510)
+    assert fake.lib.grf_features_free(feat) == 0 and fake.lib.grf_ctx_destroy(ctx) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
