@@ -65,7 +65,8 @@ int grf_deconvolve(const double* alpha, int32_t len, double* f_out);
  *   n_walks >= 1, 0 <= p_halt < 1, 0 <= max_len <= GRF_MAX_WALK_LEN
  *   f_phi[max_len+1], f_psi[max_len+1]  HOST  modulation coefficients; f_psi == NULL means f_phi
  *   *inout   NULL: a new feature object is created; otherwise that object's buffers are reused
- *            (regrown if needed) and its previous contents are overwritten.
+ *            (regrown if needed) and its previous contents are overwritten; a call that fails on the way (memory,
+ *            CUDA errors; not invalid arguments) leaves it without matrices, fit for sampling again or freeing.
  *
  * Walk rule: the walk from node i deposits f_t * load_t / n_walks at the node reached after t hops
  * (nothing when f_t == 0), load_0 = 1 and load_{t+1} = load_t * W_uv * deg(u) / (1 - p_halt) for the hop

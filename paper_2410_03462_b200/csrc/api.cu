@@ -146,6 +146,17 @@ int grf_features_new(grf_features** out, int device)
     return GRF_OK;
 }
 
+// Empties an object (its buffers stay for the next sample): no call finds a matrix in it.
+void grf_features_clear(grf_features* feat)
+{
+    for (grf_csr_dev* m : {&feat->phi, &feat->psi, &feat->psit}) { m->rows = m->cols = 0; m->nnz = 0; }
+    feat->sizes_pending = false;
+    feat->kept.valid = feat->kept.perm_valid = false;
+    feat->plan_stale = true;
+    feat->plan_ready = feat->plan_coef_ready = false;
+    grf_mask_invalidate(feat);
+}
+
 int grf_settle_sizes(grf_features* feat)
 {
     GRF_CUDA_TRY(cudaEventSynchronize(feat->sizes.ready));
@@ -393,7 +404,7 @@ extern "C" int grf_features_copy(grf_ctx* ctx, const grf_features* feat, int whi
     if (!ctx || !feat || which < 0 || which > 2 || !rowptr) return GRF_ERR_INVALID;
     GRF_TRY(grf_features_sizes(feat));
     const grf_csr_dev& m = which == 0 ? feat->phi : (which == 1 ? feat->psi : feat->psit);
-    if (m.nnz > 0 && (!col || !val)) return GRF_ERR_INVALID;
+    if (m.rows == 0 || (m.nnz > 0 && (!col || !val))) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
     GRF_CUDA_TRY(cudaMemcpyAsync(rowptr, m.rowptr.ptr, sizeof(int32_t) * ((size_t)m.rows + 1), cudaMemcpyDeviceToDevice,
                                  ctx->stream));

@@ -151,6 +151,7 @@ int grf_buf_reserve(grf_buf* b, size_t bytes);          // grows (contents not p
 void grf_buf_release(grf_buf* b);
 int grf_csr_reserve(grf_csr_dev* m, int32_t rows, int32_t cols, int64_t nnz_cap);
 int grf_features_new(grf_features** out, int device);   // empty; `device` is current
+void grf_features_clear(grf_features* feat);
 int grf_settle_sizes(grf_features* feat);
 // before nnz of a matrix is read: waits for the sample's sizes if they have not been read yet
 static inline int grf_features_sizes(const grf_features* feat)

@@ -695,7 +695,8 @@ extern "C" int grf_sample(grf_ctx* ctx, int32_t N, const int32_t* rowptr, const 
     if (!feat) GRF_TRY(grf_features_new(&feat, ctx->device));
     const int rc = sample_into(ctx, feat, P, rowptr, col, w);
     if (rc != GRF_OK) {
-        if (!*inout) grf_features_free(feat);
+        if (*inout) grf_features_clear(feat);       // some of its arrays may be the new sample's already
+        else grf_features_free(feat);
         return rc;
     }
     *inout = feat;

@@ -25,6 +25,7 @@ def build(directory):
 
 class Fake:
     """Sizes that the kernels report are set with `report`; NNZ etc. index them."""
+    INVALID, NOMEM, TOO_LARGE = -1, -5, -2
     PHI, PSI, DEP_PHI, DEP_PSI, EDGES, PLAN, KEYS, POSITIONS, LONGEST = range(9)
 
     def __init__(self, so):
@@ -67,3 +68,11 @@ class Fake:
         """(code, non-zeros)"""
         n = C.c_int64(-1)
         return self.lib.grf_features_view(feat, which, None, None, C.byref(n), None, None, None), n.value
+
+    def linear(self, ctx, feat, G, N, m, d, dtype):
+        """grf_masked_linear_attn on arrays that nobody reads, with a workspace for one problem."""
+        code = 1 if dtype == "bf16" else 0
+        need = self.lib.grf_attn_workspace_bytes(1, N, m, d, code)
+        some = C.c_void_p(4096)
+        return self.lib.grf_masked_linear_attn(ctx, feat, G, N, m, d, code, some, some, some, some, None, some,
+                                               C.c_size_t(need))

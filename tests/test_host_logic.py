@@ -78,3 +78,25 @@ def test_a_sample_does_not_wait_for_the_one_before(fake):
     assert fake.nnz(feat) == (0, 510)
     assert fake.lib.grf_features_free(feat) == 0 and fake.lib.grf_ctx_destroy(ctx) == 0
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
+def test_an_object_whose_resampling_failed_is_empty(fake):
+    """Not one with the new row count and the old, or no, arrays behind it."""
+    ctx = fake.context(0)
+    fake.report(PHI=5000, PSI=6000, EDGES=900)
+    rc, feat = fake.sample(ctx, 100)
+    assert rc == 0 and fake.nnz(feat) == (0, 5000)
+    fake.lib.fake_limit(0, 300 << 20)             # the staging area fits, the matrices do not
+    fake.report(PHI=40 << 20, PSI=40 << 20)
+    assert fake.sample(ctx, 40000, feat)[0] == fake.NOMEM
+    fake.lib.fake_log_clear()
+    assert fake.linear(ctx, feat, 1, 40000, 32, 64, "fp32") == fake.INVALID
+    assert fake.linear(ctx, feat, 1, 100, 32, 64, "fp32") == fake.INVALID
+    assert fake.lib.grf_features_materialise(ctx, feat) != 0
+    assert fake.launched("kernel") == 0 and fake.nnz(feat) == (0, 0)
+    fake.lib.fake_limit(0, 1 << 40)
+    fake.report(PHI=5000, PSI=6000)
+    assert fake.sample(ctx, 100, feat)[0] == 0 and fake.nnz(feat) == (0, 5000)
+    assert fake.linear(ctx, feat, 1, 100, 32, 64, "fp32") == 0
+    assert fake.lib.grf_features_free(feat) == 0 and fake.lib.grf_ctx_destroy(ctx) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
