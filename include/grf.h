@@ -192,7 +192,11 @@ size_t grf_attn_workspace_bytes(int32_t G, int32_t R, int32_t m, int32_t d, int 
  * m, d in {8, 16, 32, 64, 128}.  workspace: DEVICE, 256-byte aligned.  Summation order is fixed, so
  * results are run-to-run identical.  Where the same sum is cheaper in the other order (Mhat = Phi Psi^T first, as
  * grf_masked_attn_mhat evaluates it), a bf16 batch takes that order; the choice depends on the features' sizes and on
- * G, m, d only, never on earlier calls, and the workspace is then not touched.
+ * G, m, d only, never on earlier calls, and the workspace is then not touched.  The mask lies inside the feature object
+ * (260 bytes per key entry, at most 8 GiB, and while it is formed 2 bytes per (block, node, key) beside it) until the
+ * object is resampled or freed.  If the device has no memory left for it, this call and later ones on the same features
+ * take the per-node states instead, which need the caller's workspace only (equal calls then differ by rounding from
+ * those made with memory at hand); grf_ctx_use_tensor_cores(ctx, 2) keeps to the states from the start.
  * Asynchronous, except that the first bf16 call with m and d multiples of 16
  * after the features were created, resampled or re-modulated prepares a per-block plan of Phi, and where it takes the
  * other order the mask, inside the feature object, which waits for the stream (so a feature object must not be used by two threads at the same time).

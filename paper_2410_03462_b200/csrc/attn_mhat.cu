@@ -908,7 +908,7 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
 void grf_mask_invalidate(grf_features* feat)
 {
     grf_mask_dev& K = feat->mask;
-    K.ready = K.requested = K.refused = K.lists_ready = K.structure_ready = false;
+    K.ready = K.requested = K.refused = K.no_room = K.lists_ready = K.structure_ready = false;
 }
 // Phi's and Psi's values changed, their structure did not (re-modulation): key lists and positions stay
 void grf_mask_values_stale(grf_features* feat) { feat->mask.ready = feat->mask.requested = false; }
@@ -1059,6 +1059,7 @@ extern "C" int grf_features_materialise(grf_ctx* ctx, grf_features* feat)
     feat->mask.requested = false;
     GRF_TRY(build_mask(ctx, feat));
     feat->mask.requested = true;
+    feat->mask.no_room = false;
     return GRF_OK;
 }
 
@@ -1096,7 +1097,7 @@ int grf_linear_by_mask(grf_ctx* ctx, const grf_features* cfeat, int32_t G, int32
     const double rows = grf_gather_rows_ns(feat, G, m, d);
     if (rows < GRF_PLAN_WORTH_NS) return GRF_OK;
     GRF_TRY(grf_ensure_block_plan(ctx, feat, false));
-    if (!feat->plan_ready || K.refused) return GRF_OK;
+    if (!feat->plan_ready || K.refused || K.no_room) return GRF_OK;
     const double state_scale = (m + 16) / 48.0, mask_scale = (m + 48) / 80.0;
     const double nnz = 0.5 * ((double)feat->phi.nnz + (double)feat->psi.nnz);
     const double tiles = grf_gather_tiles_ns(feat, G, m);
@@ -1113,13 +1114,25 @@ int grf_linear_by_mask(grf_ctx* ctx, const grf_features* cfeat, int32_t G, int32
     const double shared = 2.5 * list < N ? 2.5 * list : N;
     const double keys = 1.8 * (double)feat->plan_entries > (double)feat->phi.nnz ? drawn : shared;
     if (build + rest(keys * feat->plan_blocks) > states) return GRF_OK;
-    if (!K.lists_ready) GRF_TRY(prepare_mask_lists(ctx, feat));
+    // Memory for the mask is the library's own wish: without it the states serve the call, and later ones on these features
+    auto without_mask = [&](int rc) {
+        if (rc != GRF_ERR_NOMEM) return rc;
+        cudaDeviceSynchronize();                                // the structure kernel may still be writing to what goes
+        grf_mask_release(feat);
+        K.no_room = true;
+        return (int)GRF_OK;
+    };
+    if (!K.lists_ready) {
+        GRF_TRY(without_mask(prepare_mask_lists(ctx, feat)));
+        if (K.no_room) return GRF_OK;
+    }
     if (K.refused || (int64_t)G * K.blocks > 0x7fffffffll || (int64_t)G * N > 0x7fffffffll) return GRF_OK;
     if (0.75 * build + rest((double)K.entries) > states) return GRF_OK;
     if (!K.ready) {
         const int rc = build_mask(ctx, feat);
-        if (rc == GRF_ERR_TOO_LARGE || rc == GRF_ERR_NOMEM) { K.refused = true; return GRF_OK; }
-        GRF_TRY(rc);
+        if (rc == GRF_ERR_TOO_LARGE) { K.refused = true; return GRF_OK; }
+        GRF_TRY(without_mask(rc));
+        if (K.no_room) return GRF_OK;
     }
     *by_mask = true;
     return GRF_OK;

@@ -107,6 +107,7 @@ struct grf_mask_dev {
     bool ready = false;             // the blocks hold the mask of the present features
     bool requested = false;         // the caller asked for it (grf_features_materialise); else it is grf_masked_linear_attn's own
     bool refused = false;           // its blocks would be too large for the present structure: not tried again
+    bool no_room = false;           // its memory could not be had for grf_masked_linear_attn, which then keeps to the states
     bool lists_ready = false;       // key sets, counts and sizes match the features' structure (what deciding the route needs)
     int64_t positions = 0;          // (node, key) pairs over all blocks, -1 when they passed 2^31
     int32_t longest = 0;            // longest key list of a block

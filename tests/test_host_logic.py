@@ -100,3 +100,36 @@ def test_an_object_whose_resampling_failed_is_empty(fake):
     assert fake.linear(ctx, feat, 1, 100, 32, 64, "fp32") == 0
     assert fake.lib.grf_features_free(feat) == 0 and fake.lib.grf_ctx_destroy(ctx) == 0
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
+def _cloud_like(fake, ctx):
+    """An object whose reported sizes are those of a cloud of 4096 points: the cost rule takes the mask."""
+    fake.report(PHI=400_000, PSI=400_000, EDGES=40_000, PLAN=25_600, KEYS=64_000, POSITIONS=2_500_000, LONGEST=4096)
+    rc, feat = fake.sample(ctx, 4096)
+    assert rc == 0
+    assert fake.lib.grf_plan_stats(ctx, feat, None, None) == 0
+    return feat
+
+
+def test_no_memory_for_the_mask_means_the_states(fake):
+    """The main call does not fail for want of memory that the per-node states do without, and such a call does not keep
+    grf_features_materialise from trying again."""
+    ctx = fake.context(0)
+    taken = {}
+    for mib in (1, 2, 4, 6, 8, 12, 16, 20, 24, 32, 64):
+        feat = _cloud_like(fake, ctx)
+        fake.lib.fake_limit(0, fake.lib.fake_live(0) + (mib << 20))
+        for _ in range(2):                        # the second call takes the same route
+            fake.lib.fake_log_clear()
+            assert fake.linear(ctx, feat, 8, 4096, 32, 64, "bf16") == 0, f"{mib} MiB left"
+            mask, states = fake.launched("mhat_attention_kernel"), fake.launched("build_states")
+            assert (mask > 0) != (states > 0)
+            assert taken.setdefault(mib, mask > 0) == (mask > 0)
+        fake.lib.fake_limit(0, 1 << 40)
+        assert fake.lib.grf_features_materialise(ctx, feat) == 0
+        assert fake.lib.grf_features_free(feat) == 0
+        assert fake.lib.grf_ctx_destroy(ctx) == 0                 # gives the pool back
+        ctx = fake.context(0)
+    assert not taken[1] and taken[64] and len(set(taken.values())) == 2
+    assert fake.lib.grf_ctx_destroy(ctx) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
