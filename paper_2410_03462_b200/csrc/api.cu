@@ -603,6 +603,7 @@ extern "C" int grf_step_host(grf_ctx* ctx, int32_t N, const int32_t* rowptr, con
     if (ctx->prefer_mask_route && dtype == GRF_DTYPE_BF16 && d == 64 && (m == 16 || m == 32 || m == 64)) {
         const int rc = grf_features_materialise(ctx, ctx->h_feat);
         if (rc == GRF_OK) by_mask = true;
+        else if (rc == GRF_ERR_NOMEM) { cudaDeviceSynchronize(); grf_mask_release(ctx->h_feat); }     // the states need less
         else if (rc != GRF_ERR_TOO_LARGE) return rc;          // too large = no locality: the S/z route serves it
     } else {
         GRF_TRY(grf_linear_by_mask(ctx, ctx->h_feat, G, N, m, d, dtype, &by_mask));

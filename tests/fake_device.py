@@ -76,3 +76,15 @@ class Fake:
         some = C.c_void_p(4096)
         return self.lib.grf_masked_linear_attn(ctx, feat, G, N, m, d, code, some, some, some, some, None, some,
                                                C.c_size_t(need))
+
+    def step_host(self, ctx, N, G, m, d, walks=32, length=12):
+        """grf_step_host in bf16 on a ring of N nodes."""
+        rowptr = np.arange(0, 2 * N + 1, 2, dtype=np.int32)
+        col = np.stack([np.arange(N) - 1, np.arange(N) + 1], 1).astype(np.int32).ravel() % N
+        w = np.full(2 * N, 0.25, np.float32)
+        f = np.ones(length + 1, np.float32)
+        q, v = np.zeros(G * N * m, np.uint16), np.zeros(G * N * d, np.uint16)
+        out = np.zeros_like(v)
+        p = lambda a: a.ctypes.data_as(C.c_void_p)  # noqa: E731
+        return self.lib.grf_step_host(ctx, N, p(rowptr), p(col), p(w), C.c_uint64(1), walks, C.c_float(0.1), length, p(f), None,
+                                      G, m, d, 1, p(q), p(q), p(v), p(out))

@@ -133,3 +133,22 @@ def test_no_memory_for_the_mask_means_the_states(fake):
     assert not taken[1] and taken[64] and len(set(taken.values())) == 2
     assert fake.lib.grf_ctx_destroy(ctx) == 0
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
+def test_host_path_without_memory_for_the_preferred_mask(fake):
+    ctx = fake.context(0)
+    fake.report(PHI=400_000, PSI=400_000, EDGES=8192, PLAN=25_600, KEYS=64_000, POSITIONS=2_500_000, LONGEST=4096)
+    assert fake.lib.grf_ctx_use_tensor_cores(ctx, 2) == 0
+    for _ in range(2):                            # the second pass has made the object's arrays as large as they get
+        assert fake.step_host(ctx, 4096, 8, 32, 64) == 0
+    assert fake.lib.grf_ctx_prefer_mask_route(ctx, 1) == 0
+    fake.lib.fake_limit(0, fake.lib.fake_live(0) + (1 << 20))
+    fake.lib.fake_log_clear()
+    assert fake.step_host(ctx, 4096, 8, 32, 64) == 0
+    assert fake.launched("build_states") > 0 and fake.launched("mhat_attention_kernel") == 0
+    fake.lib.fake_limit(0, 1 << 40)
+    fake.lib.fake_log_clear()
+    assert fake.step_host(ctx, 4096, 8, 32, 64) == 0
+    assert fake.launched("build_states") == 0 and fake.launched("mhat_attention_kernel") > 0
+    assert fake.lib.grf_ctx_destroy(ctx) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
