@@ -253,7 +253,7 @@ int grf_masked_attn_mhat(grf_ctx* ctx, const grf_features* feat, int32_t G, int3
 /*
  * The whole path of Alg. 1 from HOST buffers, for callers that keep nothing on the device:
  * copies the graph and phi(Q), phi(K), V to the device, samples features, evaluates the attention and
- * copies `out` ([G][N][d], dtype) back; returns after the result is in `out`.  Device buffers and the
+ * copies `out` ([G][N][d], dtype) back; returns after the result is in `out`, with an error after its copies have ended.  Device buffers and the
  * feature object are owned by the context and reused by later calls.  Graph consistency (monotone
  * rowptr, indices in range) is checked on the host: GRF_ERR_BADGRAPH.
  */

@@ -546,11 +546,9 @@ static int check_graph_host(int32_t N, const int32_t* rowptr, const int32_t* col
     return GRF_OK;
 }
 
-extern "C" int grf_step_host(grf_ctx* ctx, int32_t N, const int32_t* rowptr, const int32_t* col, const float* w,
-                             uint64_t seed, int32_t n_walks, float p_halt, int32_t max_len,
-                             const float* f_phi, const float* f_psi,
-                             int32_t G, int32_t m, int32_t d, int dtype,
-                             const void* phiQ, const void* phiK, const void* V, void* out)
+static int step_host(grf_ctx* ctx, int32_t N, const int32_t* rowptr, const int32_t* col, const float* w, uint64_t seed,
+                     int32_t n_walks, float p_halt, int32_t max_len, const float* f_phi, const float* f_psi, int32_t G, int32_t m,
+                     int32_t d, int dtype, const void* phiQ, const void* phiK, const void* V, void* out)
 {
     if (!ctx || !rowptr || !col || !w || !phiQ || !phiK || !V || !out || N <= 0 || G <= 0) return GRF_ERR_INVALID;
     if (!dim_ok(m) || !dim_ok(d) || (dtype != GRF_DTYPE_F32 && dtype != GRF_DTYPE_BF16)) return GRF_ERR_INVALID;
@@ -636,6 +634,22 @@ extern "C" int grf_step_host(grf_ctx* ctx, int32_t N, const int32_t* rowptr, con
     GRF_CUDA_TRY(cudaEventRecord(ctx->down_done, ctx->down_stream));
     GRF_CUDA_TRY(cudaStreamWaitEvent(s, ctx->down_done, 0));
     return grf_ctx_check(ctx);
+}
+
+extern "C" int grf_step_host(grf_ctx* ctx, int32_t N, const int32_t* rowptr, const int32_t* col, const float* w,
+                             uint64_t seed, int32_t n_walks, float p_halt, int32_t max_len,
+                             const float* f_phi, const float* f_psi,
+                             int32_t G, int32_t m, int32_t d, int dtype,
+                             const void* phiQ, const void* phiK, const void* V, void* out)
+{
+    const int rc = step_host(ctx, N, rowptr, col, w, seed, n_walks, p_halt, max_len, f_phi, f_psi, G, m, d, dtype, phiQ, phiK, V,
+                             out);
+    if (rc != GRF_OK && ctx) {                      // copies from and to the caller's buffers may be on their way
+        cudaStreamSynchronize(ctx->stream);
+        if (ctx->copy_stream) cudaStreamSynchronize(ctx->copy_stream);
+        if (ctx->down_stream) cudaStreamSynchronize(ctx->down_stream);
+    }
+    return rc;
 }
 
 extern "C" const char* grf_strerror(int code)

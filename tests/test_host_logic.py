@@ -152,3 +152,16 @@ def test_host_path_without_memory_for_the_preferred_mask(fake):
     assert fake.launched("build_states") == 0 and fake.launched("mhat_attention_kernel") > 0
     assert fake.lib.grf_ctx_destroy(ctx) == 0
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
+def test_host_path_that_fails_waits_for_its_copies(fake):
+    """The caller may free or change its buffers once the call has returned, with an error as well."""
+    ctx = fake.context(0)
+    fake.report(PHI=5000, PSI=6000, EDGES=800)
+    fake.lib.fake_log_clear()
+    assert fake.step_host(ctx, 400, 8, 32, 64, walks=0) == fake.INVALID
+    waited = {x for x in fake.log() if x.startswith("sync stream")}
+    assert len(waited) >= 2                       # the context's stream and the one that the inputs travel on
+    assert fake.step_host(ctx, 400, 8, 32, 64) == 0
+    assert fake.lib.grf_ctx_destroy(ctx) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
