@@ -47,9 +47,13 @@ typedef struct grf_ctx grf_ctx;            /* device id, stream, reusable scratc
 typedef struct grf_features grf_features;  /* device-resident Phi (N x R), Psi (N x R), Psi^T (R x N)     */
 
 /* Context bound to `device` and to the CUDA stream `cuda_stream` (a cudaStream_t passed as void*;
- * NULL = the default stream).  Scratch buffers grow on demand and live until destroy. */
+ * NULL = the default stream).  Scratch buffers grow on demand and live until destroy.
+ * Device memory that scratch or feature objects give back is kept for later buffers of the same device, at most 1 GiB per
+ * device, while any context exists; it is freed when the last context of the process is destroyed, and earlier when one of
+ * the library's own allocations would fail.  It is not available to other allocators of the process meanwhile. */
 int grf_ctx_create(grf_ctx** out, int device, void* cuda_stream);
-int grf_ctx_destroy(grf_ctx* ctx);   /* waits for the stream, frees scratch; features are freed separately */
+/* Waits for the device and gives the scratch back; features are freed separately. */
+int grf_ctx_destroy(grf_ctx* ctx);
 
 /* Remark 3.1: f with sum_{p=0..k} f_p f_{k-p} = alpha_k, k < len (fp64 recurrence on the host).
  * HOST pointers.  GRF_ERR_INVALID unless alpha[0] > 0. */
@@ -76,8 +80,10 @@ int grf_deconvolve(const double* alpha, int32_t len, double* f_out);
  * Deposits of a row that hit the same column are added in ascending (walk, t) order.
  *
  * Limits: n_walks*(max_len+1) <= 16384 and N * 2^ceil(log2(n_walks*(max_len+1))) <= 2^32, else
- * GRF_ERR_TOO_LARGE.  Samples of more than 4 M possible entries per matrix make the call wait once for the device (it reads
- * back the two nonzero counts); smaller ones do not wait, and the first call that needs the counts does.
+ * GRF_ERR_TOO_LARGE.  The call waits once for the device (it reads back the two nonzero counts) for an object's first
+ * sample and for samples of more than 4 M possible entries, N * min(N, n_walks*(max_len+1)), per matrix; the object's
+ * arrays then hold the non-zeros and an eighth more.  Smaller samples into an object that has been sampled before do not
+ * wait (the first call that needs the counts does); its arrays then grow to the possible entries, 100 MB at most.
  */
 int grf_sample(grf_ctx* ctx, int32_t N, const int32_t* rowptr, const int32_t* col, const float* w,
                uint64_t seed, int32_t n_walks, float p_halt, int32_t max_len,

@@ -136,6 +136,7 @@ struct grf_features {
     grf_csr_dev phi, psi, psit;
     grf_size_slot sizes;
     bool sizes_pending = false;     // nnz of the matrices is still to be read from `sizes` (grf_features_sizes)
+    bool sampled = false;           // holds, or has held, a sample
     grf_kept_walks kept;
     grf_mask_dev mask;
     // block plan of Phi: per block of GRF_PLAN_BLOCK rows, the sorted distinct columns

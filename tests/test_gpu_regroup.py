@@ -80,3 +80,20 @@ def test_objects_handed_from_one_context_to_another():
         feat.free()
     producer.close()
     consumer.close()
+
+
+def test_one_object_resampled_without_reading_its_sizes():
+    """First sample (exact arrays), later ones (arrays for the largest sample), on graphs that grow and shrink."""
+    from paper_2410_03462_b200 import api
+    ctx = api.Context(0)
+    w = configs.tiny()
+    f = oracle.deconvolve(w.alpha).astype(np.float32)
+    feat = None
+    for n, reads in ((9, False), (6, True), (15, False), (15, False), (4, True), (17, True)):
+        g = graphs.grid_graph(n, n + 1, 0.25, True)
+        feat = api.sample(ctx, api.DeviceGraph(g), n, w.n_walks, w.p_halt, w.max_len, f, features=feat)
+        if reads:
+            for which, want in enumerate(oracle.sample(g.rowptr, g.col, g.w, n, w.n_walks, w.p_halt, w.max_len, f)[:3]):
+                helpers.assert_csr_equal(feat.to_host(which), want, f"n={n} matrix {which}", val_rtol=0)
+    feat.free()
+    ctx.close()

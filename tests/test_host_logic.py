@@ -137,7 +137,7 @@ def test_no_memory_for_the_mask_means_the_states(fake):
 
 def test_host_path_without_memory_for_the_preferred_mask(fake):
     ctx = fake.context(0)
-    fake.report(PHI=400_000, PSI=400_000, EDGES=8192, PLAN=25_600, KEYS=64_000, POSITIONS=2_500_000, LONGEST=4096)
+    fake.report(PHI=400_000, PSI=400_000, EDGES=8192, PLAN=25_600, KEYS=640_000, POSITIONS=2_500_000, LONGEST=40_000)
     assert fake.lib.grf_ctx_use_tensor_cores(ctx, 2) == 0
     for _ in range(2):                            # the second pass has made the object's arrays as large as they get
         assert fake.step_host(ctx, 4096, 8, 32, 64) == 0
@@ -163,5 +163,28 @@ def test_host_path_that_fails_waits_for_its_copies(fake):
     waited = {x for x in fake.log() if x.startswith("sync stream")}
     assert len(waited) >= 2                       # the context's stream and the one that the inputs travel on
     assert fake.step_host(ctx, 400, 8, 32, 64) == 0
+    assert fake.lib.grf_ctx_destroy(ctx) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
+def test_objects_sampled_once_hold_what_their_entries_need(fake):
+    """A model freezes one object per layer and head: its arrays follow the number of non-zeros.  An object that is sampled
+    again and again has arrays for the largest sample, and its samples do not wait."""
+    ctx = fake.context(0)
+    nnz = 400_000
+    fake.report(PHI=nnz, PSI=nnz, EDGES=40_000)
+    rc, first = fake.sample(ctx, 4096)            # makes the context's scratch
+    assert rc == 0
+    live = fake.lib.fake_live(0)
+    rc, frozen = fake.sample(ctx, 4096)
+    assert rc == 0 and fake.nnz(frozen) == (0, nnz)
+    assert fake.lib.fake_live(0) - live < 1.3 * 3 * (8 * nnz + 4 * 4097)
+    for _ in range(2):
+        assert fake.sample(ctx, 4096, first)[0] == 0
+    fake.lib.fake_log_clear()
+    assert fake.sample(ctx, 4096, first)[0] == 0
+    assert not [x for x in fake.log() if x.startswith("sync")]
+    for h in (first, frozen):
+        assert fake.lib.grf_features_free(h) == 0
     assert fake.lib.grf_ctx_destroy(ctx) == 0
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
