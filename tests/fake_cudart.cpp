@@ -192,7 +192,7 @@ cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void** args, size_t, cud
     } else if (is("block_plan_kernel")) {
         **(int32_t**)args[7] = (int32_t)report[5];
     } else if (is("mask_structure_kernel")) {
-        int32_t* host = *(int32_t**)args[18];
+        int32_t* host = *(int32_t**)args[20];
         host[0] = (int32_t)report[6]; host[1] = (int32_t)report[7]; host[2] = (int32_t)report[8];
     }
     return cudaSuccess;
