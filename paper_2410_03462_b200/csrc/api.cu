@@ -42,7 +42,8 @@ struct block_pool {
     {
         std::lock_guard<std::mutex> g(lock);
         if (contexts == 0 || held[dev] + bytes > POOL_BYTES) return false;
-        blocks[dev].emplace(bytes, p);
+        try { blocks[dev].emplace(bytes, p); }
+        catch (const std::bad_alloc&) { return false; }
         held[dev] += bytes;
         return true;
     }
@@ -224,16 +225,17 @@ extern "C" int grf_ctx_destroy(grf_ctx* ctx)
     for (auto& t : ctx->timed) { cudaEventDestroy(t.beg); cudaEventDestroy(t.end); }
     for (cudaEvent_t e : ctx->free_events) cudaEventDestroy(e);
     delete ctx;
-    bool last = false;
+    bool last = false, holds[block_pool::DEVICES];
     {
         std::lock_guard<std::mutex> g(pool().lock);
         last = --pool().contexts == 0;
+        for (int dev = 0; dev < block_pool::DEVICES; ++dev) holds[dev] = pool().held[dev] > 0 || pool().slots_held[dev] > 0;
     }
     if (last) {
         int before = 0;
         cudaGetDevice(&before);
         for (int dev = 0; dev < block_pool::DEVICES; ++dev)
-            if ((pool().held[dev] > 0 || pool().slots_held[dev] > 0) && cudaSetDevice(dev) == cudaSuccess) {
+            if (holds[dev] && cudaSetDevice(dev) == cudaSuccess) {
                 pool().empty(dev);
                 for (grf_size_slot s; pool().take_slot(dev, &s);) slot_destroy(&s);
             }
@@ -269,7 +271,8 @@ grf_launch_scope::~grf_launch_scope()
     ctx->launches += n;
     if (!ctx->timing || !beg || !end) return;
     cudaEventRecord(end, ctx->stream);
-    ctx->timed.push_back({cls, beg, end});
+    try { ctx->timed.push_back({cls, beg, end}); }
+    catch (const std::bad_alloc&) { cudaEventDestroy(beg); cudaEventDestroy(end); }     // this launch goes untimed
 }
 
 extern "C" int grf_ctx_use_tensor_cores(grf_ctx* ctx, int enable)
@@ -324,8 +327,10 @@ extern "C" int grf_ctx_kernel_times(grf_ctx* ctx, float* ms, int64_t* launches)
     for (auto& t : ctx->timed) {
         float x = 0.0f;
         if (cudaEventElapsedTime(&x, t.beg, t.end) == cudaSuccess) { ms[t.cls] += x; launches[t.cls] += 1; }
-        ctx->free_events.push_back(t.beg);
-        ctx->free_events.push_back(t.end);
+        for (cudaEvent_t e : {t.beg, t.end}) {
+            try { ctx->free_events.push_back(e); }
+            catch (const std::bad_alloc&) { cudaEventDestroy(e); }
+        }
     }
     ctx->timed.clear();
     cudaGetLastError();

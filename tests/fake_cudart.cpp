@@ -9,6 +9,7 @@
 #include <cstdlib>
 #include <map>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -36,6 +37,13 @@ thread_local cudaError_t last = cudaSuccess;
 // longest list
 int64_t report[9];
 
+bool no_heap = false;                                // the library's operator new throws
+struct Own {                                         // ... while this file's own calls do not
+    bool was = no_heap;
+    Own() { no_heap = false; }
+    ~Own() { no_heap = was; }
+};
+
 struct Stream { int device; };
 struct Event { int device; };
 
@@ -52,19 +60,32 @@ int device_of(const void* p)
 
 }  // namespace
 
+void* operator new(size_t n)
+{
+    void* p = no_heap ? nullptr : malloc(n ? n : 1);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void* operator new(size_t n, const std::nothrow_t&) noexcept { return no_heap ? nullptr : malloc(n ? n : 1); }
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
+
 extern "C" {
 
 // ---- what a test sets and reads
 void fake_reset()
 {
     std::lock_guard<std::recursive_mutex> g(lock);
+    const Own own;
     for (int d = 0; d < DEVICES; ++d) limit[d] = ~(size_t)0;
     mallocs = frees = refused = errors = 0;
+    no_heap = false;
     memset(report, 0, sizeof(report));
     log_.clear();
     current = 0;
 }
 void fake_report(int which, int64_t value) { report[which] = value; }
+void fake_no_heap(int on) { no_heap = on != 0; }
 void fake_limit(int device, size_t bytes) { limit[device] = bytes; }      // an allocation beyond it fails
 size_t fake_live(int device) { return live[device]; }
 long fake_mallocs() { return mallocs; }
@@ -89,13 +110,14 @@ cudaError_t cudaSetDevice(int d)
     return cudaSuccess;
 }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 148; return cudaSuccess; }
-cudaError_t cudaDeviceSynchronize() { log_.push_back("sync device " + std::to_string(current)); return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { const Own own; log_.push_back("sync device " + std::to_string(current)); return cudaSuccess; }
 cudaError_t cudaGetLastError() { const cudaError_t e = last; last = cudaSuccess; return e; }
 
 // ---- memory
 cudaError_t cudaMalloc(void** p, size_t bytes)
 {
     std::lock_guard<std::recursive_mutex> g(lock);
+    const Own own;
     if (bytes > limit[current] || live[current] + bytes > limit[current]) { ++refused; return fail(cudaErrorMemoryAllocation); }
     char* q = (char*)calloc(bytes ? bytes : 1, 1);
     if (!q) return fail(cudaErrorMemoryAllocation);
@@ -108,6 +130,7 @@ cudaError_t cudaMalloc(void** p, size_t bytes)
 cudaError_t cudaFree(void* p)
 {
     std::lock_guard<std::recursive_mutex> g(lock);
+    const Own own;
     if (!p) return cudaSuccess;
     auto it = blocks.find((char*)p);
     if (it == blocks.end()) return bad();
@@ -135,10 +158,11 @@ cudaError_t cudaMemset(void* p, int v, size_t bytes) { memset(p, v, bytes); retu
 cudaError_t cudaMemsetAsync(void* p, int v, size_t bytes, cudaStream_t) { memset(p, v, bytes); return cudaSuccess; }
 
 // ---- streams and events
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = (cudaStream_t) new Stream{current}; return cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { const Own own; *s = (cudaStream_t) new Stream{current}; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { delete (Stream*)s; return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t s)
 {
+    const Own own;
     char t[64];
     snprintf(t, sizeof t, "sync stream %p", (void*)s);
     log_.push_back(t);
@@ -146,12 +170,13 @@ cudaError_t cudaStreamSynchronize(cudaStream_t s)
 }
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t, unsigned)
 {
+    const Own own;
     char t[64];
     snprintf(t, sizeof t, "wait stream %p", (void*)s);
     log_.push_back(t);
     return cudaSuccess;
 }
-cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = (cudaEvent_t) new Event{current}; return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t* e) { const Own own; *e = (cudaEvent_t) new Event{current}; return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return cudaEventCreate(e); }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { delete (Event*)e; return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s)
@@ -160,7 +185,7 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s)
     if (((Event*)e)->device != (s ? ((Stream*)s)->device : current)) return bad();
     return cudaSuccess;
 }
-cudaError_t cudaEventSynchronize(cudaEvent_t) { log_.push_back("sync event"); return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { const Own own; log_.push_back("sync event"); return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 0.0f; return cudaSuccess; }
 
 // ---- kernels
@@ -175,6 +200,7 @@ cudaError_t cudaGetDriverEntryPoint(const char*, void** fn, unsigned long long, 
 cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void** args, size_t, cudaStream_t s)
 {
     std::lock_guard<std::recursive_mutex> g(lock);
+    const Own own;
     if (s && ((Stream*)s)->device != current) return bad();
     const std::string& name = kernels()[f];
     auto is = [&](const char* what) { return name.find(what) != std::string::npos; };

@@ -188,3 +188,23 @@ def test_objects_sampled_once_hold_what_their_entries_need(fake):
         assert fake.lib.grf_features_free(h) == 0
     assert fake.lib.grf_ctx_destroy(ctx) == 0
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
+def test_no_exception_leaves_the_library_when_the_heap_is_exhausted(fake):
+    """Bookkeeping that finds no host memory is left out: blocks go back to the device at once, times are not taken."""
+    ctx = fake.context(0)
+    fake.report(PHI=5000, PSI=6000, EDGES=900)
+    rc, feat = fake.sample(ctx, 100)
+    assert rc == 0 and fake.lib.grf_ctx_enable_timing(ctx, 1) == 0
+    assert fake.sample(ctx, 100, feat)[0] == 0
+    frees = fake.lib.fake_frees()
+    fake.lib.fake_no_heap(1)
+    assert fake.sample(ctx, 100, feat)[0] == 0
+    ms, n = (fake_device.C.c_float * 10)(), (fake_device.C.c_int64 * 10)()
+    assert fake.lib.grf_ctx_kernel_times(ctx, ms, n) == 0
+    assert fake.lib.grf_features_free(feat) == 0
+    assert fake.sample(ctx, 100)[0] == fake.NOMEM
+    fake.lib.fake_no_heap(0)
+    assert fake.lib.fake_frees() - frees >= 9     # three matrices of three arrays
+    assert fake.lib.grf_ctx_destroy(ctx) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
