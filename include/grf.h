@@ -12,7 +12,9 @@
  *   - all device work is enqueued on the context's stream; unless a call says otherwise it
  *     returns without waiting for that work;
  *   - a context is not thread-safe: one host thread at a time per context; a feature object likewise, but it is
- *     independent of the context that sampled it: any context of its device may use it (the caller orders the streams);
+ *     independent of the context that sampled it: any context of its device may use it.  The caller orders the streams
+ *     behind calls that sample or re-modulate; what an attention call or grf_features_materialise builds inside an object
+ *     the library orders itself (except for calls under stream capture);
  *   - matrices are CSR with int32 row pointers/column indices (ascending inside a row) and fp32 values.
  */
 #ifndef GRF_H

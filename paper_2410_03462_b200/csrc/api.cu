@@ -1,5 +1,6 @@
 // C-ABI entry points that are not kernels themselves: contexts, buffers, feature objects, the
 // attention driver (Alg. 1 step 5 in chunks of problems) and the host-buffer path.
+#include <atomic>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -73,6 +74,7 @@ struct block_pool {
 void slot_destroy(grf_size_slot* s)
 {
     if (s->ready) cudaEventDestroy(s->ready);
+    if (s->built) cudaEventDestroy(s->built);
     if (s->host) cudaFreeHost(s->host);
     *s = grf_size_slot();
 }
@@ -135,7 +137,8 @@ int grf_features_new(grf_features** out, int device)
     if (device >= block_pool::DEVICES || !pool().take_slot(device, &f->sizes)) {
         int rc = GRF_OK;
         if (cudaMallocHost((void**)&f->sizes.host, 64) != cudaSuccess) rc = GRF_ERR_NOMEM;
-        else if (cudaEventCreateWithFlags(&f->sizes.ready, cudaEventDisableTiming) != cudaSuccess) rc = GRF_ERR_CUDA;
+        else if (cudaEventCreateWithFlags(&f->sizes.ready, cudaEventDisableTiming) != cudaSuccess ||
+                 cudaEventCreateWithFlags(&f->sizes.built, cudaEventDisableTiming) != cudaSuccess) rc = GRF_ERR_CUDA;
         if (rc != GRF_OK) {
             cudaGetLastError();
             slot_destroy(&f->sizes);
@@ -167,6 +170,26 @@ int grf_settle_sizes(grf_features* feat)
     return GRF_OK;
 }
 
+static bool capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    cudaGetLastError();                                 // the default stream, while another one is captured
+    return true;
+}
+
+void grf_built_by(grf_ctx* ctx, grf_features* feat)
+{
+    if (capturing(ctx->stream)) return;
+    if (cudaEventRecord(feat->sizes.built, ctx->stream) == cudaSuccess) feat->built_by = ctx->id;
+}
+
+int grf_wait_for_build(grf_ctx* ctx, const grf_features* feat)
+{
+    if (!capturing(ctx->stream)) GRF_CUDA_TRY(cudaStreamWaitEvent(ctx->stream, feat->sizes.built, 0));
+    return GRF_OK;
+}
+
 int grf_csr_reserve(grf_csr_dev* m, int32_t rows, int32_t cols, int64_t nnz_cap)
 {
     m->rows = rows; m->cols = cols;
@@ -184,6 +207,8 @@ extern "C" int grf_ctx_create(grf_ctx** out, int device, void* cuda_stream)
     GRF_CUDA_TRY(cudaSetDevice(device));
     grf_ctx* c = new (std::nothrow) grf_ctx();
     if (!c) return GRF_ERR_NOMEM;
+    static std::atomic<uint64_t> contexts_made{0};
+    c->id = ++contexts_made;
     c->device = device;
     c->stream = (cudaStream_t)cuda_stream;
     if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
@@ -535,6 +560,7 @@ extern "C" int grf_masked_linear_attn(grf_ctx* ctx, const grf_features* feat, in
     const size_t per = ws_per_problem(R, m, d, dtype);
     if (workspace_bytes < per) return GRF_ERR_WORKSPACE;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
+    GRF_TRY(grf_wait_built(ctx, feat));
     bool by_mask = false;
     if (aligned16(phiQ, phiK, V, out)) GRF_TRY(grf_linear_by_mask(ctx, feat, G, N, m, d, dtype, &by_mask));
     return linear_attn(ctx, feat, by_mask, G, G, N, m, d, dtype, phiQ, phiK, V, out, den_out, workspace, workspace_bytes);

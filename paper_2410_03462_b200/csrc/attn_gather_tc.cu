@@ -543,6 +543,7 @@ static int build_plan_coefficients(grf_ctx* ctx, grf_features* feat)
     }
     GRF_CUDA_TRY(cudaGetLastError());
     feat->plan_coef_ready = true;
+    grf_built_by(ctx, feat);
     return GRF_OK;
 }
 
@@ -598,6 +599,7 @@ extern "C" int grf_plan_stats(grf_ctx* ctx, const grf_features* feat, int32_t* b
 {
     if (!ctx || !feat) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
+    GRF_TRY(grf_wait_built(ctx, feat));
     GRF_TRY(grf_ensure_block_plan(ctx, feat));
     if (!feat->plan_ready) return GRF_ERR_TOO_LARGE;
     if (blocks) *blocks = feat->plan_blocks;

@@ -1036,6 +1036,7 @@ static int build_mask(grf_ctx* ctx, grf_features* feat)
     if (K.structure_ready && feat->plan_ready && !feat->plan_stale) {
         // same walks, new coefficients: the key lists and positions still hold
         GRF_TRY(launch_mask_values(ctx, feat, K.by_position));
+        grf_built_by(ctx, feat);
         K.ready = true;
         return GRF_OK;
     }
@@ -1047,6 +1048,7 @@ static int build_mask(grf_ctx* ctx, grf_features* feat)
     if (K.refused) return GRF_ERR_TOO_LARGE;
     GRF_TRY(reserve_with_headroom(&K.val, (size_t)K.entries * BQ * sizeof(__nv_bfloat16)));
     GRF_TRY(launch_mask_values(ctx, feat, K.by_position));
+    grf_built_by(ctx, feat);
     K.structure_ready = true;
     K.ready = true;
     return GRF_OK;
@@ -1056,6 +1058,7 @@ extern "C" int grf_features_materialise(grf_ctx* ctx, grf_features* feat)
 {
     if (!ctx || !feat) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
+    GRF_TRY(grf_wait_built(ctx, feat));
     feat->mask.requested = false;
     GRF_TRY(build_mask(ctx, feat));
     feat->mask.requested = true;
@@ -1152,6 +1155,7 @@ extern "C" int grf_mask_rows(grf_ctx* ctx, const grf_features* feat, int32_t n, 
     if (!ctx || !feat || n <= 0 || !rows || !out) return GRF_ERR_INVALID;
     if (!feat->mask.ready || !feat->mask.requested) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
+    GRF_TRY(grf_wait_built(ctx, feat));
     const grf_mask_dev& K = feat->mask;
     {
         grf_launch_scope scope(ctx, 8);
@@ -1205,5 +1209,6 @@ extern "C" int grf_masked_attn_mhat(grf_ctx* ctx, const grf_features* feat, int3
     if ((int64_t)G * N > 0x7fffffffll || (int64_t)G * feat->mask.blocks > 0x7fffffffll) return GRF_ERR_TOO_LARGE;
     if (((uintptr_t)phiQ | (uintptr_t)phiK | (uintptr_t)V | (uintptr_t)out) & 15u) return GRF_ERR_INVALID;
     GRF_CUDA_TRY(cudaSetDevice(ctx->device));
+    GRF_TRY(grf_wait_built(ctx, feat));
     return grf_mhat_launch(ctx, feat, G, N, m, d, phiQ, phiK, V, out, den_out);
 }

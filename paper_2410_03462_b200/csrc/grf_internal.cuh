@@ -30,6 +30,7 @@ struct grf_buf {
 
 struct grf_ctx {
     int device = 0;
+    uint64_t id = 0;                // of this context alone, from 1
     cudaStream_t stream = nullptr;
     int sm_count = 0;
     int64_t launches = 0;
@@ -129,6 +130,7 @@ struct grf_mask_dev {
 struct grf_size_slot {
     int32_t* host = nullptr;        // pinned
     cudaEvent_t ready = nullptr;    // behind the kernels that write them
+    cudaEvent_t built = nullptr;    // behind what an attention call has built inside the object (grf_built_by)
 };
 
 struct grf_features {
@@ -136,6 +138,7 @@ struct grf_features {
     grf_csr_dev phi, psi, psit;
     grf_size_slot sizes;
     bool sizes_pending = false;     // nnz of the matrices is still to be read from `sizes` (grf_features_sizes)
+    uint64_t built_by = 0;          // context on whose stream sizes.built was recorded last
     bool sampled = false;           // holds, or has held, a sample
     grf_kept_walks kept;
     grf_mask_dev mask;
@@ -159,6 +162,17 @@ int grf_settle_sizes(grf_features* feat);
 static inline int grf_features_sizes(const grf_features* feat)
 {
     return feat->sizes_pending ? grf_settle_sizes(const_cast<grf_features*>(feat)) : GRF_OK;
+}
+
+// What a call builds inside an object (mask values, the gather's coefficients) is queued on that call's stream, and callers
+// that see a const object cannot order other streams behind it.  grf_built_by: after such a build.  grf_wait_built: before a
+// call uses or builds any of it; lets the stream wait if another context built last (whose stream then waited for the one
+// before it).  A stream under capture neither records nor waits: who replays a graph orders it.
+void grf_built_by(grf_ctx* ctx, grf_features* feat);
+int grf_wait_for_build(grf_ctx* ctx, const grf_features* feat);
+static inline int grf_wait_built(grf_ctx* ctx, const grf_features* feat)
+{
+    return feat->built_by == 0 || feat->built_by == ctx->id ? GRF_OK : grf_wait_for_build(ctx, feat);
 }
 
 // sample.cu

@@ -208,3 +208,31 @@ def test_no_exception_leaves_the_library_when_the_heap_is_exhausted(fake):
     assert fake.lib.fake_frees() - frees >= 9     # three matrices of three arrays
     assert fake.lib.grf_ctx_destroy(ctx) == 0
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
+def test_what_one_context_builds_inside_an_object_another_waits_for(fake):
+    """The first attention call forms the mask (or the gather's coefficients) on its own stream; the caller, who passes a
+    const object, cannot know of it.  A call of another context lets its stream wait for that."""
+    A, B = (fake.lib.fake_stream(0) for _ in range(2))
+    a, b = fake.context(0, A), fake.context(0, B)
+    wait = f"wait stream {hex(B)}"
+    for m, kernel in ((32, "mask_values"), (128, "block_coef")):
+        feat = _cloud_like(fake, a) if m == 32 else fake.sample(a, 4096)[1]
+        fake.lib.fake_log_clear()
+        assert fake.linear(a, feat, 8, 4096, m, 64, "bf16") == 0
+        assert fake.launched(kernel) == 1 and not [x for x in fake.log() if x.startswith("wait")]
+        assert fake.linear(a, feat, 8, 4096, m, 64, "bf16") == 0
+        assert not [x for x in fake.log() if x.startswith("wait")]        # its own stream is in order
+        fake.lib.fake_log_clear()
+        assert fake.linear(b, feat, 8, 4096, m, 64, "bf16") == 0
+        assert fake.log()[0] == wait
+        if m == 32:
+            assert fake.lib.grf_features_materialise(a, feat) == 0
+            fake.lib.fake_log_clear()
+            some = fake_device.C.c_void_p(4096)
+            assert fake.lib.grf_masked_attn_mhat(b, feat, 8, 4096, m, 64, 1, some, some, some, some, None) == 0
+            assert fake.lib.grf_mask_rows(b, feat, 1, some, some) == 0
+            assert fake.log()[0] == wait and fake.log()[2] == wait
+        assert fake.lib.grf_features_free(feat) == 0
+    assert fake.lib.grf_ctx_destroy(a) == 0 and fake.lib.grf_ctx_destroy(b) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
