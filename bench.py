@@ -3,14 +3,14 @@
 (walks, merge, CSR, regrouping) and evaluate the masked attention for one batch of synthetic inputs.
 Prints ONE JSON line.
 
-    python bench.py [--gpus N] [--steps K] [--warmup W] [--workload pc32768] [--route sz|mhat|asym]
+    python bench.py [--gpus N] [--steps K] [--warmup W] [--workload pc32768] [--route sz|states|mhat|asym]
                     [--frozen] [--impl ours|reference]
     python bench.py --suite        every workload, the unsorted point cloud, the scaling sweep and the operation
                                    counts of Sec. 4: a summary (.md) and one JSON line per run (.jsonl) in --suite-dir
 
 Routes: sz = grf_masked_linear_attn (the headline): Alg. 1 through the per-node states S_l, z_l of Eq. 12 or over the mask,
-whichever the library's cost rule finds cheaper for the batch (`evaluated_by` in the output says which); mhat = Eqs. 1-2 over the
-materialised mask Phi Psi^T; asym = Alg. 2 (asymmetric features, Psi = I).
+whichever the library's cost rule finds cheaper for the batch (`evaluated_by` in the output says which); states = the same call
+held to the per-node states; mhat = Eqs. 1-2 over the materialised mask Phi Psi^T; asym = Alg. 2 (asymmetric features, Psi = I).
 
 With N > 1 (launched by torch.distributed.run) every rank runs the same-sized, independently seeded batch
 on its own GPU (the problems are independent: no data-path collective); the value is the sum of all
@@ -176,7 +176,8 @@ def algorithmic_bytes(w, N, nnz_phi, nnz_psi, E):
     }
 
 
-def binding_report(w, N, nnz_phi, nnz_psi, ktimes, steps, pk, counters, plan_entries, mask_entries):
+def binding_report(w, N, nnz_phi, nnz_psi, ktimes, steps, pk, counters, plan_entries, mask_entries,
+                   mask_values_ms=None):
     """For each big kernel, the rates of the resources that can bind it (from counts of this run and the CUDA-event
     time of the kernel) and, where the tracked profile of the same sources exists, the profiler's busy fractions.
     `binds` names the resource with the largest fraction of its peak."""
@@ -234,15 +235,22 @@ def binding_report(w, N, nnz_phi, nnz_psi, ktimes, steps, pk, counters, plan_ent
             fr["integer_issue"] = issue
         finish("walk_merge", r, fr)
     ms, n = ktimes.get("mask_build", (0.0, 0))
-    if n and mask_entries:
-        # every multiply-add of Phi Psi^T reads a position and a value and reads and writes an accumulator: four accesses of
-        # the load/store unit, which takes one warp-wide access a cycle (148 SMs at 1.965 GHz)
-        t = ms / steps * 1e-3
+    if n and mask_entries and mask_values_ms:
+        # The values kernel.  Every multiply-add of Phi Psi^T reads a position and a value and reads and writes an accumulator:
+        # four accesses of the load/store unit, which takes one warp-wide access a cycle (148 SMs at 1.965 GHz) where no two
+        # lanes meet in a bank.  Here lanes do meet, so `conflict_free_fraction` is what a layout without conflicts could
+        # gain; how busy the unit is only the profiler can say.
+        t = mask_values_ms * 1e-3
         macs = nnz_phi * nnz_psi / N / t / 1e9
         peak = 148 * 32 * 1.965 / 4
-        hbm = (mask_entries * 260 + 2 * (nnz_phi + nnz_psi) * 8) / t / 1e9
-        finish("mask_build", {"multiply_adds_g_per_s": macs, "multiply_adds_peak_g_per_s": peak, "hbm_algorithmic_gbs": hbm},
-               {"load_store_unit": macs / peak, "hbm": hbm / pk["hbm_gbs"]})
+        hbm = (mask_entries * 260 + (nnz_phi + nnz_psi) * 8) / t / 1e9
+        c = counters.get("mask_build")
+        fr = {"hbm": hbm / pk["hbm_gbs"]}
+        if c and not c["stale"]:
+            fr["load_store_unit"] = c["lsu_pct"] / 100.0
+        finish("mask_build", {"values_ms": mask_values_ms, "structure_ms": max(ms / steps - mask_values_ms, 0.0),
+                              "multiply_adds_g_per_s": macs, "multiply_adds_conflict_free_g_per_s": peak,
+                              "conflict_free_fraction": macs / peak, "hbm_algorithmic_gbs": hbm}, fr)
     t = per_launch_s("mhat_attention")
     if t and mask_entries:
         issued = mask_entries * G * 2.0 * 128 * (m + d) / t / 1e12
@@ -295,7 +303,9 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
         w.name += f"-heads{args.heads}"
     g = w.graph()
     N, E = g.N, g.E
-    asym, mhat = route == "asym", route == "mhat"
+    asym, mhat, states_only = route == "asym", route == "mhat", route == "states"
+    if states_only:
+        route = "sz"
     if asym:      # Alg. 2: f_phi = alpha, f_psi = delta_0 (no key-side walks contribute, Psi = I)
         f = w.alpha.astype(np.float32)
         f_psi = np.zeros(w.max_len + 1, np.float32); f_psi[0] = 1.0
@@ -303,6 +313,8 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
         f = B.grf_deconvolve(w.alpha).astype(np.float32)
         f_psi = None
     ctx = api.Context(local)
+    if states_only:
+        B.grf_ctx_use_tensor_cores(ctx.handle, 2)
     dg = api.DeviceGraph(g, local)
     # every rank has its own batch of the same shape (weak scaling over independent problems)
     q, k, v = tensors.qkv(w.G, N, w.m, w.d, w.dtype, rank_seed(configs.QKV_SEED, rank))
@@ -396,7 +408,7 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
     ktimes = B.grf_ctx_kernel_times(ctx.handle)
     B.grf_ctx_enable_timing(ctx.handle, False)
     nnz_phi, nnz_psi = feat.shape(0)[2], feat.shape(1)[2]
-    plan_entries = mask_entries = None
+    plan_entries = mask_entries = mask_values_ms = None
     by_mask = mhat or ktimes.get("mhat_attention", (0.0, 0))[1] > 0      # what grf_masked_linear_attn chose
     if route == "sz" and w.dtype == "bf16" and not by_mask:
         try:
@@ -407,6 +419,15 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
         if not mhat:
             B.grf_features_materialise(ctx.handle, feat.handle)          # outside the timed region: the sizes are told to who asked
         mask_entries = B.grf_mask_stats(feat.handle)[1]
+        # the class "mask_build" is two kernels (structure, values); a mask formed again on lists that are in place is the
+        # values kernel alone
+        B.grf_ctx_enable_timing(ctx.handle, True)
+        for _ in range(5):
+            flush.zero_()
+            B.grf_features_materialise(ctx.handle, feat.handle)
+        ms, n = B.grf_ctx_kernel_times(ctx.handle)["mask_build"]
+        B.grf_ctx_enable_timing(ctx.handle, False)
+        mask_values_ms = ms / n
 
     # ---- end to end through the host-buffer entry point (pinned host memory; copies inside the timing)
     e2e = None
@@ -470,9 +491,9 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
             per_kernel[name] = {"ms_per_step": ms / steps, "launch_groups": n, "algorithmic_gb": a / 1e9,
                                 "achieved_gbs": a / 1e9 / (per * 1e-3), "hbm_frac": a / 1e9 / (per * 1e-3) / pk["hbm_gbs"]}
         dom = max(ktimes, key=lambda kname: ktimes[kname][0])
-        dom_ms = ktimes[dom][0] / max(ktimes[dom][1], 1)
         achieved = alg.get(dom, 0) / 1e9 / (ktimes[dom][0] / steps * 1e-3)
-        binding = binding_report(w, N, nnz_phi, nnz_psi, ktimes, steps, pk, counters, plan_entries, mask_entries)
+        binding = binding_report(w, N, nnz_phi, nnz_psi, ktimes, steps, pk, counters, plan_entries, mask_entries,
+                                 mask_values_ms)
         # DRAM traffic of the dominant kernel from the tracked profile of the same sources, scaled to this run's heads
         traffic = None
         c = counters.get(dom)
@@ -496,7 +517,7 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
             "scaling": "weak", "vs_baseline": None,
             "dtype": ("bf16" if w.dtype == "bf16" else "f32"), "dtype_note": DTYPE_NOTE[note] if w.dtype == "bf16" else "fp32 throughout",
             "data": "synthetic",
-            "config": {"workload": w.name, "route": route, "evaluated_by": "rows" if asym else "mask" if by_mask else "states",
+            "config": {"workload": w.name, "route": "states" if states_only else route, "evaluated_by": "rows" if asym else "mask" if by_mask else "states",
                        "N": N, "edges": E, "batch": w.batch, "heads": w.heads, "m": w.m,
                        "d": w.d, "n_walks": w.n_walks, "p_halt": w.p_halt, "max_len": w.max_len,
                        "nnz_phi": nnz_phi, "nnz_psi": nnz_psi,
@@ -517,7 +538,7 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
             "roofline": {"kernel": dom, "bound": bound, "frac_of": "hbm (the metric's roofline)", "achieved": achieved,
                          "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": achieved / pk["hbm_gbs"], "peak_source": pk["source"],
                          "traffic": traffic, "algorithmic_bytes": alg.get(dom, 0),
-                         "algorithmic_bytes_per_token_head": alg.get(dom, 0) / (w.G * N), "ms_per_launch": dom_ms,
+                         "algorithmic_bytes_per_token_head": alg.get(dom, 0) / (w.G * N), "ms_per_step": ktimes[dom][0] / steps,
                          "binding_resource": binds,
                          "fraction_of_binding_peak": binding.get(dom, {}).get("fraction_of_binding_peak")},
             "binding": binding,
@@ -655,7 +676,7 @@ def loglog_slope(xs, ys):
 
 
 def run_suite(args):
-    """All workloads on both symmetric routes, the unsorted point cloud, frozen and re-modulated features, the sweep 2^10..2^20 (sz
+    """All workloads, by cost and held to either symmetric route, the unsorted point cloud, frozen and re-modulated features, the sweep 2^10..2^20 (sz
     route) with the fitted slopes, and the operation counts; writes <dir>/bench_suite.jsonl and <dir>/bench_suite.md."""
     os.makedirs(args.suite_dir, exist_ok=True)
     lines, md = [], []
@@ -686,10 +707,12 @@ def run_suite(args):
         md.append(f"| {r['suite_case']} | {c['N']} | {c['batch'] * c['heads']} | {r['ms_per_step']:.3f} | {ph['sample_ms']:.3f} | "
                   f"{ph['attn_ms']:.3f} | {r['value'] / 1e6:.2f} | "
                   f"{'-' if ph['walks_per_s'] is None else format(ph['walks_per_s'] / 1e9, '.2f')} | {rf['kernel']} | "
-                  f"{rf['ms_per_launch']:.3f} | {rf['frac']:.3f} | {rf['binding_resource']} ({'-' if fb is None else format(fb, '.2f')}) |")
+                  f"{rf['ms_per_step']:.3f} | {rf['frac']:.3f} | {rf['binding_resource']} ({'-' if fb is None else format(fb, '.2f')}) |")
 
     for name in ("tiny", "vit", "pc4096", "pc32768", "pc32768-unsorted"):
         row(run(name, "sz"))
+        if name in ("vit", "pc4096", "pc32768"):
+            row(run(name, "states"))
         if name != "tiny":
             row(run(name, "sz", frozen=True))
             row(run(name, "mhat"))
@@ -742,10 +765,10 @@ def main():
     ap.add_argument("--impl", choices=["ours", "reference"], default="ours")
     ap.add_argument("--workload", default="pc32768")
     ap.add_argument("--no-cpu-baseline", action="store_true")
-    ap.add_argument("--route", choices=["sz", "asym", "mhat"], default="sz",
-                    help="sz: grf_masked_linear_attn, states or mask by cost (the default and the headline); mhat: Eqs. 1-2 over the "
-                         "materialised mask Phi Psi^T; asym: Alg. 2 (asymmetric features, Psi = I); the last two are "
-                         "variants outside the headline metric")
+    ap.add_argument("--route", choices=["sz", "states", "asym", "mhat"], default="sz",
+                    help="sz: grf_masked_linear_attn, states or mask by cost (the default and the headline); states: the same "
+                         "held to the per-node states; mhat: Eqs. 1-2 over the materialised mask Phi Psi^T; asym: Alg. 2 "
+                         "(asymmetric features, Psi = I); the last three are variants outside the headline metric")
     ap.add_argument("--frozen", action="store_true", help="features sampled (and prepared) once, outside the timed steps")
     ap.add_argument("--remodulate", action="store_true",
                     help="walks sampled once and kept; every timed step re-modulates them with new coefficients")
@@ -753,7 +776,7 @@ def main():
     ap.add_argument("--heads", type=int, default=0, help="override the workload's head count (profiling of a smaller case)")
     ap.add_argument("--no-other-routes", action="store_true", help="skip the short runs of the other routes beside the headline")
     ap.add_argument("--suite", action="store_true")
-    ap.add_argument("--suite-dir", default=os.path.join(ROOT, "gpurun_out"))
+    ap.add_argument("--suite-dir", default=os.path.join(ROOT, "build", "suite"))
     args = ap.parse_args()
     if args.warmup < 3 and args.impl == "ours":
         args.warmup = 3
