@@ -238,7 +238,8 @@ int grf_masked_attn_asym(grf_ctx* ctx, const grf_features* feat, int32_t G, int3
  *
  * grf_features_materialise: forms Mhat once for a feature object (N x N; Phi and Psi may be N x R) as dense bf16
  * blocks, one per 128 consecutive rows, over the sorted list of keys the block reaches (sums in fp32, fixed order).
- * Needs the node lists of Phi's block plan (built here if absent).  Waits for the stream twice.  The mask is dropped
+ * Needs the node lists of Phi's block plan (built here if absent).  Waits for the stream: once for the length of the node
+ * lists and once for that of the key lists, again where these outgrow the room at hand.  The mask is dropped
  * when the object is resampled; after grf_remodulate its values are stale (grf_mask_stats, grf_mask_rows and
  * grf_masked_attn_mhat return GRF_ERR_INVALID) until this call forms them again, which then takes one kernel over
  * the key lists already in place and does not wait for the stream.  GRF_ERR_TOO_LARGE when N > 294912 or the blocks would exceed 8 GiB (no
@@ -284,10 +285,10 @@ int grf_ctx_check_graphs(grf_ctx* ctx, int enable);
  * stays usable.  Asynchronous. */
 int grf_debug_wait_timeout(grf_ctx* ctx, int64_t limit_cycles);
 
-/* Route of grf_step_host: 0 (default) = through the per-node states (grf_masked_linear_attn); 1 = over the materialised
- * mask (grf_features_materialise + grf_masked_attn_mhat) whenever the shape allows it (bf16, d = 64, m in {16, 32, 64})
- * and the mask can be built; otherwise the call falls back to the default route.  Same outputs within the stated
- * tolerance. */
+/* Route of grf_step_host: 0 (default) = as grf_masked_linear_attn decides for the whole batch (states or mask by cost); 1 =
+ * over the materialised mask (grf_features_materialise + grf_masked_attn_mhat) whenever the shape allows it (bf16, d = 64,
+ * m in {16, 32, 64}) and the mask can be built; otherwise through the per-node states for that call (mask too large or no
+ * memory for it), or as 0 (other shapes).  Same outputs within the stated tolerance. */
 int grf_ctx_prefer_mask_route(grf_ctx* ctx, int enable);
 
 /* Waits for the context's stream and reports whether any kernel since the previous check gave up one of its

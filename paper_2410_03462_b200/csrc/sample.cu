@@ -63,7 +63,7 @@ struct Walker {
 // One 16-byte record per edge u -> v: v, the factor of the hop's load, and where v's own edges are.  A hop of a warp's 32
 // walkers then costs one gather instead of four, and fewer instructions.  Eight lanes per row.  (How many edges a graph has
 // is known on the device only: the records have the room that earlier graphs needed, and a larger graph is walked through
-// its CSR arrays once.)
+// its CSR arrays until its number has reached the host.)
 // It also clears what the walk kernel counts into and tells the host how many edges there are.
 __global__ void __launch_bounds__(256)
 edge_records_kernel(int32_t N, int64_t room, float inv_keep, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
