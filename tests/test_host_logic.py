@@ -236,3 +236,27 @@ def test_what_one_context_builds_inside_an_object_another_waits_for(fake):
         assert fake.lib.grf_features_free(feat) == 0
     assert fake.lib.grf_ctx_destroy(a) == 0 and fake.lib.grf_ctx_destroy(b) == 0
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
+def test_the_pool_holds_at_most_one_gib_and_goes_with_the_last_context(fake):
+    ctx, other = fake.context(0), fake.context(1)
+    fake.report(PHI=12 << 20, PSI=12 << 20, EDGES=900)
+    feats = [fake.sample(ctx, 100) for _ in range(6)]             # 0.3 GiB of matrices each
+    assert all(rc == 0 for rc, _ in feats) and fake.lib.fake_live(0) > 3 << 29
+    before = fake.lib.fake_live(0)
+    for _, h in feats:
+        assert fake.lib.grf_features_free(h) == 0
+    left = fake.lib.fake_live(0)
+    assert before - left > 1 << 29                # more than the pool takes has gone back to the device
+    mallocs = fake.lib.fake_mallocs()
+    rc, h = fake.sample(ctx, 100)                 # served by blocks of the freed objects
+    assert rc == 0 and fake.lib.fake_mallocs() == mallocs and fake.lib.fake_live(0) == left
+    fake.lib.fake_limit(0, left)                  # an allocation that fails empties the pool and tries again
+    fake.report(PHI=18 << 20, PSI=18 << 20)
+    rc, big = fake.sample(ctx, 100)
+    assert rc == 0 and fake.lib.fake_refused() > 0
+    for x in (h, big):
+        assert fake.lib.grf_features_free(x) == 0
+    assert fake.lib.grf_ctx_destroy(ctx) == 0 and fake.lib.fake_live(0) <= (1 << 30) + (1 << 20)
+    assert fake.lib.grf_ctx_destroy(other) == 0 and fake.lib.fake_live(0) == 0 and fake.lib.fake_live(1) == 0
+    assert fake.errors() == 0
