@@ -561,9 +561,15 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     GRF_TRY(grf_buf_reserve(&ctx->stage_val, rows2 * stride * sizeof(float)));
     GRF_TRY(grf_buf_reserve(&ctx->counts, 3 * (size_t)stride_counts * sizeof(int32_t)));
     GRF_TRY(grf_buf_reserve(&ctx->t_cursor, sizeof(int32_t) * (3 * (size_t)N + 1)));
-    GRF_TRY(grf_csr_reserve(&feat->phi, N, N, whole ? most : 0));
-    GRF_TRY(grf_csr_reserve(&feat->psi, N, N, whole ? most : 0));
-    GRF_TRY(grf_csr_reserve(&feat->psit, N, N, whole ? most : 0));
+    grf_csr_dev* const mats[3] = {&feat->phi, &feat->psi, &feat->psit};
+    for (grf_csr_dev* m : mats) {
+        if (whole) {
+            GRF_TRY(grf_csr_reserve(m, N, N, most));
+        } else {                                    // columns and values when their number is known
+            m->rows = m->cols = N;
+            GRF_TRY(grf_buf_reserve(&m->rowptr, sizeof(int32_t) * ((size_t)N + 1)));
+        }
+    }
     if (whole) GRF_TRY(grf_reserve_buckets(ctx, most));
     int32_t* counts = (int32_t*)ctx->counts.ptr;
     int32_t *long_count = (int32_t*)ctx->t_cursor.ptr, *cursor = long_count + 1, *long_list = cursor + N;
@@ -627,12 +633,10 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     if (!whole) {
         // column/value arrays, grown with head-room so that resampling rarely reallocates
         GRF_TRY(grf_settle_sizes(feat));
-        const int64_t nnz_phi = feat->phi.nnz, nnz_psi = feat->psi.nnz;
-        const int64_t cap_phi = nnz_phi + nnz_phi / 8 + 64, cap_psi = nnz_psi + nnz_psi / 8 + 64;
-        if (feat->phi.col.bytes < (size_t)nnz_phi * 4) GRF_TRY(grf_csr_reserve(&feat->phi, N, N, cap_phi));
-        if (feat->psi.col.bytes < (size_t)nnz_psi * 4) GRF_TRY(grf_csr_reserve(&feat->psi, N, N, cap_psi));
-        if (feat->psit.col.bytes < (size_t)nnz_psi * 4) GRF_TRY(grf_csr_reserve(&feat->psit, N, N, cap_psi));
-        GRF_TRY(grf_reserve_buckets(ctx, nnz_psi));
+        for (grf_csr_dev* m : mats)
+            if (!m->col.ptr || !m->val.ptr || m->col.bytes < (size_t)m->nnz * 4 || m->val.bytes < (size_t)m->nnz * 4)
+                GRF_TRY(grf_csr_reserve(m, N, N, m->nnz + m->nnz / 8 + 64));
+        GRF_TRY(grf_reserve_buckets(ctx, feat->psi.nnz));
     }
     int2* buckets = (int2*)ctx->t_tmp.ptr;
     {
