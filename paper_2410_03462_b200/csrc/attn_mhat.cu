@@ -38,7 +38,7 @@ constexpr int KT = GRF_MASK_TILE;       // keys per tile
 // depends on it.  A block whose part does not fit the room that the host has made writes none of it: the totals tell
 // the host how much is needed.  The last CTA to finish orders the blocks by decreasing key count.
 // One kernel for all of this, at the N = 32768 cloud: 237 us in five kernels and two prefix sums before, 178 us now (issue
-// slots 69 % busy while an SM has blocks, the blocks with the longest lists end last).
+// slots 77 % busy while an SM has blocks, 59 % of the warps there; the blocks with the longest lists end last).
 // Grid of 196 nodes: structure and values together 56 us with 32 nodes a warp and turn whatever the list's length, 40 now.
 
 constexpr int MS_THREADS = 768;
@@ -406,13 +406,13 @@ mask_values_kernel(int32_t N, int32_t Nk, const int32_t* __restrict__ phi_rowptr
 // block's list is used by nine of the block's rows on average, and the look-up (two shared-memory reads and a
 // population count per key) was most of the work of every addition.
 //
-// Bound by the load/store unit: per 32 multiply-adds two accesses of the accumulators (about three bank conflicts each) and
-// the position and value loads.  So every row makes one pass over its nodes: a warp's accumulators are as long as the block's
+// Bound by the load/store unit: per 32 multiply-adds two accesses of the accumulators (2.6 wavefronts each) and the
+// position and value loads.  So every row makes one pass over its nodes: a warp's accumulators are as long as the block's
 // key list, and the CTA runs as many of its warps as then fit its shared memory (a list beyond an eighth of it is
 // taken in segments).  Rows are handed to the warps by a counter.  N = 32768 cloud, 297 M multiply-adds: 853 -> 557 us
 // (fixed segments of 4096 keys made two passes of half the rows; four shuffles per node were 14 % of the unit's work; half
-// sectors in the output 10 %; 422 -> 222 M warp instructions).  The unit is busy 78 % of the time; what is left is its
-// bank conflicts (a node's 95 keys meet three times in a bank on average) and the loads.
+// sectors in the output 10 %; 422 -> 222 M warp instructions).  The unit is busy 76 % of the time
+// (124 M wavefronts); 40 M of them are bank conflicts in shared memory, the others would take it 0.29 ms.
 constexpr int MVP_WARPS = 16;
 constexpr int MVP_MIN_WARPS = 8;
 constexpr int MVP_ROOM = 212 * 256;      // accumulators (fp32) of a CTA at most: what an SM's shared memory holds
