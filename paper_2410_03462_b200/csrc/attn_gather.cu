@@ -3,13 +3,13 @@
 //
 // What bounds it is the delivery of state tiles: every non-zero of Phi brings m x d values to the SM, and on graphs
 // without locality nothing is shared.  From HBM that is 6 TB/s, from L2 up to 19 TB/s, so the columns of a problem's
-// tiles are taken in slices whose bytes over all nodes fit L2 (the grid runs through the rows of one slice before it
-// starts the next): HBM then sees each record once.  A group of lanes takes one node's slice, one 16-byte chunk (CH
+// tiles are taken in slices (the grid runs through the rows of one slice before it starts the next): as far as a slice of
+// all nodes fits L2, HBM sees each record once.  A group of lanes takes one node's slice, one 16-byte chunk (CH
 // consecutive feature rows a of one column b) per lane, and adds Phi_il times it to T_i = sum_l Phi_il S_l in registers;
 // phi(q_i) enters once, at the end.  What limits a slice is then the latency of L2 at one load per warp and 64 warps per
-// SM; fewer warps with more loads each were slower.  Expanders, 4 heads, m = 32, d = 64, bf16: N = 2^18 34.0 -> 23.5 ms
-// (10.4 TB/s into the SMs), N = 2^16 6.8 ms by the tensor-core gather -> 3.6 ms (17 TB/s).  Sums are carried in fp32 in a
-// fixed order.
+// SM; fewer warps with more loads each were slower.  Expanders, 2 heads, m = 32, d = 64, bf16: N = 2^18 16.8 ms with
+// whole tiles -> 9.4 (12.9 TB/s into the SMs), N = 2^20 71.4 -> 60.9 (8 TB/s: 512 MB per slice).  Sums are carried in fp32
+// in a fixed order.
 #include <type_traits>
 
 #include "grf_internal.cuh"
@@ -102,11 +102,11 @@ gather_denominators_kernel(int32_t N, int32_t R, const int32_t* __restrict__ row
     if (lane == 0) den[(size_t)g * N + i] = d;
 }
 
-// Lanes of one node's slice and columns of a slice, for LANES lanes wanted and CPL chunks per lane.
-template <typename T, int M, int D, int LANES, int CPL> struct SliceShape {
+// Lanes of one node's slice (32, fewer where a whole tile has fewer chunks) and columns of a slice, for CPL chunks per lane.
+template <typename T, int M, int D, int CPL> struct SliceShape {
     static constexpr int CH = grf_tile_chunk<T>();
     static constexpr int KC = M / CH;                                        // chunks along the feature rows a
-    static constexpr int LPN = KC >= LANES ? KC : (KC * D < LANES ? KC * D : LANES);
+    static constexpr int LPN = KC >= 32 ? KC : (KC * D < 32 ? KC * D : 32);
     static constexpr int SB = LPN / KC;                                      // columns side by side
     static constexpr int NB = SB * CPL <= D ? CPL : D / SB;                  // columns per lane
     static constexpr int COLS = SB * NB;                                     // columns of a slice
@@ -122,13 +122,13 @@ __device__ __forceinline__ uint4 load_tile(const unsigned char* p, uint64_t poli
     return x;
 }
 
-template <typename T, int M, int D, int LANES, int CPL>
+template <typename T, int M, int D, int CPL>
 __global__ void __launch_bounds__(GATHER_WARPS * 32, CPL == 1 ? 16 : 6)
 gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                      const float* __restrict__ val, const T* __restrict__ phiQ, const unsigned char* __restrict__ states,
                      T* __restrict__ out, const float* __restrict__ den)
 {
-    using Sh = SliceShape<T, M, D, LANES, CPL>;
+    using Sh = SliceShape<T, M, D, CPL>;
     constexpr int CH = Sh::CH, LPN = Sh::LPN, NPS = 32 / LPN, NB = Sh::NB, KC = Sh::KC, P = Chunk<T>::PAIRS;
     const int lane = threadIdx.x & 31, sub = lane / LPN, pl = lane % LPN;
     const int kc = pl % KC, b = pl / KC;                 // this lane's chunk along a, and its first column of the slice
@@ -204,8 +204,12 @@ gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, c
     }
 }
 
-// Bytes of a slice over all nodes that still stay in L2 beside the streams.  (Measured at 2^17 and 2^18 nodes: half of it
-// doubles the passes over the matrix, 23 -> 36 ms; twice of it misses L2, 23 -> 31 ms.)
+// Bytes of a slice over all nodes that stay in L2 beside the streams.  Slices of 2 KB, four loads per lane and node, are
+// taken where they fit it; all other graphs take 512 bytes, one load of every lane per node, which costs more passes over the
+// matrix but hits L2 in part however large the graph.  ms, 2 KB / 512 bytes, expanders, 2 heads, m = 32, d = 64, bf16:
+// N = 36000 0.92 / 0.98, 60000 1.79 / 1.63, 147000 7.2 / 4.2, 2^18 14.8 / 9.4, 2^19 32.1 / 26.1, 2^20 66.8 / 60.9; fp32, 3 heads,
+// N = 20000 1.37 / 1.45.  (Narrower slices, with two or four nodes side by side, never win: 256 bytes 1.47, 2.45, 6.6, 13.6, 33.5,
+// 76 ms, 128 bytes 1.75, 3.03, 10.3, 19.0, 40.6, 88.)
 constexpr size_t SLICE_L2_BYTES = (size_t)72 << 20;
 
 template <typename T, int M, int D>
@@ -227,19 +231,13 @@ int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, const 
             N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, den);
     }
     grf_launch_scope scope(ctx, 5);
-    // The widest slice that fits L2: fewer passes over the matrix.
-    auto launch = [&](auto lanes, auto cpl) {
-        using Sh = SliceShape<T, M, D, decltype(lanes)::value, decltype(cpl)::value>;
-        gather_sliced_kernel<T, M, D, decltype(lanes)::value, decltype(cpl)::value>
-            <<<dim3(blocks, Sh::SLICES, G), GATHER_WARPS * 32, 0, ctx->stream>>>(
-                N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, (T*)out, den);
+    auto launch = [&](auto cpl) {
+        using Sh = SliceShape<T, M, D, decltype(cpl)::value>;
+        gather_sliced_kernel<T, M, D, decltype(cpl)::value><<<dim3(blocks, Sh::SLICES, G), GATHER_WARPS * 32, 0, ctx->stream>>>(
+            N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, (T*)out, den);
     };
-    using std::integral_constant;
-    const size_t R = (size_t)phi.cols;
-    if (R * 2048 <= SLICE_L2_BYTES) launch(integral_constant<int, 32>(), integral_constant<int, 4>());
-    else if (R * 512 <= SLICE_L2_BYTES) launch(integral_constant<int, 32>(), integral_constant<int, 1>());
-    else if (R * 256 <= SLICE_L2_BYTES) launch(integral_constant<int, 16>(), integral_constant<int, 1>());
-    else launch(integral_constant<int, 8>(), integral_constant<int, 1>());
+    if ((size_t)phi.cols * 2048 <= SLICE_L2_BYTES) launch(std::integral_constant<int, 4>());
+    else launch(std::integral_constant<int, 1>());
     return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
 }
 

@@ -47,7 +47,7 @@ def test_both_routes_match_oracle(N, G, d, m):
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
 @pytest.mark.parametrize("R,m,d", [(300, 32, 64), (36863, 32, 64), (36865, 128, 8), (147457, 16, 32), (294913, 8, 16)])
 def test_sliced_gather_widths(R, m, d, dtype):
-    """The plain-ALU gather takes tiles whole or in slices of 512, 256 or 128 bytes by the number of nodes: rows of Phi
+    """The plain-ALU gather takes tiles in slices of 2 KB or 512 bytes by the number of nodes (smaller tiles whole): rows of Phi
     with 0, 1, 31, 32, 33 and 70 non-zeros over few and many nodes."""
     from paper_2410_03462_b200 import api, binding as B
     ctx = api.Context(0)
@@ -78,5 +78,22 @@ def test_sliced_gather_widths(R, m, d, dtype):
     out, den = api.masked_linear_attn(ctx, feat, q.cuda(), k.cuda(), v.cuda(), want_den=True)
     B.grf_ctx_check(ctx.handle)
     helpers.assert_attn_close(out.float().cpu().numpy(), ref, helpers.TOL[dtype], den.cpu().numpy(), f"R={R}", min_ok=0.3)
+    feat.free()
+    ctx.close()
+
+
+@pytest.mark.parametrize("N,G", [(1000, 2), (1000, 96)])        # by the states, over the mask
+def test_a_mask_that_the_caller_formed_changes_no_bit_of_the_main_call(N, G):
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    w = configs.point_cloud_4096(N)
+    f = oracle.deconvolve(w.alpha).astype(np.float32)
+    feat = api.sample(ctx, api.DeviceGraph(w.graph()), 3, w.n_walks, w.p_halt, w.max_len, f)
+    q, k, v = (t.cuda() for t in tensors.qkv(G, N, 32, 64, "bf16", 4))
+    before = api.masked_linear_attn(ctx, feat, q, k, v)
+    B.grf_features_materialise(ctx.handle, feat.handle)
+    assert torch.equal(before, api.masked_linear_attn(ctx, feat, q, k, v))
+    api.masked_attn_mhat(ctx, feat, q, k, v)
+    assert torch.equal(before, api.masked_linear_attn(ctx, feat, q, k, v))
     feat.free()
     ctx.close()
