@@ -54,7 +54,7 @@ struct grf_ctx {
     static constexpr int HOST_PARTS = 4;     // most parts grf_step_host splits a batch into
     cudaStream_t copy_stream = nullptr, down_stream = nullptr;
     cudaEvent_t up_done[HOST_PARTS] = {}, part_done[HOST_PARTS] = {}, down_done = nullptr;
-    // small pinned host block for read-backs; [PINNED_EDGES]: edges of the graph of some earlier sample, written by its kernel
+    // small pinned host block for read-backs; [PINNED_EDGES]: edges of a graph whose records found no room, written by its sample
     static constexpr int PINNED_EDGES = 10;
     int32_t* pinned = nullptr;
     int* error_word = nullptr;      // device word set by a kernel that gave up a bounded wait

@@ -64,14 +64,17 @@ struct Walker {
 // walkers then costs one gather instead of four, and fewer instructions.  Eight lanes per row.  (How many edges a graph has
 // is known on the device only: the records have the room that earlier graphs needed, and a larger graph is walked through
 // its CSR arrays until its number has reached the host.)
-// It also clears what the walk kernel counts into and tells the host how many edges there are.
+// It also clears what the walk kernel counts into, and tells the host how many edges there are if they found no room.
 __global__ void __launch_bounds__(256)
 edge_records_kernel(int32_t N, int64_t room, float inv_keep, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                     const float* __restrict__ w, int4* __restrict__ edges, int32_t* __restrict__ col_counts,
                     int32_t* __restrict__ long_count, int32_t* __restrict__ host_edges)
 {
     const int32_t E = rowptr[N];
-    if (blockIdx.x == 0 && threadIdx.x == 0) { *host_edges = E; *long_count = 0; }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (E > room) *host_edges = E;
+        *long_count = 0;
+    }
     const int32_t u = blockIdx.x * 32 + (threadIdx.x >> 3);
     if (u >= N) return;
     if ((threadIdx.x & 7) == 0) col_counts[u] = 0;
@@ -574,8 +577,9 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     int32_t* counts = (int32_t*)ctx->counts.ptr;
     int32_t *long_count = (int32_t*)ctx->t_cursor.ptr, *cursor = long_count + 1, *long_list = cursor + N;
 
-    // Room for the edge records by the last graph that is known: the kernels compare it with their own graph's edges and
-    // read the CSR arrays where it is too small.  (An earlier sample may be writing the number just now; either value will do.)
+    // Room for the edge records by the last graph that is known to have found none: the kernels compare it with their own
+    // graph's edges and read the CSR arrays where it is too small.  (An earlier sample may be writing the number just now;
+    // either value will do.)
     const int64_t edges_seen = *(volatile const int32_t*)(ctx->pinned + grf_ctx::PINNED_EDGES);
     if (edges_seen > (int64_t)(ctx->edge_records.bytes / sizeof(int4)))
         (void)grf_buf_reserve(&ctx->edge_records, sizeof(int4) * ((size_t)edges_seen + (size_t)edges_seen / 8 + 64));

@@ -208,7 +208,7 @@ cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void** args, size_t, cud
     log_.push_back("launch " + name);
     if (is("edge_records_kernel")) {
         if (*(int64_t*)args[1] > 0 && device_of(*(void**)args[6]) != current) ++errors;     // the room for the records
-        **(int32_t**)args[9] = (int32_t)report[4];
+        if (report[4] > *(int64_t*)args[1]) **(int32_t**)args[9] = (int32_t)report[4];
     } else if (is("scan_direct_kernel")) {
         const grf_scan_jobs& j = *(const grf_scan_jobs*)args[0];
         for (int x = 0; x < 3; ++x) {
