@@ -82,10 +82,10 @@ int grf_deconvolve(const double* alpha, int32_t len, double* f_out);
  * Deposits of a row that hit the same column are added in ascending (walk, t) order.
  *
  * Limits: n_walks*(max_len+1) <= 16384 and N * 2^ceil(log2(n_walks*(max_len+1))) <= 2^32, else
- * GRF_ERR_TOO_LARGE.  The call waits once for the device (it reads back the two nonzero counts) for an object's first
- * sample and for samples of more than 4 M possible entries, N * min(N, n_walks*(max_len+1)), per matrix; the object's
- * arrays then hold the non-zeros and an eighth more.  Smaller samples into an object that has been sampled before do not
- * wait (the first call that needs the counts does); its arrays then grow to the possible entries, 100 MB at most.
+ * GRF_ERR_TOO_LARGE.  The call waits once for the device (it reads back the two nonzero counts) for samples of more than
+ * 4 M possible entries, N * min(N, n_walks*(max_len+1)), per matrix, and for an object's first sample from 8 K possible
+ * entries on; the object's arrays then hold the non-zeros and an eighth more.  Other samples do not wait (the first call
+ * that needs the counts does); the arrays are then made for the possible entries, 100 MB an object at most.
  */
 int grf_sample(grf_ctx* ctx, int32_t N, const int32_t* rowptr, const int32_t* col, const float* w,
                uint64_t seed, int32_t n_walks, float p_halt, int32_t max_len,

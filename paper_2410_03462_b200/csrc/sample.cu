@@ -548,8 +548,9 @@ static int sample_row_pointers(grf_ctx* ctx, grf_features* feat, int32_t N, int3
 // Up to this many entries per matrix the arrays of an object that is sampled again are made for the largest sample there can
 // be, so that nothing has to be known about it before the kernels are queued, and grf_sample does not wait.  The first sample
 // of an object waits and takes what it needs: features that are frozen (one object per layer and head) hold their non-zeros,
-// where the bound is several times as much (cloud of 4096 points: 41 MB against 10).
-constexpr int64_t SAMPLE_WHOLE_ENTRIES = 4 << 20;
+// where the bound is several times as much (cloud of 4096 points: 41 MB against 10).  Where the bound is 0.2 MB an object at
+// most, it is not worth the wait (10 us of 86 for the first pass on a lattice of 64 nodes).
+constexpr int64_t SAMPLE_WHOLE_ENTRIES = 4 << 20, SAMPLE_SMALL_ENTRIES = 8 << 10;
 
 static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& P,
                        const int32_t* rowptr, const int32_t* col, const float* w)
@@ -558,7 +559,7 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
     const int32_t stride = P.cap < N ? P.cap : N;   // a row cannot hold more distinct columns than N
     const size_t rows2 = 2 * (size_t)N;
     const int64_t most = (int64_t)N * stride;
-    const bool whole = most <= SAMPLE_WHOLE_ENTRIES && feat->sampled && !ctx->keep_walks;
+    const bool whole = most <= (feat->sampled ? SAMPLE_WHOLE_ENTRIES : SAMPLE_SMALL_ENTRIES) && !ctx->keep_walks;
     const int32_t stride_counts = (N + 3) & ~3;
     GRF_TRY(grf_buf_reserve(&ctx->stage_col, rows2 * stride * sizeof(int32_t)));
     GRF_TRY(grf_buf_reserve(&ctx->stage_val, rows2 * stride * sizeof(float)));
