@@ -14,8 +14,13 @@
 //            per query.
 // The exponentials are taken relative to a running maximum of the scores, which cancels in the quotient; sums are carried
 // in fp32 in a fixed order, so results are run-to-run identical.
-// N = 32768 cloud, 8 problems, m = 32, d = 64, bf16, softmax: 684 us with a lane per key and a warp per value row, 584 now:
-// latency, at the 32 warps per SM that 64 registers allow (48 registers spill: 759 us; 80 leave 24 warps: 723 us).
+// Batches of 32 non-zeros, and steps of value rows within a last batch that are whole, take loads without conditions: a
+// conditional load also zeroes its registers, and at d >= 8 m these instructions made the kernel slower than a lane per key and
+// a warp per value row.  N = 32768 cloud, 8 problems, bf16, softmax, us: lane per key / whole rows, conditional / now: m = 32,
+// d = 64 669 / 580 / 493; m = 16, d = 128 671 / 718 / 610; linear: 629 / 519 / 463 and 637 / 715 / 570.  Bound by
+// instructions and latency, at the 32 warps per SM that 64 registers allow (80 registers: 531, 48 spill).
+#include <type_traits>
+
 #include "grf_internal.cuh"
 
 namespace {
@@ -114,9 +119,10 @@ asym_attention_kernel(int32_t G, int32_t N, const int32_t* __restrict__ rowptr, 
     }
 
     const int32_t beg = rowptr[i], end = rowptr[i + 1];
-    for (int32_t p0 = beg; p0 < end; p0 += 32) {
-        const int32_t n = min(32, end - p0);
-        const bool valid = own < n;
+    // full: all 32 non-zeros are there, and no load or weight is conditional
+    auto batch = [&](int32_t p0, int32_t n, auto full) {
+        constexpr bool FULL = decltype(full)::value;
+        const bool valid = FULL || own < n;
         const int32_t l = valid ? __ldg(col + p0 + own) : 0;
         const float phi = valid ? __ldg(val + p0 + own) : 0.0f;
         float w[GH];
@@ -131,7 +137,7 @@ asym_attention_kernel(int32_t G, int32_t N, const int32_t* __restrict__ rowptr, 
 #pragma unroll
                 for (int u = 0; u < KB; ++u) {
                     const int32_t lk = __shfl_sync(0xffffffffu, l, (lane / KL) * KL + i0 + u);
-                    x[u] = row_piece(Kh[h] + (size_t)lk * M, (i0 + u) * KPI + lane / KL < n);
+                    x[u] = row_piece(Kh[h] + (size_t)lk * M, FULL || (i0 + u) * KPI + lane / KL < n);
                 }
 #pragma unroll
                 for (int u = 0; u < KB; ++u) {
@@ -176,7 +182,7 @@ asym_attention_kernel(int32_t G, int32_t N, const int32_t* __restrict__ rowptr, 
         }
         // the batch's value rows, VPI at a time
         constexpr int VB = 32 / VPI < 4 ? 32 / VPI : 4;              // loads of a problem on their way together
-        for (int t0 = 0; t0 < n; t0 += VPI * VB) {
+        auto values = [&](int t0, auto whole) {
 #pragma unroll
             for (int h = 0; h < GH; ++h) {
                 uint4 x[VB];
@@ -186,7 +192,7 @@ asym_attention_kernel(int32_t G, int32_t N, const int32_t* __restrict__ rowptr, 
                     const int b = t0 + u * VPI + vg, src = (b % KPI) * KL + b / KPI;     // the lane that owns number b
                     const int32_t lv = __shfl_sync(0xffffffffu, l, src & 31);
                     wt[u] = __shfl_sync(0xffffffffu, w[h], src & 31);
-                    x[u] = row_piece(Vh[h] + (size_t)lv * D, b < n);
+                    x[u] = row_piece(Vh[h] + (size_t)lv * D, decltype(whole)::value || b < n);
                 }
 #pragma unroll
                 for (int u = 0; u < VB; ++u) {
@@ -197,8 +203,14 @@ asym_attention_kernel(int32_t G, int32_t N, const int32_t* __restrict__ rowptr, 
                     for (int e = 0; e < P; ++e) acc[h][e] = fma_pair(w2, v[e], acc[h][e]);
                 }
             }
-        }
-    }
+        };
+        int t0 = 0;
+        for (; t0 + VPI * VB <= (FULL ? 32 : n); t0 += VPI * VB) values(t0, std::true_type());
+        if (!FULL && t0 < n) values(t0, std::false_type());
+    };
+    int32_t p0 = beg;
+    for (; p0 + 32 <= end; p0 += 32) batch(p0, 32, std::true_type());
+    if (p0 < end) batch(p0, end - p0, std::false_type());
 #pragma unroll
     for (int h = 0; h < GH; ++h) {
         float dn = den[h];
