@@ -205,9 +205,14 @@ size_t grf_attn_workspace_bytes(int32_t G, int32_t R, int32_t m, int32_t d, int 
  * object is resampled or freed.  If the device has no memory left for it, this call and later ones on the same features
  * take the per-node states instead, which need the caller's workspace only (equal calls then differ by rounding from
  * those made with memory at hand); grf_ctx_use_tensor_cores(ctx, 2) keeps to the states from the start.
- * Asynchronous, except that the first bf16 call with m and d multiples of 16
- * after the features were created, resampled or re-modulated prepares a per-block plan of Phi, and where it takes the
- * other order the mask, inside the feature object, which waits for the stream (so a feature object must not be used by two threads at the same time).
+ * Where the states are cheaper used at once than stored and gathered (m in {16, 32, 64}, d in {32, 64}; graphs without
+ * locality, fp32), every (row, node) pair leaves a record of d fp32 values in the workspace, or, where that holds fewer
+ * problems, in up to 512 MiB of scratch of the context (up to 1 GiB where the workspace is smaller than one problem's narrowest
+ * records); a call under stream capture keeps to whole states, which need the workspace only (and differ by rounding).
+ * Asynchronous, except that a call may wait for the sizes of a sample that is still running, and that the first bf16 call
+ * with m and d multiples of 16 after the features were created, resampled or re-modulated prepares a per-block plan of Phi,
+ * and where it takes the other order the mask, inside the feature object, which waits for the stream (so a feature object
+ * must not be used by two threads at the same time).
  */
 int grf_masked_linear_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d,
                            int dtype, const void* phiQ, const void* phiK, const void* V,

@@ -170,7 +170,7 @@ int grf_settle_sizes(grf_features* feat)
     return GRF_OK;
 }
 
-static bool capturing(cudaStream_t stream)
+bool grf_capturing(cudaStream_t stream)
 {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
@@ -180,13 +180,13 @@ static bool capturing(cudaStream_t stream)
 
 void grf_built_by(grf_ctx* ctx, grf_features* feat)
 {
-    if (capturing(ctx->stream)) return;
+    if (grf_capturing(ctx->stream)) return;
     if (cudaEventRecord(feat->sizes.built, ctx->stream) == cudaSuccess) feat->built_by = ctx->id;
 }
 
 int grf_wait_for_build(grf_ctx* ctx, const grf_features* feat)
 {
-    if (!capturing(ctx->stream)) GRF_CUDA_TRY(cudaStreamWaitEvent(ctx->stream, feat->sizes.built, 0));
+    if (!grf_capturing(ctx->stream)) GRF_CUDA_TRY(cudaStreamWaitEvent(ctx->stream, feat->sizes.built, 0));
     return GRF_OK;
 }
 
@@ -235,7 +235,7 @@ extern "C" int grf_ctx_destroy(grf_ctx* ctx)
     cudaDeviceSynchronize();
     grf_buf* bufs[] = {&ctx->edge_records, &ctx->stage_col, &ctx->stage_val, &ctx->counts, &ctx->scan_blocks,
                        &ctx->stage_dep_start, &ctx->stage_dep_t, &ctx->stage_dep_load, &ctx->dep_counts, &ctx->dep_rowptr2,
-                       &ctx->t_cursor, &ctx->t_tmp, &ctx->den_scratch, &ctx->h_rowptr, &ctx->h_col, &ctx->h_w,
+                       &ctx->t_cursor, &ctx->t_tmp, &ctx->den_scratch, &ctx->pair_scratch, &ctx->h_rowptr, &ctx->h_col, &ctx->h_w,
                        &ctx->h_q, &ctx->h_k, &ctx->h_v, &ctx->h_out, &ctx->h_ws};
     for (grf_buf* b : bufs) grf_buf_release(b);
     if (ctx->h_feat) grf_features_free(ctx->h_feat);
@@ -506,6 +506,46 @@ extern "C" size_t grf_attn_workspace_bytes(int32_t G, int32_t R, int32_t m, int3
     return ws_per_problem(R, m, d, dtype) * (size_t)G;
 }
 
+// The tensor-core build takes 35 us at least (a bucket's chain of segments); the plain one 8 us and 0.27 ns per non-zero
+// and problem at m = 32, d = 64.  us measured, plain / tensor cores: lattice of 400 nodes, 4 problems 10 / 36, grid of
+// 196, 8 problems 29 / 44, expander of 1024, 2 problems, m = 16 29 / 44, 4 problems, m = 32 69 / 47.
+static double plain_build_ns(const grf_features* feat, int32_t G, int32_t m, int32_t d)
+{
+    return 0.27 * ((double)m * d + 512.0) / 2560.0 * (double)G * (double)feat->psit.nnz;
+}
+constexpr double PLAIN_BUILD_WORTH_NS = 25000.0;
+
+// Whether the states of a batch are used where they are made (attn_pairs.cu) instead of being stored and gathered.  Decided by
+// the features' sizes, the shape and the whole batch's G_all, so that parts of a batch give the bits of the whole.  The sizes
+// of a sample whose kernels may still be running are waited for only where its walks' expectation leaves the choice open.  A
+// call under stream capture keeps to whole states, whose only memory is the caller's: the pairs lie in buffers of the context
+// that a later call may replace while the graph still names them.
+static int states_by_pairs(grf_ctx* ctx, const grf_features* feat, int32_t G_all, int32_t m, int32_t d, int dtype, const void* phiQ,
+                           const void* phiK, const void* V, const void* out, bool* yes)
+{
+    *yes = false;
+    if (!grf_pairs_shape(ctx, m, d) || !aligned16(phiQ, phiK, V, out)) return GRF_OK;
+    const size_t per = ws_per_problem(feat->phi.cols, m, d, dtype);
+    auto cheaper = [&](double nnz) {
+        return grf_pairs_ns(nnz, G_all, m, d, dtype, per) < grf_states_by_rows_ns(nnz, feat->phi.cols, G_all, m, d, dtype);
+    };
+    if (feat->sizes_pending && !cheaper(feat->expected_entries)) return GRF_OK;
+    if (grf_capturing(ctx->stream)) return GRF_OK;
+    GRF_TRY(grf_features_sizes(feat));
+    const double nnz = 0.5 * ((double)feat->phi.nnz + (double)feat->psit.nnz);
+    if (!cheaper(nnz) || !grf_pairs_fit(feat->phi.nnz, dtype)) return GRF_OK;
+    if (dtype == GRF_DTYPE_BF16) {
+        // (the plain build of small batches does not round Psi phi(k) to bf16: outputs 2.0e-3 off fp64 against 2.05e-3)
+        if (plain_build_ns(feat, G_all, m, d) <= PLAIN_BUILD_WORTH_NS) return GRF_OK;
+        // whole states by tiles, where rows of a block share their nodes
+        GRF_TRY(grf_ensure_block_plan(ctx, feat, false));
+        if (feat->plan_ready && grf_gather_tiles_ns(feat, G_all, m) + 45000.0 + G_all * nnz * (0.03 + 0.001 * m) <
+                                    grf_pairs_ns(nnz, G_all, m, d, dtype, per)) return GRF_OK;
+    }
+    *yes = true;
+    return GRF_OK;
+}
+
 // The attention of G problems once the route is known: over the mask in one launch, or through the per-node states in
 // chunks of as many problems as the workspace holds.  G_all is the size of the whole batch that they belong to: it picks
 // the kernels, so that parts of a batch give the bits of the whole.
@@ -514,6 +554,12 @@ static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int
                        void* workspace, size_t workspace_bytes)
 {
     if (by_mask) return grf_mhat_launch(ctx, feat, G, N, m, d, phiQ, phiK, V, out, den_out);
+    bool by_pairs = false;
+    GRF_TRY(states_by_pairs(ctx, feat, G_all, m, d, dtype, phiQ, phiK, V, out, &by_pairs));
+    if (by_pairs) {
+        const int rc = grf_pairs_attn(ctx, feat, G, N, m, d, dtype, phiQ, phiK, V, out, den_out, workspace, workspace_bytes);
+        if (rc != GRF_ERR_NOMEM) return rc;                     // its scratch could not be had: whole states need none
+    }
     const size_t per = ws_per_problem(feat->phi.cols, m, d, dtype);
     int64_t chunk = (int64_t)(workspace_bytes / per);
     if (chunk > G) chunk = G;
@@ -523,11 +569,7 @@ static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int
     bool tc_gather = false;
     const bool tensor_cores = dtype == GRF_DTYPE_BF16 && ctx->use_tensor_cores;
     if (tensor_cores) GRF_TRY(grf_features_sizes(feat));        // the choices below read them
-    // The tensor-core build takes 35 us at least (a bucket's chain of segments); the plain one 8 us and 0.27 ns per non-zero
-    // and problem at m = 32, d = 64.  us measured, plain / tensor cores: lattice of 400 nodes, 4 problems 10 / 36, grid of
-    // 196, 8 problems 29 / 44, expander of 1024, 2 problems, m = 16 29 / 44, 4 problems, m = 32 69 / 47.
-    const double plain_ns = 0.27 * ((double)m * d + 512.0) / 2560.0 * (double)G_all * (double)feat->psit.nnz;
-    const bool tc_states = tensor_cores && (plain_ns > 25000.0 || ctx->tiles_only);
+    const bool tc_states = tensor_cores && (plain_build_ns(feat, G_all, m, d) > PLAIN_BUILD_WORTH_NS || ctx->tiles_only);
     GRF_TRY(grf_gather_by_tensor_cores(ctx, feat, G_all, m, d, dtype, &tc_gather));
     for (int64_t g0 = 0; g0 < G; g0 += chunk) {
         const int32_t gc = (int32_t)((G - g0) < chunk ? (G - g0) : chunk);

@@ -46,6 +46,7 @@ struct grf_ctx {
     grf_buf t_cursor;               // per column: count, then scatter cursor; number of long buckets; their list
     grf_buf t_tmp;                  // unordered buckets of (row, value)
     grf_buf den_scratch;            // denominators of the tensor-core gather path when the caller wants none
+    grf_buf pair_scratch;           // records of (row, node) pairs that the caller's workspace has no room for
     // host-buffer path
     grf_buf h_rowptr, h_col, h_w, h_q, h_k, h_v, h_out, h_ws;
     grf_features* h_feat = nullptr;
@@ -138,6 +139,7 @@ struct grf_features {
     grf_csr_dev phi, psi, psit;
     grf_size_slot sizes;
     bool sizes_pending = false;     // nnz of the matrices is still to be read from `sizes` (grf_features_sizes)
+    double expected_entries = 0.0;  // non-zeros per matrix that the walks leave at most on average (0: not sampled)
     uint64_t built_by = 0;          // context on whose stream sizes.built was recorded last
     bool sampled = false;           // holds, or has held, a sample
     grf_kept_walks kept;
@@ -157,6 +159,7 @@ void grf_buf_release(grf_buf* b);
 int grf_csr_reserve(grf_csr_dev* m, int32_t rows, int32_t cols, int64_t nnz_cap);
 int grf_features_new(grf_features** out, int device);   // empty; `device` is current
 void grf_features_clear(grf_features* feat);
+bool grf_capturing(cudaStream_t stream);
 int grf_settle_sizes(grf_features* feat);
 // before nnz of a matrix is read: waits for the sample's sizes if they have not been read yet
 static inline int grf_features_sizes(const grf_features* feat)
@@ -220,6 +223,13 @@ int grf_build_states_tc(grf_ctx* ctx, const grf_csr_dev& psit, int32_t G, int32_
                         const void* phiK, const void* V, void* states, bool by_column);
 int grf_gather_contract_alu(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t m, int32_t d,
                             int dtype, const void* phiQ, const void* states, void* out, float* den_out);
+// attn_pairs.cu
+bool grf_pairs_shape(const grf_ctx* ctx, int32_t m, int32_t d);
+double grf_pairs_ns(double nnz, int32_t G, int32_t m, int32_t d, int dtype, size_t workspace_per_problem);
+double grf_states_by_rows_ns(double nnz, int32_t nodes, int32_t G, int32_t m, int32_t d, int dtype);
+bool grf_pairs_fit(int64_t nnz, int dtype);
+int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, int dtype, const void* phiQ,
+                   const void* phiK, const void* V, void* out, float* den_out, void* workspace, size_t workspace_bytes);
 // attn_mhat.cu
 void grf_mask_invalidate(grf_features* feat);
 void grf_mask_values_stale(grf_features* feat);

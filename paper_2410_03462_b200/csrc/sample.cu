@@ -632,6 +632,13 @@ static int sample_into(grf_ctx* ctx, grf_features* feat, const grf_walk_params& 
         }
     GRF_CUDA_TRY(cudaEventRecord(feat->sizes.ready, ctx->stream));
     feat->sizes_pending = true;
+    {
+        // expected deposits of a walk: 1 + keep + ... + keep^max_len
+        double deposits = 0.0, reached = 1.0;
+        for (int32_t t = 0; t <= P.max_len; ++t) { deposits += reached; reached /= P.inv_keep; }
+        deposits *= P.n_walks;
+        feat->expected_entries = (double)N * (deposits < N ? deposits : N);
+    }
     feat->plan_stale = true;       // the block plan of Phi is built by the first attention call that needs it
     feat->plan_ready = false;
     grf_mask_invalidate(feat);

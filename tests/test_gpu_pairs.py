@@ -1,0 +1,131 @@
+"""States used where they are made (records of (row, node) pairs): lists of every length class against the oracle, both types, all
+shapes of the route; records of every width give the same bits; the route agrees with whole states."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from tests import helpers
+from workloads import configs, tensors
+
+pytestmark = pytest.mark.gpu
+
+
+def kernel_classes(B, ctx, call):
+    """The kernel classes that a call launched."""
+    B.grf_ctx_enable_timing(ctx.handle, True)
+    B.grf_ctx_kernel_times(ctx.handle)
+    out = call()
+    times = B.grf_ctx_kernel_times(ctx.handle)
+    B.grf_ctx_enable_timing(ctx.handle, False)
+    return out, {name for name, (_, launches) in times.items() if launches}
+
+
+def csr(rng, rows, cols, lengths):
+    c = [np.sort(rng.choice(cols, size=min(n, cols), replace=False)) for n in lengths]
+    rp = np.concatenate([[0], np.cumsum([len(x) for x in c])]).astype(np.int32)
+    c = np.concatenate(c).astype(np.int32)
+    return oracle.CSR(rp, c, rng.uniform(0.1, 1.0, c.size).astype(np.float32), None, (rows, cols))
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("m", [16, 32, 64])
+@pytest.mark.parametrize("d", [32, 64])
+def test_lists_of_every_length(m, d, dtype):
+    """Nodes with 0, 1, 7 .. 9, 15 .. 17, 31 .. 33 and 100 keys and as many queries (chunks are of 8, 16 and 32), rows with none."""
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    rng = np.random.default_rng(m + d)
+    N, R, G = 3001, 2569, 24
+    lengths = (0, 1, 7, 8, 9, 15, 16, 17, 31, 32, 33, 100)
+    # columns of these lengths: every node's queries and keys in two different orders
+    phi_t = csr(rng, R, N, [lengths[l % 12] for l in range(R)])
+    psi_t = csr(rng, R, N, [lengths[(l + l // 12) % 12] for l in range(R)])
+    Phi, Psi = oracle.transpose(phi_t), oracle.transpose(psi_t)
+    feat = api.features_from_csr(ctx, N, R, (Phi.rowptr, Phi.col, Phi.val), (Psi.rowptr, Psi.col, Psi.val))
+    q, k, v = tensors.qkv(G, N, m, d, dtype, 5)
+    qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
+    B.grf_ctx_use_tensor_cores(ctx.handle, 2)               # never over the mask
+    (out, den), ran = kernel_classes(B, ctx, lambda: api.masked_linear_attn(ctx, feat, qd, kd, vd, want_den=True))
+    assert "row_denominators" not in ran and "mhat_attention" not in ran, ran
+    pick = [0, 1, G - 1]
+    ref = oracle.attn_sparse(tensors.widen(q[pick]), tensors.widen(k[pick]), tensors.widen(v[pick]), Phi, oracle.transpose(Psi))
+    helpers.assert_attn_close(out[pick].float().cpu().numpy(), ref, helpers.TOL[dtype], den[pick].cpu().numpy(), min_ok=0.3)
+    # one problem's workspace: the same bits; whole states: the same values (every difference is within both routes' bounds)
+    small = B.grf_attn_workspace_bytes(1, R, m, d, B.dtype_code(vd))
+    assert torch.equal(out, api.masked_linear_attn(ctx, feat, qd, kd, vd, workspace_bytes=small))
+    B.grf_ctx_use_tensor_cores(ctx.handle, 0)
+    other, ran = kernel_classes(B, ctx, lambda: api.masked_linear_attn(ctx, feat, qd, kd, vd))
+    assert "row_denominators" in ran
+    helpers.assert_attn_close(other[pick].float().cpu().numpy(), ref, helpers.TOL[dtype], min_ok=0.3)
+    feat.free()
+    ctx.close()
+
+
+@pytest.mark.parametrize("m,d", [(32, 64), (32, 32), (16, 64)])
+def test_records_of_every_width_give_the_same_bits(m, d):
+    """An expander whose whole records are larger than the context's scratch: a full workspace holds them, one problem's only
+    records of 16 columns."""
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    w = configs.sweep(17)
+    N = 1 << 17
+    f = oracle.deconvolve(w.alpha).astype(np.float32)
+    feat = api.sample(ctx, api.DeviceGraph(w.graph()), 3, w.n_walks, w.p_halt, w.max_len, f)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    G = 4
+    q = torch.relu(torch.randn(G, N, m, generator=gen, device="cuda")).bfloat16()
+    k = torch.relu(torch.randn(G, N, m, generator=gen, device="cuda")).bfloat16()
+    v = torch.randn(G, N, d, generator=gen, device="cuda").bfloat16()
+    out, ran = kernel_classes(B, ctx, lambda: api.masked_linear_attn(ctx, feat, q, k, v))
+    assert "row_denominators" not in ran, ran
+    for problems in (1, 2, 3):
+        small = B.grf_attn_workspace_bytes(problems, N, m, d, B.GRF_DTYPE_BF16)
+        assert torch.equal(out, api.masked_linear_attn(ctx, feat, q, k, v, workspace_bytes=small))
+    B.grf_ctx_use_tensor_cores(ctx.handle, 0)
+    other = api.masked_linear_attn(ctx, feat, q, k, v)
+    # both round S and the outputs to bf16 (2^-9 each): the relative difference of two such results is below 2^-7
+    assert float((out.float() - other.float()).norm() / other.float().norm()) < 2.0 ** -7
+    feat.free()
+    ctx.close()
+
+
+def test_capture_keeps_to_whole_states():
+    """The pairs' buffers belong to the context and may be replaced later: a captured call, also one on a sample whose sizes are
+    not known yet, uses the caller's memory only, and its replay gives the bits of whole states."""
+    from paper_2410_03462_b200 import api, binding as B
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        ctx = api.Context(0)
+        w = configs.point_cloud_4096(1500)
+        f = oracle.deconvolve(w.alpha).astype(np.float32)
+        q, k, v = (t.cuda() for t in tensors.qkv(4, 1500, 32, 64, "fp32", 4))
+        ws = torch.empty(B.grf_attn_workspace_bytes(4, 1500, 32, 64, B.GRF_DTYPE_F32), dtype=torch.uint8, device="cuda")
+        den = torch.empty(4, 1500, device="cuda")
+        out = torch.empty_like(v)
+        dg = api.DeviceGraph(w.graph())
+        feat = api.sample(ctx, dg, 3, w.n_walks, w.p_halt, w.max_len, f)
+
+        def call():
+            B.grf_masked_linear_attn(ctx.handle, feat.handle, 4, 1500, 32, 64, B.GRF_DTYPE_F32, q, k, v, out, den, ws, ws.numel())
+            return out.clone()
+
+        direct, ran = kernel_classes(B, ctx, call)
+        assert "row_denominators" not in ran, ran
+        B.grf_ctx_use_tensor_cores(ctx.handle, 0)
+        whole = call()
+        B.grf_ctx_use_tensor_cores(ctx.handle, 1)
+        feat.handle = B.grf_sample(ctx.handle, dg.N, dg.rowptr, dg.col, dg.w, 3, w.n_walks, w.p_halt, w.max_len, f, None, feat.handle)
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            call()
+        out.zero_()
+        graph.replay()
+        s.synchronize()
+        assert torch.equal(out, whole)
+        # two fp32 evaluations of the same sums: the bound of fp32 outputs
+        assert float((out - direct).norm() / direct.norm()) < 1e-5
+        del graph
+        feat.free()
+        ctx.close()
