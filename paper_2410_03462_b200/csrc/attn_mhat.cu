@@ -174,6 +174,16 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
         if (!(kbits[k >> 5] >> (k & 31) & 1u)) atomicOr(&kbits[k >> 5], 1u << (k & 31));
     });
     __syncthreads();
+    if (Nk <= GRF_MASK_SMALL) {                                 // every key of the tiles from the first to the last one reached
+        if (warp == 0) {
+            const uint32_t any = __ballot_sync(0xffffffffu, lane < wk && kbits[min(lane, wk - 1)] != 0u);
+            if (any) {
+                const int32_t first = (__ffs(any) - 1) & ~1, last = (31 - __clz(any)) | 1;       // two words a tile
+                if (lane >= first && lane <= last && lane < wk) kbits[lane] = lane * 32 + 32 <= Nk ? 0xffffffffu : (1u << (Nk & 31)) - 1u;
+            }
+        }
+        __syncthreads();
+    }
     const int32_t keys = ms_ranks(kbits, kbefore, wk, warp_sums, &total);
     ms_ranks(nbits, nbefore, wr, warp_sums, &total);
     const int32_t padded = (keys + KT - 1) / KT * KT;
@@ -604,34 +614,6 @@ template <int M, int D> struct MhShape {
 
 constexpr int MH_THREADS = 448;
 
-// two fp32 values in one 64-bit register: the packed multiply and add take one issue slot for both
-__device__ __forceinline__ uint64_t pack_f32x2(uint32_t lo, uint32_t hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b)
-{
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b)
-{
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ void ld_nc_32bytes(const uint4* p, uint4& a, uint4& b)
-{
-    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
-}
 constexpr int MH_ISSUER_S = 8, MH_ISSUER_O = 9, MH_PRODUCER0 = 10;
 
 template <int M, int D>
@@ -1195,6 +1177,7 @@ static int launch_mhat_values(grf_ctx* ctx, const grf_features* feat, int32_t G,
 int grf_mhat_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, const void* phiQ,
                     const void* phiK, const void* V, void* out, float* den_out)
 {
+    if (N <= GRF_MASK_SMALL) return grf_mhat_small_launch(ctx, feat, G, N, m, d, phiQ, phiK, V, out, den_out);
     if (m == 16) return launch_mhat_values<16>(ctx, feat, G, N, d, phiQ, phiK, V, out, den_out);
     if (m == 32) return launch_mhat_values<32>(ctx, feat, G, N, d, phiQ, phiK, V, out, den_out);
     return launch_mhat_values<64>(ctx, feat, G, N, d, phiQ, phiK, V, out, den_out);

@@ -105,6 +105,9 @@ struct grf_kept_walks {
 // sorted list of the keys j that any of its rows reaches (padded to a multiple of GRF_MASK_TILE with the last key
 // and zero values) and the block's values in bf16, laid out [group of 16 keys][row of the block][16 keys].
 #define GRF_MASK_TILE 64
+// Up to this many keys a block's list is made of whole aligned tiles, all of them between its first and last key
+// (attn_mhat_small.cu): at most eight.
+#define GRF_MASK_SMALL 512
 struct grf_mask_dev {
     bool ready = false;             // the blocks hold the mask of the present features
     bool requested = false;         // the caller asked for it (grf_features_materialise); else it is grf_masked_linear_attn's own
@@ -239,6 +242,9 @@ int grf_linear_by_mask(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_
 int grf_mhat_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, const void* phiQ,
                     const void* phiK, const void* V, void* out, float* den_out);
 void grf_mask_release(grf_features* feat);
+// attn_mhat_small.cu: the same for N <= GRF_MASK_SMALL
+int grf_mhat_small_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, const void* phiQ,
+                          const void* phiK, const void* V, void* out, float* den_out);
 // attn_gather_tc.cu
 int grf_build_block_plan(grf_ctx* ctx, grf_features* feat, bool with_coef = true);
 int grf_ensure_block_plan(grf_ctx* ctx, const grf_features* feat, bool with_coef = true);   // builds it if Phi changed since the last build

@@ -188,6 +188,44 @@ __device__ __forceinline__ void fence_before_sync() { asm volatile("tcgen05.fenc
 __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// two fp32 values in one 64-bit register: the packed multiply and add take one issue slot for both
+__device__ __forceinline__ uint64_t pack_f32x2(uint32_t lo, uint32_t hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ void ld_nc_32bytes(const uint4* p, uint4& a, uint4& b)
+{
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
+}
+// A box of a 3-D tensor (columns, rows, problems) into shared memory by the tensor-map copy engine, by one elected lane.
+__device__ __forceinline__ void tma_load3_elected(uint32_t dst, const CUtensorMap* map, int32_t row, int32_t problem, uint32_t bar)
+{
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n\t}"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(problem), "r"(bar) : "memory");
+}
+
 // Four rows of a 2-D tensor (row indices in registers) into shared memory by the tensor-map copy engine.
 __device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap* map, int32_t r0, int32_t r1, int32_t r2,
                                             int32_t r3, uint32_t bar)
@@ -204,3 +242,5 @@ __device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap* map
 // Host side: a [rows x cols] bf16 matrix whose rows are gathered one at a time (box = one row of at most 64
 // elements; swizzle = the row's byte length).  False when the encoder is unavailable or the base is misaligned.
 bool grf_make_row_gather_map(CUtensorMap* map, const void* base, uint64_t rows, uint32_t cols);
+// [problems][rows][cols] bf16, cols in {16, 32, 64}: boxes of box_rows whole rows of one problem, swizzled over a row's length.
+bool grf_make_row_box_map(CUtensorMap* map, const void* base, uint32_t problems, uint32_t rows, uint32_t cols, uint32_t box_rows);

@@ -1,4 +1,4 @@
-// Tensor maps for row gathers (host side).
+// Tensor maps for row gathers and boxes of rows (host side).
 #include "tc_common.cuh"
 
 // cuTensorMapEncodeTiled, looked up through the runtime (the library does not link the driver directly)
@@ -32,3 +32,16 @@ bool grf_make_row_gather_map(CUtensorMap* map, const void* base, uint64_t rows, 
                CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool grf_make_row_box_map(CUtensorMap* map, const void* base, uint32_t problems, uint32_t rows, uint32_t cols, uint32_t box_rows)
+{
+    encode_tiled_fn enc = tensor_map_encoder();
+    if (!enc || (reinterpret_cast<uintptr_t>(base) & 15u) != 0) return false;
+    const cuuint64_t dims[3] = {cols, rows, problems};
+    const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)rows * cols * 2};
+    const cuuint32_t box[3] = {cols, box_rows, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    const CUtensorMapSwizzle sw = cols * 2 == 32 ? CU_TENSOR_MAP_SWIZZLE_32B
+                                : (cols * 2 == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
