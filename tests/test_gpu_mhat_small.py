@@ -1,0 +1,65 @@
+"""Masked attention on graphs of at most 512 nodes: key lists of whole aligned tiles, several problems per CTA."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from tests import helpers
+from workloads import tensors
+
+pytestmark = pytest.mark.gpu
+
+
+def band_features(N, kind, rng):
+    """Phi, Psi (N x N) whose blocks of 128 rows reach: every key; a few keys of one tile; nothing; keys far apart."""
+    rows_phi, rows_psi = [], []
+    for i in range(N):
+        blk = i // 128
+        if kind == "dense":
+            c = rng.choice(N, size=min(N, 20), replace=False)
+        elif kind == "local" or (kind == "mixed" and blk % 4 == 0):
+            c = np.unique(np.clip(i + rng.integers(-2, 3, size=4), 0, N - 1))
+        elif kind == "mixed" and blk % 4 == 1:
+            c = np.array([], dtype=np.int64)
+        else:
+            c = np.unique(rng.choice([0, N // 2, N - 1], size=2))
+        rows_phi.append(np.sort(c))
+        rows_psi.append(np.unique(np.clip([i, i + 1], 0, N - 1)))
+
+    def csr(rows):
+        rp = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
+        col = np.concatenate(rows).astype(np.int32) if rp[-1] else np.zeros(0, np.int32)
+        return oracle.CSR(rp, col, rng.uniform(0.1, 1.0, col.size).astype(np.float32), None, (N, N))
+
+    return csr(rows_phi), csr(rows_psi)
+
+
+@pytest.mark.parametrize("kind", ["dense", "local", "mixed"])
+@pytest.mark.parametrize("N,G,m,d", [(1, 3, 16, 64), (63, 40, 32, 64), (64, 1, 64, 64), (65, 700, 16, 64), (128, 5, 32, 32),
+                                     (129, 300, 64, 32), (196, 777, 64, 64), (257, 150, 32, 64), (320, 64, 16, 32),
+                                     (449, 130, 64, 64), (512, 200, 32, 64), (513, 20, 32, 64)])
+def test_small_graphs(N, G, m, d, kind):
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    rng = np.random.default_rng(N + m)
+    Phi, Psi = band_features(N, kind, rng)
+    feat = api.features_from_csr(ctx, N, N, (Phi.rowptr, Phi.col, Phi.val), (Psi.rowptr, Psi.col, Psi.val))
+    q, k, v = tensors.qkv(G, N, m, d, "bf16", 5)
+    qd, kd, vd = q.cuda() + 0.125, k.cuda() + 0.125, v.cuda()
+    B.grf_features_materialise(ctx.handle, feat.handle)
+    if d == 64:
+        out, den = api.masked_attn_mhat(ctx, feat, qd, kd, vd, want_den=True)
+    else:
+        out, den = api.masked_linear_attn(ctx, feat, qd, kd, vd, want_den=True)
+    B.grf_ctx_check(ctx.handle)
+    pick = sorted({0, G // 2, G - 1})
+    ref = oracle.attn_sparse(tensors.widen(qd[pick].cpu()), tensors.widen(kd[pick].cpu()), tensors.widen(v[pick]), Phi, oracle.transpose(Psi))
+    helpers.assert_attn_close(out[pick].float().cpu().numpy(), ref, helpers.TOL["bf16"], den[pick].cpu().numpy(), min_ok=0.0)
+    # every problem against whole states on the plain ALUs: both round to bf16 (2^-9) at most three times
+    B.grf_ctx_use_tensor_cores(ctx.handle, 0)
+    other = api.masked_linear_attn(ctx, feat, qd, kd, vd)
+    assert float((out.float() - other.float()).norm()) <= 2.0 ** -7 * float(other.float().norm())
+    empty = np.diff(Phi.rowptr) == 0
+    assert not out[:, torch.from_numpy(empty).cuda()].any() and not out.isnan().any()
+    feat.free()
+    ctx.close()
