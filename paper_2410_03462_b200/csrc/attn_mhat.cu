@@ -633,9 +633,12 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
     __shared__ int abort_flag;
     __shared__ float den_odd[BQ];                  // row sums of the odd tiles, handed to the first group
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // what the whole warp shares is read from one lane, so that the compiler keeps it (and what follows from it) in uniform registers:
+    // a tensor-pipe instruction then costs its warp a quarter of the cycles
+    auto uniform = [](int32_t x) { return __shfl_sync(0xffffffffu, x, 0); };
+    const int tid = threadIdx.x, lane = tid & 31, warp = uniform(tid >> 5);
     const int32_t g = (int32_t)(blockIdx.x % (uint32_t)G);
-    const int32_t blk = mk_cnt[nblocks + (int32_t)(blockIdx.x / (uint32_t)G)];   // blocks by decreasing key count
+    const int32_t blk = uniform(mk_cnt[nblocks + (int32_t)(blockIdx.x / (uint32_t)G)]);   // blocks by decreasing key count
     const uint32_t stage_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     unsigned char* stage_generic = smem_dyn + (stage_base - smem_u32(smem_dyn));
     const uint32_t q_base = stage_base + (uint32_t)NS * Sh::STAGE;
@@ -673,10 +676,10 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    const uint32_t tmem_base = tmem_slot;
+    const uint32_t tmem_base = (uint32_t)uniform((int32_t)tmem_slot);
 
-    const int32_t off = mk_off[blk];
-    const int32_t T = mk_cnt[blk] / KT;                   // key tiles of this block
+    const int32_t off = uniform(mk_off[blk]);
+    const int32_t T = uniform(mk_cnt[blk] / KT);                   // key tiles of this block
 
     if (warp < 8) {
         // ------------------------------------------------------------ row threads: P = S * Mhat, row sums, epilogue
@@ -724,12 +727,12 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
                 }
                 tmem_st8(s_addr + (uint32_t)(c16 * 8), pw);
             }
-            // this group's next tile: its mask values travel while the products run
-            if (t + 2 < T) load_mask(t + 2);
             tmem_st_wait();
             fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(p_full(buf));
+            // this group's next tile: its mask values travel while the products run
+            if (t + 2 < T) load_mask(t + 2);
             buf += 2;
             if (buf >= NB) { buf -= NB; par ^= 1u; }
         }
@@ -824,23 +827,28 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
         // ------------------------------------------------------------ S_t = Q K_t^T (the whole warp runs the loop in step)
         constexpr uint32_t idesc_s = instr_desc(KT, false, false);     // both operands K-major
         bool ok = true;
-        int buf = 0;
+        int buf = 0, s = 0, back = 0;                                  // back: the stage of the tile NB back
+        uint32_t par = 0u, par_back = 0u;
+        // operands by one addition each: an issuing warp's instructions count
+        const uint64_t q_op = operand_desc(q_base, BQ * 16, 128), k_op = operand_desc(stage_base + Sh::V_BYTES, KT * 16, 128);
+        const uint32_t q_hi = (uint32_t)(q_op >> 32), k_hi = (uint32_t)(k_op >> 32);
         for (int32_t t = 0; t < T; ++t) {
-            const int s = t % NS;
-            if (!__all_sync(0xffffffffu, mbar_wait(kv_full(s), (uint32_t)(t / NS) & 1u, &abort_flag))) { ok = false; break; }
+            if (!__all_sync(0xffffffffu, mbar_wait(kv_full(s), par, &abort_flag))) { ok = false; break; }
             // the score buffer is free once the second product of the tile three back, which read its P, is complete
-            if (t >= NB && !__all_sync(0xffffffffu, mbar_wait(kv_empty((t - NB) % NS), (uint32_t)((t - NB) / NS) & 1u, &abort_flag))) { ok = false; break; }
+            if (t >= NB) {
+                if (!__all_sync(0xffffffffu, mbar_wait(kv_empty(back), par_back, &abort_flag))) { ok = false; break; }
+                if (++back == NS) { back = 0; par_back ^= 1u; }
+            }
             fence_async_smem();                                        // the copies wrote through the generic proxy
             fence_after_sync();
-            const uint32_t k_st = stage_base + (uint32_t)s * Sh::STAGE + Sh::V_BYTES;
+            const uint32_t q_lo = (uint32_t)q_op, k_lo = (uint32_t)k_op + (uint32_t)(s * (Sh::STAGE / 16));
+            const uint32_t to = tmem_base + (uint32_t)(buf * Sh::S_COLS);
+            mma_bf16_ss_halves<false>(to, q_lo, q_hi, k_lo, k_hi, idesc_s);
 #pragma unroll
-            for (int k = 0; k < M / 16; ++k) {
-                const uint64_t ad = operand_desc(q_base + (uint32_t)k * 2u * (BQ * 16), BQ * 16, 128);
-                const uint64_t bd = operand_desc(k_st + (uint32_t)k * 2u * (KT * 16), KT * 16, 128);
-                mma_bf16_ss(tmem_base + (uint32_t)(buf * Sh::S_COLS), ad, bd, idesc_s, k > 0 ? 1u : 0u);
-            }
+            for (int k = 1; k < M / 16; ++k) mma_bf16_ss_halves<true>(to, q_lo + k * 2 * BQ, q_hi, k_lo + k * 2 * KT, k_hi, idesc_s);
             mma_commit(s_full(buf));
             if (++buf == NB) buf = 0;
+            if (++s == NS) { s = 0; par ^= 1u; }
         }
         if (!ok) {
             mma_commit(drain_s);
@@ -852,24 +860,24 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
         constexpr uint32_t idesc_o = instr_desc(D, false, true);       // V is MN-major (rows of d values)
         constexpr uint32_t ATOM = 8u * D * 2u;                         // eight value rows
         bool ok = true;
-        int buf = 0;
-        uint32_t par = 0u;
+        int buf = 0, s = 0;
+        uint32_t par = 0u, par_s = 0u;
+        const uint64_t v_op = swizzled_desc(stage_base, ATOM, ATOM, Sh::V_SWIZZLE);
+        const uint32_t v_hi = (uint32_t)(v_op >> 32);
         for (int32_t t = 0; t < T; ++t) {
-            const int s = t % NS;
             if (!__all_sync(0xffffffffu, mbar_wait(p_full(buf), par, &abort_flag))) { ok = false; break; }
             // (complete since the first product of this tile ran; waited on here for this thread's own view of the stage)
-            if (!__all_sync(0xffffffffu, mbar_wait(kv_full(s), (uint32_t)(t / NS) & 1u, &abort_flag))) { ok = false; break; }
+            if (!__all_sync(0xffffffffu, mbar_wait(kv_full(s), par_s, &abort_flag))) { ok = false; break; }
             fence_async_smem();
             fence_after_sync();
             const uint32_t p_op = tmem_base + (uint32_t)(buf * Sh::S_COLS);
-            const uint32_t v_st = stage_base + (uint32_t)s * Sh::STAGE;
+            const uint32_t v_lo = (uint32_t)v_op + (uint32_t)(s * (Sh::STAGE / 16)), acc = tmem_base + (uint32_t)Sh::O_COL;
+            mma_bf16_ts_halves(acc, p_op, v_lo, v_hi, idesc_o, t > 0 ? 1u : 0u);
 #pragma unroll
-            for (int ks = 0; ks < KT / 16; ++ks) {
-                const uint64_t bd = swizzled_desc(v_st + (uint32_t)ks * 2u * ATOM, ATOM, ATOM, Sh::V_SWIZZLE);
-                mma_bf16_ts(tmem_base + (uint32_t)Sh::O_COL, p_op + (uint32_t)ks * 8u, bd, idesc_o, (t > 0 || ks > 0) ? 1u : 0u);
-            }
+            for (int ks = 1; ks < KT / 16; ++ks) mma_bf16_ts_halves(acc, p_op + ks * 8, v_lo + ks * (2 * ATOM / 16), v_hi, idesc_o, 1u);
             mma_commit(kv_empty(s));                                   // frees the stage and the score buffer
             if (++buf == NB) { buf = 0; par ^= 1u; }
+            if (++s == NS) { s = 0; par_s ^= 1u; }
         }
         if (ok && T > 0) mma_commit(acc_done);
         if (!ok) {
