@@ -17,6 +17,8 @@
 // Building the mask (once per feature object): the key list of a block is the union of the rows of Psi^T over the
 // block's node list (the block plan of Phi); the values are accumulated row by row, one warp per row, in ascending
 // order of the node l, each lane owning distinct keys, so the sums are reproducible without atomics.
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace {
@@ -37,9 +39,12 @@ constexpr int KT = GRF_MASK_TILE;       // keys per tile
 // Blocks take their places in the lists by atomic additions, so the order of the blocks inside the arrays varies; nothing
 // depends on it.  A block whose part does not fit the room that the host has made writes none of it: the totals tell
 // the host how much is needed.  The last CTA to finish orders the blocks by decreasing key count.
-// One kernel for all of this, at the N = 32768 cloud: 237 us in five kernels and two prefix sums before, 178 us now (issue
+// One kernel for all of this, at the N = 32768 cloud: 237 us in five kernels and two prefix sums before, 160 us now (issue
 // slots 77 % busy while an SM has blocks, 59 % of the warps there; the blocks with the longest lists end last).
-// Grid of 196 nodes: structure and values together 56 us with 32 nodes a warp and turn whatever the list's length, 40 now.
+// Few blocks leave SMs idle, so a cluster of C CTAs builds each: they share out the nodes, merge their key bitmaps through each
+// other's shared memory, and share out list, positions and non-zeros; ranks and prefix sums are formed by each for itself (cheaper
+// than asking).  Structure and values together, us, one CTA a block / cluster: clouds of 2048 (8 CTAs) 91 / 62, 4096 (8) 124 / 89,
+// 6000 (4) 167 / 127, 9000 (4) 203 / 166, 16000 (2) 318 / 302.
 
 constexpr int MS_THREADS = 768;
 
@@ -94,7 +99,19 @@ __device__ __forceinline__ int32_t ms_ranks(const uint32_t* bits, int32_t* befor
 // groups, so that lanes which read whole neighbouring groups meet in no bank.
 __host__ __device__ __forceinline__ uint32_t mask_slot(uint32_t p) { return p ^ ((p >> 5 & 3u) << 2); }
 
-__global__ void __launch_bounds__(MS_THREADS, 2)
+// Cluster of CTAs on one block: barrier, and a word of another CTA's shared memory (the same place as `local` in this one's).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_ld(const void* local, uint32_t rank)
+{
+    uint32_t a, x;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(local)), "r"(rank));
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(x) : "r"(a) : "memory");
+    return x;
+}
+
+template <int C>
+__global__ void __launch_bounds__(MS_THREADS, 2) __cluster_dims__(C, 1, 1)
 mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restrict__ phi_rowptr, const int32_t* __restrict__ phi_col,
                       const int32_t* __restrict__ plan_off, const int32_t* __restrict__ plan_cnt,
                       const int32_t* __restrict__ plan_col, const int32_t* __restrict__ t_rowptr,
@@ -108,7 +125,8 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
     __shared__ int32_t total, last_cta;
     __shared__ unsigned long long base_keys, base_pos;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t blk = blockIdx.x, nblocks = gridDim.x;
+    const int32_t part = C > 1 ? (int32_t)(blockIdx.x % C) : 0;                 // of the block's CTAs
+    const int32_t blk = blockIdx.x / C, nblocks = gridDim.x / C;
     const int32_t wk = (Nk + 31) >> 5, wr = (R + 31) >> 5;
     uint32_t* kbits = smem_ms;
     int32_t* kbefore = reinterpret_cast<int32_t*>(smem_ms + wk);
@@ -140,11 +158,12 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
     // ---- keys
     // nodes per warp and turn, at most 32: equal shares for all warps in as few turns as it takes (with 32 each, a list of
     // 166 nodes kept 6 warps busy and one of 908 took 5 of them a second turn)
-    const int32_t turns = (ucnt + MS_THREADS - 1) / MS_THREADS;
-    const int32_t turn = min(32, ((ucnt + turns * (MS_THREADS / 32) - 1) / max(1, turns * (MS_THREADS / 32)) + 1) & ~1);
+    constexpr int32_t WARPS = C * MS_THREADS / 32;
+    const int32_t turns = (ucnt + WARPS * 32 - 1) / (WARPS * 32);
+    const int32_t turn = min(32, ((ucnt + turns * WARPS - 1) / max(1, turns * WARPS) + 1) & ~1);
     // (a node's number `of` comes with its extent, one load for 32 nodes, not with every key)
     auto each_key = [&](const int32_t* of, auto&& use) {
-        for (int32_t u0 = warp * turn; u0 < ucnt; u0 += turn * (MS_THREADS / 32)) {
+        for (int32_t u0 = (part * (MS_THREADS / 32) + warp) * turn; u0 < ucnt; u0 += turn * WARPS) {
             const int32_t n = min(turn, ucnt - u0);
             const int32_t my_l = lane < n ? __ldg(ulist + u0 + lane) : 0;
             const int32_t my_beg = lane < n ? __ldg(t_rowptr + my_l) : 0;
@@ -174,6 +193,20 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
         if (!(kbits[k >> 5] >> (k & 31) & 1u)) atomicOr(&kbits[k >> 5], 1u << (k & 31));
     });
     __syncthreads();
+    if (C > 1) {                                                // what the block's other CTAs have marked (gathered where the ranks will be)
+        cluster_arrive();
+        cluster_wait();
+        for (int32_t x = tid; x < wk; x += MS_THREADS) {
+            uint32_t b = kbits[x];
+#pragma unroll
+            for (int r = 1; r < C; ++r) b |= cluster_ld(kbits + x, (uint32_t)((part + r) % C));
+            kbefore[x] = (int32_t)b;
+        }
+        cluster_arrive();
+        cluster_wait();
+        for (int32_t x = tid; x < wk; x += MS_THREADS) kbits[x] = (uint32_t)kbefore[x];
+        __syncthreads();
+    }
     if (Nk <= GRF_MASK_SMALL) {                                 // every key of the tiles from the first to the last one reached
         if (warp == 0) {
             const uint32_t any = __ballot_sync(0xffffffffu, lane < wk && kbits[min(lane, wk - 1)] != 0u);
@@ -187,7 +220,7 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
     const int32_t keys = ms_ranks(kbits, kbefore, wk, warp_sums, &total);
     ms_ranks(nbits, nbefore, wr, warp_sums, &total);
     const int32_t padded = (keys + KT - 1) / KT * KT;
-    if (tid == 0) {
+    if (tid == 0 && part == 0) {
         base_keys = atomicAdd(&totals->entries, (unsigned long long)padded);
         base_pos = atomicAdd(&totals->positions, (unsigned long long)npos);
         atomicMax(&totals->longest, padded);
@@ -195,10 +228,22 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
         mk_off[blk] = (int32_t)base_keys;
     }
     __syncthreads();
+    if (C > 1) {                                                // the places that the first CTA has taken
+        cluster_arrive();
+        cluster_wait();
+        if (part > 0 && tid == 0) {
+            const uint32_t* keys_at = reinterpret_cast<const uint32_t*>(&base_keys);
+            const uint32_t* pos_at = reinterpret_cast<const uint32_t*>(&base_pos);
+            base_keys = cluster_ld(keys_at, 0) | (unsigned long long)cluster_ld(keys_at + 1, 0) << 32;
+            base_pos = cluster_ld(pos_at, 0) | (unsigned long long)cluster_ld(pos_at + 1, 0) << 32;
+        }
+        __syncthreads();
+        cluster_arrive();                                       // waited for at the end: no CTA leaves while another one reads it
+    }
     if ((int64_t)base_keys + padded <= key_room) {
         int32_t* list = mk_key + base_keys;
-        const int32_t per = (wk + MS_THREADS - 1) / MS_THREADS;
-        const int32_t w0 = min(wk, tid * per), w1 = min(wk, w0 + per);
+        const int32_t per = (wk + C * MS_THREADS - 1) / (C * MS_THREADS);
+        const int32_t w0 = min(wk, (part * MS_THREADS + tid) * per), w1 = min(wk, w0 + per);
         for (int32_t x = w0; x < w1; ++x) {
             uint32_t b = kbits[x];
             int32_t o = kbefore[x];
@@ -211,7 +256,7 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
             }
         }
     }
-    if (bits_out) {                             // for the kernel that looks positions up row by row
+    if (bits_out && part == 0) {                // for the kernel that looks positions up row by row
         uint32_t* dst = bits_out + (size_t)blk * 2 * wk;
         for (int32_t x = tid; x < wk; x += MS_THREADS) { dst[x] = kbits[x]; dst[wk + x] = (uint32_t)kbefore[x]; }
     }
@@ -222,7 +267,7 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
         });
         const int32_t r0 = blk * BQ, r1 = min(N, r0 + BQ);
         const int32_t end = phi_rowptr[r1];
-        for (int32_t p0 = phi_rowptr[r0] + tid; p0 < end; p0 += 4 * MS_THREADS) {
+        for (int32_t p0 = phi_rowptr[r0] + part * (4 * MS_THREADS) + tid; p0 < end; p0 += C * 4 * MS_THREADS) {
             int32_t at[4];                      // four in flight: two dependent loads each
 #pragma unroll
             for (int q = 0; q < 4; ++q) at[q] = p0 + q * MS_THREADS < end ? __ldg(phi_col + p0 + q * MS_THREADS) : -1;
@@ -236,7 +281,12 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
         }
     }
 
-    // ---- the last CTA: sizes to the host, blocks by decreasing key count (ties: lower index first) behind the counts
+    if (C > 1) {
+        __syncthreads();
+        cluster_wait();
+        if (part > 0) return;
+    }
+    // ---- the last block's first CTA: sizes to the host, blocks by decreasing key count (ties: lower index first) behind the counts
     __threadfence();
     __syncthreads();
     if (tid == 0) last_cta = atomicAdd(&totals->finished, 1) == nblocks - 1;
@@ -595,8 +645,8 @@ mask_rows_kernel(int32_t Nk, const int32_t* __restrict__ rows, const int32_t* __
 template <int M, int D> struct MhShape {
     // key/value stages in flight: two CTAs' rings then leave the SM the larger part of its L1, which serves the mask
     // values and the rows that neighbouring keys share (eight stages were 8 % slower at the point cloud, 25 % at the grid)
-    // (m = 64, d = 64, 8 problems at 32768 points: three stages 481 us, four 440, five 449; d = 32: 465, 418, 400;
-    // m = 32: four 324, five 313, six 313)
+    // (m = 64, d = 64, 8 problems at 32768 points: four stages 398 us, five 421, six 469; d = 32: 379, 369, 370;
+    // m = 32, d = 64: four 293, five 282, six 282)
     static constexpr int NS = M <= 32 || D == 32 ? 5 : 4;
     static constexpr int NB = 3;                          // score buffers
     static constexpr int V_BYTES = KT * D * 2;            // 64 value rows of 128 or 64 bytes, swizzled over that length
@@ -961,7 +1011,6 @@ static int prepare_mask_lists(grf_ctx* ctx, grf_features* feat)
     GRF_TRY(grf_buf_reserve(&K.totals, sizeof(grf_mask_totals)));
     GRF_TRY(reserve_with_headroom(&K.node_off, sizeof(int32_t) * (size_t)(feat->plan_entries > 0 ? feat->plan_entries : 1)));
     GRF_TRY(reserve_with_headroom(&K.phi_pos, sizeof(int32_t) * (size_t)(feat->phi.nnz + 1)));
-    GRF_CUDA_TRY(cudaFuncSetAttribute(mask_structure_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     K.by_position = true;
     if (!K.key.ptr) {
         // a first guess, so that the kernel need not run twice: 3 keys per node-list entry (1.8 to 2.8 were counted on clouds
@@ -978,14 +1027,25 @@ static int prepare_mask_lists(grf_ctx* ctx, grf_features* feat)
         const int64_t pos_room = K.by_position ? (int64_t)(K.pos16.bytes / sizeof(unsigned short)) : -1;
         GRF_CUDA_TRY(cudaMemsetAsync(K.totals.ptr, 0, sizeof(grf_mask_totals), ctx->stream));
         {
-            grf_launch_scope scope(ctx, 8);
-            mask_structure_kernel<<<nblocks, MS_THREADS, smem, ctx->stream>>>(
-                N, Nk, R, (const int32_t*)feat->phi.rowptr.ptr, (const int32_t*)feat->phi.col.ptr,
-                (const int32_t*)feat->plan_off.ptr, (const int32_t*)feat->plan_cnt.ptr, (const int32_t*)feat->plan_col.ptr,
-                (const int32_t*)feat->psit.rowptr.ptr, (const int32_t*)feat->psit.col.ptr, key_room, pos_room,
-                K.by_position ? nullptr : (uint32_t*)K.bits.ptr, (int32_t*)K.node_off.ptr, (int32_t*)K.off.ptr,
-                (int32_t*)K.cnt.ptr, (int32_t*)K.key.ptr, (unsigned short*)K.pos16.ptr, (int32_t*)K.phi_pos.ptr,
-                (grf_mask_totals*)K.totals.ptr, ctx->pinned + 5);
+            auto launch = [&](auto cluster) {
+                constexpr int C = decltype(cluster)::value;
+                GRF_CUDA_TRY(cudaFuncSetAttribute(mask_structure_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+                grf_launch_scope scope(ctx, 8);
+                mask_structure_kernel<C><<<nblocks * C, MS_THREADS, smem, ctx->stream>>>(
+                    N, Nk, R, (const int32_t*)feat->phi.rowptr.ptr, (const int32_t*)feat->phi.col.ptr,
+                    (const int32_t*)feat->plan_off.ptr, (const int32_t*)feat->plan_cnt.ptr, (const int32_t*)feat->plan_col.ptr,
+                    (const int32_t*)feat->psit.rowptr.ptr, (const int32_t*)feat->psit.col.ptr, key_room, pos_room,
+                    K.by_position ? nullptr : (uint32_t*)K.bits.ptr, (int32_t*)K.node_off.ptr, (int32_t*)K.off.ptr,
+                    (int32_t*)K.cnt.ptr, (int32_t*)K.key.ptr, (unsigned short*)K.pos16.ptr, (int32_t*)K.phi_pos.ptr,
+                    (grf_mask_totals*)K.totals.ptr, ctx->pinned + 5);
+                return GRF_OK;
+            };
+            // as many CTAs per block as find room at once, two on an SM
+            const int64_t room = 2 * (int64_t)ctx->sm_count / nblocks;
+            if (room >= 8) GRF_TRY(launch(std::integral_constant<int, 8>()));
+            else if (room >= 4) GRF_TRY(launch(std::integral_constant<int, 4>()));
+            else if (room >= 2) GRF_TRY(launch(std::integral_constant<int, 2>()));
+            else GRF_TRY(launch(std::integral_constant<int, 1>()));
         }
         GRF_CUDA_TRY(cudaGetLastError());
         GRF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));      // the sizes of the key lists are known only now

@@ -56,3 +56,16 @@ def test_lists_around_accumulator_segments(N):
     Psi = oracle.CSR(rp, col, rng.standard_normal(col.size).astype(np.float32), None, (N, R))
     Phi = _csr([4] * N, R, rng)
     _check(N, R, Phi, Psi, [0, 1, 127, 128, N // 2, N - 1])
+
+
+@pytest.mark.parametrize("blocks", [2, 36, 37, 38, 74, 75, 148, 149])
+def test_several_ctas_per_block(blocks):
+    """Few blocks are each built by a cluster of 8, 4 or 2 CTAs (as many as fit 148 SMs twice over): nodes with one key, a warp's and
+    several warps' shares of nodes, and a last block of one row."""
+    N = 128 * (blocks - 1) + 1
+    rng = np.random.default_rng(blocks)
+    R = N // 4 + 700
+    Psi = _csr([(1, 3, 0, 5)[i % 4] for i in range(N)], R, rng)
+    Phi = _csr([(3, 0, 9, 1, 40)[i % 5] for i in range(N)], R, rng)
+    rows = sorted({0, 1, 2, 127, 128 % N, N // 2, N // 2 + 1, N - 129 if N > 129 else 0, N - 2, N - 1})
+    _check(N, R, Phi, Psi, rows)
