@@ -59,17 +59,14 @@ template <> struct Chunk<__nv_bfloat16> {
 
 constexpr int GATHER_WARPS = 4;
 
-// Denominators: a warp per (problem, query), M / 4 lanes per node on z_l in fp32.
+// Denominator of row i of problem g, by a warp: M / 4 lanes per node on z_l in fp32.
 template <typename T, int M, int D>
-__global__ void __launch_bounds__(GATHER_WARPS * 32)
-gather_denominators_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                           const float* __restrict__ val, const T* __restrict__ phiQ,
-                           const unsigned char* __restrict__ states, float* __restrict__ den)
+__device__ __forceinline__ float row_denominator(int32_t N, int32_t R, int32_t i, int32_t g, int lane, const int32_t* __restrict__ rowptr,
+                                                 const int32_t* __restrict__ col, const float* __restrict__ val,
+                                                 const T* __restrict__ phiQ, const unsigned char* __restrict__ states)
 {
     constexpr int LPN = M / 4, NPS = 32 / LPN;          // lanes per node, nodes side by side
-    const int lane = threadIdx.x & 31, sub = lane / LPN, pl = lane % LPN;
-    const int32_t i = blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5), g = blockIdx.y;
-    if (i >= N) return;
+    const int sub = lane / LPN, pl = lane % LPN;
     const unsigned char* zbase = states + (size_t)g * grf_states_stride<T>(R, M, D) + grf_z_at<T>(true, 0, R, M, D) + (size_t)pl * 16;
     uint64_t z[2] = {0ull, 0ull};
     const int32_t beg = rowptr[i], end = rowptr[i + 1];
@@ -99,6 +96,19 @@ gather_denominators_kernel(int32_t N, int32_t R, const int32_t* __restrict__ row
     for (int e = 0; e < 4; ++e) d = fmaf(Chunk<T>::get(qrow + e), a[e], d);
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
+    return d;
+}
+
+template <typename T, int M, int D>
+__global__ void __launch_bounds__(GATHER_WARPS * 32)
+gather_denominators_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                           const float* __restrict__ val, const T* __restrict__ phiQ,
+                           const unsigned char* __restrict__ states, float* __restrict__ den)
+{
+    const int lane = threadIdx.x & 31;
+    const int32_t i = blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5), g = blockIdx.y;
+    if (i >= N) return;
+    const float d = row_denominator<T, M, D>(N, R, i, g, lane, rowptr, col, val, phiQ, states);
     if (lane == 0) den[(size_t)g * N + i] = d;
 }
 
@@ -122,11 +132,12 @@ __device__ __forceinline__ uint4 load_tile(const unsigned char* p, uint64_t poli
     return x;
 }
 
-template <typename T, int M, int D, int CPL>
+// DEN: every slice adds up the row's denominator itself, the first one writes it (few slices: see the launch).
+template <typename T, int M, int D, int CPL, bool DEN>
 __global__ void __launch_bounds__(GATHER_WARPS * 32, CPL == 1 ? 16 : 6)
 gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                      const float* __restrict__ val, const T* __restrict__ phiQ, const unsigned char* __restrict__ states,
-                     T* __restrict__ out, const float* __restrict__ den)
+                     T* __restrict__ out, float* __restrict__ den)
 {
     using Sh = SliceShape<T, M, D, CPL>;
     constexpr int CH = Sh::CH, LPN = Sh::LPN, NPS = 32 / LPN, NB = Sh::NB, KC = Sh::KC, P = Chunk<T>::PAIRS;
@@ -135,6 +146,11 @@ gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, c
     const int32_t i = blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5);
     const int32_t slice = blockIdx.y, g = blockIdx.z;
     if (i >= N) return;
+    float dn = 0.0f;
+    if (DEN) {
+        dn = row_denominator<T, M, D>(N, R, i, g, lane, rowptr, col, val, phiQ, states);
+        if (den && slice == 0 && lane == 0) den[(size_t)g * N + i] = dn;
+    }
     const int b0 = slice * Sh::COLS + b;
     // this lane's first chunk; chunk y lies y * SB columns further on: LPN consecutive chunks per group of lanes
     const unsigned char* base = states + (size_t)g * grf_states_stride<T>(R, M, D) + grf_chunk_at<T>(true, 0, kc * CH, b0, M, D);
@@ -179,7 +195,7 @@ gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, c
     }
     // contract with phi(q): over this lane's rows a, then over the lanes along a and the nodes side by side
     const T* qrow = phiQ + ((size_t)g * N + i) * M;
-    const float dn = den[(size_t)g * N + i];
+    if (!DEN) dn = den[(size_t)g * N + i];
     float s[NB];
     uint64_t qv[P];
     Chunk<T>::widen(__ldg(reinterpret_cast<const uint4*>(qrow + kc * CH)), qv);
@@ -212,32 +228,44 @@ gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, c
 // 76 ms, 128 bytes 1.75, 3.03, 10.3, 19.0, 40.6, 88.)
 constexpr size_t SLICE_L2_BYTES = (size_t)72 << 20;
 
+constexpr int64_t DEN_INSIDE_ROWS = 2048;
+
 template <typename T, int M, int D>
 int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, const void* phiQ, const void* states, void* out,
               float* den_out)
 {
+    const int32_t* rp = (const int32_t*)phi.rowptr.ptr;
+    const int32_t* cl = (const int32_t*)phi.col.ptr;
+    const float* vl = (const float*)phi.val.ptr;
+    const int blocks = grf_ceil_div(N, GATHER_WARPS);
+    auto launch = [&](auto cpl, auto with_den, float* den) {
+        using Sh = SliceShape<T, M, D, decltype(cpl)::value>;
+        grf_launch_scope scope(ctx, 5);
+        gather_sliced_kernel<T, M, D, decltype(cpl)::value, decltype(with_den)::value><<<dim3(blocks, Sh::SLICES, G), GATHER_WARPS * 32, 0, ctx->stream>>>(
+            N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, (T*)out, den);
+    };
+    const bool wide = (size_t)phi.cols * 2048 <= SLICE_L2_BYTES;
+    // Small calls form the denominators inside, once more for each of up to four slices: what a launch costs is more than that.
+    // us measured, whole attention, separate / inside: fp32 lattice of 64 nodes, m = d = 16 23.0 / 18.0, of 400, 4 problems, m = 32,
+    // d = 64 35.1 / 29.6, bf16 30.6 / 25.3; cloud of 1024, fp32 68.0 / 66.7, of 3000, m = 16 110.2 / 111.7.
+    if constexpr (SliceShape<T, M, D, 4>::SLICES <= 4) {
+        if (wide && (int64_t)G * N <= DEN_INSIDE_ROWS) {
+            launch(std::integral_constant<int, 4>(), std::true_type(), den_out);
+            return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
+        }
+    }
     float* den = den_out;
     if (!den) {
         GRF_TRY(grf_buf_reserve(&ctx->den_scratch, sizeof(float) * (size_t)G * N));
         den = (float*)ctx->den_scratch.ptr;
     }
-    const int32_t* rp = (const int32_t*)phi.rowptr.ptr;
-    const int32_t* cl = (const int32_t*)phi.col.ptr;
-    const float* vl = (const float*)phi.val.ptr;
-    const int blocks = grf_ceil_div(N, GATHER_WARPS);
     {
         grf_launch_scope scope(ctx, 6);
         gather_denominators_kernel<T, M, D><<<dim3(blocks, G), GATHER_WARPS * 32, 0, ctx->stream>>>(
             N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, den);
     }
-    grf_launch_scope scope(ctx, 5);
-    auto launch = [&](auto cpl) {
-        using Sh = SliceShape<T, M, D, decltype(cpl)::value>;
-        gather_sliced_kernel<T, M, D, decltype(cpl)::value><<<dim3(blocks, Sh::SLICES, G), GATHER_WARPS * 32, 0, ctx->stream>>>(
-            N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, (T*)out, den);
-    };
-    if ((size_t)phi.cols * 2048 <= SLICE_L2_BYTES) launch(std::integral_constant<int, 4>());
-    else launch(std::integral_constant<int, 1>());
+    if (wide) launch(std::integral_constant<int, 4>(), std::false_type(), den);
+    else launch(std::integral_constant<int, 1>(), std::false_type(), den);
     return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
 }
 
