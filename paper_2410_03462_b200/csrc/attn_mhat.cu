@@ -41,10 +41,10 @@ constexpr int KT = GRF_MASK_TILE;       // keys per tile
 // the host how much is needed.  The last CTA to finish orders the blocks by decreasing key count.
 // One kernel for all of this, at the N = 32768 cloud: 237 us in five kernels and two prefix sums before, 160 us now (issue
 // slots 77 % busy while an SM has blocks, 59 % of the warps there; the blocks with the longest lists end last).
-// Few blocks leave SMs idle, so a cluster of C CTAs builds each: they share out the nodes, merge their key bitmaps through each
+// A cluster of C CTAs builds each block (one CTA a block leaves SMs idle where there are few): they share out the nodes, merge their key bitmaps through each
 // other's shared memory, and share out list, positions and non-zeros; ranks and prefix sums are formed by each for itself (cheaper
 // than asking).  Structure and values together, us, one CTA a block / cluster: clouds of 2048 (8 CTAs) 91 / 62, 4096 (8) 124 / 89,
-// 6000 (4) 167 / 127, 9000 (4) 203 / 166, 16000 (2) 318 / 302.
+// 6000 (4) 167 / 127, 9000 (4) 203 / 166, 22000 (2) 419 / 393.
 
 constexpr int MS_THREADS = 768;
 
@@ -125,7 +125,7 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
     __shared__ int32_t total, last_cta;
     __shared__ unsigned long long base_keys, base_pos;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t part = C > 1 ? (int32_t)(blockIdx.x % C) : 0;                 // of the block's CTAs
+    const int32_t part = (int32_t)(blockIdx.x % C);                             // of the block's CTAs
     const int32_t blk = blockIdx.x / C, nblocks = gridDim.x / C;
     const int32_t wk = (Nk + 31) >> 5, wr = (R + 31) >> 5;
     uint32_t* kbits = smem_ms;
@@ -193,7 +193,7 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
         if (!(kbits[k >> 5] >> (k & 31) & 1u)) atomicOr(&kbits[k >> 5], 1u << (k & 31));
     });
     __syncthreads();
-    if (C > 1) {                                                // what the block's other CTAs have marked (gathered where the ranks will be)
+    {                                                           // what the block's other CTAs have marked (gathered where the ranks will be)
         cluster_arrive();
         cluster_wait();
         for (int32_t x = tid; x < wk; x += MS_THREADS) {
@@ -228,7 +228,7 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
         mk_off[blk] = (int32_t)base_keys;
     }
     __syncthreads();
-    if (C > 1) {                                                // the places that the first CTA has taken
+    {                                                           // the places that the first CTA has taken
         cluster_arrive();
         cluster_wait();
         if (part > 0 && tid == 0) {
@@ -281,11 +281,9 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
         }
     }
 
-    if (C > 1) {
-        __syncthreads();
-        cluster_wait();
-        if (part > 0) return;
-    }
+    __syncthreads();
+    cluster_wait();
+    if (part > 0) return;
     // ---- the last block's first CTA: sizes to the host, blocks by decreasing key count (ties: lower index first) behind the counts
     __threadfence();
     __syncthreads();
@@ -1040,12 +1038,13 @@ static int prepare_mask_lists(grf_ctx* ctx, grf_features* feat)
                     (grf_mask_totals*)K.totals.ptr, ctx->pinned + 5);
                 return GRF_OK;
             };
-            // as many CTAs per block as find room at once, two on an SM
+            // about as many CTAs per block as find room at once, two on an SM; two also where a block finds room for one only, as
+            // the halves fill the SMs more evenly.  Structure and values, us, with 1 / 2 / 4 / 8 CTAs a block: clouds of 9000 points
+            // 203 / - / 165 / 178, 14000 - / 257 / 250 / -, 22000 419 / 393 / 396 / -, 32768 575 / 565 / 582 / -, 60000 1092 / 1091 / 1090
             const int64_t room = 2 * (int64_t)ctx->sm_count / nblocks;
             if (room >= 8) GRF_TRY(launch(std::integral_constant<int, 8>()));
-            else if (room >= 4) GRF_TRY(launch(std::integral_constant<int, 4>()));
-            else if (room >= 2) GRF_TRY(launch(std::integral_constant<int, 2>()));
-            else GRF_TRY(launch(std::integral_constant<int, 1>()));
+            else if (room >= 2) GRF_TRY(launch(std::integral_constant<int, 4>()));
+            else GRF_TRY(launch(std::integral_constant<int, 2>()));
         }
         GRF_CUDA_TRY(cudaGetLastError());
         GRF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));      // the sizes of the key lists are known only now

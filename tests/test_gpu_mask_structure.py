@@ -60,7 +60,7 @@ def test_lists_around_accumulator_segments(N):
 
 @pytest.mark.parametrize("blocks", [2, 36, 37, 38, 74, 75, 148, 149])
 def test_several_ctas_per_block(blocks):
-    """Few blocks are each built by a cluster of 8, 4 or 2 CTAs (as many as fit 148 SMs twice over): nodes with one key, a warp's and
+    """A block is built by a cluster of 8, 4 or 2 CTAs, by the number of blocks: nodes with one key, a warp's and
     several warps' shares of nodes, and a last block of one row."""
     N = 128 * (blocks - 1) + 1
     rng = np.random.default_rng(blocks)
