@@ -634,8 +634,9 @@ mask_rows_kernel(int32_t Nk, const int32_t* __restrict__ rows, const int32_t* __
 //   warp 8          issues S_t = Q K_t^T into one of three score buffers
 //   warp 9          issues O += P_t V_t once the rows of tile t are masked, and frees the tile's stage and buffer
 //   warps 10-13     producers: a quarter of every tile's key-feature and value rows each, by 16-byte async copies
-// An instruction of the tensor pipe costs its issuing thread about fifty cycles, whatever its size, so the two
-// products have a thread each; three score buffers let the first product run two tiles ahead of the masking.
+// An instruction of the tensor pipe costs its issuing warp 25 cycles with operands in uniform registers (100 with operands that
+// the compiler takes for per-thread: 306 us instead of 282 on the N = 32768 cloud), so the two products have a warp each; three
+// score buffers let the first product run two tiles ahead of the masking.
 // (A round trip to tensor memory is about 230 cycles and the hand-overs add several hundred per tile: what bounds
 // the kernel is the length of that chain, not a pipe.)
 
