@@ -39,10 +39,23 @@ pair_ranks_kernel(int64_t nnz, const int32_t* __restrict__ col, int32_t* __restr
     }
 }
 
+// The first blocks take a row of Phi per warp, the others a node per thread: nodes with more than `limit` keys and queries are
+// listed for the kernels of long nodes (below), in any order, those with more than `huge` from the list's end.
 __global__ void __launch_bounds__(256)
-pair_slots_kernel(int32_t N, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                  const int32_t* __restrict__ start, int32_t* __restrict__ slot, int32_t* __restrict__ query)
+pair_slots_kernel(int32_t N, int32_t R, int32_t row_blocks, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                  const int32_t* __restrict__ start, const int32_t* __restrict__ t_rowptr, int32_t limit, int32_t huge,
+                  int32_t* __restrict__ slot, int32_t* __restrict__ query, int32_t* __restrict__ long_count,
+                  int32_t* __restrict__ long_nodes)
 {
+    if ((int32_t)blockIdx.x >= row_blocks) {
+        const int32_t l = ((int32_t)blockIdx.x - row_blocks) * 256 + (int32_t)threadIdx.x;
+        if (l >= R) return;
+        const int32_t nq = start[l + 1] - start[l], nk = t_rowptr[l + 1] - t_rowptr[l];
+        if (nq == 0 || nk <= limit - nq) return;
+        if (nk > huge - nq) long_nodes[R - 1 - atomicAdd(long_count + 1, 1)] = l;
+        else long_nodes[atomicAdd(long_count, 1)] = l;
+        return;
+    }
     const int lane = threadIdx.x & 31;
     const int32_t i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (i >= N) return;
@@ -137,10 +150,127 @@ struct PairArgs {
     int32_t width;                          // columns of a record: columns col0 .. col0 + width - 1 of V
     int32_t col0;
     int32_t slices;                         // of DS columns each, side by side in a record
+    int32_t long_limit;                     // keys and queries of a node beyond which it is one of the long ones
+    int32_t items;                          // problems times slices
+    const int32_t *long_count, *long_nodes; // long ones and very long ones; their nodes from the front and from the end (R places)
 };
 
+// Long nodes.  A node is one warp's work, at 0.7 us a chunk (bf16) once the other warps of its SM have finished: a hub that all
+// 2^15 nodes of an expander visit kept its warp busy for 1.4 ms a problem where all other nodes take 0.14.  So a node with many
+// keys and queries is the work of a CTA, one with very many that of a cluster: the warps share its keys, add their parts of S and z
+// up in shared memory (a CTA's warps first, then the CTAs), and share its queries.  The shares depend on the node alone, so the
+// bits do not depend on the batch or the workspace.
+// Whole attention, us, whole states / one warp a node / this: expanders with a hub, 4 problems, m = 32, d = 64, bf16: 2^15 nodes
+// 2099 / 6060 / 1224 (eight hubs 3272 / 6910 / 1302), 2^17 9380 / 26400 / 4697; 2 problems, 2^13 321 / 489 / 176; graph grown by
+// preferential attachment, 2^15 2254 / 1804 / 1416, 2^17 10146 / 6365 / 5092; fp32, 3 problems: 5003 1161 / 1435 / 349, 2^15 10813 /
+// 25422 / 2436.
+constexpr int PAIR_WARPS = 8, PAIR_CLUSTER = 8;
+// Keys and queries of a node beyond which it is long: 512 (a warp then needs as long as the launches of a small batch take), or
+// twice what a warp has to do on average where that is more.  Few nodes: warps go without work, so the average does not matter.
+// Beyond PAIR_HUGE it is a cluster's: that is 32 chunks for each warp of a CTA, at 1.2 us with eight warps on an SM.
+constexpr int PAIR_HUGE = 8192;
+int32_t pair_long_limit(int64_t entries, int32_t R)
+{
+    const int64_t twice = R < 512 ? 0 : 2 * entries / (R < 16384 ? R : 16384);
+    return (int32_t)(twice > 512 ? twice : 512);
+}
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float cluster_ld(const float* local, uint32_t rank)
+{
+    uint32_t a;
+    float x;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(local)), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(a) : "memory");
+    return x;
+}
+
+// the share of n rows, in whole chunks, that a warp of `ctas` CTAs has
+__device__ __forceinline__ void pair_share(int32_t& first, int32_t& n, int32_t ctas, int chunk)
+{
+    const int32_t warps = ctas * PAIR_WARPS, who = (ctas > 1 ? (int32_t)cluster_rank() * PAIR_WARPS : 0) + (int32_t)(threadIdx.x >> 5);
+    const int32_t per = ((n + warps - 1) / warps + chunk - 1) / chunk * chunk;
+    const int32_t skip = min((int64_t)n, (int64_t)who * per);
+    first += skip;
+    n = min(per, n - skip);
+}
+
+// Sums COUNT values per lane over the warps of a CTA or of the cluster's CTAs, in their order; all receive them.  `area` is the
+// first warp's room of `stride` floats, the others' follow; a warp may write to its own again afterwards.  (value(i) names value
+// i: unrolled, so that values stay in registers)
+template <int COUNT, typename Value>
+__device__ __forceinline__ void pair_add_up(float* area, int stride, int32_t ctas, Value&& value)
+{
+    constexpr int EACH = (COUNT + PAIR_WARPS - 1) / PAIR_WARPS;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float* own = area + (size_t)warp * stride + lane;
+#pragma unroll
+    for (int i = 0; i < COUNT; ++i) own[i * 32] = value(i);
+    __syncthreads();
+    float sum[EACH];
+#pragma unroll
+    for (int e = 0; e < EACH; ++e) {
+        const int at = min(e * PAIR_WARPS + warp, COUNT - 1) * 32 + lane;
+        sum[e] = area[at];
+#pragma unroll
+        for (int w = 1; w < PAIR_WARPS; ++w) sum[e] += area[(size_t)w * stride + at];
+    }
+    __syncthreads();
+    auto spread = [&]() {
+#pragma unroll
+        for (int e = 0; e < EACH; ++e)
+            if (e * PAIR_WARPS + warp < COUNT) area[(e * PAIR_WARPS + warp) * 32 + lane] = sum[e];
+    };
+    spread();
+    if (ctas > 1) {
+        cluster_sync();
+#pragma unroll
+        for (int e = 0; e < EACH; ++e) {
+            const int at = min(e * PAIR_WARPS + warp, COUNT - 1) * 32 + lane;
+            sum[e] = 0.0f;
+            for (int32_t r = 0; r < ctas; ++r) sum[e] += cluster_ld(area + at, (uint32_t)r);
+        }
+        cluster_sync();
+        spread();
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < COUNT; ++i) value(i) = area[i * 32 + lane];
+    __syncthreads();
+}
+
+// The long nodes' kernels: clusters take the very long ones, then every CTA for itself the others, all in turn.  They need nothing
+// of the kernel for the other nodes, so they may start as soon as that one's last CTAs have (it says so by pair_let_next_start);
+// before they end they wait for it to be complete, so that what follows finds all records.  Without long nodes this kernel costs a
+// launch 1.2 us (4.5 when it starts behind the other one: fp32 cloud of 5003, 3 problems, 509.7 -> 511.1 and 514.2).
+__device__ __forceinline__ void pair_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename Node>
+__device__ __forceinline__ void pair_long_nodes(const PairArgs& A, Node&& node)
+{
+    const int64_t huge = (int64_t)__ldg(A.long_count + 1) * A.items, end = (int64_t)__ldg(A.long_count) * A.items;
+    for (int64_t x = blockIdx.x / PAIR_CLUSTER; x < huge; x += gridDim.x / PAIR_CLUSTER) {
+        node(__ldg(A.long_nodes + (A.R - 1 - x / A.items)), (int32_t)(x % A.items), PAIR_CLUSTER);
+        __syncthreads();
+    }
+    for (int64_t x = blockIdx.x; x < end; x += gridDim.x) {
+        node(__ldg(A.long_nodes + x / A.items), (int32_t)(x % A.items), 1);
+        __syncthreads();
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------------------------------
-// bf16.  A warp takes a node and problem by itself.  Keys and queries come in chunks of 32 rows through a ring of two slots
+// bf16.  A warp takes a node and problem by itself (the long ones' kernel: all warps of a CTA).  Keys and queries come in chunks of 32 rows through a ring of two slots
 // (the next chunk's copies are under way while one is used; three slots and twelve warps an SM instead of sixteen: 678 us against
 // 621 at 2^15 nodes, 4 problems).
 //   keys      S^T (DS columns b x M features a) += V^T (b x keys) . (Psi phi(K)) (keys x a): both operands by transposing
@@ -163,20 +293,22 @@ template <int M, int DS> struct PairShape {
     static constexpr int CTAS = 4;
 };
 
-template <int M, int DS>
-__global__ void __launch_bounds__(PairShape<M, DS>::WARPS * 32, PairShape<M, DS>::CTAS)
-pair_records_bf16_kernel(const __grid_constant__ PairArgs A)
+// TOGETHER: by all warps of `ctas` CTAs
+template <int M, int DS, bool TOGETHER>
+__device__ __forceinline__ void pair_node_bf16(const PairArgs& A, int32_t l, int32_t item, unsigned char* smem_pairs, int32_t ctas = 1)
 {
     using Sh = PairShape<M, DS>;
     constexpr int BT = DS / 16, AT = M / 8;                     // 16-column tiles of V, 8-feature tiles
-    extern __shared__ __align__(128) unsigned char smem_pairs[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int32_t l = blockIdx.x * Sh::WARPS + warp;
-    if (l >= A.R) return;
-    const int32_t slice = blockIdx.y % A.slices, g = blockIdx.y / A.slices;
-    const int32_t q_beg = __ldg(A.start + l), nq = __ldg(A.start + l + 1) - q_beg;
-    if (nq == 0) return;
-    const int32_t k_beg = __ldg(A.t_rowptr + l), nk = __ldg(A.t_rowptr + l + 1) - k_beg;
+    const int32_t slice = item % A.slices, g = item / A.slices;
+    int32_t q_beg = __ldg(A.start + l), nq = __ldg(A.start + l + 1) - q_beg;
+    if (!TOGETHER && nq == 0) return;
+    int32_t k_beg = __ldg(A.t_rowptr + l), nk = __ldg(A.t_rowptr + l + 1) - k_beg;
+    if (!TOGETHER && nk > A.long_limit - nq) return;
+    if (TOGETHER) {
+        pair_share(k_beg, nk, ctas, PB_CHUNK);
+        pair_share(q_beg, nq, ctas, PB_CHUNK);
+    }
     const int32_t c0 = A.col0 + slice * DS;
     const bool with_den = c0 == 0;
     const __nv_bfloat16* Kg = (const __nv_bfloat16*)A.phiK + (size_t)g * A.N * M;
@@ -257,7 +389,7 @@ pair_records_bf16_kernel(const __grid_constant__ PairArgs A)
         }
 
     fetch_rows(0);
-    issue(0, 0);
+    if (!TOGETHER || kc > 0) issue(0, 0);
     const int mi = lane >> 3, mr = lane & 7, fq = lane & 3, fr = lane >> 2;     // ldmatrix: matrix, row; fragment: quarter, row
     // this lane's row in the three kinds of ldmatrix: keys (8-key halves, then features), values (columns, then keys), queries
     const uint32_t k_lane = (uint32_t)(((mi & 1) * 8 + mr) * Sh::KROW + (((mi >> 1) ^ piece_turn<Sh::KROW>(mr)) << 4));
@@ -266,7 +398,7 @@ pair_records_bf16_kernel(const __grid_constant__ PairArgs A)
     for (int32_t c = 0; c < kc; ++c) {
         copy_wait<0>();
         __syncwarp();
-        issue(c + 1, slot ^ 1);                 // the slot that chunk c - 1 has left
+        if (!TOGETHER || c + 1 < kc) issue(c + 1, slot ^ 1);    // the slot that chunk c - 1 has left
         const uint32_t kbase = ring_addr + (uint32_t)slot * Sh::SLOT, vbase = kbase + PB_CHUNK * Sh::KROW;
         const int32_t n = min(PB_CHUNK, nk - c * PB_CHUNK);
 #pragma unroll
@@ -298,6 +430,15 @@ pair_records_bf16_kernel(const __grid_constant__ PairArgs A)
             }
         }
         slot ^= 1;
+    }
+    if (TOGETHER) {                             // in place of the ring, which holds nothing now
+        constexpr int SV = BT * AT * 4, ZV = AT * 2;
+        static_assert((SV + ZV) * 128 <= Sh::WARP_BYTES, "parts of S and z");
+        __syncwarp();
+        pair_add_up<SV + ZV>(reinterpret_cast<float*>(smem_pairs), Sh::WARP_BYTES / 4, ctas, [&](int i) -> float& {
+            return i < SV ? S[i / (AT * 4)][i / 4 % AT][i % 4] : z[(i - SV) / 2][i % 2];
+        });
+        issue(kc, slot);
     }
 
     // S in the second product's operand layout; z's three columns
@@ -373,6 +514,26 @@ pair_records_bf16_kernel(const __grid_constant__ PairArgs A)
     copy_wait<0>();
 }
 
+template <int M, int DS>
+__global__ void __launch_bounds__(PairShape<M, DS>::WARPS * 32, PairShape<M, DS>::CTAS)
+pair_records_bf16_kernel(const __grid_constant__ PairArgs A)
+{
+    extern __shared__ __align__(128) unsigned char smem_pairs[];
+    pair_let_next_start();
+    const int32_t l = blockIdx.x * PairShape<M, DS>::WARPS + (threadIdx.x >> 5);
+    if (l < A.R) pair_node_bf16<M, DS, false>(A, l, blockIdx.y, smem_pairs);
+}
+
+template <int M, int DS>
+__global__ void __launch_bounds__(PAIR_WARPS * 32, 2) __cluster_dims__(PAIR_CLUSTER, 1, 1)
+pair_long_bf16_kernel(const __grid_constant__ PairArgs A)
+{
+    extern __shared__ __align__(128) unsigned char smem_pairs[];
+    pair_long_nodes(A, [&](int32_t l, int32_t item, int32_t ctas) {
+        pair_node_bf16<M, DS, true>(A, l, item, smem_pairs, ctas);
+    });
+}
+
 // ---------------------------------------------------------------------------------------------------
 // fp32.  The same walk over a node's keys and queries on the plain ALUs, chunks of 8 keys or 16 queries.  The 32 lanes are 4
 // groups along the features times 8 along the columns; a lane keeps M / 4 x DS / 8 sums of S in registers and multiplies with
@@ -386,6 +547,8 @@ template <int M, int DS> struct PairShapeF {
     static constexpr int SLOT = KEY_FLOATS > QUERY_FLOATS ? KEY_FLOATS : QUERY_FLOATS;
     static constexpr int S_FLOATS = M;                          // z, for the queries
     static constexpr int WARP_FLOATS = PF_RING * (SLOT + PF_KEYS) + S_FLOATS;
+    static constexpr int PART_FLOATS = M * DS + (M + 31) / 32 * 32;                     // a warp's part of S and z, for long nodes
+    static constexpr int LONG_FLOATS = WARP_FLOATS > PART_FLOATS ? WARP_FLOATS : PART_FLOATS;
     static constexpr int WARPS = 2;
     static constexpr int FIT = 227 * 1024 / (WARPS * WARP_FLOATS * 4 + 1024), CTAS = FIT < 6 ? FIT : 6;
 };
@@ -395,28 +558,30 @@ template <int M> __device__ __forceinline__ int query_at(int r, int p)
     return r * M + ((p ^ (r & (M / 4 - 1))) << 2);
 }
 
-template <int M, int DS>
-__global__ void __launch_bounds__(PairShapeF<M, DS>::WARPS * 32, PairShapeF<M, DS>::CTAS)
-pair_records_f32_kernel(const __grid_constant__ PairArgs A)
+template <int M, int DS, bool TOGETHER>
+__device__ __forceinline__ void pair_node_f32(const PairArgs& A, int32_t l, int32_t item, float* smem_pairs, int32_t ctas = 1)
 {
     using Sh = PairShapeF<M, DS>;
     constexpr int MA = M / 4, NB = DS / 8;                      // features and columns of a lane
     constexpr int NQ = NB / 4;                                  // 16-byte pieces of its columns: 4 x at 32 y + 4 bg
     static_assert(NB % 4 == 0 && MA % 4 == 0, "whole pieces");
-    extern __shared__ __align__(128) unsigned char smem_pairs[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int32_t l = blockIdx.x * Sh::WARPS + warp;
-    if (l >= A.R) return;
-    const int32_t slice = blockIdx.y % A.slices, g = blockIdx.y / A.slices;
-    const int32_t q_beg = __ldg(A.start + l), nq = __ldg(A.start + l + 1) - q_beg;
-    if (nq == 0) return;
-    const int32_t k_beg = __ldg(A.t_rowptr + l), nk = __ldg(A.t_rowptr + l + 1) - k_beg;
+    const int32_t slice = item % A.slices, g = item / A.slices;
+    int32_t q_beg = __ldg(A.start + l), nq = __ldg(A.start + l + 1) - q_beg;
+    if (!TOGETHER && nq == 0) return;
+    int32_t k_beg = __ldg(A.t_rowptr + l), nk = __ldg(A.t_rowptr + l + 1) - k_beg;
+    if (!TOGETHER && nk > A.long_limit - nq) return;
+    if (TOGETHER) {
+        pair_share(k_beg, nk, ctas, PF_KEYS);
+        pair_share(q_beg, nq, ctas, PF_QUERIES);
+    }
     const int32_t c0 = A.col0 + slice * DS;
     const bool with_den = c0 == 0;
     const float* Kg = (const float*)A.phiK + (size_t)g * A.N * M;
     const float* Vg = (const float*)A.V + (size_t)g * A.N * A.d + c0;
     const float* Qg = (const float*)A.phiQ + (size_t)g * A.N * M;
-    float* ring = reinterpret_cast<float*>(smem_pairs) + (size_t)warp * Sh::WARP_FLOATS;
+    constexpr int STRIDE = TOGETHER ? Sh::LONG_FLOATS : Sh::WARP_FLOATS;
+    float* ring = smem_pairs + (size_t)warp * STRIDE;
     float* psi_ring = ring + PF_RING * Sh::SLOT;
     float* z_tile = psi_ring + PF_RING * PF_KEYS;
 
@@ -479,12 +644,12 @@ pair_records_f32_kernel(const __grid_constant__ PairArgs A)
     for (int y = 0; y < ZL; ++y) z[y] = 0.0f;
 
     fetch_rows(0);
-    issue(0, 0);
+    if (!TOGETHER || kc > 0) issue(0, 0);
     int slot = 0;
     for (int32_t c = 0; c < kc; ++c) {
         copy_wait<0>();
         __syncwarp();
-        issue(c + 1, slot ^ 1);
+        if (!TOGETHER || c + 1 < kc) issue(c + 1, slot ^ 1);
         float* kt = ring + slot * Sh::SLOT;
         const float* vt = kt + PF_KEYS * M;
         const int32_t n4 = min(PF_KEYS, (nk - c * PF_KEYS + 3) & ~3);
@@ -524,6 +689,26 @@ pair_records_f32_kernel(const __grid_constant__ PairArgs A)
             }
         }
         slot ^= 1;
+    }
+    if (TOGETHER) {
+        constexpr int SV = MA * NB;
+        static_assert((SV + ZL) * 32 <= Sh::LONG_FLOATS, "parts of S and z");
+        float part[SV + ZL];
+#pragma unroll
+        for (int i = 0; i < SV; i += 2) {
+            const float2 x = unpack2(S[i / NB][i % NB / 2]);
+            part[i] = x.x;
+            part[i + 1] = x.y;
+        }
+#pragma unroll
+        for (int y = 0; y < ZL; ++y) part[SV + y] = z[y];
+        __syncwarp();
+        pair_add_up<SV + ZL>(smem_pairs, STRIDE, ctas, [&](int i) -> float& { return part[i]; });
+#pragma unroll
+        for (int i = 0; i < SV; i += 2) S[i / NB][i % NB / 2] = pack2(part[i], part[i + 1]);
+#pragma unroll
+        for (int y = 0; y < ZL; ++y) z[y] = part[SV + y];
+        issue(kc, slot);
     }
 #pragma unroll
     for (int y = 0; y < ZL; ++y)
@@ -593,6 +778,26 @@ pair_records_f32_kernel(const __grid_constant__ PairArgs A)
         slot ^= 1;
     }
     copy_wait<0>();
+}
+
+template <int M, int DS>
+__global__ void __launch_bounds__(PairShapeF<M, DS>::WARPS * 32, PairShapeF<M, DS>::CTAS)
+pair_records_f32_kernel(const __grid_constant__ PairArgs A)
+{
+    extern __shared__ __align__(128) unsigned char smem_pairs[];
+    pair_let_next_start();
+    const int32_t l = blockIdx.x * PairShapeF<M, DS>::WARPS + (threadIdx.x >> 5);
+    if (l < A.R) pair_node_f32<M, DS, false>(A, l, blockIdx.y, reinterpret_cast<float*>(smem_pairs));
+}
+
+template <int M, int DS>
+__global__ void __launch_bounds__(PAIR_WARPS * 32, 1) __cluster_dims__(PAIR_CLUSTER, 1, 1)
+pair_long_f32_kernel(const __grid_constant__ PairArgs A)
+{
+    extern __shared__ __align__(128) unsigned char smem_pairs[];
+    pair_long_nodes(A, [&](int32_t l, int32_t item, int32_t ctas) {
+        pair_node_f32<M, DS, true>(A, l, item, reinterpret_cast<float*>(smem_pairs), ctas);
+    });
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -698,24 +903,36 @@ pair_sums_kernel(int32_t N, int32_t d, int32_t col0, int64_t nnz, const int32_t*
 }
 
 template <int M, int DS>
-int launch_records(grf_ctx* ctx, const PairArgs& A, int32_t G, bool bf16)
+int launch_records(grf_ctx* ctx, const PairArgs& A, bool bf16)
 {
+    auto launch = [&](auto kernel, auto long_kernel, int warps, size_t warp_bytes, size_t long_bytes, int long_ctas) {
+        GRF_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(warps * warp_bytes)));
+        GRF_CUDA_TRY(cudaFuncSetAttribute(long_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(PAIR_WARPS * long_bytes)));
+        kernel<<<dim3(grf_ceil_div(A.R, warps), A.items), warps * 32, warps * warp_bytes, ctx->stream>>>(A);
+        const int ctas = ctx->sm_count * long_ctas / PAIR_CLUSTER * PAIR_CLUSTER;
+        cudaLaunchAttribute beside = {};
+        beside.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        beside.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t config = {};
+        config.gridDim = dim3(ctas > 0 ? ctas : PAIR_CLUSTER);
+        config.blockDim = dim3(PAIR_WARPS * 32);
+        config.dynamicSmemBytes = PAIR_WARPS * long_bytes;
+        config.stream = ctx->stream;
+        config.attrs = &beside;
+        config.numAttrs = 1;
+        GRF_CUDA_TRY(cudaLaunchKernelEx(&config, long_kernel, A));
+        return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
+    };
     if (bf16) {
         using Sh = PairShape<M, DS>;
-        const size_t smem = (size_t)Sh::WARPS * Sh::WARP_BYTES;
-        GRF_CUDA_TRY(cudaFuncSetAttribute(pair_records_bf16_kernel<M, DS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        pair_records_bf16_kernel<M, DS><<<dim3(grf_ceil_div(A.R, Sh::WARPS), G * A.slices), Sh::WARPS * 32, smem, ctx->stream>>>(A);
-    } else {
-        if constexpr (DS >= 32) {
-            using Sh = PairShapeF<M, DS>;
-            const size_t smem = (size_t)Sh::WARPS * Sh::WARP_FLOATS * sizeof(float);
-            GRF_CUDA_TRY(cudaFuncSetAttribute(pair_records_f32_kernel<M, DS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            pair_records_f32_kernel<M, DS><<<dim3(grf_ceil_div(A.R, Sh::WARPS), G * A.slices), Sh::WARPS * 32, smem, ctx->stream>>>(A);
-        } else {
-            return GRF_ERR_INVALID;
-        }
+        return launch(pair_records_bf16_kernel<M, DS>, pair_long_bf16_kernel<M, DS>, Sh::WARPS, Sh::WARP_BYTES, Sh::WARP_BYTES, 2);
     }
-    return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
+    if constexpr (DS >= 32) {
+        using Sh = PairShapeF<M, DS>;
+        return launch(pair_records_f32_kernel<M, DS>, pair_long_f32_kernel<M, DS>, Sh::WARPS, Sh::WARP_FLOATS * sizeof(float),
+                      Sh::LONG_FLOATS * sizeof(float), 1);
+    }
+    return GRF_ERR_INVALID;
 }
 
 template <int M>
@@ -724,11 +941,12 @@ int launch_records_m(grf_ctx* ctx, PairArgs& A, int32_t G, bool bf16)
     // M x DS sums are held in registers: at most 2048 a warp
     const int32_t ds = M == 64 && A.width > 32 ? 32 : A.width;
     A.slices = A.width / ds;
+    A.items = G * A.slices;
     switch (ds) {
-        case 16: return launch_records<M, 16>(ctx, A, G, bf16);
-        case 32: return launch_records<M, 32>(ctx, A, G, bf16);
+        case 16: return launch_records<M, 16>(ctx, A, bf16);
+        case 32: return launch_records<M, 32>(ctx, A, bf16);
         default:
-            if constexpr (M <= 32) return launch_records<M, 64>(ctx, A, G, bf16);
+            if constexpr (M <= 32) return launch_records<M, 64>(ctx, A, bf16);
             return GRF_ERR_INVALID;
     }
 }
@@ -789,7 +1007,7 @@ PairRoom pair_room(int64_t nnz, int32_t G, int32_t d, int dtype, size_t workspac
 //         m = 16, d = 64: 8192 235 / 213, 200000 8765 / 7365, 50000 (records of 32 columns) 1774 / 1839;  m = 64, d = 32: 533 / 201
 //   fp32  m = 32, d = 64: cloud of 1024, 1 problem 71 / 74, 4 problems 174 / 134, 5003, 3 problems 687 / 441;
 //         m = d = 64: 8192, 4 problems 2784 / 1696;  m = 16, d = 32: 487 / 454;  lattice of 400, 4 problems 36 / 40
-// (the fixed part of the pairs is five launches: regrouping Phi's entries by column takes three).
+// (the fixed part of the pairs is six launches: regrouping Phi's entries by column takes three).
 double grf_pairs_ns(double nnz, int32_t G, int32_t m, int32_t d, int dtype, size_t workspace_per_problem)
 {
     double each;
@@ -834,16 +1052,18 @@ int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N,
 
     // Phi's entries by column
     const int32_t counts_len = (R + 3) & ~3;
-    GRF_TRY(grf_buf_reserve(&ctx->t_cursor, sizeof(int32_t) * (2 * (size_t)counts_len + 4)));
+    GRF_TRY(grf_buf_reserve(&ctx->t_cursor, sizeof(int32_t) * (3 * (size_t)counts_len + 8)));
     GRF_TRY(grf_reserve_buckets(ctx, nnz + 4));
     float* den = den_out;
     if (!den && width < d) {
         GRF_TRY(grf_buf_reserve(&ctx->den_scratch, sizeof(float) * (size_t)G * N));
         den = (float*)ctx->den_scratch.ptr;
     }
-    int32_t *counts = (int32_t*)ctx->t_cursor.ptr, *start = counts + counts_len;
+    int32_t *counts = (int32_t*)ctx->t_cursor.ptr, *long_count = counts + counts_len, *start = long_count + 4;
+    int32_t* long_nodes = start + counts_len + 4;
+    const int32_t long_limit = pair_long_limit(nnz + feat->psit.nnz, R);
     int32_t *slot = (int32_t*)ctx->t_tmp.ptr, *query = slot + ((nnz + 3) & ~(int64_t)3);
-    GRF_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(int32_t) * (size_t)R, ctx->stream));
+    GRF_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(int32_t) * ((size_t)counts_len + 2), ctx->stream));
     {
         grf_launch_scope scope(ctx, 3);
         pair_ranks_kernel<<<grf_ceil_div(nnz, 1024), 256, 0, ctx->stream>>>(nnz, (const int32_t*)feat->phi.col.ptr, counts, slot);
@@ -857,8 +1077,10 @@ int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N,
     }
     {
         grf_launch_scope scope(ctx, 3);
-        pair_slots_kernel<<<grf_ceil_div(N, 8), 256, 0, ctx->stream>>>(N, (const int32_t*)feat->phi.rowptr.ptr,
-                                                                       (const int32_t*)feat->phi.col.ptr, start, slot, query);
+        const int row_blocks = grf_ceil_div(N, 8);
+        pair_slots_kernel<<<row_blocks + grf_ceil_div(R, 256), 256, 0, ctx->stream>>>(
+            N, R, row_blocks, (const int32_t*)feat->phi.rowptr.ptr, (const int32_t*)feat->phi.col.ptr, start,
+            (const int32_t*)feat->psit.rowptr.ptr, long_limit, long_limit > PAIR_HUGE ? long_limit : PAIR_HUGE, slot, query, long_count, long_nodes);
     }
 
     for (int64_t g0 = 0; g0 < G; g0 += chunk) {
@@ -868,6 +1090,7 @@ int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N,
         A.t_rowptr = (const int32_t*)feat->psit.rowptr.ptr; A.t_col = (const int32_t*)feat->psit.col.ptr;
         A.t_val = (const float*)feat->psit.val.ptr;
         A.start = start; A.query = query;
+        A.long_limit = long_limit; A.long_count = long_count; A.long_nodes = long_nodes;
         A.phiQ = (const char*)phiQ + (size_t)g0 * N * m * es;
         A.phiK = (const char*)phiK + (size_t)g0 * N * m * es;
         A.V = (const char*)V + (size_t)g0 * N * d * es;
@@ -876,7 +1099,7 @@ int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N,
         A.den = A.rec + (size_t)gc * nnz * width;
         for (A.col0 = 0; A.col0 < d; A.col0 += width) {
             {
-                grf_launch_scope scope(ctx, 4);
+                grf_launch_scope scope(ctx, 4, 2);
                 GRF_TRY(m == 16 ? launch_records_m<16>(ctx, A, gc, bf16)
                                 : m == 32 ? launch_records_m<32>(ctx, A, gc, bf16) : launch_records_m<64>(ctx, A, gc, bf16));
             }

@@ -224,6 +224,10 @@ cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void** args, size_t, cud
     }
     return cudaSuccess;
 }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args)
+{
+    return cudaLaunchKernel(f, c->gridDim, c->blockDim, args, c->dynamicSmemBytes, c->stream);
+}
 static thread_local struct { dim3 g, b; size_t smem; void* s; } config;
 unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t smem, void* s) { config = {g, b, smem, s}; return 0; }
 cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* smem, void* s)

@@ -62,6 +62,58 @@ def test_lists_of_every_length(m, d, dtype):
     ctx.close()
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("m,d", [(16, 32), (16, 64), (32, 32), (32, 64), (64, 32), (64, 64)])
+def test_hub_nodes(m, d, dtype):
+    """Nodes with more than 512 keys and queries are a CTA's work, with more than 8192 a cluster's: right below, at and above that, one side long only, nodes
+    without keys or with a few (warps without a share), hubs that every row visits."""
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    rng = np.random.default_rng(m + d)
+    N, R, G = 6001, 1500, 24
+    sides = [(256, 256), (256, 257), (1, 511), (511, 1), (1, 512), (512, 1), (0, 600), (600, 0), (7, 700), (700, 7), (6001, 6001),
+             (2049, 33), (31, 2051), (513, 6001), (4096, 4096), (4096, 4097), (6001, 2192)]
+    sides += [(40, 30)] * (R - len(sides))
+    order = rng.permutation(R)
+    phi_t = csr(rng, R, N, [sides[x][1] for x in order])
+    psi_t = csr(rng, R, N, [sides[x][0] for x in order])
+    Phi, Psi = oracle.transpose(phi_t), oracle.transpose(psi_t)
+    feat = api.features_from_csr(ctx, N, R, (Phi.rowptr, Phi.col, Phi.val), (Psi.rowptr, Psi.col, Psi.val))
+    q, k, v = tensors.qkv(G, N, m, d, dtype, 5)
+    qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
+    B.grf_ctx_use_tensor_cores(ctx.handle, 2)
+    (out, den), ran = kernel_classes(B, ctx, lambda: api.masked_linear_attn(ctx, feat, qd, kd, vd, want_den=True))
+    assert "scan" in ran, ran
+    pick = [0, G - 1]
+    ref = oracle.attn_sparse(tensors.widen(q[pick]), tensors.widen(k[pick]), tensors.widen(v[pick]), Phi, oracle.transpose(Psi))
+    helpers.assert_attn_close(out[pick].float().cpu().numpy(), ref, helpers.TOL[dtype], den[pick].cpu().numpy(), min_ok=0.3)
+    # other shares of the batch: the same bits, every time
+    small = B.grf_attn_workspace_bytes(1, R, m, d, B.dtype_code(vd))
+    for _ in range(3):
+        assert torch.equal(out, api.masked_linear_attn(ctx, feat, qd, kd, vd, workspace_bytes=small))
+    feat.free()
+    ctx.close()
+
+
+def test_few_nodes_for_many_rows():
+    """Three nodes: all of them long, whatever the average.  (bf16 takes whole states by tiles there.)"""
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    rng = np.random.default_rng(3)
+    N, R, G, m, d, dtype = 20011, 3, 16, 32, 64, "fp32"
+    Phi, Psi = csr(rng, N, R, [1 + i % 3 for i in range(N)]), csr(rng, N, R, [2] * N)
+    feat = api.features_from_csr(ctx, N, R, (Phi.rowptr, Phi.col, Phi.val), (Psi.rowptr, Psi.col, Psi.val))
+    q, k, v = tensors.qkv(G, N, m, d, dtype, 5)
+    B.grf_ctx_use_tensor_cores(ctx.handle, 2)
+    (out, den), ran = kernel_classes(B, ctx, lambda: api.masked_linear_attn(ctx, feat, q.cuda(), k.cuda(), v.cuda(), want_den=True))
+    assert "scan" in ran, ran
+    pick = [0, G - 1]
+    ref = oracle.attn_sparse(tensors.widen(q[pick]), tensors.widen(k[pick]), tensors.widen(v[pick]), Phi, oracle.transpose(Psi))
+    helpers.assert_attn_close(out[pick].float().cpu().numpy(), ref, helpers.TOL[dtype], den[pick].cpu().numpy(), min_ok=0.3)
+    feat.free()
+    ctx.close()
+
+
 @pytest.mark.parametrize("m,d", [(32, 64), (32, 32), (16, 64)])
 def test_records_of_every_width_give_the_same_bits(m, d):
     """An expander whose whole records are larger than the context's scratch: a full workspace holds them, one problem's only
