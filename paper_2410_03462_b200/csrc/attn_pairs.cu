@@ -11,6 +11,7 @@
 // 0.64 read at random, but 0.66 (whole rows per instruction) to 1.23 ms (fragments) written at random.  What a row adds, and in
 // which order, depends on Phi alone, so results do not depend on the order inside a node's run, which the regrouping leaves to
 // chance.
+#include <cfloat>
 #include <type_traits>
 
 #include "grf_internal.cuh"
@@ -813,7 +814,7 @@ __device__ __forceinline__ void put_pair(__nv_bfloat16* dst, float x, float y) {
 __device__ __forceinline__ void add_carried(float& sum, float& lost, float phi, float y)
 {
     const float x = fmaf(phi, y, -lost), t = sum + x;
-    lost = (t - sum) - x;
+    lost = fabsf(t) <= FLT_MAX ? (t - sum) - x : 0.0f;          // an infinite sum rounds nothing off (inf - inf would make it NaN)
     sum = t;
 }
 

@@ -114,6 +114,41 @@ def test_few_nodes_for_many_rows():
     ctx.close()
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("m,d", [(16, 32), (32, 64), (64, 32)])
+def test_infinite_sums_stay_infinite(m, d, dtype):
+    """Positive features throughout: a row that uses an infinite value, or whose sum leaves the range of fp32, gives infinity of
+    that sign as a plain sum does, other columns and other rows what they give without it."""
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    rng = np.random.default_rng(m)
+    N, R, G = 2003, 1500, 24
+    Phi, Psi = csr(rng, N, R, [25 + i % 40 for i in range(N)]), csr(rng, N, R, [25] * N)
+    feat = api.features_from_csr(ctx, N, R, (Phi.rowptr, Phi.col, Phi.val), (Psi.rowptr, Psi.col, Psi.val))
+    q, k, v = (t.cuda() for t in tensors.qkv(G, N, m, d, dtype, 5))
+    q, k = q.abs() + 0.25, k.abs() + 0.25
+    B.grf_ctx_use_tensor_cores(ctx.handle, 2)
+    want = api.masked_linear_attn(ctx, feat, q, k, v)
+    bad = v.clone()
+    bad[1, 7, 3], bad[2, 11, 5] = float("inf"), -float("inf")
+    bad[3, 13, 9] = 2.0 ** 126                                   # finite; its sums are not
+    out, ran = kernel_classes(B, ctx, lambda: api.masked_linear_attn(ctx, feat, q, k, bad))
+    assert "scan" in ran, ran
+    # rows that reach a node: the support of Phi Psi^T
+    rows = np.zeros((N, R), bool)
+    rows[np.repeat(np.arange(N), np.diff(Phi.rowptr)), Phi.col] = True
+    for g, node, column, sign in ((1, 7, 3, 1), (2, 11, 5, -1)):
+        reached = torch.from_numpy(rows[:, Psi.col[Psi.rowptr[node]:Psi.rowptr[node + 1]]].any(1)).cuda()
+        assert reached.any() and not reached.all()
+        assert (out[g, reached, column] == sign * float("inf")).all()
+        out[g, reached, column] = want[g, reached, column]
+    assert not out.isnan().any() and (out[3, :, 9] == float("inf")).any()
+    out[3, :, 9] = want[3, :, 9]
+    assert torch.equal(out, want)
+    feat.free()
+    ctx.close()
+
+
 @pytest.mark.parametrize("m,d", [(32, 64), (32, 32), (16, 64)])
 def test_records_of_every_width_give_the_same_bits(m, d):
     """An expander whose whole records are larger than the context's scratch: a full workspace holds them, one problem's only
