@@ -256,7 +256,8 @@ int grf_masked_attn_asym(grf_ctx* ctx, const grf_features* feat, int32_t G, int3
  * grf_masked_attn_mhat: out_i = sum_j Mhat_ij (phi(q_i).phi(k_j)) v_j / sum_j Mhat_ij (phi(q_i).phi(k_j)) for G
  * problems; arguments as grf_masked_linear_attn, no workspace.  dtype GRF_DTYPE_BF16, d = 64, m in {16, 32, 64}
  * (other shapes: GRF_ERR_INVALID); scores are fp32, the masked scores are added into the denominator in fp32 and
- * rounded to bf16 before they multiply V.  Summation order is fixed.  Asynchronous.
+ * rounded to bf16 before they multiply V.  Summation order is fixed.  Asynchronous.  An infinity or NaN in the K or V row of
+ * a key reaches the rows of those blocks (128 consecutive rows) of which at least one row reaches that key, and no others.
  */
 int grf_features_materialise(grf_ctx* ctx, grf_features* feat);
 int grf_mask_stats(const grf_features* feat, int32_t* blocks, int64_t* key_entries, int64_t* bytes);

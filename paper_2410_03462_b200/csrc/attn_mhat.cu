@@ -32,7 +32,10 @@ constexpr int KT = GRF_MASK_TILE;       // keys per tile
 // Structure of the mask: one CTA per block of rows, everything that does not depend on values.
 //   keys       the union of Psi^T's rows over the block's node list, marked in a bitmap (a bit is looked at before it is
 //              set: a block reaches each of its keys about thirty times), counted, and written as the block's key list,
-//              padded to whole tiles with the last key (whose mask values there are zeros);
+//              padded to whole tiles with the last key (whose mask values there are zeros); on graphs of GRF_MASK_SMALL nodes
+//              and fewer the list has a place for every key of the aligned tiles from the first to the last one reached, and
+//              places of keys that no row of the block reaches are padding as well (a key of the block, zeros in the mask):
+//              what such a key's rows of K and V hold must not matter;
 //   positions  for every node of the list the accumulator (by position in the key list) of each of its keys, 16 bits each;
 //              for every non-zero Phi_il of the block's rows where node l's positions begin.
 // A warp takes 32 nodes at a time (lane x holds node x's extent in Psi^T) and fetches the keys of two nodes together.
@@ -207,8 +210,11 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
         for (int32_t x = tid; x < wk; x += MS_THREADS) kbits[x] = (uint32_t)kbefore[x];
         __syncthreads();
     }
-    if (Nk <= GRF_MASK_SMALL) {                                 // every key of the tiles from the first to the last one reached
+    __shared__ uint32_t reached[GRF_MASK_SMALL / 32];
+    const bool whole_tiles = Nk <= GRF_MASK_SMALL;
+    if (whole_tiles) {                                          // a place for every key of the tiles from the first to the last one reached
         if (warp == 0) {
+            if (lane < GRF_MASK_SMALL / 32) reached[lane] = lane < wk ? kbits[lane] : 0u;
             const uint32_t any = __ballot_sync(0xffffffffu, lane < wk && kbits[min(lane, wk - 1)] != 0u);
             if (any) {
                 const int32_t first = (__ffs(any) - 1) & ~1, last = (31 - __clz(any)) | 1;       // two words a tile
@@ -242,6 +248,16 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
     }
     if ((int64_t)base_keys + padded <= key_room) {
         int32_t* list = mk_key + base_keys;
+        // the key that stands at key k's place: itself, or the nearest one before it that is reached, or else the first one
+        auto standing = [&](int32_t k) {
+            if (!whole_tiles) return k;
+            int32_t x = k >> 5;
+            uint32_t b = reached[x] & (0xffffffffu >> (31 - (k & 31)));
+            while (b == 0u && x > 0) b = reached[--x];
+            if (b) return (x << 5) + 31 - __clz(b);
+            while (reached[x] == 0u) ++x;
+            return (x << 5) + __ffs(reached[x]) - 1;
+        };
         const int32_t per = (wk + C * MS_THREADS - 1) / (C * MS_THREADS);
         const int32_t w0 = min(wk, (part * MS_THREADS + tid) * per), w1 = min(wk, w0 + per);
         for (int32_t x = w0; x < w1; ++x) {
@@ -250,9 +266,10 @@ mask_structure_kernel(int32_t N, int32_t Nk, int32_t R, const int32_t* __restric
             while (b) {
                 const int k = (x << 5) + __ffs(b) - 1;
                 b &= b - 1;
+                const int32_t key = standing(k);
                 if (o == keys - 1)
-                    for (int32_t e = keys; e < padded; ++e) list[e] = k;
-                list[o++] = k;
+                    for (int32_t e = keys; e < padded; ++e) list[e] = key;
+                list[o++] = key;
             }
         }
     }
@@ -619,10 +636,12 @@ mask_rows_kernel(int32_t Nk, const int32_t* __restrict__ rows, const int32_t* __
     __syncthreads();
     const int32_t blk = r / BQ, rr = r % BQ;
     const int32_t off = mk_off[blk], cnt = mk_cnt[blk];
-    // padding entries repeat the last key with the value 0: skip an entry whose predecessor has the same key
+    // padding entries repeat another key with the value 0: skip an entry whose predecessor has the same key, in lists of whole
+    // aligned tiles one that holds another key than its place's
+    const int32_t first = cnt > 0 ? mk_key[off] & ~(KT - 1) : 0;
     for (int32_t e = threadIdx.x; e < cnt; e += 256) {
         const int32_t j = mk_key[off + e];
-        if (e > 0 && mk_key[off + e - 1] == j) continue;
+        if (Nk <= GRF_MASK_SMALL ? j != first + e : e > 0 && mk_key[off + e - 1] == j) continue;
         o[j] = __bfloat162float(mk_val[((size_t)((off + e) / 16) * BQ + rr) * 16 + ((off + e) & 15)]);
     }
 }

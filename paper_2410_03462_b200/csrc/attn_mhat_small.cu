@@ -5,6 +5,12 @@
 // 1000 to 2300 cycles, and every CTA started over (5900 cycles before its first product).  Here, 25.9 us:
 //   * a block's key list is a run of whole aligned tiles of 64 keys (mask_structure_kernel fills the gaps, whose mask values are
 //     zeros), so key, value and query tiles are boxes of consecutive rows: one instruction of the copy engine each;
+//   * rows of keys that no row of the block reaches come with such a box, and an infinity or NaN in one (a padded node's row) would
+//     meet the mask's zeros: every row of the block would be NaN.  So a group whose outputs hold a NaN goes over its problems a
+//     second time and clears these rows in shared memory before it multiplies.  (Clearing them always: grid of 400, 200 problems
+//     20.6 -> 21.8 us, cloud of 512, 600 problems, m = 64, a third of whose places are such keys, 51.5 -> 57.5; looking at the
+//     outputs instead 20.6 -> 20.6, 51.5 -> 51.8; lattice of 484, 300 problems 22.8 -> 23.7, the grid of 196 24.7 -> 24.7.  Both passes
+//     in one loop needed more registers than there are: 27.2);
 //   * a CTA has an SM and its tensor memory to itself and stays with one block for many problems, of which it works on four at a
 //     time, each with a group of row threads, an issuing warp, a score buffer and an accumulator of its own.  Nothing is exchanged
 //     between groups, and while one waits for its products the others use the issue slots.
@@ -17,6 +23,8 @@
 // follows from uniform registers, below); one block, six score buffers, the groups in turn over its tiles (30.4: the row sums of four
 // groups meet in every epilogue); four problems with common issuing warps (29.4: a fixed order makes the groups wait together); the
 // mask in shared memory (no change).
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace {
@@ -61,6 +69,7 @@ mhat_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     __shared__ __align__(8) unsigned long long bars[GROUPS * PER_GROUP];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ int nan_seen[GROUPS];        // in outputs of a group's problems
 
     // what the whole warp shares is read from one lane, so that the compiler keeps it (and what follows from it) in uniform
     // registers: a tensor-pipe instruction then costs its warp 25 cycles instead of 100
@@ -122,11 +131,12 @@ mhat_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         __syncwarp();
         if (g_copy < G) {
             copy_queries(mine);
-            first_row = uniform(__ldg(mk_key + off));
+            first_row = uniform(__ldg(mk_key + off) & ~(KT - 1));
             for (int s = 0; s < NS; ++s) copy_tile();
         }
     }
     if (tid == 0) abort_flag = 0;
+    if (tid < GROUPS) nan_seen[tid] = 0;
     if (warp == 0) tmem_alloc(&tmem_slot, 512u);
     fence_before_sync();
     __syncthreads();
@@ -134,6 +144,27 @@ mhat_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     const uint32_t tmem_base = (uint32_t)uniform((int32_t)tmem_slot);
     auto score_col = [&](int x) { return tmem_base + (uint32_t)(x * KT); };
     auto acc_col = [&](int x) { return tmem_base + (uint32_t)(Sh::O_COL + x * D); };
+    // The keys of every tile that no row of the block reaches: bits 32 h .. 32 h + 31 of tile t in lane 2 t + h.  (Their places hold
+    // another key; rows behind the last key are zeros as they come.)
+    auto unreached = [&]() {
+        const int32_t first = __ldg(mk_key + off) & ~(KT - 1);
+        uint32_t mine_bits = 0u;
+        for (int32_t e = 0; e < 2 * T; ++e) {
+            const int32_t k = first + e * 32 + lane;
+            const uint32_t b = __ballot_sync(0xffffffffu, k < N && __ldg(mk_key + off + e * 32 + lane) != k);
+            if (lane == e) mine_bits = b;
+        }
+        return mine_bits;
+    };
+    // After a group's last problem: whether it goes over them once more (the same answer in its five warps; all of their products
+    // are complete, as the row threads have waited for every accumulator)
+    auto once_more = [&](int x, uint32_t& gaps) {
+        __syncwarp();
+        asm volatile("bar.sync %0, 160;" ::"r"(1 + x) : "memory");
+        if (nan_seen[x] == 0 || *(volatile int*)&abort_flag != 0) return false;
+        gaps = unreached();
+        return __any_sync(0xffffffffu, gaps != 0u) != 0;
+    };
     if (warp < 16) {
         // ------------------------------------------------------------ row threads
         const int x = warp >> 2;
@@ -150,93 +181,110 @@ mhat_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         uint32_t par = 0u, acc_par = 0u;                         // of this group's present tile and problem
         const uint32_t s_addr = score_col(x) + lane_field, o_addr = acc_col(x) + lane_field;
         const bool whole = ((uintptr_t)out & 31u) == 0;          // whole sectors at once where the outputs allow it
-        if (T > 0) load_mask(0);
-        for (int32_t g = g_first + x * g_step; g < G; g += g_round) {
-            uint64_t den2[2] = {0ull, 0ull};                     // row sums, four partial sums in two packed pairs
-            for (int32_t t = 0; t < T; ++t) {
-                if (!mbar_wait(s_full(x), par, &abort_flag)) ok = false;
+        auto problems = [&](auto again) {
+            if (T > 0) load_mask(0);
+            for (int32_t g = g_first + x * g_step; g < G; g += g_round) {
+                uint64_t den2[2] = {0ull, 0ull};                     // row sums, four partial sums in two packed pairs
+                for (int32_t t = 0; t < T; ++t) {
+                    if (!mbar_wait(s_full(x), par, &abort_flag)) ok = false;
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    par ^= 1u;
+                    fence_after_sync();
+                    uint32_t sv[2][16];
+                    tmem_ld16_nowait(s_addr, sv[0]);
+#pragma unroll
+                    for (int c16 = 0; c16 < KT / 16; ++c16) {
+                        tmem_ld_wait();
+                        if (c16 + 1 < KT / 16) tmem_ld16_nowait(s_addr + (uint32_t)((c16 + 1) * 16), sv[(c16 + 1) & 1]);
+                        const uint32_t (&sc)[16] = sv[c16 & 1];
+                        uint32_t pw[8];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const uint4 mm = mk[2 * c16 + h];
+                            const uint32_t mw[4] = {mm.x, mm.y, mm.z, mm.w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                // two masked scores at a time; the denominator adds them in fp32, before the rounding to bf16
+                                const uint64_t p2 = mul_f32x2(pack_f32x2(sc[8 * h + 2 * e], sc[8 * h + 2 * e + 1]),
+                                                              pack_f32x2(mw[e] << 16, mw[e] & 0xffff0000u));
+                                den2[e & 1] = add_f32x2(den2[e & 1], p2);
+                                float p0, p1;
+                                unpack_f32x2(p2, p0, p1);
+                                const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
+                                pw[4 * h + e] = *reinterpret_cast<const uint32_t*>(&pb);
+                            }
+                        }
+                        tmem_st8(s_addr + (uint32_t)(c16 * 8), pw);
+                    }
+                    tmem_st_wait();
+                    fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(p_full(x));
+                    // the next tile's mask values travel while the products run
+                    if (t + 1 < T) load_mask(t + 1);
+                    else if (T > 1 && g + g_round < G) load_mask(0);
+                }
+                if (ok && T > 0) ok = mbar_wait(acc_done(x), acc_par, &abort_flag);
+                acc_par ^= 1u;
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                par ^= 1u;
                 fence_after_sync();
-                uint32_t sv[2][16];
-                tmem_ld16_nowait(s_addr, sv[0]);
+                float d0, d1, d2, d3;
+                unpack_f32x2(den2[0], d0, d1);
+                unpack_f32x2(den2[1], d2, d3);
+                const float den = (d0 + d1) + (d2 + d3), inv = (den != 0.0f) ? 1.0f / den : 0.0f;
+                __nv_bfloat16* dst = out + ((size_t)g * N + row) * D;
+                bool not_a_number = den != den;
+                uint32_t o[2][16];
 #pragma unroll
-                for (int c16 = 0; c16 < KT / 16; ++c16) {
-                    tmem_ld_wait();
-                    if (c16 + 1 < KT / 16) tmem_ld16_nowait(s_addr + (uint32_t)((c16 + 1) * 16), sv[(c16 + 1) & 1]);
-                    const uint32_t (&sc)[16] = sv[c16 & 1];
-                    uint32_t pw[8];
+                for (int e = 0; e < 16; ++e) o[0][e] = o[1][e] = 0u;
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint4 mm = mk[2 * c16 + h];
-                        const uint32_t mw[4] = {mm.x, mm.y, mm.z, mm.w};
+                for (int c = 0; c < D / 32; ++c) {
+                    if (T > 0) {
+                        tmem_ld16_nowait(o_addr + (uint32_t)(c * 32), o[0]);
+                        tmem_ld16_nowait(o_addr + (uint32_t)(c * 32 + 16), o[1]);
+                        tmem_ld_wait();
+                    }
+                    // what an unreached key does it does to every lane: each of the four warps looks at its share of the columns
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            // two masked scores at a time; the denominator adds them in fp32, before the rounding to bf16
-                            const uint64_t p2 = mul_f32x2(pack_f32x2(sc[8 * h + 2 * e], sc[8 * h + 2 * e + 1]),
-                                                          pack_f32x2(mw[e] << 16, mw[e] & 0xffff0000u));
-                            den2[e & 1] = add_f32x2(den2[e & 1], p2);
-                            float p0, p1;
-                            unpack_f32x2(p2, p0, p1);
-                            const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
-                            pw[4 * h + e] = *reinterpret_cast<const uint32_t*>(&pb);
+                    for (int h = 0; h < 2 && !decltype(again)::value; ++h) {
+                        if ((warp & (D / 16 - 1)) == 2 * c + h) {
+                            float y[2] = {0.0f, 0.0f};
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) y[e & 1] += __uint_as_float(o[h][e]);
+                            not_a_number |= y[0] + y[1] != y[0] + y[1];
                         }
                     }
-                    tmem_st8(s_addr + (uint32_t)(c16 * 8), pw);
+                    if (row < N) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t w[8];
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) {
+                                const __nv_bfloat162 y = __floats2bfloat162_rn(__uint_as_float(o[h][2 * e]) * inv, __uint_as_float(o[h][2 * e + 1]) * inv);
+                                w[e] = *reinterpret_cast<const uint32_t*>(&y);
+                            }
+                            if (whole) {
+                                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                                             ::"l"(dst + c * 32 + h * 16), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+                            } else {
+                                uint4* half = reinterpret_cast<uint4*>(dst + c * 32 + h * 16);
+                                half[0] = make_uint4(w[0], w[1], w[2], w[3]);
+                                half[1] = make_uint4(w[4], w[5], w[6], w[7]);
+                            }
+                        }
+                    }
                 }
-                tmem_st_wait();
+                // (read before this group hands its next tile over, which is when the accumulator is written again)
                 fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(p_full(x));
-                // the next tile's mask values travel while the products run
-                if (t + 1 < T) load_mask(t + 1);
-                else if (T > 1 && g + g_round < G) load_mask(0);
+                if (row < N && den_out) den_out[(size_t)g * N + row] = den;
+                if (!decltype(again)::value && not_a_number) nan_seen[x] = 1;
             }
-            if (ok && T > 0) ok = mbar_wait(acc_done(x), acc_par, &abort_flag);
-            acc_par ^= 1u;
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            fence_after_sync();
-            float d0, d1, d2, d3;
-            unpack_f32x2(den2[0], d0, d1);
-            unpack_f32x2(den2[1], d2, d3);
-            const float den = (d0 + d1) + (d2 + d3), inv = (den != 0.0f) ? 1.0f / den : 0.0f;
-            __nv_bfloat16* dst = out + ((size_t)g * N + row) * D;
-            uint32_t o[2][16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) o[0][e] = o[1][e] = 0u;
-#pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
-                if (T > 0) {
-                    tmem_ld16_nowait(o_addr + (uint32_t)(c * 32), o[0]);
-                    tmem_ld16_nowait(o_addr + (uint32_t)(c * 32 + 16), o[1]);
-                    tmem_ld_wait();
-                }
-                if (row < N) {
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        uint32_t w[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const __nv_bfloat162 y = __floats2bfloat162_rn(__uint_as_float(o[h][2 * e]) * inv, __uint_as_float(o[h][2 * e + 1]) * inv);
-                            w[e] = *reinterpret_cast<const uint32_t*>(&y);
-                        }
-                        if (whole) {
-                            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                                         ::"l"(dst + c * 32 + h * 16), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-                        } else {
-                            uint4* half = reinterpret_cast<uint4*>(dst + c * 32 + h * 16);
-                            half[0] = make_uint4(w[0], w[1], w[2], w[3]);
-                            half[1] = make_uint4(w[4], w[5], w[6], w[7]);
-                        }
-                    }
-                }
-            }
-            // (read before this group hands its next tile over, which is when the accumulator is written again)
-            fence_before_sync();
-            if (row < N && den_out) den_out[(size_t)g * N + row] = den;
-        }
+        };
+        uint32_t gaps;
+        problems(std::false_type());
+        if (once_more(x, gaps)) problems(std::true_type());
     } else {
         // ------------------------------------------------------------ copies and products of one group (the whole warp in step)
         const int x = warp - ISSUER;
@@ -251,11 +299,29 @@ mhat_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         bool ok = true;
         auto wait = [&](uint32_t b, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(b, parity, &abort_flag)); };
         uint32_t i = 0;                                                // tiles so far
-        // S of tile i, which is a problem's first where `queries` says so
-        auto scores = [&](bool queries) {
+        // Clears the rows of unreached keys in the t-th tile of a problem (`at`: the first stage's; P pieces of 16 bytes each); a
+        // swizzle moves pieces inside a row only.  Neighbouring lanes take the pieces of a row, so that they meet in no bank.
+        uint32_t gaps = 0u;
+        auto clear = [&](int32_t t, uint32_t at, auto pieces) {
+            constexpr int P = decltype(pieces)::value, ROWS = 32 / P;              // of a row; rows at a time
+            const uint32_t gap[2] = {__shfl_sync(0xffffffffu, gaps, 2 * t), __shfl_sync(0xffffffffu, gaps, 2 * t + 1)};
+            const uint32_t to = at + (i & (NS - 1)) * Sh::STAGE + (uint32_t)lane * 16u;
+#pragma unroll
+            for (int y = 0; y < 2 * P; ++y)
+                if (gap[y / P] >> (y % P * ROWS + lane / P) & 1u)
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(to + (uint32_t)(y * 512)), "r"(0u) : "memory");
+        };
+        // S of tile i, the t-th of its problem
+        auto scores = [&](int32_t t, auto again) {
             const int s = i & (NS - 1);
-            if (queries && !wait(q_full(x), (uint32_t)(asked - 1) & 1u)) return false;
+            if (t == 0 && !wait(q_full(x), (uint32_t)(asked - 1) & 1u)) return false;
             if (!wait(kv_full(x, s), (i / NS) & 1u)) return false;
+            if (decltype(again)::value) {
+                clear(t, my_stages, std::integral_constant<int, M / 8>());
+                clear(t, my_stages + Sh::K_BYTES, std::integral_constant<int, D / 8>());
+                fence_async_smem();                             // the products read through the asynchronous proxy
+                __syncwarp();
+            }
             fence_after_sync();
             const uint32_t k_lo = (uint32_t)k_op + (uint32_t)(s * (Sh::STAGE / 16));
             mma_bf16_ss_halves<false>(score, q_lo, q_hi, k_lo, k_hi, idesc_s);
@@ -264,8 +330,8 @@ mhat_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             mma_commit(s_full(x));
             return true;
         };
-        if (T > 0 && mine < G) {
-            ok = scores(true);
+        auto problems = [&](auto again) {
+            ok = scores(0, again);
             for (int32_t g = mine; g < G && ok; g += g_round) {
                 const bool more = g + g_round < G;
                 for (int32_t t = 0; t < T && ok; ++t, ++i) {
@@ -288,11 +354,19 @@ mhat_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     if (last && !more) continue;
                     if (!wait(kv_done(x, s), (i / NS) & 1u)) { ok = false; break; }
                     ++i;
-                    ok = scores(last);
+                    ok = scores(last ? 0 : t + 1, again);
                     --i;
                     copy_tile();
                 }
             }
+        };
+        if (T > 0 && mine < G) problems(std::false_type());
+        if (once_more(x, gaps) && ok && T > 0 && mine < G) {            // from the first one again
+            g_copy = mine;
+            t_copy = 0;
+            copy_queries(mine);
+            for (int s = 0; s < NS; ++s) copy_tile();
+            problems(std::true_type());
         }
         if (!ok) {
             // products and copies under way end before the CTA does

@@ -103,10 +103,10 @@ struct grf_kept_walks {
 
 // The mask estimate Mhat = Phi Psi^T held as dense blocks: for every block of GRF_PLAN_BLOCK consecutive rows the
 // sorted list of the keys j that any of its rows reaches (padded to a multiple of GRF_MASK_TILE with the last key
-// and zero values) and the block's values in bf16, laid out [group of 16 keys][row of the block][16 keys].
+// and zero values; see GRF_MASK_SMALL) and the block's values in bf16, laid out [group of 16 keys][row of the block][16 keys].
 #define GRF_MASK_TILE 64
 // Up to this many keys a block's list is made of whole aligned tiles, all of them between its first and last key
-// (attn_mhat_small.cu): at most eight.
+// (attn_mhat_small.cu): at most eight.  Places of keys that no row of the block reaches are padding too: they hold another key.
 #define GRF_MASK_SMALL 512
 struct grf_mask_dev {
     bool ready = false;             // the blocks hold the mask of the present features

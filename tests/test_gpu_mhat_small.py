@@ -63,3 +63,60 @@ def test_small_graphs(N, G, m, d, kind):
     assert not out[:, torch.from_numpy(empty).cuda()].any() and not out.isnan().any()
     feat.free()
     ctx.close()
+
+
+def reached_keys(Phi, Psi, N, rows):
+    """Keys that any of the rows reaches: the support of Phi Psi^T."""
+    nodes = np.zeros(N, bool)
+    for r in rows:
+        nodes[Phi.col[Phi.rowptr[r]:Phi.rowptr[r + 1]]] = True
+    keys = np.zeros(N, bool)
+    for j in range(N):
+        keys[j] = nodes[Psi.col[Psi.rowptr[j]:Psi.rowptr[j + 1]]].any()
+    return keys
+
+
+@pytest.mark.parametrize("kind", ["local", "mixed", "far"])
+@pytest.mark.parametrize("N,G,m,d", [(65, 9, 16, 64), (129, 7, 32, 64), (196, 40, 64, 64), (300, 150, 32, 64), (449, 300, 64, 32), (512, 400, 16, 32), (650, 8, 32, 64)])
+def test_keys_that_no_row_of_a_block_reaches_do_not_matter(N, G, m, d, kind):
+    """Infinities and NaNs in their rows of K and V (padded nodes, say) leave the block's bits alone, also where they lie between,
+    before or behind keys that it does reach; the mask's own rows hold zeros there."""
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    rng = np.random.default_rng(N + m)
+    Phi, Psi = band_features(N, kind, rng)
+    feat = api.features_from_csr(ctx, N, N, (Phi.rowptr, Phi.col, Phi.val), (Psi.rowptr, Psi.col, Psi.val))
+    q, k, v = (t.cuda() for t in tensors.qkv(G, N, m, d, "bf16", 5))
+    B.grf_features_materialise(ctx.handle, feat.handle)
+    if d == 64:
+        def attn(k, v):
+            return api.masked_attn_mhat(ctx, feat, q, k, v, want_den=True)
+    else:
+        B.grf_ctx_use_tensor_cores(ctx.handle, 1)
+
+        def attn(k, v):
+            return api.masked_linear_attn(ctx, feat, q, k, v, want_den=True)
+    want, want_den = attn(k, v)
+    for first in range(0, N, 128):
+        rows = np.arange(first, min(N, first + 128))
+        free = torch.from_numpy(~reached_keys(Phi, Psi, N, rows)).cuda()
+        for bad in (float("nan"), float("inf")):
+            k2, v2 = k.clone(), v.clone()
+            k2[:, free], v2[:, free] = bad, -bad
+            out, den = attn(k2, v2)
+            at = slice(first, first + len(rows))
+            assert torch.equal(out[:, at], want[:, at]) and torch.equal(den[:, at], want_den[:, at])
+    # and a NaN that rows do reach stays one, in its own problem
+    k2 = k.clone()
+    k2[G // 2, N // 2, 3] = float("nan")
+    out, den = attn(k2, v)
+    assert out[G // 2].isnan().any() and not out[:G // 2].isnan().any() and not out[G // 2 + 1:].isnan().any()
+    mask = torch.empty((N, N), device="cuda")
+    B.grf_mask_rows(ctx.handle, feat.handle, N, torch.arange(N, dtype=torch.int32, device="cuda"), mask)
+    import scipy.sparse as sp
+    dense = (sp.csr_matrix((Phi.val, Phi.col, Phi.rowptr), (N, N)) @ sp.csr_matrix((Psi.val, Psi.col, Psi.rowptr), (N, N)).T).toarray()
+    # sums of at most N positive products in fp32, rounded to bf16 once
+    assert np.abs(mask.cpu().numpy() - dense).max() <= 2.0 ** -8 * np.abs(dense).max()
+    assert (mask.cpu().numpy()[dense == 0] == 0).all()
+    feat.free()
+    ctx.close()
