@@ -1264,7 +1264,10 @@ static int launch_mhat_values(grf_ctx* ctx, const grf_features* feat, int32_t G,
 int grf_mhat_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, const void* phiQ,
                     const void* phiK, const void* V, void* out, float* den_out)
 {
-    if (N <= GRF_MASK_SMALL && G <= (1 << 30)) return grf_mhat_small_launch(ctx, feat, G, N, m, d, phiQ, phiK, V, out, den_out);
+    if (N <= GRF_MASK_SMALL && G <= (1 << 30)) {
+        const int rc = grf_mhat_small_launch(ctx, feat, G, N, m, d, phiQ, phiK, V, out, den_out);
+        if (rc <= 0) return rc;                                 // (the kernel below gathers rows and needs no tensor maps)
+    }
     if (m == 16) return launch_mhat_values<16>(ctx, feat, G, N, d, phiQ, phiK, V, out, den_out);
     if (m == 32) return launch_mhat_values<32>(ctx, feat, G, N, d, phiQ, phiK, V, out, den_out);
     return launch_mhat_values<64>(ctx, feat, G, N, d, phiQ, phiK, V, out, den_out);

@@ -392,7 +392,7 @@ int launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, const v
     const grf_mask_dev& K = feat->mask;
     CUtensorMap mq, mk, mv;
     if (!grf_make_row_box_map(&mq, phiQ, (uint32_t)G, (uint32_t)N, M, BQ) || !grf_make_row_box_map(&mk, phiK, (uint32_t)G, (uint32_t)N, M, KT) ||
-        !grf_make_row_box_map(&mv, V, (uint32_t)G, (uint32_t)N, D, KT)) return GRF_ERR_CUDA;
+        !grf_make_row_box_map(&mv, V, (uint32_t)G, (uint32_t)N, D, KT)) return 1;
     // a CTA per SM, but no more than there are problems; at least as many as all blocks' shares, of which each has one or more: so
     // every block gets a CTA
     const int64_t least = (int64_t)K.blocks * (K.longest / KT + 1), items = (int64_t)K.blocks * G;

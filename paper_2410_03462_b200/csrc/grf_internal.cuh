@@ -242,7 +242,7 @@ int grf_linear_by_mask(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_
 int grf_mhat_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, const void* phiQ,
                     const void* phiK, const void* V, void* out, float* den_out);
 void grf_mask_release(grf_features* feat);
-// attn_mhat_small.cu: the same for N <= GRF_MASK_SMALL
+// attn_mhat_small.cu: the same for N <= GRF_MASK_SMALL; 1 (nothing launched) where no tensor map can be made of the operands
 int grf_mhat_small_launch(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, const void* phiQ,
                           const void* phiK, const void* V, void* out, float* den_out);
 // attn_gather_tc.cu

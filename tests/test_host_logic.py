@@ -135,6 +135,22 @@ def test_no_memory_for_the_mask_means_the_states(fake):
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
 
 
+def test_small_graphs_without_tensor_maps(fake):
+    """The kernel for up to 512 nodes copies boxes through tensor maps, which the pretended driver does not make: the kernel that
+    gathers rows takes the call."""
+    ctx = fake.context(0)
+    fake.report(PHI=40_000, PSI=40_000, EDGES=3200, PLAN=1600, KEYS=1664, POSITIONS=200_000, LONGEST=448)
+    rc, feat = fake.sample(ctx, 400)
+    assert rc == 0 and fake.lib.grf_features_materialise(ctx, feat) == 0
+    some = fake_device.C.c_void_p(4096)
+    for m in (16, 32, 64):
+        fake.lib.fake_log_clear()
+        assert fake.lib.grf_masked_attn_mhat(ctx, feat, 200, 400, m, 64, 1, some, some, some, some, None) == 0
+        assert fake.launched("mhat_attention_kernel") == 1 and fake.launched("mhat_small_kernel") == 0
+    assert fake.lib.grf_features_free(feat) == 0 and fake.lib.grf_ctx_destroy(ctx) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
 def test_host_path_without_memory_for_the_preferred_mask(fake):
     ctx = fake.context(0)
     fake.report(PHI=400_000, PSI=400_000, EDGES=8192, PLAN=25_600, KEYS=640_000, POSITIONS=2_500_000, LONGEST=40_000)
