@@ -208,7 +208,10 @@ size_t grf_attn_workspace_bytes(int32_t G, int32_t R, int32_t m, int32_t d, int 
  * Where the states are cheaper used at once than stored and gathered (m in {16, 32, 64}, d in {32, 64}; graphs without
  * locality, fp32), every (row, node) pair leaves a record of d fp32 values in the workspace, or, where that holds fewer
  * problems, in up to 512 MiB of scratch of the context (up to 1 GiB where the workspace is smaller than one problem's narrowest
- * records); a call under stream capture keeps to whole states, which need the workspace only (and differ by rounding).
+ * records), which the context keeps until it is destroyed.  A workspace of G * (4 (d + 1) nnz(Phi) + 512) bytes means that no such
+ * scratch is taken.  Where the scratch cannot be had, fewer columns at a time lie in the workspace, with the same bits; if that is
+ * too small for them as well, whole states serve the call (and differ by rounding), as they do for a call under stream capture.
+ * grf_ctx_use_tensor_cores(ctx, 0) and 3 keep to whole states from the start.
  * Asynchronous, except that a call may wait for the sizes of a sample that is still running, and that the first bf16 call
  * with m and d multiples of 16 after the features were created, resampled or re-modulated prepares a per-block plan of Phi,
  * and where it takes the other order the mask, inside the feature object, which waits for the stream (so a feature object

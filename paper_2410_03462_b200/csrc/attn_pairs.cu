@@ -980,11 +980,11 @@ constexpr size_t PAIR_MOST = (size_t)1 << 30;
 static int32_t least_width(int dtype) { return dtype == GRF_DTYPE_BF16 ? 16 : 32; }
 
 namespace {
-struct PairRoom { int32_t width; int64_t chunk; size_t scratch; };     // columns of a record, problems a launch, own scratch (0: the workspace)
-PairRoom pair_room(int64_t nnz, int32_t G, int32_t d, int dtype, size_t workspace_bytes)
+struct PairRoom { int32_t width; int64_t chunk; size_t scratch; };     // columns of a record, problems a launch (0: no room), own scratch (0: the workspace)
+PairRoom pair_room(int64_t nnz, int32_t G, int32_t d, int dtype, size_t workspace_bytes, bool own_scratch = true)
 {
     const size_t whole = pair_bytes(nnz, d);
-    int64_t in_ws = (int64_t)(workspace_bytes / whole), in_scratch = (int64_t)(PAIR_SCRATCH / whole);
+    int64_t in_ws = (int64_t)(workspace_bytes / whole), in_scratch = own_scratch ? (int64_t)(PAIR_SCRATCH / whole) : 0;
     if (in_ws > G) in_ws = G;
     if (in_scratch > G) in_scratch = G;
     PairRoom r = {d, in_ws, 0};
@@ -994,7 +994,7 @@ PairRoom pair_room(int64_t nnz, int32_t G, int32_t d, int dtype, size_t workspac
     } else if (in_ws == 0) {
         while (r.width > least_width(dtype) && pair_bytes(nnz, r.width) > workspace_bytes) r.width >>= 1;
         r.chunk = (int64_t)(workspace_bytes / pair_bytes(nnz, r.width));
-        if (r.chunk == 0) { r.chunk = 1; r.scratch = pair_bytes(nnz, r.width); }
+        if (r.chunk == 0 && own_scratch) { r.chunk = 1; r.scratch = pair_bytes(nnz, r.width); }
         if (r.chunk > G) r.chunk = G;
     }
     if (r.chunk > 16000) r.chunk = 16000;                       // the grid's second dimension, two slices a problem
@@ -1045,10 +1045,14 @@ int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N,
     const size_t es = bf16 ? 2 : 4;
     const int64_t nnz = feat->phi.nnz;
     const int32_t R = feat->phi.cols;
-    const PairRoom room = pair_room(nnz, G, d, dtype, workspace_bytes);
+    PairRoom room = pair_room(nnz, G, d, dtype, workspace_bytes);
+    if (room.scratch > 0) {
+        const int rc = grf_buf_reserve(&ctx->pair_scratch, room.scratch);
+        if (rc == GRF_ERR_NOMEM) room = pair_room(nnz, G, d, dtype, workspace_bytes, false);     // narrower records, fewer problems: the same bits
+        if (rc != GRF_OK && (rc != GRF_ERR_NOMEM || room.chunk == 0)) return rc;
+    }
     const int32_t width = room.width;
     const int64_t chunk = room.chunk;
-    if (room.scratch > 0) GRF_TRY(grf_buf_reserve(&ctx->pair_scratch, room.scratch));
     float* records = (float*)(room.scratch > 0 ? ctx->pair_scratch.ptr : workspace);
 
     // Phi's entries by column

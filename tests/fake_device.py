@@ -69,10 +69,10 @@ class Fake:
         n = C.c_int64(-1)
         return self.lib.grf_features_view(feat, which, None, None, C.byref(n), None, None, None), n.value
 
-    def linear(self, ctx, feat, G, N, m, d, dtype):
-        """grf_masked_linear_attn on arrays that nobody reads, with a workspace for one problem."""
+    def linear(self, ctx, feat, G, N, m, d, dtype, workspace=None):
+        """grf_masked_linear_attn on arrays that nobody reads, with a workspace for one problem if not stated."""
         code = 1 if dtype == "bf16" else 0
-        need = self.lib.grf_attn_workspace_bytes(1, N, m, d, code)
+        need = workspace or self.lib.grf_attn_workspace_bytes(1, N, m, d, code)
         some = C.c_void_p(4096)
         return self.lib.grf_masked_linear_attn(ctx, feat, G, N, m, d, code, some, some, some, some, None, some,
                                                C.c_size_t(need))

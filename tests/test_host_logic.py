@@ -135,6 +135,36 @@ def test_no_memory_for_the_mask_means_the_states(fake):
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
 
 
+def test_pair_records_without_memory_or_with_the_callers(fake):
+    """Records find room in the context's scratch; without memory for that, narrower ones in the workspace (two launches a problem
+    instead of one, the same bits); whole states only where these do not fit either.  A workspace that holds all records means
+    that no scratch is taken at all."""
+    N, G, m, d = 20011, 3, 32, 64
+    for nnz, narrow in ((1_200_000, True), (1_500_000, False)):
+        ctx = fake.context(0)
+        fake.report(PHI=nnz, PSI=nnz, EDGES=160_000)
+        rc, feat = fake.sample(ctx, N)
+        assert rc == 0
+        live = fake.lib.fake_live(0)
+        records = nnz * (d + 1) * 4 + 512
+        fake.lib.fake_log_clear()
+        assert fake.linear(ctx, feat, G, N, m, d, "fp32", workspace=G * records) == 0
+        assert fake.launched("pair_records") == 1 and fake.lib.fake_live(0) == live
+        fake.lib.fake_limit(0, live + (64 << 20))
+        for _ in range(2):
+            fake.lib.fake_log_clear()
+            assert fake.linear(ctx, feat, G, N, m, d, "fp32") == 0
+            assert fake.launched("pair_records") == (2 * G if narrow else 0)
+            assert (fake.launched("build_states") == 0) == narrow
+        fake.lib.fake_limit(0, 1 << 40)
+        fake.lib.fake_log_clear()
+        assert fake.linear(ctx, feat, G, N, m, d, "fp32") == 0
+        assert fake.launched("pair_records") == G and fake.launched("build_states") == 0
+        assert fake.lib.fake_live(0) - live <= (512 << 20) + (4 << 20)
+        assert fake.lib.grf_features_free(feat) == 0 and fake.lib.grf_ctx_destroy(ctx) == 0
+        assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
 def test_small_graphs_without_tensor_maps(fake):
     """The kernel for up to 512 nodes copies boxes through tensor maps, which the pretended driver does not make: the kernel that
     gathers rows takes the call."""
