@@ -212,7 +212,8 @@ size_t grf_attn_workspace_bytes(int32_t G, int32_t R, int32_t m, int32_t d, int 
  * scratch is taken.  Where the scratch cannot be had, fewer columns at a time lie in the workspace, with the same bits; if that is
  * too small for them as well, whole states serve the call (and differ by rounding), as they do for a call under stream capture.
  * grf_ctx_use_tensor_cores(ctx, 0) and 3 keep to whole states from the start.
- * Asynchronous, except that a call may wait for the sizes of a sample that is still running, and that the first bf16 call
+ * Asynchronous, except that a call may wait for the sizes of a sample that is still running (an fp32 call where its choice between
+ * records and whole states needs them; never after grf_ctx_use_tensor_cores(ctx, 0) or 3), and that the first bf16 call
  * with m and d multiples of 16 after the features were created, resampled or re-modulated prepares a per-block plan of Phi,
  * and where it takes the other order the mask, inside the feature object, which waits for the stream (so a feature object
  * must not be used by two threads at the same time).

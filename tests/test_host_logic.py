@@ -165,6 +165,25 @@ def test_pair_records_without_memory_or_with_the_callers(fake):
         assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
 
 
+def test_fp32_calls_that_wait_for_a_running_sample(fake):
+    """Only one whose choice between records and whole states needs the sizes; none in the modes that keep to whole states."""
+    ctx = fake.context(0)
+    N, m, d = 4096, 32, 64
+    fake.report(PHI=400_000, PSI=400_000, EDGES=40_000)
+    rc, feat = fake.sample(ctx, N)
+    assert rc == 0
+    for mode, G, walks, waits in ((1, 3, 32, True), (2, 3, 32, True), (0, 3, 32, False), (3, 3, 32, False), (1, 1, 1, False)):
+        assert fake.lib.grf_ctx_use_tensor_cores(ctx, mode) == 0
+        for _ in range(2):                        # the second sample finds arrays that are large enough
+            assert fake.sample(ctx, N, feat, walks=walks)[0] == 0
+        fake.lib.fake_log_clear()
+        assert fake.linear(ctx, feat, G, N, m, d, "fp32") == 0
+        assert ("sync event" in fake.log()) == waits, (mode, G)
+        assert (fake.launched("pair_records") > 0) == waits
+    assert fake.lib.grf_features_free(feat) == 0 and fake.lib.grf_ctx_destroy(ctx) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
 def test_small_graphs_without_tensor_maps(fake):
     """The kernel for up to 512 nodes copies boxes through tensor maps, which the pretended driver does not make: the kernel that
     gathers rows takes the call."""
