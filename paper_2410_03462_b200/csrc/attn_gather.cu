@@ -228,11 +228,14 @@ gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, c
 // 76 ms, 128 bytes 1.75, 3.03, 10.3, 19.0, 40.6, 88.)
 constexpr size_t SLICE_L2_BYTES = (size_t)72 << 20;
 
+// Calls whose denominators are formed inside: at most so many rows, mean entries of a row, and look-ups of z_l over all slices.
 constexpr int64_t DEN_INSIDE_ROWS = 2048;
+template <typename T> constexpr double DEN_INSIDE_MEAN = sizeof(T) == 4 ? 48.0 : 96.0;
+template <typename T> constexpr double DEN_INSIDE_ENTRIES = (sizeof(T) == 4 ? 256.0 : 192.0) * 1024.0;
 
 template <typename T, int M, int D>
-int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, const void* phiQ, const void* states, void* out,
-              float* den_out)
+int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, double entries, int32_t G, int32_t N, const void* phiQ, const void* states,
+              void* out, float* den_out)
 {
     const int32_t* rp = (const int32_t*)phi.rowptr.ptr;
     const int32_t* cl = (const int32_t*)phi.col.ptr;
@@ -245,11 +248,15 @@ int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, const 
             N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, (T*)out, den);
     };
     const bool wide = (size_t)phi.cols * 2048 <= SLICE_L2_BYTES;
-    // Small calls form the denominators inside, once more for each of up to four slices: what a launch costs is more than that.
-    // us measured, whole attention, separate / inside: fp32 lattice of 64 nodes, m = d = 16 23.0 / 18.0, of 400, 4 problems, m = 32,
-    // d = 64 35.1 / 29.6, bf16 30.6 / 25.3; cloud of 1024, fp32 68.0 / 66.7, of 3000, m = 16 110.2 / 111.7.
+    // Small calls form the denominators inside, once more for each of up to four slices: what a launch costs (3 us) is more than
+    // that while rows are short (a warp looks 32 entries up at a time) and few in all.  us measured, whole attention, separate /
+    // inside: fp32 lattice of 64 nodes, m = d = 16 23.0 / 18.0, of 400, 4 problems, m = 32, d = 64 (four slices) 35.1 / 29.6; grid
+    // of 1024 (37 entries a row), four slices, 0.15 M look-ups 49 / 47.5, 0.3 M 96 / 98; expanders (65 to 72 entries a row) of 300,
+    // 1200 and 2000 nodes, four slices 47.5 / 48.5, 86.0 / 91.5, 112.8 / 121.1, of 600, one slice, m = 8, d = 64 45.1 / 49.2;
+    // bf16, m = d = 64, four slices, cloud of 512, 0.1 M 60.0 / 57.2, expander of 900, 0.25 M 101.1 / 103.1, 2000, 0.58 M 173 / 185.
     if constexpr (SliceShape<T, M, D, 4>::SLICES <= 4) {
-        if (wide && (int64_t)G * N <= DEN_INSIDE_ROWS) {
+        if (wide && (int64_t)G * N <= DEN_INSIDE_ROWS && entries <= DEN_INSIDE_MEAN<T> * N &&
+            G * entries * SliceShape<T, M, D, 4>::SLICES <= DEN_INSIDE_ENTRIES<T>) {
             launch(std::integral_constant<int, 4>(), std::true_type(), den_out);
             return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
         }
@@ -270,40 +277,43 @@ int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, const 
 }
 
 template <typename T, int M>
-int launch_m(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t d,
+int launch_m(grf_ctx* ctx, const grf_csr_dev& phi, double entries, int32_t G, int32_t N, int32_t d,
              const void* phiQ, const void* states, void* out, float* den_out)
 {
     switch (d) {
-        case 8: return launch_md<T, M, 8>(ctx, phi, G, N, phiQ, states, out, den_out);
-        case 16: return launch_md<T, M, 16>(ctx, phi, G, N, phiQ, states, out, den_out);
-        case 32: return launch_md<T, M, 32>(ctx, phi, G, N, phiQ, states, out, den_out);
-        case 64: return launch_md<T, M, 64>(ctx, phi, G, N, phiQ, states, out, den_out);
-        case 128: return launch_md<T, M, 128>(ctx, phi, G, N, phiQ, states, out, den_out);
+        case 8: return launch_md<T, M, 8>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
+        case 16: return launch_md<T, M, 16>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
+        case 32: return launch_md<T, M, 32>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
+        case 64: return launch_md<T, M, 64>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
+        case 128: return launch_md<T, M, 128>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
         default: return GRF_ERR_INVALID;
     }
 }
 
 template <typename T>
-int launch_t(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t m, int32_t d,
+int launch_t(grf_ctx* ctx, const grf_csr_dev& phi, double entries, int32_t G, int32_t N, int32_t m, int32_t d,
              const void* phiQ, const void* states, void* out, float* den_out)
 {
     switch (m) {
-        case 8: return launch_m<T, 8>(ctx, phi, G, N, d, phiQ, states, out, den_out);
-        case 16: return launch_m<T, 16>(ctx, phi, G, N, d, phiQ, states, out, den_out);
-        case 32: return launch_m<T, 32>(ctx, phi, G, N, d, phiQ, states, out, den_out);
-        case 64: return launch_m<T, 64>(ctx, phi, G, N, d, phiQ, states, out, den_out);
-        case 128: return launch_m<T, 128>(ctx, phi, G, N, d, phiQ, states, out, den_out);
+        case 8: return launch_m<T, 8>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
+        case 16: return launch_m<T, 16>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
+        case 32: return launch_m<T, 32>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
+        case 64: return launch_m<T, 64>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
+        case 128: return launch_m<T, 128>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
         default: return GRF_ERR_INVALID;
     }
 }
 
 }  // namespace
 
-int grf_gather_contract_alu(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t m, int32_t d,
+int grf_gather_contract_alu(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d,
                             int dtype, const void* phiQ, const void* states, void* out, float* den_out)
 {
+    const grf_csr_dev& phi = feat->phi;
+    // (a running sample's sizes are not waited for: both ways to form the denominators give the same bits)
+    const double entries = feat->sizes_pending ? feat->expected_entries : (double)phi.nnz;
     if (G > 65535) return GRF_ERR_TOO_LARGE;
-    if (dtype == GRF_DTYPE_F32) return launch_t<float>(ctx, phi, G, N, m, d, phiQ, states, out, den_out);
-    if (dtype == GRF_DTYPE_BF16) return launch_t<__nv_bfloat16>(ctx, phi, G, N, m, d, phiQ, states, out, den_out);
+    if (dtype == GRF_DTYPE_F32) return launch_t<float>(ctx, phi, entries, G, N, m, d, phiQ, states, out, den_out);
+    if (dtype == GRF_DTYPE_BF16) return launch_t<__nv_bfloat16>(ctx, phi, entries, G, N, m, d, phiQ, states, out, den_out);
     return GRF_ERR_INVALID;
 }

@@ -97,3 +97,39 @@ def test_a_mask_that_the_caller_formed_changes_no_bit_of_the_main_call(N, G):
     assert torch.equal(before, api.masked_linear_attn(ctx, feat, q, k, v))
     feat.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("m,d", [(16, 16), (32, 64), (8, 64), (16, 128), (8, 8)])
+def test_denominators_inside_and_by_themselves_give_the_same_bits(m, d, dtype):
+    """While a sample runs only the expected number of its entries is known (several times the real one here), which makes
+    the plain gather form the denominators by themselves; afterwards it forms them inside: 48 (fp32) and 96 (bf16) entries a row
+    lie between."""
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    B.grf_ctx_use_tensor_cores(ctx.handle, 0)
+    w = configs.point_cloud_4096(200)
+    dg = api.DeviceGraph(w.graph())
+    f = oracle.deconvolve(w.alpha).astype(np.float32)
+    q, k, v = (t.cuda() for t in tensors.qkv(1, 200, m, d, dtype, 4))
+    ws = torch.empty(B.grf_attn_workspace_bytes(1, 200, m, d, B.dtype_code(v)), dtype=torch.uint8, device="cuda")
+    out, den = torch.empty_like(v), torch.empty((1, 200), device="cuda")
+    feat = api.sample(ctx, dg, 3, w.n_walks, w.p_halt, w.max_len, f)
+
+    def call():
+        B.grf_ctx_enable_timing(ctx.handle, True)
+        B.grf_masked_linear_attn(ctx.handle, feat.handle, 1, 200, m, d, B.dtype_code(v), q, k, v, out, den, ws, ws.numel())
+        launches = B.grf_ctx_kernel_times(ctx.handle)["row_denominators"][1]
+        B.grf_ctx_enable_timing(ctx.handle, False)
+        return launches, out.clone(), den.clone()
+
+    for _ in range(2):                      # the second sample leaves its sizes open
+        feat.handle = B.grf_sample(ctx.handle, dg.N, dg.rowptr, dg.col, dg.w, 3, 12 if dtype == "fp32" else 20, w.p_halt, w.max_len, f, None,
+                                     feat.handle)
+    running = call()
+    feat.shape(0)                           # reads the sizes
+    settled = call()
+    assert torch.equal(running[1], settled[1]) and torch.equal(running[2], settled[2])
+    assert (running[0], settled[0]) == (1, 0)       # both ways were taken
+    feat.free()
+    ctx.close()
