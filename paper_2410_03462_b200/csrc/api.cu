@@ -519,7 +519,8 @@ constexpr double PLAIN_BUILD_WORTH_NS = 25000.0;
 // the features' sizes, the shape and the whole batch's G_all, so that parts of a batch give the bits of the whole.  The sizes
 // of a sample whose kernels may still be running are waited for only where its walks' expectation leaves the choice open.  A
 // call under stream capture keeps to whole states, whose only memory is the caller's: the pairs lie in buffers of the context
-// that a later call may replace while the graph still names them.
+// that a later call may replace while the graph still names them, and their places and launches follow the number of non-zeros,
+// which a graph would keep while the kernels of whole states read the row pointers of whatever sample the object then holds.
 static int states_by_pairs(grf_ctx* ctx, const grf_features* feat, int32_t G_all, int32_t m, int32_t d, int dtype, const void* phiQ,
                            const void* phiK, const void* V, const void* out, bool* yes)
 {

@@ -275,7 +275,8 @@ __device__ __forceinline__ void pair_long_nodes(const PairArgs& A, Node&& node)
 // (the next chunk's copies are under way while one is used; three slots and twelve warps an SM instead of sixteen: 678 us against
 // 621 at 2^15 nodes, 4 problems).
 //   keys      S^T (DS columns b x M features a) += V^T (b x keys) . (Psi phi(K)) (keys x a): both operands by transposing
-//             ldmatrix from the rows as they lie; Psi_jl enters in registers, rounded to bf16 once, as the other builds do.
+//             ldmatrix from the rows as they lie; Psi_jl enters in registers, in fp32, and the product is rounded to bf16 (once:
+//             the tensor-core builds of whole states round Psi_jl as well, which is why their outputs are further from fp64).
 //             z is added up in fp32 from the same rounded products.
 //   S         rounded to bf16, as the stored states are: the accumulators' layout is the second product's operand layout
 //   queries   records (queries x b) = phi(Q) . S; z rides along as three bf16 columns that add up to its fp32 value
