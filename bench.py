@@ -8,9 +8,9 @@ Prints ONE JSON line.
     python bench.py --suite        every workload, the unsorted point cloud, the scaling sweep and the operation
                                    counts of Sec. 4: a summary (.md) and one JSON line per run (.jsonl) in --suite-dir
 
-Routes: sz = grf_masked_linear_attn (the headline): Alg. 1 through the per-node states S_l, z_l of Eq. 12 or over the mask,
-whichever the library's cost rule finds cheaper for the batch (`evaluated_by` in the output says which); states = the same call
-held to the per-node states; mhat = Eqs. 1-2 over the materialised mask Phi Psi^T; asym = Alg. 2 (asymmetric features, Psi = I).
+Routes: sz = grf_masked_linear_attn (the headline): Alg. 1 through the per-node states S_l, z_l of Eq. 12, stored or used where
+they are made, or over the mask, whichever the library's cost rule finds cheaper for the batch (`evaluated_by` in the output says
+which: states, pairs, mask); states = the same call held to the per-node states; mhat = Eqs. 1-2 over the materialised mask Phi Psi^T; asym = Alg. 2 (asymmetric features, Psi = I).
 
 With N > 1 (launched by torch.distributed.run) every rank runs the same-sized, independently seeded batch
 on its own GPU (the problems are independent: no data-path collective); the value is the sum of all
@@ -151,7 +151,7 @@ class ClockSampler:
         return out
 
 
-def algorithmic_bytes(w, N, nnz_phi, nnz_psi, E):
+def algorithmic_bytes(w, N, nnz_phi, nnz_psi, E, by_pairs=False):
     """Bytes each kernel class must move per step if every operand crosses HBM exactly once."""
     es = 2 if w.dtype == "bf16" else 4
     G, m, d = w.G, w.m, w.d
@@ -159,7 +159,9 @@ def algorithmic_bytes(w, N, nnz_phi, nnz_psi, E):
     z = G * N * m * 4
     zb = G * N * m * 2 if w.dtype == "bf16" else 0          # bf16 copy of z in the records
     csr = lambda nnz: nnz * 8 + (N + 1) * 4
-    return {
+    # states used where they are made: a record of d fp32 values and a denominator per (row, node) pair and problem
+    records = G * nnz_phi * (d + 1) * 4
+    out = {
         # graph read once; merged rows written once
         "walk_merge": E * 8 + (N + 1) * 4 + (nnz_phi + nnz_psi) * 8 + 2 * N * 4,
         "scan": 2 * N * 4 * 3,
@@ -174,10 +176,15 @@ def algorithmic_bytes(w, N, nnz_phi, nnz_psi, E):
         # Phi read twice (union lists, coefficient table)
         "block_plan": 2 * csr(nnz_phi),
     }
+    if by_pairs:
+        # phi(K), V, phi(Q), Psi^T and Phi's order by column read once, the records written once; then read once, with Phi
+        out["build_states"] = G * N * (2 * m + d) * es + csr(nnz_psi) + csr(nnz_phi) + records
+        out["gather_contract"] = records + csr(nnz_phi) + nnz_phi * 4 + G * N * d * es
+    return out
 
 
 def binding_report(w, N, nnz_phi, nnz_psi, ktimes, steps, pk, counters, plan_entries, mask_entries,
-                   mask_values_ms=None):
+                   mask_values_ms=None, by_pairs=False):
     """For each big kernel, the rates of the resources that can bind it (from counts of this run and the CUDA-event
     time of the kernel) and, where the tracked profile of the same sources exists, the profiler's busy fractions.
     `binds` names the resource with the largest fraction of its peak."""
@@ -202,8 +209,16 @@ def binding_report(w, N, nnz_phi, nnz_psi, ktimes, steps, pk, counters, plan_ent
         r.update(prof(name))
         rep[name] = r
 
+    if by_pairs:                                        # the records and their sums: what is known without a profile is their traffic
+        alg = algorithmic_bytes(w, N, nnz_phi, nnz_psi, 0, by_pairs=True)
+        for name in ("build_states", "gather_contract"):
+            ms = ktimes.get(name, (0.0, 0))[0]
+            if ms:
+                hbm = alg[name] / (ms / steps * 1e-3) / 1e9
+                rep[name] = {"hbm_algorithmic_gbs": hbm, "binds": "hbm", "fraction_of_binding_peak": hbm / pk["hbm_gbs"],
+                             "profile": "none for these sources"}
     t = per_launch_s("gather_contract")
-    if t and plan_entries and w.dtype == "bf16":
+    if t and plan_entries and w.dtype == "bf16" and not by_pairs:
         issued = plan_entries * G * 2.0 * 128 * m * d / t / 1e12
         useful = 2.0 * nnz_phi * m * d * G / t / 1e12
         fill = plan_entries * G * m * d * es / t / 1e9
@@ -213,7 +228,7 @@ def binding_report(w, N, nnz_phi, nnz_psi, ktimes, steps, pk, counters, plan_ent
             "smem_fill_gbs": fill, "smem_fill_peak_gbs": SMEM_FILL_PEAK_GBS, "hbm_algorithmic_gbs": hbm},
             {"tensor_issue": issued / pk["bf16_tflops"], "smem_fill": fill / SMEM_FILL_PEAK_GBS, "hbm": hbm / pk["hbm_gbs"]})
     t = per_launch_s("build_states")
-    if t and w.dtype == "bf16":
+    if t and w.dtype == "bf16" and not by_pairs:
         gathered = (nnz_psi * G * (m + d) * es + G * N * (m * d * es + m * 6)) / t / 1e9
         issued = 2.0 * 128 * m * (nnz_psi + 8 * N) * G / t / 1e12       # keys padded to steps of 16 (8 on average)
         hbm = G * N * (m * d * es + m * 6) / t / 1e9
@@ -277,6 +292,7 @@ def aggregate_over_ranks(local_ms: float, tokens_per_rank_step: int, steps: int,
 DTYPE_NOTE = {
     "sz": "bf16 storage, fp32 accumulation; tensor-core path multiplies bf16(Phi_il)*phi(q) and bf16(Psi_jl)*phi(k) rounded to bf16",
     "mhat": "bf16 storage, fp32 scores and mask sums; the mask and the masked scores are rounded to bf16",
+    "pairs": "bf16 storage, fp32 accumulation; Psi_jl phi(k) and S_l are rounded to bf16, the records are fp32",
     "asym": "bf16 storage, fp32 accumulation",
 }
 
@@ -410,7 +426,13 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
     nnz_phi, nnz_psi = feat.shape(0)[2], feat.shape(1)[2]
     plan_entries = mask_entries = mask_values_ms = None
     by_mask = mhat or ktimes.get("mhat_attention", (0.0, 0))[1] > 0      # what grf_masked_linear_attn chose
-    if route == "sz" and w.dtype == "bf16" and not by_mask:
+    by_pairs = False
+    if route == "sz" and not by_mask:                   # such a call alone regroups Phi's entries by column
+        B.grf_ctx_enable_timing(ctx.handle, True)
+        attention()
+        by_pairs = B.grf_ctx_kernel_times(ctx.handle)["scan"][1] > 0
+        B.grf_ctx_enable_timing(ctx.handle, False)
+    if route == "sz" and w.dtype == "bf16" and not by_mask and not by_pairs:
         try:
             plan_entries = B.grf_plan_stats(ctx.handle, feat.handle)[1]
         except B.GrfError:
@@ -474,7 +496,7 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
     if rank == 0:
         pk = peaks()
         counters = load_counters()
-        alg = algorithmic_bytes(w, N, nnz_phi, nnz_psi, E)
+        alg = algorithmic_bytes(w, N, nnz_phi, nnz_psi, E, by_pairs)
         es = 2 if w.dtype == "bf16" else 4
         if by_mask:   # Q, K, V read once, out written once; the mask blocks written once, read once
             mbytes = B.grf_mask_stats(feat.handle)[2]
@@ -493,7 +515,7 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
         dom = max(ktimes, key=lambda kname: ktimes[kname][0])
         achieved = alg.get(dom, 0) / 1e9 / (ktimes[dom][0] / steps * 1e-3)
         binding = binding_report(w, N, nnz_phi, nnz_psi, ktimes, steps, pk, counters, plan_entries, mask_entries,
-                                 mask_values_ms)
+                                 mask_values_ms, by_pairs)
         # DRAM traffic of the dominant kernel from the tracked profile of the same sources, scaled to this run's heads
         traffic = None
         c = counters.get(dom)
@@ -502,11 +524,11 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
                 traffic = c["dram_bytes"]
             elif dom == "mhat_attention":                      # the mask is read once whatever the head count: no scaling rule
                 traffic = c["dram_bytes"] if w.G == c["heads"] else None
-            else:
+            elif not by_pairs:
                 traffic = c["dram_bytes"] * w.G / c["heads"]
         binds = binding.get(dom, {}).get("binds")
         bound = {"tensor_issue": "tensor", "hbm": "hbm", "integer_issue": "alu"}.get(binds, "hbm" if binds is None else "smem")
-        note = "mhat" if by_mask else route
+        note = "mhat" if by_mask else "pairs" if by_pairs else route
         step_text = {"sz": "grf_sample (both ensembles) + grf_masked_linear_attn",
                      "mhat": "grf_sample (both ensembles) + grf_features_materialise + grf_masked_attn_mhat",
                      "asym": "grf_sample (f_psi = delta_0) + grf_masked_attn_asym (Alg. 2, %s similarity)"
@@ -517,7 +539,7 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
             "scaling": "weak", "vs_baseline": None,
             "dtype": ("bf16" if w.dtype == "bf16" else "f32"), "dtype_note": DTYPE_NOTE[note] if w.dtype == "bf16" else "fp32 throughout",
             "data": "synthetic",
-            "config": {"workload": w.name, "route": "states" if states_only else route, "evaluated_by": "rows" if asym else "mask" if by_mask else "states",
+            "config": {"workload": w.name, "route": "states" if states_only else route, "evaluated_by": "rows" if asym else "mask" if by_mask else "pairs" if by_pairs else "states",
                        "N": N, "edges": E, "batch": w.batch, "heads": w.heads, "m": w.m,
                        "d": w.d, "n_walks": w.n_walks, "p_halt": w.p_halt, "max_len": w.max_len,
                        "nnz_phi": nnz_phi, "nnz_psi": nnz_psi,
@@ -548,7 +570,7 @@ def measure(args, workload_name, route, with_cpu_baseline, with_e2e, frozen=Fals
                        "walks_per_s": None if (frozen or remodulate) else 2 * N * w.n_walks / (statistics.mean(sample_ms) * 1e-3),
                        "attn_tokens_per_s": w.batch * N / (statistics.mean(attn_ms) * 1e-3),
                        "attn_hbm_frac": (2 * w.G * N * w.m * w.d * es + w.G * N * (2 * w.m + 2 * w.d) * es) / 1e9 /
-                                        (statistics.mean(attn_ms) * 1e-3) / pk["hbm_gbs"] if route == "sz" and not by_mask else None,
+                                        (statistics.mean(attn_ms) * 1e-3) / pk["hbm_gbs"] if route == "sz" and not by_mask and not by_pairs else None,
                        "wall_s_timed_region": wall},
             "kernels": per_kernel,
         }

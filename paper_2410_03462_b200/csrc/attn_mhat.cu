@@ -42,11 +42,11 @@ constexpr int KT = GRF_MASK_TILE;       // keys per tile
 // Blocks take their places in the lists by atomic additions, so the order of the blocks inside the arrays varies; nothing
 // depends on it.  A block whose part does not fit the room that the host has made writes none of it: the totals tell
 // the host how much is needed.  The last CTA to finish orders the blocks by decreasing key count.
-// One kernel for all of this, at the N = 32768 cloud: 237 us in five kernels and two prefix sums before, 160 us now (issue
-// slots 77 % busy while an SM has blocks, 59 % of the warps there; the blocks with the longest lists end last).
-// A cluster of C CTAs builds each block (one CTA a block leaves SMs idle where there are few): they share out the nodes, merge their key bitmaps through each
-// other's shared memory, and share out list, positions and non-zeros; ranks and prefix sums are formed by each for itself (cheaper
-// than asking).  Structure and values together, us, one CTA a block / cluster: clouds of 2048 (8 CTAs) 91 / 62, 4096 (8) 124 / 89,
+// One kernel for all of this, at the N = 32768 cloud: 237 us in five kernels and two prefix sums before, 160 us with a CTA per
+// block, 150 now (profiled: issue slots 75 % busy, 65 % of the warps there; the blocks with the longest lists end last).
+// A cluster of C CTAs builds each block (one CTA a block leaves SMs idle where there are few): they share out the nodes, merge their
+// key bitmaps through each other's shared memory, and share out list, positions and non-zeros; ranks and prefix sums are formed by
+// each for itself (cheaper than asking).  Structure and values together, us, one CTA a block / cluster: clouds of 2048 (8 CTAs) 91 / 62, 4096 (8) 124 / 89,
 // 6000 (4) 167 / 127, 9000 (4) 203 / 166, 22000 (2) 419 / 393.
 
 constexpr int MS_THREADS = 768;

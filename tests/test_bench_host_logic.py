@@ -58,6 +58,21 @@ def test_binding_report_arithmetic():
     assert np.isclose(rep["walk_merge"]["walks_per_s"], 2 * 32768 * 32 / 0.25e-3)
 
 
+def test_records_of_pairs_are_counted_as_such():
+    """Expanders do not gather stored states: the two classes move the records, and no fraction of a delivery that did not happen
+    is reported."""
+    w = configs.sweep(18)
+    N, nnz = 1 << 18, 14_600_000
+    a = bench.algorithmic_bytes(w, N, nnz, nnz, 8 * N, by_pairs=True)
+    records = w.G * nnz * (w.d + 1) * 4
+    assert records < a["build_states"] < 1.05 * records and records < a["gather_contract"] < 1.05 * records
+    ktimes = {"gather_contract": (3.3 * 4, 16), "build_states": (5.0 * 4, 16), "walk_merge": (1.3 * 4, 4)}
+    rep = bench.binding_report(w, N, nnz, nnz, ktimes, 4, {"hbm_gbs": 6500.0, "bf16_tflops": 1600.0}, {}, None, None, by_pairs=True)
+    for name, ms in (("build_states", 5.0), ("gather_contract", 3.3)):
+        assert rep[name]["binds"] == "hbm"
+        assert np.isclose(rep[name]["fraction_of_binding_peak"], a[name] / (ms * 1e-3) / 6500e9)
+
+
 def test_loglog_slope():
     xs = [2 ** k for k in range(14, 21)]
     assert np.isclose(bench.loglog_slope(xs, [3e-6 * x for x in xs]), 1.0)
