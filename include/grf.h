@@ -211,6 +211,8 @@ size_t grf_attn_workspace_bytes(int32_t G, int32_t R, int32_t m, int32_t d, int 
  * records), which the context keeps until it is destroyed.  A workspace of G * (4 (d + 1) nnz(Phi) + 512) bytes means that no such
  * scratch is taken.  Where the scratch cannot be had, fewer columns at a time lie in the workspace, with the same bits; if that is
  * too small for them as well, whole states serve the call (and differ by rounding), as they do for a call under stream capture.
+ * A captured call without den_out keeps its denominators in the context, which therefore has to outlive the graph; a later, larger
+ * call leaves that memory to it.
  * grf_ctx_use_tensor_cores(ctx, 0) and 3 keep to whole states from the start.
  * Asynchronous, except that a call may wait for the sizes of a sample that is still running (an fp32 call where its choice between
  * records and whole states needs them; never after grf_ctx_use_tensor_cores(ctx, 0) or 3), and that the first bf16 call

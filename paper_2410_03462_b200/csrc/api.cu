@@ -178,6 +178,30 @@ bool grf_capturing(cudaStream_t stream)
     return true;
 }
 
+// Room for denominators that nobody asked for.  A graph goes on naming the block that it was captured with: such a block stays until
+// the context goes, and a larger call takes another one, at least twice as large (so that there are few).  A captured call may
+// be the first that needs one: eager calls of its shape may have taken another route.
+int grf_den_scratch(grf_ctx* ctx, int64_t count, float** den)
+{
+    const size_t bytes = sizeof(float) * (size_t)count;
+    const bool captured = grf_capturing(ctx->stream);
+    grf_buf& b = ctx->den_scratch;
+    if (b.bytes < bytes && (captured || ctx->den_in_graphs)) {
+        constexpr int KEPT = sizeof(ctx->den_kept) / sizeof(ctx->den_kept[0]);
+        if (ctx->den_kept_count == KEPT) return GRF_ERR_NOMEM;
+        const grf_relaxed_capture relaxed;
+        grf_buf larger;
+        GRF_TRY(grf_buf_reserve(&larger, bytes > 2 * b.bytes ? bytes : 2 * b.bytes));
+        if (b.ptr) ctx->den_kept[ctx->den_kept_count++] = b;
+        b = larger;
+        ctx->den_in_graphs = false;
+    }
+    GRF_TRY(grf_buf_reserve(&b, bytes));
+    if (captured) ctx->den_in_graphs = true;
+    *den = (float*)b.ptr;
+    return GRF_OK;
+}
+
 void grf_built_by(grf_ctx* ctx, grf_features* feat)
 {
     if (grf_capturing(ctx->stream)) return;
@@ -238,6 +262,7 @@ extern "C" int grf_ctx_destroy(grf_ctx* ctx)
                        &ctx->t_cursor, &ctx->t_tmp, &ctx->den_scratch, &ctx->pair_scratch, &ctx->h_rowptr, &ctx->h_col, &ctx->h_w,
                        &ctx->h_q, &ctx->h_k, &ctx->h_v, &ctx->h_out, &ctx->h_ws};
     for (grf_buf* b : bufs) grf_buf_release(b);
+    for (grf_buf& b : ctx->den_kept) grf_buf_release(&b);
     if (ctx->h_feat) grf_features_free(ctx->h_feat);
     if (ctx->pinned) cudaFreeHost(ctx->pinned);
     if (ctx->error_word) cudaFree(ctx->error_word);
@@ -518,8 +543,8 @@ constexpr double PLAIN_BUILD_WORTH_NS = 25000.0;
 // Whether the states of a batch are used where they are made (attn_pairs.cu) instead of being stored and gathered.  Decided by
 // the features' sizes, the shape and the whole batch's G_all, so that parts of a batch give the bits of the whole.  The sizes
 // of a sample whose kernels may still be running are waited for only where its walks' expectation leaves the choice open.  A
-// call under stream capture keeps to whole states, whose only memory is the caller's: the pairs lie in buffers of the context
-// that a later call may replace while the graph still names them, and their places and launches follow the number of non-zeros,
+// call under stream capture keeps to whole states, which need the caller's memory and denominators (grf_den_scratch): the pairs lie in
+// buffers of the context that a later call may replace while the graph still names them, and their places and launches follow the number of non-zeros,
 // which a graph would keep while the kernels of whole states read the row pointers of whatever sample the object then holds.
 static int states_by_pairs(grf_ctx* ctx, const grf_features* feat, int32_t G_all, int32_t m, int32_t d, int dtype, const void* phiQ,
                            const void* phiK, const void* V, const void* out, bool* yes)

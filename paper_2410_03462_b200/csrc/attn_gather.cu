@@ -262,10 +262,7 @@ int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, double entries, int32_t G, i
         }
     }
     float* den = den_out;
-    if (!den) {
-        GRF_TRY(grf_buf_reserve(&ctx->den_scratch, sizeof(float) * (size_t)G * N));
-        den = (float*)ctx->den_scratch.ptr;
-    }
+    if (!den) GRF_TRY(grf_den_scratch(ctx, (int64_t)G * N, &den));
     {
         grf_launch_scope scope(ctx, 6);
         gather_denominators_kernel<T, M, D><<<dim3(blocks, G), GATHER_WARPS * 32, 0, ctx->stream>>>(

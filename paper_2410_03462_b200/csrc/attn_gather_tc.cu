@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(256) block_order_kernel(int32_t nblocks, int32
 }  // namespace
 
 // The coefficient table of the tensor-core gather (Phi's values per union entry and row), for a plan that is ready.
-static int build_plan_coefficients(grf_ctx* ctx, grf_features* feat)
+static int launch_plan_coefficients(grf_ctx* ctx, grf_features* feat, cudaStream_t stream)
 {
     grf_csr_dev& phi = feat->phi;
     const int32_t N = phi.rows, R = phi.cols;
@@ -537,14 +537,36 @@ static int build_plan_coefficients(grf_ctx* ctx, grf_features* feat)
     GRF_CUDA_TRY(cudaFuncSetAttribute(block_coef_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(words * 8)));
     {
         grf_launch_scope scope(ctx, 7);
-        block_coef_kernel<<<feat->plan_blocks, PLAN_THREADS, words * 8, ctx->stream>>>(
+        block_coef_kernel<<<feat->plan_blocks, PLAN_THREADS, words * 8, stream>>>(
             N, R, (const int32_t*)phi.rowptr.ptr, (const int32_t*)phi.col.ptr, (const float*)phi.val.ptr,
             (const int32_t*)feat->plan_off.ptr, (const int32_t*)feat->plan_cnt.ptr, (__nv_bfloat16*)feat->plan_coef.ptr);
     }
     GRF_CUDA_TRY(cudaGetLastError());
-    feat->plan_coef_ready = true;
-    grf_built_by(ctx, feat);
     return GRF_OK;
+}
+
+// A captured call may be the first that takes the tiles (eager calls of its shape may use the states where they are made).  As long
+// as Phi is what the plan was made of, the table is then built at once and beside the graph, whose replays would otherwise write
+// what other contexts read.  Values that a re-modulation has changed, perhaps one in this very graph, are the graph's to read:
+// the table is part of it, and whether it holds the present values is not known here.
+static int build_plan_coefficients(grf_ctx* ctx, grf_features* feat)
+{
+    if (!grf_capturing(ctx->stream)) {
+        GRF_TRY(launch_plan_coefficients(ctx, feat, ctx->stream));
+        feat->plan_coef_ready = true;
+        grf_built_by(ctx, feat);
+        return GRF_OK;
+    }
+    const grf_relaxed_capture relaxed;
+    if (feat->plan_coef.bytes < (size_t)feat->plan_entries * BQ * sizeof(__nv_bfloat16)) grf_buf_release(&feat->plan_coef);   // (of an earlier plan: nothing uses it any more)
+    if (!feat->plan_settled) return launch_plan_coefficients(ctx, feat, ctx->stream);
+    cudaStream_t beside;
+    GRF_CUDA_TRY(cudaStreamCreateWithFlags(&beside, cudaStreamNonBlocking));
+    int rc = launch_plan_coefficients(ctx, feat, beside);
+    if (cudaStreamSynchronize(beside) != cudaSuccess && rc == GRF_OK) rc = GRF_ERR_CUDA;
+    cudaStreamDestroy(beside);
+    feat->plan_coef_ready = rc == GRF_OK;
+    return rc;
 }
 
 int grf_build_block_plan(grf_ctx* ctx, grf_features* feat, bool with_coef)
@@ -582,7 +604,7 @@ int grf_build_block_plan(grf_ctx* ctx, grf_features* feat, bool with_coef)
     if (table_bytes > ((size_t)2 << 30)) return GRF_OK;           // too little sharing between neighbouring rows
     feat->plan_blocks = nblocks;
     feat->plan_entries = (int64_t)entries;
-    feat->plan_ready = true;
+    feat->plan_ready = feat->plan_settled = true;
     return with_coef ? build_plan_coefficients(ctx, feat) : GRF_OK;
 }
 
@@ -616,10 +638,7 @@ static int launch_tc(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t 
     GRF_CUDA_TRY(cudaFuncSetAttribute(gather_contract_tc_kernel<M, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)Sh::SMEM));
     float* den = den_out;
-    if (!den) {
-        GRF_TRY(grf_buf_reserve(&ctx->den_scratch, sizeof(float) * (size_t)G * N));
-        den = (float*)ctx->den_scratch.ptr;
-    }
+    if (!den) GRF_TRY(grf_den_scratch(ctx, (int64_t)G * N, &den));
     // (Running the denominators on a side stream beside the gather kernel was measured: both draw on the same
     // L2 bandwidth, the pair ends 0.1 ms earlier at most, and the rows then need a second pass to be divided.)
     {

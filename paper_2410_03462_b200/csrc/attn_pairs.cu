@@ -1061,10 +1061,7 @@ int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N,
     GRF_TRY(grf_buf_reserve(&ctx->t_cursor, sizeof(int32_t) * (3 * (size_t)counts_len + 8)));
     GRF_TRY(grf_reserve_buckets(ctx, nnz + 4));
     float* den = den_out;
-    if (!den && width < d) {
-        GRF_TRY(grf_buf_reserve(&ctx->den_scratch, sizeof(float) * (size_t)G * N));
-        den = (float*)ctx->den_scratch.ptr;
-    }
+    if (!den && width < d) GRF_TRY(grf_den_scratch(ctx, (int64_t)G * N, &den));
     int32_t *counts = (int32_t*)ctx->t_cursor.ptr, *long_count = counts + counts_len, *start = long_count + 4;
     int32_t* long_nodes = start + counts_len + 4;
     const int32_t long_limit = pair_long_limit(nnz + feat->psit.nnz, R);

@@ -45,7 +45,11 @@ struct grf_ctx {
     // transpose scratch
     grf_buf t_cursor;               // per column: count, then scatter cursor; number of long buckets; their list
     grf_buf t_tmp;                  // unordered buckets of (row, value)
-    grf_buf den_scratch;            // denominators of the tensor-core gather path when the caller wants none
+    // denominators of whole states when the caller wants none (grf_den_scratch); what graphs still name beside the present block,
+    // every one at most half as large as the next
+    grf_buf den_scratch, den_kept[40];
+    int den_kept_count = 0;
+    bool den_in_graphs = false;     // a captured call names the present block
     grf_buf pair_scratch;           // records of (row, node) pairs that the caller's workspace has no room for
     // host-buffer path
     grf_buf h_rowptr, h_col, h_w, h_q, h_k, h_v, h_out, h_ws;
@@ -155,6 +159,7 @@ struct grf_features {
     bool plan_ready = false;
     bool plan_coef_ready = false;   // the gather kernel's coefficient table exists for the present plan
     bool plan_stale = true;         // Phi changed since the plan was built: the gather kernel's launcher rebuilds it
+    bool plan_settled = false;      // Phi has not changed at all since then, and the device had finished with it
 };
 
 int grf_buf_reserve(grf_buf* b, size_t bytes);          // grows (contents not preserved)
@@ -163,6 +168,13 @@ int grf_csr_reserve(grf_csr_dev* m, int32_t rows, int32_t cols, int64_t nnz_cap)
 int grf_features_new(grf_features** out, int device);   // empty; `device` is current
 void grf_features_clear(grf_features* feat);
 bool grf_capturing(cudaStream_t stream);
+// For as long as it lives this thread may allocate while a stream is captured.
+struct grf_relaxed_capture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    grf_relaxed_capture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~grf_relaxed_capture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+int grf_den_scratch(grf_ctx* ctx, int64_t count, float** den);
 int grf_settle_sizes(grf_features* feat);
 // before nnz of a matrix is read: waits for the sample's sizes if they have not been read yet
 static inline int grf_features_sizes(const grf_features* feat)

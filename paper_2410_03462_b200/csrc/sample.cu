@@ -806,7 +806,7 @@ extern "C" int grf_remodulate(grf_ctx* ctx, grf_features* feat, int32_t max_len,
     GRF_CUDA_TRY(cudaGetLastError());
     // the structure is the same: the block plan's node lists and the mask's key lists stay; the gather kernel's
     // coefficient table and the mask's values hold the old values
-    feat->plan_coef_ready = false;
+    feat->plan_coef_ready = feat->plan_settled = false;
     grf_mask_values_stale(feat);
     return GRF_OK;
 }

@@ -37,6 +37,10 @@ thread_local cudaError_t last = cudaSuccess;
 // longest list
 int64_t report[9];
 
+void* captured = nullptr;                            // the stream that is captured
+cudaStreamCaptureMode capture_mode = cudaStreamCaptureModeGlobal;
+void* denominators = nullptr;                        // where the last launch of the plain gather's kernel writes them
+
 bool no_heap = false;                                // the library's operator new throws
 struct Own {                                         // ... while this file's own calls do not
     bool was = no_heap;
@@ -49,6 +53,9 @@ struct Event { int device; };
 
 cudaError_t fail(cudaError_t e) { last = e; return e; }
 cudaError_t bad() { ++errors; return fail(cudaErrorInvalidValue); }
+// calls that a thread may not make while a stream is captured, unless it says that it knows what it does
+bool unsafe() { return captured && capture_mode != cudaStreamCaptureModeRelaxed; }
+cudaError_t invalidates() { ++errors; return fail(cudaErrorStreamCaptureUnsupported); }
 
 int device_of(const void* p)
 {
@@ -83,7 +90,11 @@ void fake_reset()
     memset(report, 0, sizeof(report));
     log_.clear();
     current = 0;
+    captured = denominators = nullptr;
+    capture_mode = cudaStreamCaptureModeGlobal;
 }
+void fake_capture(void* stream) { captured = stream; }
+void* fake_denominators() { return denominators; }
 void fake_report(int which, int64_t value) { report[which] = value; }
 void fake_no_heap(int on) { no_heap = on != 0; }
 void fake_limit(int device, size_t bytes) { limit[device] = bytes; }      // an allocation beyond it fails
@@ -110,7 +121,14 @@ cudaError_t cudaSetDevice(int d)
     return cudaSuccess;
 }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 148; return cudaSuccess; }
-cudaError_t cudaDeviceSynchronize() { const Own own; log_.push_back("sync device " + std::to_string(current)); return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize()
+{
+    if (captured) return invalidates();
+    const Own own;
+    log_.push_back("sync device " + std::to_string(current));
+    return cudaSuccess;
+}
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode* m) { std::swap(*m, capture_mode); return cudaSuccess; }
 cudaError_t cudaGetLastError() { const cudaError_t e = last; last = cudaSuccess; return e; }
 
 // ---- memory
@@ -118,6 +136,7 @@ cudaError_t cudaMalloc(void** p, size_t bytes)
 {
     std::lock_guard<std::recursive_mutex> g(lock);
     const Own own;
+    if (unsafe()) return invalidates();
     if (bytes > limit[current] || live[current] + bytes > limit[current]) { ++refused; return fail(cudaErrorMemoryAllocation); }
     char* q = (char*)calloc(bytes ? bytes : 1, 1);
     if (!q) return fail(cudaErrorMemoryAllocation);
@@ -132,6 +151,7 @@ cudaError_t cudaFree(void* p)
     std::lock_guard<std::recursive_mutex> g(lock);
     const Own own;
     if (!p) return cudaSuccess;
+    if (unsafe()) return invalidates();
     auto it = blocks.find((char*)p);
     if (it == blocks.end()) return bad();
     live[it->second.device] -= it->second.bytes;
@@ -162,6 +182,7 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { const Own own
 cudaError_t cudaStreamDestroy(cudaStream_t s) { delete (Stream*)s; return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t s)
 {
+    if (captured && (s == captured || unsafe())) return invalidates();
     const Own own;
     char t[64];
     snprintf(t, sizeof t, "sync stream %p", (void*)s);
@@ -186,7 +207,11 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s)
     return cudaSuccess;
 }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { const Own own; log_.push_back("sync event"); return cudaSuccess; }
-cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* st) { *st = cudaStreamCaptureStatusNone; return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* st)
+{
+    *st = captured && s == captured ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 0.0f; return cudaSuccess; }
 
 // ---- kernels
@@ -205,7 +230,7 @@ cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void** args, size_t, cud
     if (s && ((Stream*)s)->device != current) return bad();
     const std::string& name = kernels()[f];
     auto is = [&](const char* what) { return name.find(what) != std::string::npos; };
-    log_.push_back("launch " + name);
+    log_.push_back("launch " + name + (captured && s != captured ? " beside" : ""));
     if (is("edge_records_kernel")) {
         if (*(int64_t*)args[1] > 0 && device_of(*(void**)args[6]) != current) ++errors;     // the room for the records
         if (report[4] > *(int64_t*)args[1]) **(int32_t**)args[9] = (int32_t)report[4];
@@ -216,6 +241,8 @@ cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void** args, size_t, cud
             if (j.job[x].out) j.job[x].out[n] = (int32_t)report[x > 1 ? 1 : x];
             if (j.job[x].host_total) *j.job[x].host_total = (int32_t)report[x];
         }
+    } else if (is("gather_denominators_kernel")) {
+        denominators = *(void**)args[7];
     } else if (is("block_plan_kernel")) {
         **(int32_t**)args[7] = (int32_t)report[5];
     } else if (is("mask_structure_kernel")) {

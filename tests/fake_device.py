@@ -30,8 +30,9 @@ class Fake:
 
     def __init__(self, so):
         self.lib = C.CDLL(so)
-        for name in ("fake_stream", "fake_live"):
-            getattr(self.lib, name).restype = C.c_void_p if name == "fake_stream" else C.c_size_t
+        for name in ("fake_stream", "fake_denominators", "fake_live"):
+            getattr(self.lib, name).restype = C.c_size_t if name == "fake_live" else C.c_void_p
+        self.lib.fake_capture.argtypes = [C.c_void_p]
         self.lib.fake_log.restype = C.c_char_p
         self.lib.fake_limit.argtypes = [C.c_int, C.c_size_t]
         self.lib.fake_report.argtypes = [C.c_int, C.c_int64]

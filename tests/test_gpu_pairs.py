@@ -179,7 +179,7 @@ def test_records_of_every_width_give_the_same_bits(m, d):
 
 def test_capture_keeps_to_whole_states():
     """The pairs' buffers belong to the context and may be replaced later: a captured call, also one on a sample whose sizes are
-    not known yet, uses the caller's memory only, and its replay gives the bits of whole states."""
+    not known yet, uses the caller's, and its replay gives the bits of whole states."""
     from paper_2410_03462_b200 import api, binding as B
     s = torch.cuda.Stream()
     with torch.cuda.stream(s):
@@ -213,6 +213,89 @@ def test_capture_keeps_to_whole_states():
         assert torch.equal(out, whole)
         # two fp32 evaluations of the same sums: the bound of fp32 outputs
         assert float((out - direct).norm() / direct.norm()) < 1e-5
+        del graph
+        feat.free()
+        ctx.close()
+
+
+@pytest.mark.parametrize("dtype,N,G,walks,length", [("fp32", 1500, 4, 32, 12), ("bf16", 20000, 8, 8, 6)])
+def test_capture_behind_calls_by_pairs_and_before_larger_ones(dtype, N, G, walks, length):
+    """On a fresh context, without room for denominators: the eager call uses the states where they are made, the captured one needs
+    memory (bf16: and the coefficients of the gather by tiles) that no call has asked for yet, and larger calls leave it to the graph."""
+    from paper_2410_03462_b200 import api, binding as B
+    m, d = 32, 64
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        ctx = api.Context(0)
+        w = configs.point_cloud_4096(N)
+        f = oracle.deconvolve(w.alpha).astype(np.float32)[:length + 1]
+        feat = api.sample(ctx, api.DeviceGraph(w.graph()), 3, walks, w.p_halt, length, f)
+        q, k, v = (t.cuda() for t in tensors.qkv(G, N, m, d, dtype, 4))
+        ws = torch.empty(B.grf_attn_workspace_bytes(G, N, m, d, B.dtype_code(v)), dtype=torch.uint8, device="cuda")
+        B.grf_ctx_use_tensor_cores(ctx.handle, 2)
+        direct, ran = kernel_classes(B, ctx, lambda: api.masked_linear_attn(ctx, feat, q, k, v, workspace=ws))
+        assert "scan" in ran, ran
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            out = api.masked_linear_attn(ctx, feat, q, k, v, workspace=ws)
+        B.grf_ctx_use_tensor_cores(ctx.handle, 0 if dtype == "fp32" else 3)
+        whole = api.masked_linear_attn(ctx, feat, q, k, v, workspace=ws)
+        q2, k2, v2 = (t.cuda() for t in tensors.qkv(2 * G, N, m, d, dtype, 5))
+        larger = api.masked_linear_attn(ctx, feat, q2, k2, v2)
+        other = api.Context(0)                          # blocks that have been given back would come to it
+        B.grf_ctx_use_tensor_cores(other.handle, 0 if dtype == "fp32" else 3)
+        beside = api.masked_linear_attn(other, feat, q2[:G], k2[:G], v2[:G])
+        for _ in range(2):
+            out.zero_()
+            graph.replay()
+            s.synchronize()
+            assert torch.equal(out, whole)
+        assert torch.equal(larger[:G], beside)
+        # both round S and the outputs to bf16 (2^-9 each); fp32: two evaluations of the same sums
+        assert float((out.float() - direct.float()).norm() / direct.float().norm()) < (1e-5 if dtype == "fp32" else 2.0 ** -7)
+        del graph
+        feat.free()
+        ctx.close()
+        other.close()
+
+
+def test_captured_remodulation_before_the_gather_by_tiles():
+    """The coefficients that the gather reads follow the values that the graph itself gives Phi, replay after replay, and eager calls
+    between replays see the features as they are."""
+    from paper_2410_03462_b200 import api, binding as B
+    N, m, d = 2048, 128, 64
+    w = configs.point_cloud_4096(N)
+    f = oracle.deconvolve(w.alpha).astype(np.float32)
+    new = (f * np.linspace(1.0, 1.3, f.size)).astype(np.float32)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        ctx = api.Context(0)
+        B.grf_ctx_use_tensor_cores(ctx.handle, 3)
+        B.grf_ctx_keep_walks(ctx.handle, True)
+        feat = api.sample(ctx, api.DeviceGraph(w.graph()), 7, w.n_walks, w.p_halt, w.max_len, f)
+        q, k, v = (t.cuda() for t in tensors.qkv(4, N, m, d, "bf16", 5))
+        ws = torch.empty(B.grf_attn_workspace_bytes(4, N, m, d, B.dtype_code(v)), dtype=torch.uint8, device="cuda")
+
+        def attend():
+            return api.masked_linear_attn(ctx, feat, q, k, v, workspace=ws)
+
+        def step(coefficients):
+            B.grf_remodulate(ctx.handle, feat.handle, w.max_len, coefficients, None)
+            return attend()
+
+        want, old = step(new).clone(), step(f).clone()
+        assert not torch.equal(want, old)
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            got = step(new)
+        assert torch.equal(attend(), old)               # nothing of the graph has run
+        for _ in range(2):
+            got.zero_()
+            graph.replay()
+            assert torch.equal(got, want) and torch.equal(attend(), want)
+            assert torch.equal(step(f), old)
         del graph
         feat.free()
         ctx.close()

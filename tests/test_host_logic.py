@@ -184,6 +184,60 @@ def test_fp32_calls_that_wait_for_a_running_sample(fake):
     assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
 
 
+def test_a_captured_call_without_room_for_denominators(fake):
+    """Eager calls of its shape use the states where they are made and need none for a caller who asks for none.  The captured call
+    finds its room all the same, and no later call takes that away from the graph."""
+    A, B = (fake.lib.fake_stream(0) for _ in range(2))
+    ctx, other = fake.context(0, A), fake.context(0, B)
+    N, m, d = 4096, 32, 64
+    fake.report(PHI=400_000, PSI=400_000, EDGES=40_000)
+    rc, feat = fake.sample(ctx, N)
+    assert rc == 0
+    fake.lib.fake_log_clear()
+    assert fake.linear(ctx, feat, 3, N, m, d, "fp32") == 0
+    assert fake.launched("pair_records") > 0 and fake.launched("gather_denominators") == 0
+    named, room = [], fake.lib.grf_attn_workspace_bytes(1, N, m, d, 0)
+    for G in (3, 3, 4):                           # the last graph's block is another one than that of the first two
+        fake.lib.fake_capture(A)
+        assert fake.linear(ctx, feat, G, N, m, d, "fp32", workspace=G * room) == 0
+        fake.lib.fake_capture(None)
+        named.append(fake.lib.fake_denominators())
+    assert fake.launched("pair_records") == 1 and fake.launched("gather_denominators") == 3
+    assert named[0] == named[1] != named[2] and fake.errors() == 0
+    assert fake.lib.grf_ctx_use_tensor_cores(ctx, 0) == 0 and fake.lib.grf_ctx_use_tensor_cores(other, 0) == 0
+    for c in (ctx, other):                        # larger and equal calls
+        for G in (3, 4, 6, 40):
+            assert fake.linear(c, feat, G, N, m, d, "fp32", workspace=G * room) == 0
+            if c is other or G == 40:
+                assert fake.lib.fake_denominators() not in named
+    assert fake.lib.grf_features_free(feat) == 0
+    assert fake.lib.grf_ctx_destroy(ctx) == 0 and fake.lib.grf_ctx_destroy(other) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
+def test_a_captured_call_without_the_gathers_coefficients(fake):
+    """Rows that share some of their nodes: eager calls use the states where they are made, a captured one gathers them by tiles.  The
+    coefficients are built once, beside the graph."""
+    A = fake.lib.fake_stream(0)
+    ctx = fake.context(0, A)
+    N, G, m, d = 20000, 8, 32, 64
+    fake.report(PHI=500_000, PSI=500_000, EDGES=160_000, PLAN=78_000)
+    rc, feat = fake.sample(ctx, N)
+    assert rc == 0 and fake.lib.grf_ctx_use_tensor_cores(ctx, 2) == 0
+    room = G * fake.lib.grf_attn_workspace_bytes(1, N, m, d, 1)
+    assert fake.linear(ctx, feat, G, N, m, d, "bf16", workspace=room) == 0
+    assert fake.launched("pair_records") > 0 and fake.launched("block_coef") == 0
+    fake.lib.fake_log_clear()
+    for _ in range(2):
+        fake.lib.fake_capture(A)
+        assert fake.linear(ctx, feat, G, N, m, d, "bf16", workspace=room) == 0
+        fake.lib.fake_capture(None)
+    assert fake.launched("gather_contract_tc") == 2 and fake.launched("pair_records") == 0
+    assert [x for x in fake.log() if "block_coef" in x and x.endswith("beside")] and fake.launched("block_coef") == 1
+    assert fake.lib.grf_features_free(feat) == 0 and fake.lib.grf_ctx_destroy(ctx) == 0
+    assert fake.errors() == 0 and fake.lib.fake_live(0) == 0
+
+
 def test_small_graphs_without_tensor_maps(fake):
     """The kernel for up to 512 nodes copies boxes through tensor maps, which the pretended driver does not make: the kernel that
     gathers rows takes the call."""
