@@ -70,3 +70,13 @@ def assert_attn_close(out_gpu: np.ndarray, ref: dict, tol: float, den_gpu: np.nd
 def qkv_for(w, N, G=None, seed=None):
     from workloads import configs
     return tensors.qkv(G or w.G, N, w.m, w.d, w.dtype, configs.QKV_SEED if seed is None else seed)
+
+
+def kernel_classes(B, ctx, call):
+    """The kernel classes that a call launched (the pairs alone regroup Phi: a scan)."""
+    B.grf_ctx_enable_timing(ctx.handle, True)
+    B.grf_ctx_kernel_times(ctx.handle)
+    out = call()
+    times = B.grf_ctx_kernel_times(ctx.handle)
+    B.grf_ctx_enable_timing(ctx.handle, False)
+    return out, {name for name, (_, launches) in times.items() if launches}

@@ -6,19 +6,10 @@ import torch
 
 import oracle
 from tests import helpers
+from tests.helpers import kernel_classes
 from workloads import configs, tensors
 
 pytestmark = pytest.mark.gpu
-
-
-def kernel_classes(B, ctx, call):
-    """The kernel classes that a call launched (the pairs alone regroup Phi: a scan)."""
-    B.grf_ctx_enable_timing(ctx.handle, True)
-    B.grf_ctx_kernel_times(ctx.handle)
-    out = call()
-    times = B.grf_ctx_kernel_times(ctx.handle)
-    B.grf_ctx_enable_timing(ctx.handle, False)
-    return out, {name for name, (_, launches) in times.items() if launches}
 
 
 def csr(rng, rows, cols, lengths):
