@@ -22,28 +22,9 @@
 #include <type_traits>
 
 #include "grf_internal.cuh"
+#include "packed.cuh"
 
 namespace {
-
-__device__ __forceinline__ uint64_t pair_of(float lo, float hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void split_pair(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ uint64_t fma_pair(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul_pair(uint64_t a, uint64_t b)
-{
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 
 // sixteen bytes of a row as packed pairs of fp32, and back
 template <typename T> struct Row;
@@ -51,8 +32,8 @@ template <> struct Row<float> {
     static constexpr int CH = 4;
     __device__ static __forceinline__ void widen(const uint4& x, uint64_t (&v)[2])
     {
-        v[0] = pair_of(__uint_as_float(x.x), __uint_as_float(x.y));
-        v[1] = pair_of(__uint_as_float(x.z), __uint_as_float(x.w));
+        v[0] = pack2(__uint_as_float(x.x), __uint_as_float(x.y));
+        v[1] = pack2(__uint_as_float(x.z), __uint_as_float(x.w));
     }
     __device__ static __forceinline__ void store(float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
 };
@@ -62,7 +43,7 @@ template <> struct Row<__nv_bfloat16> {
     {
         const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = pair_of(__uint_as_float(w[q] << 16), __uint_as_float(w[q] & 0xffff0000u));
+        for (int q = 0; q < 4; ++q) v[q] = pack2(__uint_as_float(w[q] << 16), __uint_as_float(w[q] & 0xffff0000u));
     }
     __device__ static __forceinline__ void store(__nv_bfloat16* p, const float (&v)[8])
     {
@@ -144,9 +125,9 @@ asym_attention_kernel(int32_t G, int32_t N, const int32_t* __restrict__ rowptr, 
                     uint64_t k[P], s2 = 0ull;
                     Row<T>::widen(x[u], k);
 #pragma unroll
-                    for (int e = 0; e < P; ++e) s2 = fma_pair(k[e], q[h][e], s2);
+                    for (int e = 0; e < P; ++e) s2 = fma2(k[e], q[h][e], s2);
                     float lo, hi;
-                    split_pair(s2, lo, hi);
+                    unpack2(s2, lo, hi);
                     part[i0 + u] = lo + hi;
                 }
             }
@@ -168,9 +149,9 @@ asym_attention_kernel(int32_t G, int32_t N, const int32_t* __restrict__ rowptr, 
                 const float new_max = fmaxf(run_max[h], bmax);
                 if (new_max > run_max[h]) {
                     const float rescale = __expf(run_max[h] - new_max);     // 0 on the first batch (run_max = -inf)
-                    const uint64_t r2 = pair_of(rescale, rescale);
+                    const uint64_t r2 = pack2(rescale, rescale);
 #pragma unroll
-                    for (int e = 0; e < P; ++e) acc[h][e] = mul_pair(acc[h][e], r2);
+                    for (int e = 0; e < P; ++e) acc[h][e] = mul2(acc[h][e], r2);
                     den[h] *= rescale;
                     run_max[h] = new_max;
                 }
@@ -198,9 +179,9 @@ asym_attention_kernel(int32_t G, int32_t N, const int32_t* __restrict__ rowptr, 
                 for (int u = 0; u < VB; ++u) {
                     uint64_t v[P];
                     Row<T>::widen(x[u], v);
-                    const uint64_t w2 = pair_of(wt[u], wt[u]);
+                    const uint64_t w2 = pack2(wt[u], wt[u]);
 #pragma unroll
-                    for (int e = 0; e < P; ++e) acc[h][e] = fma_pair(w2, v[e], acc[h][e]);
+                    for (int e = 0; e < P; ++e) acc[h][e] = fma2(w2, v[e], acc[h][e]);
                 }
             }
         };
@@ -220,7 +201,7 @@ asym_attention_kernel(int32_t G, int32_t N, const int32_t* __restrict__ rowptr, 
         const float inv = dn != 0.0f ? 1.0f / dn : 0.0f;
         float o[CH];
 #pragma unroll
-        for (int e = 0; e < P; ++e) split_pair(acc[h][e], o[2 * e], o[2 * e + 1]);
+        for (int e = 0; e < P; ++e) unpack2(acc[h][e], o[2 * e], o[2 * e + 1]);
 #pragma unroll
         for (int e = 0; e < CH; ++e) {
 #pragma unroll

@@ -297,19 +297,6 @@ gather_contract_tc_kernel(int32_t G, int32_t nblocks, int32_t N, int32_t R, cons
 
 constexpr int DEN_GH = 4;   // problems per warp of the denominators kernel: they share the row's indices and coefficients
 
-__device__ __forceinline__ uint64_t den_pack2(uint32_t lo, uint32_t hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
-    return r;
-}
-__device__ __forceinline__ uint64_t den_fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 template <int M, int D>
 __global__ void __launch_bounds__(256)
 row_denominators_kernel(int32_t G, int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
@@ -345,11 +332,11 @@ row_denominators_kernel(int32_t G, int32_t N, int32_t R, const int32_t* __restri
 #pragma unroll
                 for (int h = 0; h < DEN_GH; ++h)
                     w[h] = g0 + h < G ? __ldg(reinterpret_cast<const uint2*>(zl + (size_t)h * gstride)) : make_uint2(0u, 0u);
-                const uint64_t phi2 = den_pack2(__float_as_uint(phi), __float_as_uint(phi));
+                const uint64_t phi2 = pack2(phi, phi);
 #pragma unroll
                 for (int h = 0; h < DEN_GH; ++h) {
-                    z01[h] = den_fma2(phi2, den_pack2(w[h].x << 16, w[h].x & 0xffff0000u), z01[h]);
-                    z23[h] = den_fma2(phi2, den_pack2(w[h].y << 16, w[h].y & 0xffff0000u), z23[h]);
+                    z01[h] = fma2(phi2, pack2(w[h].x << 16, w[h].x & 0xffff0000u), z01[h]);
+                    z23[h] = fma2(phi2, pack2(w[h].y << 16, w[h].y & 0xffff0000u), z23[h]);
                 }
             }
         }

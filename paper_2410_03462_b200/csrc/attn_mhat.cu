@@ -784,11 +784,11 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         // two masked scores at a time; the denominator adds them in fp32, before the rounding to bf16
-                        const uint64_t p2 = mul_f32x2(pack_f32x2(sv[8 * h + 2 * e], sv[8 * h + 2 * e + 1]),
-                                                      pack_f32x2(mw[e] << 16, mw[e] & 0xffff0000u));
-                        den2[e & 1] = add_f32x2(den2[e & 1], p2);
+                        const uint64_t p2 = mul2(pack2(sv[8 * h + 2 * e], sv[8 * h + 2 * e + 1]),
+                                                      pack2(mw[e] << 16, mw[e] & 0xffff0000u));
+                        den2[e & 1] = add2(den2[e & 1], p2);
                         float p0, p1;
-                        unpack_f32x2(p2, p0, p1);
+                        unpack2(p2, p0, p1);
                         const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
                         pw[4 * h + e] = *reinterpret_cast<const uint32_t*>(&pb);
                     }
@@ -807,8 +807,8 @@ mhat_attention_kernel(int32_t G, int32_t nblocks, int32_t N, const int32_t* __re
         float den;
         {
             float d0, d1, d2, d3;
-            unpack_f32x2(den2[0], d0, d1);
-            unpack_f32x2(den2[1], d2, d3);
+            unpack2(den2[0], d0, d1);
+            unpack2(den2[1], d2, d3);
             den = (d0 + d1) + (d2 + d3);
         }
         if (grp == 1) {

@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "grf_internal.cuh"
+#include "packed.cuh"
 
 namespace {
 
@@ -112,32 +113,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 template <int ROW> __device__ __forceinline__ constexpr int piece_turn(int r)
 {
     return ROW >= 128 ? r & 7 : ROW == 64 ? (r >> 1) & 3 : (r >> 2) & 1;
-}
-
-// two fp32 in one 64-bit register: a packed multiply-add takes one issue slot for both (and as long as two in the pipe)
-__device__ __forceinline__ uint64_t pack2(float lo, float hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(uint64_t v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
-{
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
 }
 
 struct PairArgs {
@@ -698,9 +673,7 @@ __device__ __forceinline__ void pair_node_f32(const PairArgs& A, int32_t l, int3
         float part[SV + ZL];
 #pragma unroll
         for (int i = 0; i < SV; i += 2) {
-            const float2 x = unpack2(S[i / NB][i % NB / 2]);
-            part[i] = x.x;
-            part[i + 1] = x.y;
+            unpack2(S[i / NB][i % NB / 2], part[i], part[i + 1]);
         }
 #pragma unroll
         for (int y = 0; y < ZL; ++y) part[SV + y] = z[y];
@@ -747,7 +720,7 @@ __device__ __forceinline__ void pair_node_f32(const PairArgs& A, int32_t l, int3
             }
             float u[NB], w[NB / 2], x[NB / 4];
 #pragma unroll
-            for (int b = 0; b < NB / 2; ++b) { const float2 y = unpack2(t[b]); u[2 * b] = y.x; u[2 * b + 1] = y.y; }
+            for (int b = 0; b < NB / 2; ++b) unpack2(t[b], u[2 * b], u[2 * b + 1]);
 #pragma unroll
             for (int b = 0; b < NB / 2; ++b) {
                 const float give = (ag & 1) ? u[b] : u[NB / 2 + b], keep = (ag & 1) ? u[NB / 2 + b] : u[b];
