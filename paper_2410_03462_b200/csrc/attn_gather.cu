@@ -46,14 +46,18 @@ template <> struct Chunk<__nv_bfloat16> {
 
 constexpr int GATHER_WARPS = 4;
 
-// Denominator of row i of problem g, by a warp: M / 4 lanes per node on z_l in fp32.
+// Denominators: a warp per (problem, query), M / 4 lanes per node on z_l in fp32.  The gather may start once all CTAs here have.
 template <typename T, int M, int D>
-__device__ __forceinline__ float row_denominator(int32_t N, int32_t R, int32_t i, int32_t g, int lane, const int32_t* __restrict__ rowptr,
-                                                 const int32_t* __restrict__ col, const float* __restrict__ val,
-                                                 const T* __restrict__ phiQ, const unsigned char* __restrict__ states)
+__global__ void __launch_bounds__(GATHER_WARPS * 32)
+gather_denominators_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                           const float* __restrict__ val, const T* __restrict__ phiQ,
+                           const unsigned char* __restrict__ states, float* __restrict__ den)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int LPN = M / 4, NPS = 32 / LPN;          // lanes per node, nodes side by side
-    const int sub = lane / LPN, pl = lane % LPN;
+    const int lane = threadIdx.x & 31, sub = lane / LPN, pl = lane % LPN;
+    const int32_t i = blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5), g = blockIdx.y;
+    if (i >= N) return;
     const unsigned char* zbase = states + (size_t)g * grf_states_stride<T>(R, M, D) + grf_z_at<T>(true, 0, R, M, D) + (size_t)pl * 16;
     uint64_t z[2] = {0ull, 0ull};
     const int32_t beg = rowptr[i], end = rowptr[i + 1];
@@ -83,19 +87,6 @@ __device__ __forceinline__ float row_denominator(int32_t N, int32_t R, int32_t i
     for (int e = 0; e < 4; ++e) d = fmaf(Chunk<T>::get(qrow + e), a[e], d);
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
-    return d;
-}
-
-template <typename T, int M, int D>
-__global__ void __launch_bounds__(GATHER_WARPS * 32)
-gather_denominators_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                           const float* __restrict__ val, const T* __restrict__ phiQ,
-                           const unsigned char* __restrict__ states, float* __restrict__ den)
-{
-    const int lane = threadIdx.x & 31;
-    const int32_t i = blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5), g = blockIdx.y;
-    if (i >= N) return;
-    const float d = row_denominator<T, M, D>(N, R, i, g, lane, rowptr, col, val, phiQ, states);
     if (lane == 0) den[(size_t)g * N + i] = d;
 }
 
@@ -119,12 +110,11 @@ __device__ __forceinline__ uint4 load_tile(const unsigned char* p, uint64_t poli
     return x;
 }
 
-// DEN: every slice adds up the row's denominator itself, the first one writes it (few slices: see the launch).
-template <typename T, int M, int D, int CPL, bool DEN>
+template <typename T, int M, int D, int CPL>
 __global__ void __launch_bounds__(GATHER_WARPS * 32, CPL == 1 ? 16 : 6)
 gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                      const float* __restrict__ val, const T* __restrict__ phiQ, const unsigned char* __restrict__ states,
-                     T* __restrict__ out, float* __restrict__ den)
+                     T* __restrict__ out, const float* den)
 {
     using Sh = SliceShape<T, M, D, CPL>;
     constexpr int CH = Sh::CH, LPN = Sh::LPN, NPS = 32 / LPN, NB = Sh::NB, KC = Sh::KC, P = Chunk<T>::PAIRS;
@@ -133,11 +123,6 @@ gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, c
     const int32_t i = blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5);
     const int32_t slice = blockIdx.y, g = blockIdx.z;
     if (i >= N) return;
-    float dn = 0.0f;
-    if (DEN) {
-        dn = row_denominator<T, M, D>(N, R, i, g, lane, rowptr, col, val, phiQ, states);
-        if (den && slice == 0 && lane == 0) den[(size_t)g * N + i] = dn;
-    }
     const int b0 = slice * Sh::COLS + b;
     // this lane's first chunk; chunk y lies y * SB columns further on: LPN consecutive chunks per group of lanes
     const unsigned char* base = states + (size_t)g * grf_states_stride<T>(R, M, D) + grf_chunk_at<T>(true, 0, kc * CH, b0, M, D);
@@ -182,7 +167,8 @@ gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, c
     }
     // contract with phi(q): over this lane's rows a, then over the lanes along a and the nodes side by side
     const T* qrow = phiQ + ((size_t)g * N + i) * M;
-    if (!DEN) dn = den[(size_t)g * N + i];
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // for the denominators' kernel; all before it is complete
+    const float dn = __ldcg(den + (size_t)g * N + i);
     float s[NB];
     uint64_t qv[P];
     Chunk<T>::widen(__ldg(reinterpret_cast<const uint4*>(qrow + kc * CH)), qv);
@@ -215,89 +201,80 @@ gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, c
 // 76 ms, 128 bytes 1.75, 3.03, 10.3, 19.0, 40.6, 88.)
 constexpr size_t SLICE_L2_BYTES = (size_t)72 << 20;
 
-// Calls whose denominators are formed inside: at most so many rows, mean entries of a row, and look-ups of z_l over all slices.
-constexpr int64_t DEN_INSIDE_ROWS = 2048;
-template <typename T> constexpr double DEN_INSIDE_MEAN = sizeof(T) == 4 ? 48.0 : 96.0;
-template <typename T> constexpr double DEN_INSIDE_ENTRIES = (sizeof(T) == 4 ? 256.0 : 192.0) * 1024.0;
-
 template <typename T, int M, int D>
-int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, double entries, int32_t G, int32_t N, const void* phiQ, const void* states,
-              void* out, float* den_out)
+int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, const void* phiQ, const void* states, void* out, float* den_out)
 {
+    float* den = den_out;
+    if (!den) GRF_TRY(grf_den_scratch(ctx, (int64_t)G * N, &den));
     const int32_t* rp = (const int32_t*)phi.rowptr.ptr;
     const int32_t* cl = (const int32_t*)phi.col.ptr;
     const float* vl = (const float*)phi.val.ptr;
     const int blocks = grf_ceil_div(N, GATHER_WARPS);
-    auto launch = [&](auto cpl, auto with_den, float* den) {
-        using Sh = SliceShape<T, M, D, decltype(cpl)::value>;
-        grf_launch_scope scope(ctx, 5);
-        gather_sliced_kernel<T, M, D, decltype(cpl)::value, decltype(with_den)::value><<<dim3(blocks, Sh::SLICES, G), GATHER_WARPS * 32, 0, ctx->stream>>>(
-            N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, (T*)out, den);
-    };
-    const bool wide = (size_t)phi.cols * 2048 <= SLICE_L2_BYTES;
-    // Small calls form the denominators inside, once more for each of up to four slices: what a launch costs (3 us) is more than
-    // that while rows are short (a warp looks 32 entries up at a time) and few in all.  us measured, whole attention, separate /
-    // inside: fp32 lattice of 64 nodes, m = d = 16 23.0 / 18.0, of 400, 4 problems, m = 32, d = 64 (four slices) 35.1 / 29.6; grid
-    // of 1024 (37 entries a row), four slices, 0.15 M look-ups 49 / 47.5, 0.3 M 96 / 98; expanders (65 to 72 entries a row) of 300,
-    // 1200 and 2000 nodes, four slices 47.5 / 48.5, 86.0 / 91.5, 112.8 / 121.1, of 600, one slice, m = 8, d = 64 45.1 / 49.2;
-    // bf16, m = d = 64, four slices, cloud of 512, 0.1 M 60.0 / 57.2, expander of 900, 0.25 M 101.1 / 103.1, 2000, 0.58 M 173 / 185.
-    if constexpr (SliceShape<T, M, D, 4>::SLICES <= 4) {
-        if (wide && (int64_t)G * N <= DEN_INSIDE_ROWS && entries <= DEN_INSIDE_MEAN<T> * N &&
-            G * entries * SliceShape<T, M, D, 4>::SLICES <= DEN_INSIDE_ENTRIES<T>) {
-            launch(std::integral_constant<int, 4>(), std::true_type(), den_out);
-            return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
-        }
-    }
-    float* den = den_out;
-    if (!den) GRF_TRY(grf_den_scratch(ctx, (int64_t)G * N, &den));
     {
         grf_launch_scope scope(ctx, 6);
         gather_denominators_kernel<T, M, D><<<dim3(blocks, G), GATHER_WARPS * 32, 0, ctx->stream>>>(
             N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, den);
     }
-    if (wide) launch(std::integral_constant<int, 4>(), std::false_type(), den);
-    else launch(std::integral_constant<int, 1>(), std::false_type(), den);
-    return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
+    // Beside the denominators' kernel, which it waits for before it divides.  Whole attention, us, one behind the other / this: fp32
+    // lattice of 64 nodes, m = d = 16 17.4 / 13.5, of 400, 4 problems, m = 32, d = 64 33.4 / 27.8, expander of 2000 99.4 / 87.0;
+    // bf16, m = d = 64, cloud of 512 64.3 / 52.1; 120 calls of up to 8192 rows, of equal and of very different lengths, 1 / 0.81 of the
+    // time (geometric mean), none above 0.975.  (Denominators formed inside every slice of small calls: 0.89, but up to 1.15 where some rows
+    // are long.)
+    auto launch = [&](auto cpl) {
+        using Sh = SliceShape<T, M, D, decltype(cpl)::value>;
+        grf_launch_scope scope(ctx, 5);
+        cudaLaunchAttribute beside = {};
+        beside.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        beside.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t config = {};
+        config.gridDim = dim3(blocks, Sh::SLICES, G);
+        config.blockDim = dim3(GATHER_WARPS * 32);
+        config.stream = ctx->stream;
+        config.attrs = &beside;
+        config.numAttrs = 1;
+        GRF_CUDA_TRY(cudaLaunchKernelEx(&config, gather_sliced_kernel<T, M, D, decltype(cpl)::value>, N, phi.cols, rp, cl, vl,
+                                        (const T*)phiQ, (const unsigned char*)states, (T*)out, (const float*)den));
+        return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
+    };
+    if ((size_t)phi.cols * 2048 <= SLICE_L2_BYTES) return launch(std::integral_constant<int, 4>());
+    return launch(std::integral_constant<int, 1>());
 }
 
 template <typename T, int M>
-int launch_m(grf_ctx* ctx, const grf_csr_dev& phi, double entries, int32_t G, int32_t N, int32_t d,
+int launch_m(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t d,
              const void* phiQ, const void* states, void* out, float* den_out)
 {
     switch (d) {
-        case 8: return launch_md<T, M, 8>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
-        case 16: return launch_md<T, M, 16>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
-        case 32: return launch_md<T, M, 32>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
-        case 64: return launch_md<T, M, 64>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
-        case 128: return launch_md<T, M, 128>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
+        case 8: return launch_md<T, M, 8>(ctx, phi, G, N, phiQ, states, out, den_out);
+        case 16: return launch_md<T, M, 16>(ctx, phi, G, N, phiQ, states, out, den_out);
+        case 32: return launch_md<T, M, 32>(ctx, phi, G, N, phiQ, states, out, den_out);
+        case 64: return launch_md<T, M, 64>(ctx, phi, G, N, phiQ, states, out, den_out);
+        case 128: return launch_md<T, M, 128>(ctx, phi, G, N, phiQ, states, out, den_out);
         default: return GRF_ERR_INVALID;
     }
 }
 
 template <typename T>
-int launch_t(grf_ctx* ctx, const grf_csr_dev& phi, double entries, int32_t G, int32_t N, int32_t m, int32_t d,
+int launch_t(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t m, int32_t d,
              const void* phiQ, const void* states, void* out, float* den_out)
 {
     switch (m) {
-        case 8: return launch_m<T, 8>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
-        case 16: return launch_m<T, 16>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
-        case 32: return launch_m<T, 32>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
-        case 64: return launch_m<T, 64>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
-        case 128: return launch_m<T, 128>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
+        case 8: return launch_m<T, 8>(ctx, phi, G, N, d, phiQ, states, out, den_out);
+        case 16: return launch_m<T, 16>(ctx, phi, G, N, d, phiQ, states, out, den_out);
+        case 32: return launch_m<T, 32>(ctx, phi, G, N, d, phiQ, states, out, den_out);
+        case 64: return launch_m<T, 64>(ctx, phi, G, N, d, phiQ, states, out, den_out);
+        case 128: return launch_m<T, 128>(ctx, phi, G, N, d, phiQ, states, out, den_out);
         default: return GRF_ERR_INVALID;
     }
 }
 
 }  // namespace
 
-int grf_gather_contract_alu(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d,
+int grf_gather_contract_alu(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t m, int32_t d,
                             int dtype, const void* phiQ, const void* states, void* out, float* den_out)
 {
-    const grf_csr_dev& phi = feat->phi;
-    // (a running sample's sizes are not waited for: both ways to form the denominators give the same bits)
-    const double entries = feat->sizes_pending ? feat->expected_entries : (double)phi.nnz;
     if (G > 65535) return GRF_ERR_TOO_LARGE;
-    if (dtype == GRF_DTYPE_F32) return launch_t<float>(ctx, phi, entries, G, N, m, d, phiQ, states, out, den_out);
-    if (dtype == GRF_DTYPE_BF16) return launch_t<__nv_bfloat16>(ctx, phi, entries, G, N, m, d, phiQ, states, out, den_out);
+    if (dtype == GRF_DTYPE_F32) return launch_t<float>(ctx, phi, G, N, m, d, phiQ, states, out, den_out);
+    if (dtype == GRF_DTYPE_BF16) return launch_t<__nv_bfloat16>(ctx, phi, G, N, m, d, phiQ, states, out, den_out);
     return GRF_ERR_INVALID;
 }

@@ -100,36 +100,35 @@ def test_a_mask_that_the_caller_formed_changes_no_bit_of_the_main_call(N, G):
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
-@pytest.mark.parametrize("m,d", [(16, 16), (32, 64), (8, 64), (16, 128), (8, 8)])
-def test_denominators_inside_and_by_themselves_give_the_same_bits(m, d, dtype):
-    """While a sample runs only the expected number of its entries is known (several times the real one here), which makes
-    the plain gather form the denominators by themselves; afterwards it forms them inside: 48 (fp32) and 96 (bf16) entries a row
-    lie between."""
+@pytest.mark.parametrize("m,d", [(8, 8), (16, 16), (16, 128), (64, 64), (128, 32)])
+def test_plain_gather_beside_its_denominators(m, d, dtype):
+    """The gather starts while the denominators are formed: rows of 0, 1 and 4000 entries side by side, call after call with other
+    inputs into the same outputs, so that a denominator read too early is another call's."""
     from paper_2410_03462_b200 import api, binding as B
+    rng = np.random.default_rng(m + d)
+    N, R, G = 515, 4003, 3
+    lengths = [(0, 1, 4000, 33, 32)[i % 5] if i < 40 else 20 for i in range(N)]
+    rows = [np.sort(rng.choice(R, size=n, replace=False)) for n in lengths]
+    rp = np.concatenate([[0], np.cumsum([len(c) for c in rows])]).astype(np.int32)
+    c = np.concatenate(rows).astype(np.int32)
+    Phi = oracle.CSR(rp, c, rng.uniform(0.1, 1.0, c.size).astype(np.float32), None, (N, R))
+    cols = [np.sort(rng.choice(R, size=30, replace=False)) for _ in range(N)]
+    Psi = oracle.CSR(np.arange(0, 30 * N + 1, 30, dtype=np.int32), np.concatenate(cols).astype(np.int32),
+                     rng.uniform(0.1, 1.0, 30 * N).astype(np.float32), None, (N, R))
     ctx = api.Context(0)
     B.grf_ctx_use_tensor_cores(ctx.handle, 0)
-    w = configs.point_cloud_4096(200)
-    dg = api.DeviceGraph(w.graph())
-    f = oracle.deconvolve(w.alpha).astype(np.float32)
-    q, k, v = (t.cuda() for t in tensors.qkv(1, 200, m, d, dtype, 4))
-    ws = torch.empty(B.grf_attn_workspace_bytes(1, 200, m, d, B.dtype_code(v)), dtype=torch.uint8, device="cuda")
-    out, den = torch.empty_like(v), torch.empty((1, 200), device="cuda")
-    feat = api.sample(ctx, dg, 3, w.n_walks, w.p_halt, w.max_len, f)
-
-    def call():
-        B.grf_ctx_enable_timing(ctx.handle, True)
-        B.grf_masked_linear_attn(ctx.handle, feat.handle, 1, 200, m, d, B.dtype_code(v), q, k, v, out, den, ws, ws.numel())
-        launches = B.grf_ctx_kernel_times(ctx.handle)["row_denominators"][1]
-        B.grf_ctx_enable_timing(ctx.handle, False)
-        return launches, out.clone(), den.clone()
-
-    for _ in range(2):                      # the second sample leaves its sizes open
-        feat.handle = B.grf_sample(ctx.handle, dg.N, dg.rowptr, dg.col, dg.w, 3, 12 if dtype == "fp32" else 20, w.p_halt, w.max_len, f, None,
-                                     feat.handle)
-    running = call()
-    feat.shape(0)                           # reads the sizes
-    settled = call()
-    assert torch.equal(running[1], settled[1]) and torch.equal(running[2], settled[2])
-    assert (running[0], settled[0]) == (1, 0)       # both ways were taken
+    feat = api.features_from_csr(ctx, N, R, (Phi.rowptr, Phi.col, Phi.val), (Psi.rowptr, Psi.col, Psi.val))
+    inputs = [tensors.qkv(G, N, m, d, dtype, seed) for seed in (1, 2)]
+    ws = torch.empty(B.grf_attn_workspace_bytes(G, R, m, d, B.dtype_code(inputs[0][0])), dtype=torch.uint8, device="cuda")
+    out, den = torch.empty_like(inputs[0][2], device="cuda"), torch.empty((G, N), device="cuda")
+    got = []
+    for q, k, v in [[t.cuda() * (1 + 3 * x) for t in inputs[x]] for x in (0, 1, 0, 1)]:
+        B.grf_masked_linear_attn(ctx.handle, feat.handle, G, N, m, d, B.dtype_code(v), q, k, v, out, den, ws, ws.numel())
+        got.append((out.clone(), den.clone()))
+    for x in (0, 1):
+        assert torch.equal(got[x][0], got[x + 2][0]) and torch.equal(got[x][1], got[x + 2][1])
+        q, k, v = (tensors.widen(t * (1 + 3 * x)) for t in inputs[x])
+        ref = oracle.attn_sparse(q, k, v, Phi, oracle.transpose(Psi))
+        helpers.assert_attn_close(got[x][0].float().cpu().numpy(), ref, helpers.TOL[dtype], got[x][1].cpu().numpy(), min_ok=0.3)
     feat.free()
     ctx.close()
