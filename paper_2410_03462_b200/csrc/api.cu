@@ -583,7 +583,7 @@ static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int
     bool by_pairs = false;
     GRF_TRY(states_by_pairs(ctx, feat, G_all, m, d, dtype, phiQ, phiK, V, out, &by_pairs));
     if (by_pairs) {
-        const int rc = grf_pairs_attn(ctx, feat, G, N, m, d, dtype, phiQ, phiK, V, out, den_out, workspace, workspace_bytes);
+        const int rc = grf_pairs_attn(ctx, feat, G, G_all, N, m, d, dtype, phiQ, phiK, V, out, den_out, workspace, workspace_bytes);
         if (rc != GRF_ERR_NOMEM) return rc;                     // its scratch could not be had: whole states need none
     }
     const size_t per = ws_per_problem(feat->phi.cols, m, d, dtype);

@@ -134,21 +134,28 @@ struct PairArgs {
 // Long nodes.  A node is one warp's work, at 0.7 us a chunk (bf16) once the other warps of its SM have finished: a hub that all
 // 2^15 nodes of an expander visit kept its warp busy for 1.4 ms a problem where all other nodes take 0.14.  So a node with many
 // keys and queries is the work of a CTA, one with very many that of a cluster: the warps share its keys, add their parts of S and z
-// up in shared memory (a CTA's warps first, then the CTAs), and share its queries.  The shares depend on the node alone, so the
-// bits do not depend on the batch or the workspace.
+// up in shared memory (a CTA's warps first, then the CTAs), and share its queries.  The shares depend on the node and the
+// whole batch alone, so the bits do not depend on the parts that it is taken in or the workspace.
 // Whole attention, us, whole states / one warp a node / this: expanders with a hub, 4 problems, m = 32, d = 64, bf16: 2^15 nodes
 // 2099 / 6060 / 1224 (eight hubs 3272 / 6910 / 1302), 2^17 9380 / 26400 / 4697; 2 problems, 2^13 321 / 489 / 176; graph grown by
 // preferential attachment, 2^15 2254 / 1804 / 1416, 2^17 10146 / 6365 / 5092; fp32, 3 problems: 5003 1161 / 1435 / 349, 2^15 10813 /
 // 25422 / 2436.
 constexpr int PAIR_WARPS = 8, PAIR_CLUSTER = 8;
-// Keys and queries of a node beyond which it is long: 512 (a warp then needs as long as the launches of a small batch take), or
-// twice what a warp has to do on average where that is more.  Few nodes: warps go without work, so the average does not matter.
-// Beyond PAIR_HUGE it is a cluster's: that is 32 chunks for each warp of a CTA, at 1.2 us with eight warps on an SM.
-constexpr int PAIR_HUGE = 8192;
-int32_t pair_long_limit(int64_t entries, int32_t R)
+// Keys and queries of a node beyond which it is long, or a cluster's.  Sharing a node costs adding its parts up, so it pays where
+// the node would be what the call waits for: beyond an eighth, or a quarter, of what an SM has to do for the whole batch on average, within
+// 128 .. 512 and 2048 .. 8192; and never below twice what a warp has to do in a problem (few nodes in all: warps go without work, so
+// that does not matter).  us, whole attention, 512 and 8192 throughout / this / whole states, rows of 20 entries in columns N x^4, x uniform:
+// fp32, 1 problem, m = 32, d = 64, 8060 nodes 286 / 175 / 136, 20000 349 / 292 / 316, 2697, m = 64 134 / 101 / 93; 2 problems, 30000 716 /
+// 634 / 914, 4 problems 1168 / 1185 / 6744 (at 128 and 2048 1551); bf16, 8060, 1 problem 123 / 101 / 85, 3 problems, m = 16, d = 32 124 / 116 / 118.
+// (What is left to whole states on one problem: their gather finds the few states that most rows use in L1; the regrouping's
+// additions to one column's count come one after the other, 2.4 ns each.)
+struct PairLimits { int32_t longer, huge; };
+PairLimits pair_limits(int64_t entries, int32_t R, int32_t G_all)
 {
-    const int64_t twice = R < 512 ? 0 : 2 * entries / (R < 16384 ? R : 16384);
-    return (int32_t)(twice > 512 ? twice : 512);
+    const int64_t share = entries * G_all / 148, twice = (int64_t)R * G_all < 512 ? 0 : 2 * entries / (R < 16384 ? R : 16384);
+    auto within = [](int64_t x, int64_t least, int64_t most) { return x < least ? least : x > most ? most : x; };
+    const int64_t from = within(share / 8, 128, 512), longer = from > twice ? from : twice, huge = within(share / 4, 2048, 8192);
+    return {(int32_t)longer, (int32_t)(huge > longer ? huge : longer)};
 }
 
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -1012,7 +1019,7 @@ bool grf_pairs_shape(const grf_ctx* ctx, int32_t m, int32_t d)
 
 bool grf_pairs_fit(int64_t nnz, int dtype) { return nnz > 0 && pair_bytes(nnz, least_width(dtype)) <= PAIR_MOST; }
 
-int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, int dtype, const void* phiQ,
+int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t G_all, int32_t N, int32_t m, int32_t d, int dtype, const void* phiQ,
                    const void* phiK, const void* V, void* out, float* den_out, void* workspace, size_t workspace_bytes)
 {
     const bool bf16 = dtype == GRF_DTYPE_BF16;
@@ -1037,7 +1044,7 @@ int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N,
     if (!den && width < d) GRF_TRY(grf_den_scratch(ctx, (int64_t)G * N, &den));
     int32_t *counts = (int32_t*)ctx->t_cursor.ptr, *long_count = counts + counts_len, *start = long_count + 4;
     int32_t* long_nodes = start + counts_len + 4;
-    const int32_t long_limit = pair_long_limit(nnz + feat->psit.nnz, R);
+    const PairLimits limits = pair_limits(nnz + feat->psit.nnz, R, G_all);
     int32_t *slot = (int32_t*)ctx->t_tmp.ptr, *query = slot + ((nnz + 3) & ~(int64_t)3);
     GRF_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(int32_t) * ((size_t)counts_len + 2), ctx->stream));
     {
@@ -1056,7 +1063,7 @@ int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N,
         const int row_blocks = grf_ceil_div(N, 8);
         pair_slots_kernel<<<row_blocks + grf_ceil_div(R, 256), 256, 0, ctx->stream>>>(
             N, R, row_blocks, (const int32_t*)feat->phi.rowptr.ptr, (const int32_t*)feat->phi.col.ptr, start,
-            (const int32_t*)feat->psit.rowptr.ptr, long_limit, long_limit > PAIR_HUGE ? long_limit : PAIR_HUGE, slot, query, long_count, long_nodes);
+            (const int32_t*)feat->psit.rowptr.ptr, limits.longer, limits.huge, slot, query, long_count, long_nodes);
     }
 
     for (int64_t g0 = 0; g0 < G; g0 += chunk) {
@@ -1066,7 +1073,7 @@ int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N,
         A.t_rowptr = (const int32_t*)feat->psit.rowptr.ptr; A.t_col = (const int32_t*)feat->psit.col.ptr;
         A.t_val = (const float*)feat->psit.val.ptr;
         A.start = start; A.query = query;
-        A.long_limit = long_limit; A.long_count = long_count; A.long_nodes = long_nodes;
+        A.long_limit = limits.longer; A.long_count = long_count; A.long_nodes = long_nodes;
         A.phiQ = (const char*)phiQ + (size_t)g0 * N * m * es;
         A.phiK = (const char*)phiK + (size_t)g0 * N * m * es;
         A.V = (const char*)V + (size_t)g0 * N * d * es;

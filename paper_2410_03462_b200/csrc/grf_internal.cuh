@@ -243,7 +243,7 @@ bool grf_pairs_shape(const grf_ctx* ctx, int32_t m, int32_t d);
 double grf_pairs_ns(double nnz, int32_t G, int32_t m, int32_t d, int dtype, size_t workspace_per_problem);
 double grf_states_by_rows_ns(double nnz, int32_t nodes, int32_t G, int32_t m, int32_t d, int dtype);
 bool grf_pairs_fit(int64_t nnz, int dtype);
-int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d, int dtype, const void* phiQ,
+int grf_pairs_attn(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t G_all, int32_t N, int32_t m, int32_t d, int dtype, const void* phiQ,
                    const void* phiK, const void* V, void* out, float* den_out, void* workspace, size_t workspace_bytes);
 // attn_mhat.cu
 void grf_mask_invalidate(grf_features* feat);

@@ -54,15 +54,15 @@ def test_lists_of_every_length(m, d, dtype):
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
-@pytest.mark.parametrize("m,d", [(16, 32), (16, 64), (32, 32), (32, 64), (64, 32), (64, 64)])
-def test_hub_nodes(m, d, dtype):
-    """Nodes with more than 512 keys and queries are a CTA's work, with more than 8192 a cluster's: right below, at and above that, one side long only, nodes
-    without keys or with a few (warps without a share), hubs that every row visits."""
+@pytest.mark.parametrize("m,d,G", [(16, 32, 24), (16, 64, 24), (32, 32, 24), (32, 64, 24), (64, 32, 24), (64, 64, 24), (32, 64, 2), (64, 32, 2)])
+def test_hub_nodes(m, d, G, dtype):
+    """Nodes with more than 512 keys and queries (2 problems: 280 or so) are a CTA's work, with more than 8192 (2048) a cluster's: right
+    below, at and above that, one side long only, nodes without keys or with a few (warps without a share), hubs that every row visits."""
     from paper_2410_03462_b200 import api, binding as B
     ctx = api.Context(0)
     rng = np.random.default_rng(m + d)
-    N, R, G = 6001, 1500, 24
-    sides = [(256, 256), (256, 257), (1, 511), (511, 1), (1, 512), (512, 1), (0, 600), (600, 0), (7, 700), (700, 7), (6001, 6001),
+    N, R = 6001, 1500
+    sides = [(100, x) for x in range(170, 200)] + [(1024, 1024), (1024, 1025), (1000, 1047), (256, 256), (256, 257), (1, 511), (511, 1), (1, 512), (512, 1), (0, 600), (600, 0), (7, 700), (700, 7), (6001, 6001),
              (2049, 33), (31, 2051), (513, 6001), (4096, 4096), (4096, 4097), (6001, 2192)]
     sides += [(40, 30)] * (R - len(sides))
     order = rng.permutation(R)
