@@ -610,7 +610,7 @@ static int linear_attn(grf_ctx* ctx, const grf_features* feat, bool by_mask, int
         if (rs > 0) rs = grf_build_states(ctx, feat->psit, gc, N, m, d, dtype, k_ptr, v_ptr, workspace, !tc_gather);
         GRF_TRY(rs);
         if (tc_gather) GRF_TRY(grf_gather_contract_tc(ctx, feat, gc, N, m, d, q_ptr, workspace, o_ptr, den_ptr));
-        else GRF_TRY(grf_gather_contract_alu(ctx, feat->phi, gc, N, m, d, dtype, q_ptr, workspace, o_ptr, den_ptr));
+        else GRF_TRY(grf_gather_contract_alu(ctx, feat, gc, N, m, d, dtype, q_ptr, workspace, o_ptr, den_ptr));
     }
     return GRF_OK;
 }

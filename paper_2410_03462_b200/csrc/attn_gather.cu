@@ -46,18 +46,14 @@ template <> struct Chunk<__nv_bfloat16> {
 
 constexpr int GATHER_WARPS = 4;
 
-// Denominators: a warp per (problem, query), M / 4 lanes per node on z_l in fp32.  The gather may start once all CTAs here have.
+// Denominator of row i of problem g, by a warp: M / 4 lanes per node on z_l in fp32.
 template <typename T, int M, int D>
-__global__ void __launch_bounds__(GATHER_WARPS * 32)
-gather_denominators_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                           const float* __restrict__ val, const T* __restrict__ phiQ,
-                           const unsigned char* __restrict__ states, float* __restrict__ den)
+__device__ __forceinline__ float row_denominator(int32_t N, int32_t R, int32_t i, int32_t g, int lane, const int32_t* __restrict__ rowptr,
+                                                 const int32_t* __restrict__ col, const float* __restrict__ val,
+                                                 const T* __restrict__ phiQ, const unsigned char* __restrict__ states)
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int LPN = M / 4, NPS = 32 / LPN;          // lanes per node, nodes side by side
-    const int lane = threadIdx.x & 31, sub = lane / LPN, pl = lane % LPN;
-    const int32_t i = blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5), g = blockIdx.y;
-    if (i >= N) return;
+    const int sub = lane / LPN, pl = lane % LPN;
     const unsigned char* zbase = states + (size_t)g * grf_states_stride<T>(R, M, D) + grf_z_at<T>(true, 0, R, M, D) + (size_t)pl * 16;
     uint64_t z[2] = {0ull, 0ull};
     const int32_t beg = rowptr[i], end = rowptr[i + 1];
@@ -87,6 +83,21 @@ gather_denominators_kernel(int32_t N, int32_t R, const int32_t* __restrict__ row
     for (int e = 0; e < 4; ++e) d = fmaf(Chunk<T>::get(qrow + e), a[e], d);
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
+    return d;
+}
+
+// The gather may start once all CTAs here have.
+template <typename T, int M, int D>
+__global__ void __launch_bounds__(GATHER_WARPS * 32)
+gather_denominators_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                           const float* __restrict__ val, const T* __restrict__ phiQ,
+                           const unsigned char* __restrict__ states, float* __restrict__ den)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int lane = threadIdx.x & 31;
+    const int32_t i = blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5), g = blockIdx.y;
+    if (i >= N) return;
+    const float d = row_denominator<T, M, D>(N, R, i, g, lane, rowptr, col, val, phiQ, states);
     if (lane == 0) den[(size_t)g * N + i] = d;
 }
 
@@ -110,11 +121,12 @@ __device__ __forceinline__ uint4 load_tile(const unsigned char* p, uint64_t poli
     return x;
 }
 
-template <typename T, int M, int D, int CPL>
+// DEN: every slice adds up the row's denominator itself, the first one writes it where it is asked for (see the launch).
+template <typename T, int M, int D, int CPL, bool DEN>
 __global__ void __launch_bounds__(GATHER_WARPS * 32, CPL == 1 ? 16 : 6)
 gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                      const float* __restrict__ val, const T* __restrict__ phiQ, const unsigned char* __restrict__ states,
-                     T* __restrict__ out, const float* den)
+                     T* __restrict__ out, float* den)
 {
     using Sh = SliceShape<T, M, D, CPL>;
     constexpr int CH = Sh::CH, LPN = Sh::LPN, NPS = 32 / LPN, NB = Sh::NB, KC = Sh::KC, P = Chunk<T>::PAIRS;
@@ -123,6 +135,11 @@ gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, c
     const int32_t i = blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5);
     const int32_t slice = blockIdx.y, g = blockIdx.z;
     if (i >= N) return;
+    float dn = 0.0f;
+    if (DEN) {
+        dn = row_denominator<T, M, D>(N, R, i, g, lane, rowptr, col, val, phiQ, states);
+        if (den && slice == 0 && lane == 0) den[(size_t)g * N + i] = dn;
+    }
     const int b0 = slice * Sh::COLS + b;
     // this lane's first chunk; chunk y lies y * SB columns further on: LPN consecutive chunks per group of lanes
     const unsigned char* base = states + (size_t)g * grf_states_stride<T>(R, M, D) + grf_chunk_at<T>(true, 0, kc * CH, b0, M, D);
@@ -167,8 +184,10 @@ gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, c
     }
     // contract with phi(q): over this lane's rows a, then over the lanes along a and the nodes side by side
     const T* qrow = phiQ + ((size_t)g * N + i) * M;
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // for the denominators' kernel; all before it is complete
-    const float dn = __ldcg(den + (size_t)g * N + i);
+    if (!DEN) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");       // for the denominators' kernel; all before it is complete
+        dn = __ldcg(den + (size_t)g * N + i);
+    }
     float s[NB];
     uint64_t qv[P];
     Chunk<T>::widen(__ldg(reinterpret_cast<const uint4*>(qrow + kc * CH)), qv);
@@ -201,26 +220,26 @@ gather_sliced_kernel(int32_t N, int32_t R, const int32_t* __restrict__ rowptr, c
 // 76 ms, 128 bytes 1.75, 3.03, 10.3, 19.0, 40.6, 88.)
 constexpr size_t SLICE_L2_BYTES = (size_t)72 << 20;
 
+// Objects whose rows form their denominators inside: at most so many nodes (no row is longer), and entries a row on average.
+constexpr int32_t DEN_INSIDE_NODES = 128;
+constexpr int DEN_INSIDE_MEAN = 16;
+
 template <typename T, int M, int D>
-int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, const void* phiQ, const void* states, void* out, float* den_out)
+int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, double entries, int32_t G, int32_t N, const void* phiQ, const void* states,
+              void* out, float* den_out)
 {
-    float* den = den_out;
-    if (!den) GRF_TRY(grf_den_scratch(ctx, (int64_t)G * N, &den));
     const int32_t* rp = (const int32_t*)phi.rowptr.ptr;
     const int32_t* cl = (const int32_t*)phi.col.ptr;
     const float* vl = (const float*)phi.val.ptr;
     const int blocks = grf_ceil_div(N, GATHER_WARPS);
-    {
-        grf_launch_scope scope(ctx, 6);
-        gather_denominators_kernel<T, M, D><<<dim3(blocks, G), GATHER_WARPS * 32, 0, ctx->stream>>>(
-            N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, den);
-    }
-    // Beside the denominators' kernel, which it waits for before it divides.  Whole attention, us, one behind the other / this: fp32
-    // lattice of 64 nodes, m = d = 16 17.4 / 13.5, of 400, 4 problems, m = 32, d = 64 33.4 / 27.8, expander of 2000 99.4 / 87.0;
-    // bf16, m = d = 64, cloud of 512 64.3 / 52.1; 120 calls of up to 8192 rows, of equal and of very different lengths, 1 / 0.81 of the
-    // time (geometric mean), none above 0.975.  (Denominators formed inside every slice of small calls: 0.89, but up to 1.15 where some rows
-    // are long.)
-    auto launch = [&](auto cpl) {
+    // The gather starts beside the denominators' kernel, which it waits for before it divides.  Whole attention, us, one behind the other
+    // / this: fp32 lattice of 64 nodes, m = d = 16 17.4 / 13.5, of 400, 4 problems, m = 32, d = 64 33.4 / 27.8, expander of 2000 99.4 /
+    // 87.0; bf16, m = d = 64, cloud of 512 64.3 / 52.1; 120 calls of up to 8192 rows, of equal and of very different lengths, 1 / 0.81
+    // of the time (geometric mean), none above 0.975.
+    // The smallest objects' slices form the denominators themselves: the device needs 2 us more, but such calls wait for the host, for which
+    // a launch is 2 to 3 us.  us, call after call, inside / beside: 64 and 128 nodes, 10 entries a row 14.2 / 16.4 (sample and attention
+    // 38.7 / 41.8), 64 nodes, 32 entries, m = 32, d = 64, 4 problems 22.7 / 18.8, 192 nodes, 10 entries 17.7 / 17.4.
+    auto launch = [&](auto cpl, auto inside, float* den) {
         using Sh = SliceShape<T, M, D, decltype(cpl)::value>;
         grf_launch_scope scope(ctx, 5);
         cudaLaunchAttribute beside = {};
@@ -231,50 +250,64 @@ int launch_md(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, const 
         config.blockDim = dim3(GATHER_WARPS * 32);
         config.stream = ctx->stream;
         config.attrs = &beside;
-        config.numAttrs = 1;
-        GRF_CUDA_TRY(cudaLaunchKernelEx(&config, gather_sliced_kernel<T, M, D, decltype(cpl)::value>, N, phi.cols, rp, cl, vl,
-                                        (const T*)phiQ, (const unsigned char*)states, (T*)out, (const float*)den));
+        config.numAttrs = decltype(inside)::value ? 0 : 1;
+        GRF_CUDA_TRY(cudaLaunchKernelEx(&config, gather_sliced_kernel<T, M, D, decltype(cpl)::value, decltype(inside)::value>, N, phi.cols,
+                                        rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, (T*)out, den));
         return cudaGetLastError() == cudaSuccess ? GRF_OK : GRF_ERR_CUDA;
     };
-    if ((size_t)phi.cols * 2048 <= SLICE_L2_BYTES) return launch(std::integral_constant<int, 4>());
-    return launch(std::integral_constant<int, 1>());
+    if constexpr (SliceShape<T, M, D, 4>::SLICES <= 4) {
+        if (phi.cols <= DEN_INSIDE_NODES && (int64_t)G * N <= 2048 && entries <= (double)DEN_INSIDE_MEAN * N)
+            return launch(std::integral_constant<int, 4>(), std::true_type(), den_out);
+    }
+    float* den = den_out;
+    if (!den) GRF_TRY(grf_den_scratch(ctx, (int64_t)G * N, &den));
+    {
+        grf_launch_scope scope(ctx, 6);
+        gather_denominators_kernel<T, M, D><<<dim3(blocks, G), GATHER_WARPS * 32, 0, ctx->stream>>>(
+            N, phi.cols, rp, cl, vl, (const T*)phiQ, (const unsigned char*)states, den);
+    }
+    if ((size_t)phi.cols * 2048 <= SLICE_L2_BYTES) return launch(std::integral_constant<int, 4>(), std::false_type(), den);
+    return launch(std::integral_constant<int, 1>(), std::false_type(), den);
 }
 
 template <typename T, int M>
-int launch_m(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t d,
+int launch_m(grf_ctx* ctx, const grf_csr_dev& phi, double entries, int32_t G, int32_t N, int32_t d,
              const void* phiQ, const void* states, void* out, float* den_out)
 {
     switch (d) {
-        case 8: return launch_md<T, M, 8>(ctx, phi, G, N, phiQ, states, out, den_out);
-        case 16: return launch_md<T, M, 16>(ctx, phi, G, N, phiQ, states, out, den_out);
-        case 32: return launch_md<T, M, 32>(ctx, phi, G, N, phiQ, states, out, den_out);
-        case 64: return launch_md<T, M, 64>(ctx, phi, G, N, phiQ, states, out, den_out);
-        case 128: return launch_md<T, M, 128>(ctx, phi, G, N, phiQ, states, out, den_out);
+        case 8: return launch_md<T, M, 8>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
+        case 16: return launch_md<T, M, 16>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
+        case 32: return launch_md<T, M, 32>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
+        case 64: return launch_md<T, M, 64>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
+        case 128: return launch_md<T, M, 128>(ctx, phi, entries, G, N, phiQ, states, out, den_out);
         default: return GRF_ERR_INVALID;
     }
 }
 
 template <typename T>
-int launch_t(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t m, int32_t d,
+int launch_t(grf_ctx* ctx, const grf_csr_dev& phi, double entries, int32_t G, int32_t N, int32_t m, int32_t d,
              const void* phiQ, const void* states, void* out, float* den_out)
 {
     switch (m) {
-        case 8: return launch_m<T, 8>(ctx, phi, G, N, d, phiQ, states, out, den_out);
-        case 16: return launch_m<T, 16>(ctx, phi, G, N, d, phiQ, states, out, den_out);
-        case 32: return launch_m<T, 32>(ctx, phi, G, N, d, phiQ, states, out, den_out);
-        case 64: return launch_m<T, 64>(ctx, phi, G, N, d, phiQ, states, out, den_out);
-        case 128: return launch_m<T, 128>(ctx, phi, G, N, d, phiQ, states, out, den_out);
+        case 8: return launch_m<T, 8>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
+        case 16: return launch_m<T, 16>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
+        case 32: return launch_m<T, 32>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
+        case 64: return launch_m<T, 64>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
+        case 128: return launch_m<T, 128>(ctx, phi, entries, G, N, d, phiQ, states, out, den_out);
         default: return GRF_ERR_INVALID;
     }
 }
 
 }  // namespace
 
-int grf_gather_contract_alu(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t m, int32_t d,
+int grf_gather_contract_alu(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d,
                             int dtype, const void* phiQ, const void* states, void* out, float* den_out)
 {
+    const grf_csr_dev& phi = feat->phi;
+    // (a running sample's sizes are not waited for: both ways to form the denominators give the same bits)
+    const double entries = feat->sizes_pending ? feat->expected_entries : (double)phi.nnz;
     if (G > 65535) return GRF_ERR_TOO_LARGE;
-    if (dtype == GRF_DTYPE_F32) return launch_t<float>(ctx, phi, G, N, m, d, phiQ, states, out, den_out);
-    if (dtype == GRF_DTYPE_BF16) return launch_t<__nv_bfloat16>(ctx, phi, G, N, m, d, phiQ, states, out, den_out);
+    if (dtype == GRF_DTYPE_F32) return launch_t<float>(ctx, phi, entries, G, N, m, d, phiQ, states, out, den_out);
+    if (dtype == GRF_DTYPE_BF16) return launch_t<__nv_bfloat16>(ctx, phi, entries, G, N, m, d, phiQ, states, out, den_out);
     return GRF_ERR_INVALID;
 }

@@ -236,7 +236,7 @@ int grf_build_states(grf_ctx* ctx, const grf_csr_dev& psit, int32_t G, int32_t N
                      const void* phiK, const void* V, void* states, bool by_column);
 int grf_build_states_tc(grf_ctx* ctx, const grf_csr_dev& psit, int32_t G, int32_t N, int32_t m, int32_t d,
                         const void* phiK, const void* V, void* states, bool by_column);
-int grf_gather_contract_alu(grf_ctx* ctx, const grf_csr_dev& phi, int32_t G, int32_t N, int32_t m, int32_t d,
+int grf_gather_contract_alu(grf_ctx* ctx, const grf_features* feat, int32_t G, int32_t N, int32_t m, int32_t d,
                             int dtype, const void* phiQ, const void* states, void* out, float* den_out);
 // attn_pairs.cu
 bool grf_pairs_shape(const grf_ctx* ctx, int32_t m, int32_t d);

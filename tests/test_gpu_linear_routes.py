@@ -132,3 +132,38 @@ def test_plain_gather_beside_its_denominators(m, d, dtype):
         helpers.assert_attn_close(got[x][0].float().cpu().numpy(), ref, helpers.TOL[dtype], got[x][1].cpu().numpy(), min_ok=0.3)
     feat.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("m,d", [(16, 16), (32, 64), (8, 64), (16, 128), (8, 8)])
+def test_denominators_inside_and_by_themselves_give_the_same_bits(m, d, dtype):
+    """While a sample runs only the expected number of its entries is known (more than 16 a row here; the real one is smaller), which
+    makes the plain gather form the denominators by themselves; afterwards it forms them inside."""
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    B.grf_ctx_use_tensor_cores(ctx.handle, 0)
+    N = 125
+    w = configs.point_cloud_4096(N)
+    dg = api.DeviceGraph(w.graph())
+    f = oracle.deconvolve(w.alpha).astype(np.float32)
+    q, k, v = (t.cuda() for t in tensors.qkv(1, N, m, d, dtype, 4))
+    ws = torch.empty(B.grf_attn_workspace_bytes(1, N, m, d, B.dtype_code(v)), dtype=torch.uint8, device="cuda")
+    out, den = torch.empty_like(v), torch.empty((1, N), device="cuda")
+    feat = api.sample(ctx, dg, 3, w.n_walks, w.p_halt, w.max_len, f)
+
+    def call():
+        B.grf_ctx_enable_timing(ctx.handle, True)
+        B.grf_masked_linear_attn(ctx.handle, feat.handle, 1, N, m, d, B.dtype_code(v), q, k, v, out, den, ws, ws.numel())
+        launches = B.grf_ctx_kernel_times(ctx.handle)["row_denominators"][1]
+        B.grf_ctx_enable_timing(ctx.handle, False)
+        return launches, out.clone(), den.clone()
+
+    for _ in range(2):                      # the second sample leaves its sizes open
+        feat.handle = B.grf_sample(ctx.handle, dg.N, dg.rowptr, dg.col, dg.w, 3, 3, w.p_halt, w.max_len, f, None, feat.handle)
+    running = call()
+    assert feat.shape(0)[2] <= 16 * N       # reads the sizes
+    settled = call()
+    assert torch.equal(running[1], settled[1]) and torch.equal(running[2], settled[2])
+    assert (running[0], settled[0]) == (1, 0)       # both ways were taken
+    feat.free()
+    ctx.close()
