@@ -756,8 +756,8 @@ def run_suite(args):
     md.append(f"Sweep (8-regular graphs, sz route), log-log slope of time against N for N >= 2^14: sampler "
               f"{slopes['sampler']:.3f}, attention {slopes['attention']:.3f} (1.0 = linear time).")
     md.append("Attention time per token-head (ns): " + ", ".join(
-        f"2^{int(math.log2(r['config']['N']))}: {r['phases']['attn_ms'] * 1e6 / (r['config']['N'] * r['config']['heads']):.1f}"
-        for r in sweep) + " (the per-problem records outgrow L2, 126 MB, between 2^13 and 2^15).")
+        f"2^{int(math.log2(r['config']['N']))} by {r['config']['evaluated_by']}: "
+        f"{r['phases']['attn_ms'] * 1e6 / (r['config']['N'] * r['config']['heads']):.1f}" for r in sweep) + ".")
     fl = flops_figure(args)
     md.append("")
     md.append("Operation counts (Sec. 4 \"Time complexity\": 1-D grids, n = 4, p_halt = 0.5, m = d = 8, 10 seeds):")

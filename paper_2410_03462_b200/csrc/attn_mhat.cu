@@ -29,7 +29,7 @@ constexpr int BQ = GRF_PLAN_BLOCK;      // queries per block
 constexpr int KT = GRF_MASK_TILE;       // keys per tile
 
 // ---------------------------------------------------------------------------------------------------
-// Structure of the mask: one CTA per block of rows, everything that does not depend on values.
+// Structure of the mask: a cluster of CTAs per block of rows (see below), everything that does not depend on values.
 //   keys       the union of Psi^T's rows over the block's node list, marked in a bitmap (a bit is looked at before it is
 //              set: a block reaches each of its keys about thirty times), counted, and written as the block's key list,
 //              padded to whole tiles with the last key (whose mask values there are zeros); on graphs of GRF_MASK_SMALL nodes
