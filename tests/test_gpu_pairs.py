@@ -86,6 +86,32 @@ def test_hub_nodes(m, d, G, dtype):
     ctx.close()
 
 
+@pytest.mark.parametrize("R", [3, 1023, 1024, 5000])
+def test_entries_that_do_not_fill_a_cta(R):
+    """The regrouping counts 1024 entries at a time in shared memory, in places that columns of one hash compete for: numbers of entries
+    around 1024 and 4, columns that share places by chance and one that all rows use."""
+    from paper_2410_03462_b200 import api, binding as B
+    ctx = api.Context(0)
+    rng = np.random.default_rng(R)
+    for nnz_extra in (0, 1, 2, 3):
+        N, G, m, d = 8000, 12, 32, 64
+        lengths = np.full(N, min(R, 9))
+        lengths[:nnz_extra] += 1 if R > 9 else 0
+        Phi = csr(rng, N, R, lengths)
+        hub = Phi.rowptr[:-1]
+        Phi.col[hub] = 0                        # the first entry of every row (columns ascend)
+        Psi = csr(rng, N, R, [min(R, 9)] * N)
+        feat = api.features_from_csr(ctx, N, R, (Phi.rowptr, Phi.col, Phi.val), (Psi.rowptr, Psi.col, Psi.val))
+        q, k, v = tensors.qkv(G, N, m, d, "fp32", 5)
+        B.grf_ctx_use_tensor_cores(ctx.handle, 2)
+        (out, den), ran = kernel_classes(B, ctx, lambda: api.masked_linear_attn(ctx, feat, q.cuda(), k.cuda(), v.cuda(), want_den=True))
+        assert "scan" in ran, ran
+        ref = oracle.attn_sparse(tensors.widen(q[:1]), tensors.widen(k[:1]), tensors.widen(v[:1]), Phi, oracle.transpose(Psi))
+        helpers.assert_attn_close(out[:1].float().cpu().numpy(), ref, helpers.TOL["fp32"], den[:1].cpu().numpy(), min_ok=0.3)
+        feat.free()
+    ctx.close()
+
+
 def test_few_nodes_for_many_rows():
     """Three nodes: all of them long, whatever the average.  (bf16 takes whole states by tiles there.)"""
     from paper_2410_03462_b200 import api, binding as B
