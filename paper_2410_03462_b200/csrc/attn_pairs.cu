@@ -175,7 +175,8 @@ constexpr int PAIR_WARPS = 8, PAIR_CLUSTER = 8;
 // Keys and queries of a node beyond which it is long, or a cluster's.  Sharing a node costs adding its parts up, so it pays where
 // the node would be what the call waits for: beyond an eighth, or a quarter, of what an SM has to do for the whole batch on average, within
 // 128 .. 512 and 2048 .. 8192; and never below twice what a warp has to do in a problem (few nodes in all: warps go without work, so
-// that does not matter).  us, whole attention, 512 and 8192 throughout / this / whole states, rows of 20 entries in columns N x^4, x uniform:
+// that does not matter).  us, whole attention (with one addition per entry in the regrouping, 10 to 25 us more than now), 512 and 8192
+// throughout / this / whole states, rows of 20 entries in columns N x^4, x uniform:
 // fp32, 1 problem, m = 32, d = 64, 8060 nodes 286 / 175 / 136, 20000 349 / 292 / 316, 2697, m = 64 134 / 101 / 93; 2 problems, 30000 716 /
 // 634 / 914, 4 problems 1168 / 1185 / 6744 (at 128 and 2048 1551); bf16, 8060, 1 problem 123 / 101 / 85, 3 problems, m = 16, d = 32 124 / 116 / 118.
 // (What is left to whole states on one problem: their gather finds the few states that most rows use in L1.)
